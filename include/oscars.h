@@ -452,9 +452,11 @@ oscars_status oscars_gemm_bf16_nt(const void* A, const void* B, float* C, int32_
  * in global capture mode (where cudaMalloc is refused), hosts whose memory
  * pool owns the whole GPU, and loops that cannot pay for cudaMalloc/cudaFree,
  * which may synchronise the device.  The paper has no counterpart; this is a
- * deployment convenience.  It allocates nothing: its scratch (argument tables
- * and per-step loss partials) is a fixed 64 KB array inside the library that
- * every GPU which loads the library keeps until the process exits.
+ * deployment convenience.  It allocates nothing: one launch of the context's
+ * cluster kernel, or, where a mini-batch's exchange buffers do not fit that
+ * kernel's shared memory, of a single-CTA kernel whose scratch (argument
+ * tables and per-step loss partials) is a fixed 64 KB array inside the library
+ * that every GPU which loads the library keeps until the process exits.
  *
  * params_in / params_out: device, classes*dim + classes fp32 each, canonical
  * layout (W [classes][dim], then b [classes]); they may be the same buffer.

@@ -998,6 +998,7 @@ cudaError_t enqueue_round_softreg(oscars_ctx* c, cudaStream_t st) {
   a.cursor = c->cursor;
   a.loss_part = c->loss_part;
   a.max_tau = c->max_tau;
+  a.err = c->err;
   a.loss_out = c->loss_dev;   // the round's bookkeeping in the same launch
   a.cursor_next = c->cursor;
   ProfScope ps(c, "softreg_round", st);

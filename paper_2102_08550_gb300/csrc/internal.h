@@ -44,13 +44,18 @@ struct SoftregArgs {
   int64_t offW, offB;           // element offsets inside a slot
   int D, C, B;
   float lr;
-  const int32_t* tau;           // [W]
-  const float* const* shard_x;  // [W] device pointers
-  const int32_t* const* shard_y;
-  const int64_t* shard_n;       // [W]
-  const int64_t* cursor;        // [W]
-  float* loss_part;             // [W][max_tau]  (sum of per-sample losses of one step)
-  int max_tau;
+  const int32_t* tau = nullptr; // [W]; null (cluster kernel, one worker): the values below
+  const float* const* shard_x = nullptr;  // [W] device pointers
+  const int32_t* const* shard_y = nullptr;
+  const int64_t* shard_n = nullptr;       // [W]
+  const int64_t* cursor = nullptr;        // [W]
+  int tau1 = 0;                 // one worker's step count, shard and cursor
+  const float* x1 = nullptr;
+  const int32_t* y1 = nullptr;
+  int64_t n1 = 0, cursor1 = 0;
+  float* loss_part = nullptr;   // single-CTA kernel: [W][max_tau] (sum of per-sample losses of one step)
+  int max_tau = 0;
+  int* err = nullptr;           // cluster kernel: device error word of the bounded waits, or null
   // round bookkeeping in the same launch (null: not done): the worker's mean
   // loss over its steps, and its cursor advanced by tau * B (mod the shard)
   float* loss_out = nullptr;    // [W]
@@ -62,10 +67,9 @@ size_t softreg_smem_bytes(int D, int C, int B);
 // label and softmax: B must not exceed its block size
 constexpr int kSoftregMaxBatch = 512;
 // the same round with each worker on a cluster of 8 CTAs splitting the input
-// columns (B <= 256 and a column slice plus one batch slice in shared memory)
+// columns (a column slice of the weights, two of the mini-batch and the
+// exchange buffers in shared memory); writes loss_out, which must be set
 bool softreg_cluster_supported(int D, int C, int B);
-int softreg_cluster_cols(int D);
-size_t softreg_cluster_smem_bytes(int D, int C, int B);
 cudaError_t launch_softreg_cluster_round(const SoftregArgs& a, int W, cudaStream_t s);
 
 struct SoftregEvalArgs {

@@ -8,9 +8,10 @@
 // mini-batches of its shard with the weights resident in shared memory, and
 // writes the result to the worker's replica (the push).  Workers never
 // exchange data inside a round.  Two kernels: softreg_cluster_round_kernel
-// puts each worker on a cluster of 8 CTAs that split the input columns (the
-// round kernel of a context, batch <= 256); softreg_round_kernel puts each
-// worker on one CTA (larger batches, and the allocation-free entry point).
+// puts each worker on a cluster of 8 CTAs that split the input columns;
+// softreg_round_kernel puts each worker on one CTA (only where the cluster's
+// exchange buffers do not fit: about 400 rows and more with 17 or more
+// classes).
 //
 // Per step: logits z[b][c] = sum_k x[b][k] W[c][k] + bias[c] (warp-level dot
 // products), p = softmax(z), loss_b = logsumexp(z_b) - z_b[y_b],
@@ -221,213 +222,448 @@ __global__ void __launch_bounds__(kThreads) softreg_round_kernel(const __grid_co
 }
 
 // The same round with each worker on a cluster of kCl CTAs that split the
-// input columns: CTA r owns columns [r * Dc, min(D, (r + 1) * Dc)) (Dc a
-// multiple of 4) of W and of every mini-batch row, so a step's work and the
-// shared memory it needs are divided by kCl.  Per step each CTA computes the
-// partial logits of the whole mini-batch over its columns; after one cluster
-// barrier every CTA sums the kCl partials in rank order (distributed shared
-// memory loads) and adds the bias, and runs the softmax cross-entropy of every
-// row itself (identical arithmetic in every CTA); then it updates its own
-// columns of W, and its private copy of the bias (the same update in every
-// CTA; rank 0 writes it back).  The partial logits are double-buffered by
-// step parity: a CTA rewrites a buffer two steps later, after a barrier that
-// every reader of the buffer has passed.
+// input columns: CTA r owns columns [r * Dc, (r + 1) * Dc) (Dc a multiple of
+// 4) of W and of every mini-batch row, and the rows b = r (mod kCl) of the
+// mini-batch for the softmax.  The bias is column D of W against an input of
+// 1, so it needs no code of its own.
+//
+// A step is a serial chain, so it is built from short parallel phases and
+// one-way exchanges (no cluster barrier, no remote read):
+//  1. partial logits of the whole mini-batch over the CTA's columns: a warp
+//     takes 32 rows x CC classes, a lane 4 rows and every fourth 4-column
+//     chunk (4 rows x CC classes in registers); the four lanes of a row
+//     reduce-scatter with shuffles, so a lane ends up with one row; with few
+//     rows and classes the columns are also split over the warps (KS) and
+//     summed in shared memory;
+//  2. the partials of a row go to the CTA that owns it with asynchronous
+//     16-byte stores (st.async) that complete on the owner's mbarrier; the
+//     owner adds the kCl partials in rank order and one warp per row (lane =
+//     class) computes the softmax cross-entropy;
+//  3. the row of dz goes to every CTA the same way;
+//  4. weight update of the CTA's columns: a thread sums CC classes x 4
+//     columns over a part (1 / BS) of the rows; the parts meet in shared
+//     memory.
+// Four more warps fetch: the rows of step s + 1 come by cp.async into the
+// other of two buffers (and the labels of the CTA's rows beside them) while
+// step s runs; they meet the others once a step.  Classes are kept in rows of "slots": groups of CC classes,
+// each padded to CCp = a multiple of 4 slots (at most 32 slots in all).
+// Every index a thread needs in a step is worked out before the first one or
+// by shifts: an integer division by a run-time value costs as much as a
+// whole phase of the smaller shapes.  The products are bound by the values
+// that shared memory returns (32 a clock, broadcast or not; 128 FMAs a
+// clock), hence the register tiles: 4 x CC in phase 1, CC x 4 in phase 4.
+//
+// Buffer reuse: a CTA sends the partials of step s + 1 only after it has
+// received all of dz(s), which an owner sends after it has read its partials
+// of step s: so partials(s + 1) never overwrite partials(s) in use.  An owner
+// sends dz(s + 1) only after it has received every CTA's partials(s + 1),
+// which a CTA sends after its last read of dz(s).
+//
+// What bounds it: the latency of the chain (issue slots 39% busy, 0.3% of
+// DRAM).  Eight steps of one 784 x 10 worker, batch 32: 203 us on one CTA,
+// 35 us here (about 3.9 us a step).  A round of 333 x 26, batch 100, 12
+// workers, with its merge and pull: 373 us with the earlier cluster kernel
+// (cluster barrier, remote reads, one-thread row loops), 134 us now.
+// 784 x 10, 4 workers, at most 4 steps: 49 and 37 us.
 constexpr int kCl = 8;
-constexpr int kClThreads = 256;
-// columns per CTA: D / kCl rounded up to a multiple of 4
-__host__ __device__ inline int cluster_cols(int D) { return ((D + kCl - 1) / kCl + 3) / 4 * 4; }
-constexpr int kClPrefetch = 8;   // float4 items of the next step's rows held per thread
+constexpr int kClThreads = 512;
+constexpr int kClWarps = kClThreads / 32;
+constexpr int kClFetch = 128;                        // threads of the fetching warps
+constexpr int kClBlock = kClThreads + kClFetch;
+// columns per CTA: (D + the bias column) / kCl rounded up to a multiple of 4
+__host__ __device__ inline int cluster_cols(int D) { return ((D + 1 + kCl - 1) / kCl + 3) / 4 * 4; }
+constexpr int kSlots = 32;   // class slots of a row at most (one lane each)
 
-__global__ void __launch_bounds__(kClThreads) softreg_cluster_round_kernel(const __grid_constant__ SoftregArgs a) {
+// The shape-dependent split of a step (host: shared memory; device: offsets).
+struct ClPlan {
+  int Dc, Xld;     // columns per CTA, row stride of the mini-batch tile
+  int ncg, Zp;     // class groups, slots per row
+  int KS, BS;      // column splits (logits), row splits (update)
+  int R;           // mini-batch rows a CTA owns
+  // offsets in floats from the start of shared memory
+  int oX, oRed, oPin, oZ, oZst, oEnd;
+};
+// classes per group: the least padding of C with at most kSlots slots, then
+// the larger group (more products per value read)
+__host__ __device__ inline int cluster_cc(int C) {
+  const int cand[4] = {8, 7, 5, 4};
+  int best = 0, waste = 1 << 20;
+  for (int i = 0; i < 4; ++i) {
+    const int cc = cand[i], g = (C + cc - 1) / cc;
+    if (g * ((cc + 3) / 4 * 4) > kSlots) continue;
+    if (g * cc - C < waste) {
+      waste = g * cc - C;
+      best = cc;
+    }
+  }
+  return best;
+}
+__host__ __device__ inline ClPlan cluster_plan(int D, int C, int B, int CC) {
+  ClPlan p;
+  p.Dc = cluster_cols(D);
+  p.Xld = (p.Dc / 4) % 2 ? p.Dc : p.Dc + 4;   // an odd number of 16-byte chunks: lanes = rows hit distinct banks
+  p.ncg = (C + CC - 1) / CC;
+  p.Zp = p.ncg * ((CC + 3) / 4 * 4);
+  const int nrb = (B + 31) / 32, nk4 = p.Dc / 4;
+  p.KS = kClWarps / (nrb * p.ncg);
+  p.KS = p.KS > 4 ? 4 : p.KS;                          // more splits cost more to sum than they save
+  p.KS = p.KS > (nk4 + 3) / 4 ? (nk4 + 3) / 4 : p.KS;  // a warp's lanes take 4 chunks at a time
+  p.KS = p.KS < 1 ? 1 : p.KS;
+  p.BS = kClThreads / (nk4 * p.ncg);
+  p.BS = p.BS > 8 ? 8 : p.BS;
+  p.BS = p.BS > B / 8 ? B / 8 : p.BS;                  // at least 8 rows a split: the parts are summed too
+  p.BS = p.BS < 1 ? 1 : p.BS;
+  p.R = (B + kCl - 1) / kCl;
+  const int red1 = p.KS * B * (p.Zp + 4), red2 = p.BS > 1 ? p.BS * p.ncg * CC * p.Dc : 0;
+  p.oX = p.ncg * CC * p.Dc;
+  p.oRed = p.oX + 2 * B * p.Xld;
+  p.oPin = p.oRed + (red1 > red2 ? red1 : red2);
+  p.oZ = p.oPin + kCl * p.R * p.Zp;
+  p.oZst = p.oZ + B * p.Zp;
+  p.oEnd = p.oZst + kClWarps * kSlots;
+  return p;
+}
+// after the float area (16-byte aligned): loss sums, row offsets, barriers, labels
+__host__ __device__ inline size_t cluster_tail_bytes(int B) {
+  return sizeof(double) * (kClWarps + kCl) + sizeof(int64_t) * B + 2 * sizeof(uint64_t) +
+         sizeof(int) * 2 * ((B + kCl - 1) / kCl);
+}
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+__device__ __forceinline__ float warp_max(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ __forceinline__ void fma4(float4& acc, float s, const float4& v) {
+  acc.x = fmaf(s, v.x, acc.x);
+  acc.y = fmaf(s, v.y, acc.y);
+  acc.z = fmaf(s, v.z, acc.z);
+  acc.w = fmaf(s, v.w, acc.w);
+}
+__device__ __forceinline__ void add4(float4& a, const float4& v) {
+  a.x += v.x;
+  a.y += v.y;
+  a.z += v.z;
+  a.w += v.w;
+}
+__device__ __forceinline__ void st_dsmem_f64(double* local, uint32_t rank, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(local, rank)), "d"(v) : "memory");
+}
+
+template <int CC>
+__global__ void __launch_bounds__(kClBlock, 1) softreg_cluster_round_kernel(const __grid_constant__ SoftregArgs a) {
   extern __shared__ __align__(16) float sm[];
+  constexpr int CCp = (CC + 3) / 4 * 4;
   const int D = a.D, C = a.C, B = a.B;
-  const int Dc = cluster_cols(D);
+  const ClPlan p = cluster_plan(D, C, B, CC);
+  const int Dc = p.Dc, Xld = p.Xld, Zp = p.Zp, zq = p.Zp / 4, R = p.R, ncg = p.ncg;
   const int rank = static_cast<int>(cluster_ctarank());
   const int c0 = rank * Dc;
-  const int nc = D - c0 < Dc ? (D - c0 > 0 ? D - c0 : 0) : Dc;   // this CTA's columns (may be 0)
-  float* Wsm = sm;                       // [C][Dc]
-  float* bsm = Wsm + C * Dc;             // [32]
-  float* Xsm = bsm + 32;                 // [B][Dc]
-  float* Psm = Xsm + B * Dc;             // [2][B][C] partial logits, by step parity
-  float* Zsm = Psm + 2 * B * C;          // [B][C] logits, then dz
-  float* Lsm = Zsm + B * C;              // [B]
-  int* Ysm = reinterpret_cast<int*>(Lsm + B);   // [B]
-  int64_t* Rsm = reinterpret_cast<int64_t*>((reinterpret_cast<uintptr_t>(Ysm + B) + 7) & ~uintptr_t(7));  // [B]
+  const int nc = D - c0 < Dc ? (D - c0 > 0 ? D - c0 : 0) : Dc;   // this CTA's input columns (may be 0)
+  const bool has_bias = D >= c0 && D < c0 + Dc;                  // column D: the bias
+  const int nk4 = (nc + (has_bias ? 1 : 0) + 3) / 4;             // 4-column chunks in use
+  const int R_own = (B - rank + kCl - 1) / kCl;                  // rows rank, rank + kCl, ... (rank <= B + 7)
+  float* Wsm = sm;                       // [ncg * CC][Dc], classes past C and columns past the bias zero
+  float* Xsm = sm + p.oX;                // [2][B][Xld]
+  float* red = sm + p.oRed;              // [KS][B][Zp + 4] partial logits, or [BS][ncg * CC][Dc] gradients
+  float* Pin = sm + p.oPin;              // [kCl][R][Zp] partial logits of this CTA's rows
+  float* Zsm = sm + p.oZ;                // [B][Zp] dz
+  float* zst = sm + p.oZst;              // [warps][kSlots] a row of dz on its way out
+  double* lsum = reinterpret_cast<double*>(sm + p.oEnd);    // [warps]
+  double* lrank = lsum + kClWarps;                          // [kCl] (rank 0)
+  int64_t* Rsm = reinterpret_cast<int64_t*>(lrank + kCl);   // [B] rows of the step being fetched
+  uint64_t* pbar = reinterpret_cast<uint64_t*>(Rsm + B);    // the partials of this CTA's rows have landed
+  uint64_t* zbar = pbar + 1;                                // dz has landed
+  int* Ysm = reinterpret_cast<int*>(zbar + 1);              // [2][R] labels of this CTA's rows, by step parity
 
   const int w = blockIdx.y;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int tau = a.tau[w];
+  const bool table = a.tau != nullptr;   // per-worker tables, or one worker's values in the arguments
+  const int tau = table ? a.tau[w] : a.tau1;
   const float* gsrc = a.master + static_cast<int64_t>(a.global_slot) * a.slot_stride;
   float* dst = a.master_out + static_cast<int64_t>(w) * a.slot_stride;
-  const float* X = a.shard_x[w];
-  const int32_t* Y = a.shard_y[w];
-  const int64_t n = a.shard_n[w];
-  const int64_t cur = a.cursor[w];
+  const float* X = table ? a.shard_x[w] : a.x1;
+  const int32_t* Y = table ? a.shard_y[w] : a.y1;
+  const int64_t n = table ? a.shard_n[w] : a.n1;
+  const int64_t cur = table ? a.cursor[w] : a.cursor1;
   const float invB = 1.0f / static_cast<float>(B);
-  const int nc4 = nc / 4;
 
-  // pull: this CTA's columns of the global model, and the whole bias
-  for (int i = tid; i < C * Dc; i += kClThreads) {
-    const int c = i / Dc, k = i - c * Dc;
-    Wsm[i] = k < nc ? gsrc[a.offW + static_cast<int64_t>(c) * D + c0 + k] : 0.f;
+  if (tid == 0) {
+    mbar_init(pbar, 1);
+    mbar_init(zbar, 1);
+    fence_barrier_init();
   }
-  for (int i = tid; i < C; i += kClThreads) bsm[i] = gsrc[a.offB + i];
-
-  // rows of step s: (cursor + s*B + b) mod n; this CTA's columns of each,
-  // as 16-byte loads when every row's slice is 16-byte aligned
-  const bool vec = (D & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0 && B * nc4 <= kClPrefetch * kClThreads;
-  float4 pf[kClPrefetch];
-  auto row_offsets = [&](int s) {
-    if (tid < B) {
-      const int64_t r = (cur + static_cast<int64_t>(s) * B + tid) % n;
-      Rsm[tid] = r * D + c0;
-      Ysm[tid] = Y[r];
+  // this CTA's columns of each row, in units of 16-byte chunks when every
+  // slice is 16-byte aligned, else of single floats: a warp copies 32 / 2^ush
+  // rows at a time, 2^ush (the units rounded up, at most 32) lanes a row
+  const bool vec = (D & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+  const int units = vec ? nc / 4 : nc;
+  const int ush = units <= 1 ? 0 : 32 - __clz((units < 32 ? units : 32) - 1);
+  // rows of step s: (cursor + s*B + b) mod n, kept in Rsm and advanced by the
+  // fetching threads (each the rows b = its index, in steps of kClFetch)
+  const int64_t bmod = B % n;
+  auto fetch = [&](int s) {   // the fetching warps: rows and labels of step s
+    const int ft = tid - kClThreads;
+    for (int b = ft; b < B; b += kClFetch) {
+      int64_t r = s == 0 ? (cur + b) % n : Rsm[b] + bmod;
+      if (s > 0 && r >= n) r -= n;
+      Rsm[b] = r;
     }
-  };
-  auto fetch = [&]() {
-#pragma unroll
-    for (int j = 0; j < kClPrefetch; ++j) {
-      const int i = tid + j * kClThreads;
-      if (i < B * nc4) {
-        const int b = i / nc4, k4 = i - b * nc4;
-        pf[j] = *reinterpret_cast<const float4*>(X + Rsm[b] + 4 * k4);
-      }
+    bar_named(2, kClFetch);
+    float* buf = Xsm + (s & 1) * B * Xld;
+    const int fw = warp - kClWarps, u0 = lane & ((1 << ush) - 1);
+    for (int b = (fw << (5 - ush)) + (lane >> ush); b < B; b += kClFetch >> ush) {
+      const float* from = X + Rsm[b] * D + c0;
+      float* to = buf + b * Xld;
+      if (vec)
+        for (int u = u0; u < units; u += 1 << ush) cp_async16(to + 4 * u, from + 4 * u);
+      else
+        for (int u = u0; u < units; u += 1 << ush) cp_async4(to + u, from + u);
     }
+    for (int l = ft; l < R_own; l += kClFetch) Ysm[(s & 1) * R + l] = Y[Rsm[l * kCl + rank]];
+    cp_async_wait_all();
+    bar_named(2, kClFetch);   // Rsm is read by all before the next step's rows go in
   };
-  if (vec && tau > 0) {
-    row_offsets(0);
-    __syncthreads();
-    fetch();
+  const bool fetcher = tid >= kClThreads;
+  if (fetcher) {
+    if (tau > 0) fetch(0);
+  } else {
+  // columns past nc of both buffers are never copied: the bias input, then zeros
+  for (int i = tid; i < 2 * B; i += kClThreads)
+    for (int k = nc; k < 4 * nk4; ++k) Xsm[i * Xld + k] = k == nc && has_bias ? 1.f : 0.f;
+  // pull: this CTA's columns of the global model and, in its CTA, the bias
+  for (int c = warp; c < ncg * CC; c += kClWarps)
+    for (int k = lane; k < Dc; k += 32)
+      Wsm[c * Dc + k] = c >= C ? 0.f
+                        : k < nc ? gsrc[a.offW + static_cast<int64_t>(c) * D + c0 + k]
+                        : k == nc && has_bias ? gsrc[a.offB + c] : 0.f;
   }
+  // the class of this lane's slot, or -1
+  const int cls0 = lane / CCp * CC + lane % CCp;
+  const int cls = lane < Zp && lane % CCp < CC && cls0 < C ? cls0 : -1;
+  // phase 1: this warp's column split and class group, its first row block and their step
+  const int G = ncg * p.KS, l_ks = warp % p.KS, l_cg = warp / p.KS % ncg;
+  const int l_rb = warp / G, l_rbstep = kClWarps / G;   // warps past l_rbstep * G idle
+  const int nrb = l_rb < l_rbstep ? (B + 31) / 32 : 0;
+  const int l_k0 = l_ks * nk4 / p.KS + (lane >> 3), l_k1 = (l_ks + 1) * nk4 / p.KS;
+  // phase 2: thread = (row tid / 8, 16-byte chunk tid % 8 of its slots), rows kClThreads / 8 apart, so with one owner
+  const int s_q = tid & 7, s_b = tid >> 3, s_owner = s_b & (kCl - 1);
+  static_assert(kCl == 8 && kClThreads / 8 % kCl == 0, "the rows of a thread have one owner");
+  const uint32_t s_pin = cluster_addr(Pin + rank * R * Zp + 4 * s_q, s_owner), s_bar = cluster_addr(pbar, s_owner);
+  // phase 3: lane = (destination lane % 8, chunk lane / 8)
+  const int z_to = lane & 7, z_q = lane >> 3;
+  const uint32_t z_dst = cluster_addr(Zsm, z_to), z_bar = cluster_addr(zbar, z_to);
+  // phase 4: the first item (kv, cg, bs) of this thread, and its first sum (class, kv)
+  const int nkv = Dc / 4, items = nkv * ncg * p.BS;
+  const int u_kv = tid % nkv, u_cg = tid / nkv % ncg, u_bs = tid / (nkv * ncg);
+  const int u_b0 = u_bs * B / p.BS, u_b1 = (u_bs + 1) * B / p.BS;
+  const int r_c = tid / nkv, r_cstep = kClThreads / nkv, r_kvstep = kClThreads % nkv;
+  // the warp's row losses over all steps as an unevaluated sum of two floats
+  // (2Sum): fp64 adds are two lanes a clock here and sat in the chain
+  float loss_hi = 0.f, loss_lo = 0.f;
+  bool alive = true;     // no bounded wait has run out
+  cluster_sync();        // barriers initialised everywhere; the global model read before anyone can end
 
   for (int s = 0; s < tau; ++s) {
-    float* Pp = Psm + (s & 1) * B * C;
-    __syncthreads();   // the previous step is done with Xsm and Zsm
-    int yl = 0;
-    if (vec) {
-      if (tid < B) yl = Ysm[tid];
+    __syncthreads();   // X, the labels and W of this step are in place
+    if (fetcher) {
+      if (s + 1 < tau) fetch(s + 1);
+      continue;
+    }
+    const float* Xs = Xsm + (s & 1) * B * Xld;
+    if (tid == 0) {
+      if (R_own > 0) mbar_arrive_expect_tx(pbar, static_cast<uint32_t>(kCl * R_own * Zp * 4));
+      mbar_arrive_expect_tx(zbar, static_cast<uint32_t>(B * Zp * 4));
+    }
+    // 1. partial logits over this CTA's columns
+    for (int rb = l_rb; rb < nrb; rb += l_rbstep) {
+      // lane: rows rb * 32 + lane % 8 + 8 i, chunks l_k0 (= split's first + lane / 8), + 4, ...
+      const float* xr[4];
+      float acc[4][CC];
 #pragma unroll
-      for (int j = 0; j < kClPrefetch; ++j) {
-        const int i = tid + j * kClThreads;
-        if (i < B * nc4) {
-          const int b = i / nc4, k4 = i - b * nc4;
-          reinterpret_cast<float4*>(Xsm + b * Dc)[k4] = pf[j];
+      for (int i = 0; i < 4; ++i) {
+        const int row = rb * 32 + (lane & 7) + 8 * i;
+        xr[i] = Xs + (row < B ? row : B - 1) * Xld;
+#pragma unroll
+        for (int j = 0; j < CC; ++j) acc[i][j] = 0.f;
+      }
+      const float* wr = Wsm + l_cg * CC * Dc;
+#pragma unroll 1
+      for (int k4 = l_k0; k4 < l_k1; k4 += 4) {
+        float4 xv[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) xv[i] = *reinterpret_cast<const float4*>(xr[i] + 4 * k4);
+#pragma unroll
+        for (int j = 0; j < CC; ++j) {
+          const float4 wv = *reinterpret_cast<const float4*>(wr + j * Dc + 4 * k4);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            acc[i][j] = fmaf(xv[i].x, wv.x, acc[i][j]);
+            acc[i][j] = fmaf(xv[i].y, wv.y, acc[i][j]);
+            acc[i][j] = fmaf(xv[i].z, wv.z, acc[i][j]);
+            acc[i][j] = fmaf(xv[i].w, wv.w, acc[i][j]);
+          }
         }
       }
-      if (s + 1 < tau) row_offsets(s + 1);
-      __syncthreads();
-      if (s + 1 < tau) fetch();
-    } else {
-      row_offsets(s);
-      __syncthreads();
-      for (int i = tid; i < B * nc; i += kClThreads) {
-        const int b = i / nc, k = i - b * nc;
-        Xsm[b * Dc + k] = X[Rsm[b] + k];
-      }
-      if (tid < B) yl = Ysm[tid];
-      __syncthreads();
-    }
-    // partial logits over this CTA's columns: one thread per (row, class)
-    for (int q = tid; q < B * C; q += kClThreads) {
-      const int b = q / C, c = q - b * C;
-      const float* xr = Xsm + b * Dc;
-      const float* wr = Wsm + c * Dc;
-      float acc = 0.f;
-      if ((nc & 3) == 0) {
-        for (int k4 = 0; k4 < nc4; ++k4) {
-          const float4 xv = reinterpret_cast<const float4*>(xr)[k4];
-          const float4 wv = reinterpret_cast<const float4*>(wr)[k4];
-          acc = fmaf(xv.x, wv.x, acc);
-          acc = fmaf(xv.y, wv.y, acc);
-          acc = fmaf(xv.z, wv.z, acc);
-          acc = fmaf(xv.w, wv.w, acc);
-        }
-      } else {
-        for (int k = 0; k < nc; ++k) acc = fmaf(xr[k], wr[k], acc);
-      }
-      Pp[q] = acc;
-    }
-    cluster_sync();
-    // logits: the partials of every CTA in rank order, then the bias
-    for (int q = tid; q < B * C; q += kClThreads) {
-      float part[kCl];
+      // the four lanes of a row set: lane / 8 = i keeps row i
+      const bool up = lane & 16, odd = lane & 8;
+      float v[CCp];
 #pragma unroll
-      for (int r = 0; r < kCl; ++r) part[r] = ld_dsmem_f32(Pp + q, r);
-      float acc = 0.f;
+      for (int j = 0; j < CC; ++j) {
+        const float k0 = up ? acc[2][j] : acc[0][j], k1 = up ? acc[3][j] : acc[1][j];
+        const float g0 = up ? acc[0][j] : acc[2][j], g1 = up ? acc[1][j] : acc[3][j];
+        const float h0 = k0 + __shfl_xor_sync(0xffffffffu, g0, 16), h1 = k1 + __shfl_xor_sync(0xffffffffu, g1, 16);
+        v[j] = (odd ? h1 : h0) + __shfl_xor_sync(0xffffffffu, odd ? h0 : h1, 8);
+      }
 #pragma unroll
-      for (int r = 0; r < kCl; ++r) acc += part[r];
-      Zsm[q] = acc + bsm[q % C];
-    }
-    __syncthreads();
-    // softmax cross-entropy, one thread per row
-    if (tid < B) {
-      float* z = Zsm + tid * C;
-      float m = z[0];
-      for (int c = 1; c < C; ++c) m = fmaxf(m, z[c]);
-      const int y = yl;
-      float se = 0.f, so = 0.f;
-      for (int c = 0; c < C; ++c) {
-        const float e = expf(z[c] - m);
-        se += e;
-        if (c != y) so += e;
-      }
-      Lsm[tid] = m + logf(se) - z[y];
-      for (int c = 0; c < C; ++c) z[c] = (c == y ? -(so / se) : expf(z[c] - m) / se) * invB;
-    }
-    __syncthreads();
-    if (rank == 0 && warp == 0) {   // the step's loss: rows summed in order
-      if (lane == 0) {
-        float l = 0.f;
-        for (int b = 0; b < B; ++b) l += Lsm[b];
-        a.loss_part[static_cast<int64_t>(w) * a.max_tau + s] = l;
+      for (int j = CC; j < CCp; ++j) v[j] = 0.f;
+      const int row = rb * 32 + lane;   // lane % 8 + 8 (lane / 8)
+      if (row < B) {
+        float* o = red + (l_ks * B + row) * (Zp + 4) + l_cg * CCp;
+#pragma unroll
+        for (int q = 0; q < CCp / 4; ++q)
+          *reinterpret_cast<float4*>(o + 4 * q) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
       }
     }
-    // weight gradient and update of this CTA's columns: item = (class, 4 columns)
-    if ((nc & 3) == 0) {
-      for (int q = tid; q < C * nc4; q += kClThreads) {
-        const int c = q / nc4, k4 = q - c * nc4;
-        float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int b = 0; b < B; ++b) {
-          const float d = Zsm[b * C + c];
-          const float4 xv = reinterpret_cast<const float4*>(Xsm + b * Dc)[k4];
-          g.x = fmaf(d, xv.x, g.x);
-          g.y = fmaf(d, xv.y, g.y);
-          g.z = fmaf(d, xv.z, g.z);
-          g.w = fmaf(d, xv.w, g.w);
+    bar_named(1, kClThreads);
+    // 2. each row's partials to its owner
+    if (s_q < zq)
+      for (int b = s_b; b < B; b += kClThreads / 8) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int ks = 0; ks < p.KS; ++ks)
+          add4(v, *reinterpret_cast<const float4*>(red + (ks * B + b) * (Zp + 4) + 4 * s_q));
+        st_async_v4(s_pin + static_cast<uint32_t>((b >> 3) * Zp * 4),
+                    make_uint4(__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w)),
+                    s_bar);
+      }
+    // softmax cross-entropy of this CTA's rows, one warp per row, lane = slot
+    if (warp < R_own) {
+      if (alive) alive = mbar_wait(pbar, s & 1, a.err, kDevTimeoutFull);
+      for (int l = warp; l < R_own; l += kClWarps) {
+        float part[kCl];
+#pragma unroll
+        for (int q = 0; q < kCl; ++q) part[q] = lane < Zp ? Pin[(q * R + l) * Zp + lane] : 0.f;
+        float z = 0.f;
+#pragma unroll
+        for (int q = 0; q < kCl; ++q) z += part[q];
+        z = cls >= 0 ? z : -INFINITY;
+        const int y = Ysm[(s & 1) * R + l], ys = y / CC * CCp + y % CC;
+        const float m = warp_max(z);
+        // p_c = e_c / s; 1 - p_y = (sum_{c != y} e_c) / s (no cancellation)
+        const float e = cls >= 0 ? expf(z - m) : 0.f;
+        float se = e, so = lane == ys ? 0.f : e;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          se += __shfl_xor_sync(0xffffffffu, se, o);
+          so += __shfl_xor_sync(0xffffffffu, so, o);
         }
-        float4* wp = reinterpret_cast<float4*>(Wsm + c * Dc) + k4;
-        float4 wv = *wp;
-        wv.x = fmaf(-a.lr, g.x, wv.x);
-        wv.y = fmaf(-a.lr, g.y, wv.y);
-        wv.z = fmaf(-a.lr, g.z, wv.z);
-        wv.w = fmaf(-a.lr, g.w, wv.w);
-        *wp = wv;
-      }
-    } else {
-      for (int q = tid; q < C * nc; q += kClThreads) {
-        const int c = q / nc, k = q - c * nc;
-        float g = 0.f;
-        for (int b = 0; b < B; ++b) g = fmaf(Zsm[b * C + c], Xsm[b * Dc + k], g);
-        Wsm[c * Dc + k] = fmaf(-a.lr, g, Wsm[c * Dc + k]);
+        zst[warp * kSlots + lane] = (lane == ys ? -so : e) / se * invB;
+        __syncwarp();
+        // 3. the row of dz to every CTA
+        for (int q = z_q; q < zq; q += 4)
+          st_async_v4(z_dst + static_cast<uint32_t>(((l * kCl + rank) * Zp + 4 * q) * 4),
+                      *reinterpret_cast<const uint4*>(zst + warp * kSlots + 4 * q), z_bar);
+        const float zy = __shfl_sync(0xffffffffu, z, ys);
+        const float row = m + logf(se) - zy, t = loss_hi + row, bb = t - loss_hi;
+        loss_lo += (loss_hi - (t - bb)) + (row - bb);
+        loss_hi = t;
+        __syncwarp();
       }
     }
-    for (int c = tid; c < C; c += kClThreads) {   // the bias, the same update in every CTA
-      float g = 0.f;
-      for (int b = 0; b < B; ++b) g += Zsm[b * C + c];
-      bsm[c] = fmaf(-a.lr, g, bsm[c]);
+    if (alive) alive = mbar_wait(zbar, s & 1, a.err, kDevTimeoutFull);
+    // 4. weight gradient of this CTA's columns: item = (4 columns, CC classes, 1 / BS of the rows)
+    int kv = u_kv, cg = u_cg, bs = u_bs, b0 = u_b0, b1 = u_b1;
+    for (int i = tid; i < items;) {
+      if (kv < nk4) {
+        float4 g[CC];
+#pragma unroll
+        for (int j = 0; j < CC; ++j) g[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+        for (int b = b0; b < b1; ++b) {
+          const float4 xv = *reinterpret_cast<const float4*>(Xs + b * Xld + 4 * kv);
+          const float* zr = Zsm + b * Zp + cg * CCp;
+#pragma unroll
+          for (int q = 0; q < CC / 4; ++q) {
+            const float4 d = *reinterpret_cast<const float4*>(zr + 4 * q);
+            fma4(g[4 * q], d.x, xv);
+            fma4(g[4 * q + 1], d.y, xv);
+            fma4(g[4 * q + 2], d.z, xv);
+            fma4(g[4 * q + 3], d.w, xv);
+          }
+#pragma unroll
+          for (int j = CC / 4 * 4; j < CC; ++j) fma4(g[j], zr[j], xv);
+        }
+#pragma unroll
+        for (int j = 0; j < CC; ++j) {
+          const int c = cg * CC + j;
+          if (p.BS > 1) {
+            *reinterpret_cast<float4*>(red + (bs * ncg * CC + c) * Dc + 4 * kv) = g[j];
+          } else {
+            float4* wp = reinterpret_cast<float4*>(Wsm + c * Dc + 4 * kv);
+            float4 wv = *wp;
+            fma4(wv, -a.lr, g[j]);
+            *wp = wv;
+          }
+        }
+      }
+      i += kClThreads;
+      if (i >= items) break;   // nearly always: more items than threads need over 2000 columns
+      kv = i % nkv;
+      cg = i / nkv % ncg;
+      bs = i / (nkv * ncg);
+      b0 = bs * B / p.BS;
+      b1 = (bs + 1) * B / p.BS;
+    }
+    if (p.BS > 1) {
+      bar_named(1, kClThreads);
+      int c = r_c, kv4 = u_kv;
+      while (c < C) {
+        if (kv4 < nk4) {
+          float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+          for (int q = 0; q < p.BS; ++q) add4(g, *reinterpret_cast<const float4*>(red + (q * ncg * CC + c) * Dc + 4 * kv4));
+          float4* wp = reinterpret_cast<float4*>(Wsm + c * Dc + 4 * kv4);
+          float4 wv = *wp;
+          fma4(wv, -a.lr, g);
+          *wp = wv;
+        }
+        c += r_cstep;
+        kv4 += r_kvstep;
+        if (kv4 >= nkv) {
+          kv4 -= nkv;
+          ++c;
+        }
+      }
     }
   }
+  if (!fetcher && lane == 0) lsum[warp] = static_cast<double>(loss_hi) + static_cast<double>(loss_lo);
   __syncthreads();
-  // push: this CTA's columns into the replica (rank 0 also the bias)
-  for (int i = tid; i < C * nc; i += kClThreads) {
-    const int c = i / nc, k = i - c * nc;
-    dst[a.offW + static_cast<int64_t>(c) * D + c0 + k] = Wsm[c * Dc + k];
+  // push: this CTA's columns into the replica
+  for (int c = warp; c < C; c += kClBlock / 32)
+    for (int k = lane; k < nc; k += 32) dst[a.offW + static_cast<int64_t>(c) * D + c0 + k] = Wsm[c * Dc + k];
+  if (has_bias && tid < C) dst[a.offB + tid] = Wsm[tid * Dc + nc];
+  if (tid == 0) {
+    double t = 0.0;
+    for (int i = 0; i < kClWarps; ++i) t += lsum[i];
+    st_dsmem_f64(lrank + rank, 0, t);
   }
-  if (rank == 0)
-    for (int i = tid; i < C; i += kClThreads) dst[a.offB + i] = bsm[i];
-  cluster_sync();   // no CTA leaves while a peer may still read its partial logits
-  // every CTA has read the cursor; rank 0's thread 0 wrote the loss partials
-  if (rank == 0 && tid == 0) finish_worker(a, w, tau, cur, n);
+  cluster_sync();   // the loss sums are in; every CTA has read the cursor
+  if (rank == 0 && tid == 0) {
+    double t = 0.0;
+    for (int q = 0; q < kCl; ++q) t += lrank[q];
+    // without an error word (the allocation-free entry) a wait that ran out shows as a NaN loss
+    a.loss_out[w] = alive ? static_cast<float>(t / (static_cast<double>(B) * tau)) : NAN;
+    if (a.cursor_next) a.cursor_next[w] = (cur + static_cast<int64_t>(tau) * B) % n;
+  }
 }
 
 // Mean cross-entropy of the global model: one warp per sample, partial sums
@@ -477,26 +713,25 @@ cudaError_t launch_softreg_round(const SoftregArgs& a, int W, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-int softreg_cluster_cols(int D) { return cluster_cols(D); }
-
 size_t softreg_cluster_smem_bytes(int D, int C, int B) {
-  const size_t Dc = static_cast<size_t>(softreg_cluster_cols(D));
-  return sizeof(float) * (C * Dc + 32 + static_cast<size_t>(B) * Dc + 3 * static_cast<size_t>(B) * C + B) +
-         sizeof(int) * B + 8 + sizeof(int64_t) * B;
+  const ClPlan p = cluster_plan(D, C, B, cluster_cc(C));
+  return sizeof(float) * p.oEnd + cluster_tail_bytes(B);
 }
 
 bool softreg_cluster_supported(int D, int C, int B) {
-  return B <= kClThreads && softreg_cluster_smem_bytes(D, C, B) <= 200 * 1024;
+  return B <= kClThreads && softreg_cluster_smem_bytes(D, C, B) <= 220 * 1024;
 }
 
-cudaError_t launch_softreg_cluster_round(const SoftregArgs& a, int W, cudaStream_t s) {
+namespace {
+template <int CC>
+cudaError_t launch_cluster(const SoftregArgs& a, int W, cudaStream_t s) {
   const size_t smem = softreg_cluster_smem_bytes(a.D, a.C, a.B);
-  cudaError_t e = cudaFuncSetAttribute(softreg_cluster_round_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = cudaFuncSetAttribute(softreg_cluster_round_kernel<CC>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kCl, W, 1);
-  cfg.blockDim = dim3(kClThreads, 1, 1);
+  cfg.blockDim = dim3(kClBlock, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr;
@@ -506,7 +741,18 @@ cudaError_t launch_softreg_cluster_round(const SoftregArgs& a, int W, cudaStream
   attr.val.clusterDim.z = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, softreg_cluster_round_kernel, a);
+  return cudaLaunchKernelEx(&cfg, softreg_cluster_round_kernel<CC>, a);
+}
+}  // namespace
+
+cudaError_t launch_softreg_cluster_round(const SoftregArgs& a, int W, cudaStream_t s) {
+  switch (cluster_cc(a.C)) {
+    case 4: return launch_cluster<4>(a, W, s);
+    case 5: return launch_cluster<5>(a, W, s);
+    case 7: return launch_cluster<7>(a, W, s);
+    case 8: return launch_cluster<8>(a, W, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 cudaError_t launch_softreg_eval(const SoftregEvalArgs& a, int blocks, cudaStream_t s) {
