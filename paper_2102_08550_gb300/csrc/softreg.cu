@@ -266,10 +266,15 @@ __global__ void __launch_bounds__(kThreads) softreg_round_kernel(const __grid_co
 // (cluster barrier, remote reads, one-thread row loops), 134 us now.
 // 784 x 10, 4 workers, at most 4 steps: 49 and 37 us.
 constexpr int kCl = 8;
-constexpr int kClThreads = 512;
-constexpr int kClWarps = kClThreads / 32;
-constexpr int kClFetch = 128;                        // threads of the fetching warps
-constexpr int kClBlock = kClThreads + kClFetch;
+// A CTA has NT computing threads and NT / 4 fetching ones.  NT = 512 fills the
+// SM's registers, so 17 to 19 workers run at once; a step of few products
+// leaves most of its warps without work, and NT = 128 lets four CTAs share an
+// SM.  The line: 16 x 2, batch 1, 32 workers, a round: 50 us with the earlier
+// kernel, 62 with NT = 512, 40 with 128; 333 x 26, batch
+// 100, 24 workers: 140 us with 512, 392 with the earlier 256-thread kernel.
+constexpr int kClThreads = 512, kClSmall = 128;
+constexpr int kClSmallWork = 4096;   // products of a step in a CTA, at most, for kClSmall
+constexpr int kClMaxWarps = kClThreads / 32;
 // columns per CTA: (D + the bias column) / kCl rounded up to a multiple of 4
 __host__ __device__ inline int cluster_cols(int D) { return ((D + 1 + kCl - 1) / kCl + 3) / 4 * 4; }
 constexpr int kSlots = 32;   // class slots of a row at most (one lane each)
@@ -298,18 +303,18 @@ __host__ __device__ inline int cluster_cc(int C) {
   }
   return best;
 }
-__host__ __device__ inline ClPlan cluster_plan(int D, int C, int B, int CC) {
+__host__ __device__ inline ClPlan cluster_plan(int D, int C, int B, int CC, int NT) {
   ClPlan p;
   p.Dc = cluster_cols(D);
   p.Xld = (p.Dc / 4) % 2 ? p.Dc : p.Dc + 4;   // an odd number of 16-byte chunks: lanes = rows hit distinct banks
   p.ncg = (C + CC - 1) / CC;
   p.Zp = p.ncg * ((CC + 3) / 4 * 4);
   const int nrb = (B + 31) / 32, nk4 = p.Dc / 4;
-  p.KS = kClWarps / (nrb * p.ncg);
+  p.KS = NT / 32 / (nrb * p.ncg);
   p.KS = p.KS > 4 ? 4 : p.KS;                          // more splits cost more to sum than they save
   p.KS = p.KS > (nk4 + 3) / 4 ? (nk4 + 3) / 4 : p.KS;  // a warp's lanes take 4 chunks at a time
   p.KS = p.KS < 1 ? 1 : p.KS;
-  p.BS = kClThreads / (nk4 * p.ncg);
+  p.BS = NT / (nk4 * p.ncg);
   p.BS = p.BS > 8 ? 8 : p.BS;
   p.BS = p.BS > B / 8 ? B / 8 : p.BS;                  // at least 8 rows a split: the parts are summed too
   p.BS = p.BS < 1 ? 1 : p.BS;
@@ -320,12 +325,12 @@ __host__ __device__ inline ClPlan cluster_plan(int D, int C, int B, int CC) {
   p.oPin = p.oRed + (red1 > red2 ? red1 : red2);
   p.oZ = p.oPin + kCl * p.R * p.Zp;
   p.oZst = p.oZ + B * p.Zp;
-  p.oEnd = p.oZst + kClWarps * kSlots;
+  p.oEnd = p.oZst + NT / 32 * kSlots;
   return p;
 }
 // after the float area (16-byte aligned): loss sums, row offsets, barriers, labels
 __host__ __device__ inline size_t cluster_tail_bytes(int B) {
-  return sizeof(double) * (kClWarps + kCl) + sizeof(int64_t) * B + 2 * sizeof(uint64_t) +
+  return sizeof(double) * (kClMaxWarps + kCl) + sizeof(int64_t) * B + 2 * sizeof(uint64_t) +
          sizeof(int) * 2 * ((B + kCl - 1) / kCl);
 }
 
@@ -358,12 +363,13 @@ __device__ __forceinline__ void st_dsmem_f64(double* local, uint32_t rank, doubl
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(local, rank)), "d"(v) : "memory");
 }
 
-template <int CC>
-__global__ void __launch_bounds__(kClBlock, 1) softreg_cluster_round_kernel(const __grid_constant__ SoftregArgs a) {
+template <int CC, int NT>
+__global__ void __launch_bounds__(NT + NT / 4, 1) softreg_cluster_round_kernel(const __grid_constant__ SoftregArgs a) {
+  constexpr int NW = NT / 32, NF = NT / 4;   // computing warps, fetching threads
   extern __shared__ __align__(16) float sm[];
   constexpr int CCp = (CC + 3) / 4 * 4;
   const int D = a.D, C = a.C, B = a.B;
-  const ClPlan p = cluster_plan(D, C, B, CC);
+  const ClPlan p = cluster_plan(D, C, B, CC, NT);
   const int Dc = p.Dc, Xld = p.Xld, Zp = p.Zp, zq = p.Zp / 4, R = p.R, ncg = p.ncg;
   const int rank = static_cast<int>(cluster_ctarank());
   const int c0 = rank * Dc;
@@ -378,7 +384,7 @@ __global__ void __launch_bounds__(kClBlock, 1) softreg_cluster_round_kernel(cons
   float* Zsm = sm + p.oZ;                // [B][Zp] dz
   float* zst = sm + p.oZst;              // [warps][kSlots] a row of dz on its way out
   double* lsum = reinterpret_cast<double*>(sm + p.oEnd);    // [warps]
-  double* lrank = lsum + kClWarps;                          // [kCl] (rank 0)
+  double* lrank = lsum + kClMaxWarps;                          // [kCl] (rank 0)
   int64_t* Rsm = reinterpret_cast<int64_t*>(lrank + kCl);   // [B] rows of the step being fetched
   uint64_t* pbar = reinterpret_cast<uint64_t*>(Rsm + B);    // the partials of this CTA's rows have landed
   uint64_t* zbar = pbar + 1;                                // dz has landed
@@ -408,19 +414,19 @@ __global__ void __launch_bounds__(kClBlock, 1) softreg_cluster_round_kernel(cons
   const int units = vec ? nc / 4 : nc;
   const int ush = units <= 1 ? 0 : 32 - __clz((units < 32 ? units : 32) - 1);
   // rows of step s: (cursor + s*B + b) mod n, kept in Rsm and advanced by the
-  // fetching threads (each the rows b = its index, in steps of kClFetch)
+  // fetching threads (each the rows b = its index, in steps of NF)
   const int64_t bmod = B % n;
   auto fetch = [&](int s) {   // the fetching warps: rows and labels of step s
-    const int ft = tid - kClThreads;
-    for (int b = ft; b < B; b += kClFetch) {
+    const int ft = tid - NT;
+    for (int b = ft; b < B; b += NF) {
       int64_t r = s == 0 ? (cur + b) % n : Rsm[b] + bmod;
       if (s > 0 && r >= n) r -= n;
       Rsm[b] = r;
     }
-    bar_named(2, kClFetch);
+    bar_named(2, NF);
     float* buf = Xsm + (s & 1) * B * Xld;
-    const int fw = warp - kClWarps, u0 = lane & ((1 << ush) - 1);
-    for (int b = (fw << (5 - ush)) + (lane >> ush); b < B; b += kClFetch >> ush) {
+    const int fw = warp - NW, u0 = lane & ((1 << ush) - 1);
+    for (int b = (fw << (5 - ush)) + (lane >> ush); b < B; b += NF >> ush) {
       const float* from = X + Rsm[b] * D + c0;
       float* to = buf + b * Xld;
       if (vec)
@@ -428,19 +434,19 @@ __global__ void __launch_bounds__(kClBlock, 1) softreg_cluster_round_kernel(cons
       else
         for (int u = u0; u < units; u += 1 << ush) cp_async4(to + u, from + u);
     }
-    for (int l = ft; l < R_own; l += kClFetch) Ysm[(s & 1) * R + l] = Y[Rsm[l * kCl + rank]];
+    for (int l = ft; l < R_own; l += NF) Ysm[(s & 1) * R + l] = Y[Rsm[l * kCl + rank]];
     cp_async_wait_all();
-    bar_named(2, kClFetch);   // Rsm is read by all before the next step's rows go in
+    bar_named(2, NF);   // Rsm is read by all before the next step's rows go in
   };
-  const bool fetcher = tid >= kClThreads;
+  const bool fetcher = tid >= NT;
   if (fetcher) {
     if (tau > 0) fetch(0);
   } else {
   // columns past nc of both buffers are never copied: the bias input, then zeros
-  for (int i = tid; i < 2 * B; i += kClThreads)
+  for (int i = tid; i < 2 * B; i += NT)
     for (int k = nc; k < 4 * nk4; ++k) Xsm[i * Xld + k] = k == nc && has_bias ? 1.f : 0.f;
   // pull: this CTA's columns of the global model and, in its CTA, the bias
-  for (int c = warp; c < ncg * CC; c += kClWarps)
+  for (int c = warp; c < ncg * CC; c += NW)
     for (int k = lane; k < Dc; k += 32)
       Wsm[c * Dc + k] = c >= C ? 0.f
                         : k < nc ? gsrc[a.offW + static_cast<int64_t>(c) * D + c0 + k]
@@ -451,12 +457,12 @@ __global__ void __launch_bounds__(kClBlock, 1) softreg_cluster_round_kernel(cons
   const int cls = lane < Zp && lane % CCp < CC && cls0 < C ? cls0 : -1;
   // phase 1: this warp's column split and class group, its first row block and their step
   const int G = ncg * p.KS, l_ks = warp % p.KS, l_cg = warp / p.KS % ncg;
-  const int l_rb = warp / G, l_rbstep = kClWarps / G;   // warps past l_rbstep * G idle
+  const int l_rb = warp / G, l_rbstep = NW / G;   // warps past l_rbstep * G idle
   const int nrb = l_rb < l_rbstep ? (B + 31) / 32 : 0;
   const int l_k0 = l_ks * nk4 / p.KS + (lane >> 3), l_k1 = (l_ks + 1) * nk4 / p.KS;
-  // phase 2: thread = (row tid / 8, 16-byte chunk tid % 8 of its slots), rows kClThreads / 8 apart, so with one owner
+  // phase 2: thread = (row tid / 8, 16-byte chunk tid % 8 of its slots), rows NT / 8 apart, so with one owner
   const int s_q = tid & 7, s_b = tid >> 3, s_owner = s_b & (kCl - 1);
-  static_assert(kCl == 8 && kClThreads / 8 % kCl == 0, "the rows of a thread have one owner");
+  static_assert(kCl == 8 && NT / 8 % kCl == 0, "the rows of a thread have one owner");
   const uint32_t s_pin = cluster_addr(Pin + rank * R * Zp + 4 * s_q, s_owner), s_bar = cluster_addr(pbar, s_owner);
   // phase 3: lane = (destination lane % 8, chunk lane / 8)
   const int z_to = lane & 7, z_q = lane >> 3;
@@ -465,7 +471,7 @@ __global__ void __launch_bounds__(kClBlock, 1) softreg_cluster_round_kernel(cons
   const int nkv = Dc / 4, items = nkv * ncg * p.BS;
   const int u_kv = tid % nkv, u_cg = tid / nkv % ncg, u_bs = tid / (nkv * ncg);
   const int u_b0 = u_bs * B / p.BS, u_b1 = (u_bs + 1) * B / p.BS;
-  const int r_c = tid / nkv, r_cstep = kClThreads / nkv, r_kvstep = kClThreads % nkv;
+  const int r_c = tid / nkv, r_cstep = NT / nkv, r_kvstep = NT % nkv;
   // the warp's row losses over all steps as an unevaluated sum of two floats
   // (2Sum): fp64 adds are two lanes a clock here and sat in the chain
   float loss_hi = 0.f, loss_lo = 0.f;
@@ -533,10 +539,10 @@ __global__ void __launch_bounds__(kClBlock, 1) softreg_cluster_round_kernel(cons
           *reinterpret_cast<float4*>(o + 4 * q) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
       }
     }
-    bar_named(1, kClThreads);
+    bar_named(1, NT);
     // 2. each row's partials to its owner
     if (s_q < zq)
-      for (int b = s_b; b < B; b += kClThreads / 8) {
+      for (int b = s_b; b < B; b += NT / 8) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
         for (int ks = 0; ks < p.KS; ++ks)
@@ -548,7 +554,7 @@ __global__ void __launch_bounds__(kClBlock, 1) softreg_cluster_round_kernel(cons
     // softmax cross-entropy of this CTA's rows, one warp per row, lane = slot
     if (warp < R_own) {
       if (alive) alive = mbar_wait(pbar, s & 1, a.err, kDevTimeoutFull);
-      for (int l = warp; l < R_own; l += kClWarps) {
+      for (int l = warp; l < R_own; l += NW) {
         float part[kCl];
 #pragma unroll
         for (int q = 0; q < kCl; ++q) part[q] = lane < Zp ? Pin[(q * R + l) * Zp + lane] : 0.f;
@@ -615,7 +621,7 @@ __global__ void __launch_bounds__(kClBlock, 1) softreg_cluster_round_kernel(cons
           }
         }
       }
-      i += kClThreads;
+      i += NT;
       if (i >= items) break;   // nearly always: more items than threads need over 2000 columns
       kv = i % nkv;
       cg = i / nkv % ncg;
@@ -624,7 +630,7 @@ __global__ void __launch_bounds__(kClBlock, 1) softreg_cluster_round_kernel(cons
       b1 = (bs + 1) * B / p.BS;
     }
     if (p.BS > 1) {
-      bar_named(1, kClThreads);
+      bar_named(1, NT);
       int c = r_c, kv4 = u_kv;
       while (c < C) {
         if (kv4 < nk4) {
@@ -648,12 +654,12 @@ __global__ void __launch_bounds__(kClBlock, 1) softreg_cluster_round_kernel(cons
   if (!fetcher && lane == 0) lsum[warp] = static_cast<double>(loss_hi) + static_cast<double>(loss_lo);
   __syncthreads();
   // push: this CTA's columns into the replica
-  for (int c = warp; c < C; c += kClBlock / 32)
+  for (int c = warp; c < C; c += (NT + NF) / 32)
     for (int k = lane; k < nc; k += 32) dst[a.offW + static_cast<int64_t>(c) * D + c0 + k] = Wsm[c * Dc + k];
   if (has_bias && tid < C) dst[a.offB + tid] = Wsm[tid * Dc + nc];
   if (tid == 0) {
     double t = 0.0;
-    for (int i = 0; i < kClWarps; ++i) t += lsum[i];
+    for (int i = 0; i < NW; ++i) t += lsum[i];
     st_dsmem_f64(lrank + rank, 0, t);
   }
   cluster_sync();   // the loss sums are in; every CTA has read the cursor
@@ -713,25 +719,25 @@ cudaError_t launch_softreg_round(const SoftregArgs& a, int W, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-size_t softreg_cluster_smem_bytes(int D, int C, int B) {
-  const ClPlan p = cluster_plan(D, C, B, cluster_cc(C));
+namespace {
+int cluster_threads(int D, int C, int B) {
+  return static_cast<int64_t>(B) * C * cluster_cols(D) <= kClSmallWork ? kClSmall : kClThreads;
+}
+
+size_t cluster_smem_bytes(int D, int C, int B) {
+  const ClPlan p = cluster_plan(D, C, B, cluster_cc(C), cluster_threads(D, C, B));
   return sizeof(float) * p.oEnd + cluster_tail_bytes(B);
 }
 
-bool softreg_cluster_supported(int D, int C, int B) {
-  return B <= kClThreads && softreg_cluster_smem_bytes(D, C, B) <= 220 * 1024;
-}
-
-namespace {
-template <int CC>
-cudaError_t launch_cluster(const SoftregArgs& a, int W, cudaStream_t s) {
-  const size_t smem = softreg_cluster_smem_bytes(a.D, a.C, a.B);
-  cudaError_t e = cudaFuncSetAttribute(softreg_cluster_round_kernel<CC>,
+template <int CC, int NT>
+cudaError_t launch_cluster_nt(const SoftregArgs& a, int W, cudaStream_t s) {
+  const size_t smem = cluster_smem_bytes(a.D, a.C, a.B);
+  cudaError_t e = cudaFuncSetAttribute(softreg_cluster_round_kernel<CC, NT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kCl, W, 1);
-  cfg.blockDim = dim3(kClBlock, 1, 1);
+  cfg.blockDim = dim3(NT + NT / 4, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr;
@@ -741,9 +747,19 @@ cudaError_t launch_cluster(const SoftregArgs& a, int W, cudaStream_t s) {
   attr.val.clusterDim.z = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, softreg_cluster_round_kernel<CC>, a);
+  return cudaLaunchKernelEx(&cfg, softreg_cluster_round_kernel<CC, NT>, a);
+}
+
+template <int CC>
+cudaError_t launch_cluster(const SoftregArgs& a, int W, cudaStream_t s) {
+  return cluster_threads(a.D, a.C, a.B) == kClSmall ? launch_cluster_nt<CC, kClSmall>(a, W, s)
+                                                    : launch_cluster_nt<CC, kClThreads>(a, W, s);
 }
 }  // namespace
+
+bool softreg_cluster_supported(int D, int C, int B) {
+  return B <= kSoftregMaxBatch && cluster_smem_bytes(D, C, B) <= 220 * 1024;
+}
 
 cudaError_t launch_softreg_cluster_round(const SoftregArgs& a, int W, cudaStream_t s) {
   switch (cluster_cc(a.C)) {
