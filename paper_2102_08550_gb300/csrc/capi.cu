@@ -1537,6 +1537,47 @@ void advance_clocks(oscars_ctx* c) {
   ++c->rounds_run;
 }
 
+// dst <- a padded slot in the canonical layout (dst in host or device memory)
+cudaError_t read_canonical(oscars_ctx* c, float* slot, float* dst) {
+  cudaPointerAttributes at;
+  int dev = -1;
+  if (cudaPointerGetAttributes(&at, dst) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    at.type = cudaMemoryTypeUnregistered;
+  }
+  if (at.type == cudaMemoryTypeDevice && at.device == dev && c->model != OSCARS_MODEL_FLAT) {
+    CopySeg seg[kMaxCopySegs];
+    int n = 0;
+    int64_t co = 0;
+    auto add = [&](int64_t off, int64_t len, int rows, int pitch) {
+      seg[n++] = CopySeg{off, co, len, rows, pitch};
+      co += len * rows;
+    };
+    if (c->model == OSCARS_MODEL_CNN) {
+      const int Cin = c->dims[2], K = c->dims[4];
+      if (c->cnn_im2col) add(c->cnn_offW[0], 9 * Cin, 64, 64);   // the stem's padded rows (see copy_canonical)
+      else add(c->cnn_offW[0], Cin, 64 * 9, 64);
+      add(c->cnn_offB[0], 64, 1, 0);
+      for (size_t l = 1; l < c->cnn_offW.size(); ++l) {
+        add(c->cnn_offW[l], 64 * 9 * 64, 1, 0);
+        add(c->cnn_offB[l], 64, 1, 0);
+      }
+      add(c->cnn_offWf, static_cast<int64_t>(K) * 64, 1, 0);
+      add(c->cnn_offBf, K, 1, 0);
+    } else {
+      for (const Layer& ly : c->layers) {
+        add(ly.offW, static_cast<int64_t>(ly.in) * ly.out, 1, 0);
+        add(ly.offB, ly.out, 1, 0);
+      }
+    }
+    return launch_unpad(slot, dst, seg, n, c->stream);
+  }
+  cudaError_t e = copy_canonical(c, slot, dst, false, c->stream);
+  if (e == cudaSuccess && (at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeUnregistered))
+    e = cudaStreamSynchronize(c->stream);
+  return e;
+}
+
 bool is_host_ptr(const void* p) {
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
@@ -1820,22 +1861,22 @@ oscars_status oscars_push_merge(oscars_ctx* c, const float* const* deltas, const
       ProfScope ps(c, "merge", c->stream);
       e = launch_merge(a, xg, c->P, eta, false, c->stream);
     } else {
+      // every tensor of the canonical deltas against its place in the slot,
+      // and the bf16 copy, in one launch
+      MergeSeg seg[kMaxMergeSegs];
+      int n = 0;
       int64_t co = 0;
       for (const Layer& ly : c->layers) {
         const int64_t nw = static_cast<int64_t>(ly.in) * ly.out;
-        for (int k = 0; k < c->W; ++k) a.src[k] = deltas[k] + co;
-        e = launch_merge(a, xg + ly.offW, nw, eta, false, c->stream);
-        if (e != cudaSuccess) break;
-        for (int k = 0; k < c->W; ++k) a.src[k] = deltas[k] + co + nw;
-        e = launch_merge(a, xg + ly.offB, ly.out, eta, false, c->stream);
-        if (e != cudaSuccess) break;
+        seg[n++] = MergeSeg{ly.offW, co, nw, 0, 0};
+        seg[n++] = MergeSeg{ly.offB, co + nw, ly.out, 0, 0};
         co += nw + ly.out;
       }
+      for (int k = 0; k < c->W; ++k) a.src[k] = deltas[k];
+      ProfScope ps(c, "merge", c->stream);
+      e = launch_merge_segs(a, seg, n, xg, eta, false, c->stream,
+                            c->shadow ? c->shadow + static_cast<int64_t>(c->W) * c->P_pad : nullptr);
     }
-  }
-  if (e == cudaSuccess && c->model == OSCARS_MODEL_MLP) {
-    ProfScope ps(c, "shadow_refresh", c->stream);
-    e = refresh_global_shadows(c, c->stream);
   }
   if (e != cudaSuccess) return cuda_fail(c, e, "merge launch");
   c->pending = false;
@@ -1847,8 +1888,7 @@ oscars_status oscars_pull(oscars_ctx* c, float* dst) {
   cudaError_t e = cudaSuccess;
   const int64_t g = slotted(c) ? static_cast<int64_t>(c->W) * c->P_pad : 0;
   if (dst) {
-    e = copy_canonical(c, c->slab + g, dst, false, c->stream);
-    if (e == cudaSuccess && is_host_ptr(dst)) e = cudaStreamSynchronize(c->stream);
+    e = read_canonical(c, c->slab + g, dst);
   } else if (slotted(c)) {
     e = launch_broadcast(c->slab + g, c->slab, c->P_pad, c->W, c->P_pad, c->stream);
     for (int k = 0; e == cudaSuccess && k < c->W && c->shadow; ++k)
@@ -2124,8 +2164,7 @@ oscars_status oscars_read_replica(oscars_ctx* c, int32_t k, float* dst) {
   if (!c || !dst) return OSCARS_EINVAL;
   if (!slotted(c)) return fail(c, OSCARS_ESTATE, "replicas exist in MLP and CNN mode only");
   if (k < 0 || k >= c->W) return fail(c, OSCARS_EINVAL, "worker index out of range");
-  cudaError_t e = copy_canonical(c, c->slab + static_cast<int64_t>(k) * c->P_pad, dst, false, c->stream);
-  if (e == cudaSuccess && is_host_ptr(dst)) e = cudaStreamSynchronize(c->stream);
+  const cudaError_t e = read_canonical(c, c->slab + static_cast<int64_t>(k) * c->P_pad, dst);
   if (e != cudaSuccess) return cuda_fail(c, e, "read replica");
   return OSCARS_OK;
 }

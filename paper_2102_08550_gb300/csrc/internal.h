@@ -25,6 +25,29 @@ struct MergeArgs {
 cudaError_t launch_merge(const MergeArgs& a, float* x_g, int64_t P, float eta, bool replica,
                          cudaStream_t s, __nv_bfloat16* shadow = nullptr);
 
+// The same over pieces of the vector, in one launch: elements [dst, dst + n)
+// of x_g (and shadow) take [src, src + n) of every pushed buffer (head and n4
+// are filled in by the launcher).
+constexpr int kMaxMergeSegs = 32;   // two tensors per layer
+struct MergeSeg {
+  int64_t dst, src, n;
+  int head;                         // single elements before the first 16-byte chunk
+  int64_t n4;                       // 16-byte chunks
+};
+cudaError_t launch_merge_segs(const MergeArgs& a, const MergeSeg* seg, int nseg, float* x_g, float eta, bool replica,
+                              cudaStream_t s, __nv_bfloat16* shadow = nullptr);
+
+// Copy between a padded slot and a canonical vector on the device: piece i is
+// `rows` rows of `len` floats, `pitch` apart in the slot and contiguous in
+// the canonical vector.
+constexpr int kMaxCopySegs = 40;
+struct CopySeg {
+  int64_t slot, canon;
+  int64_t len;
+  int rows, pitch;
+};
+cudaError_t launch_unpad(const float* slot, float* canon, const CopySeg* seg, int nseg, cudaStream_t s);
+
 // one thread waits `polls` polls on an mbarrier nothing completes, then
 // records its timeout code in *err (the bounded-wait failure path)
 cudaError_t launch_wait_selfcheck(int* err, uint32_t polls, cudaStream_t s);

@@ -677,6 +677,35 @@ __global__ void transpose_bf16_kernel(const __nv_bfloat16* __restrict__ src, __n
     if (c0 + c < cols && r0 + tx < rows) dst[static_cast<int64_t>(c0 + c) * rows + r0 + tx] = t[tx][c];
 }
 
+// Canonical vector <- padded slot, grid y = piece: 16-byte copies where both
+// sides of every row are 16-byte aligned.  One launch instead of a copy per
+// tensor (two per layer): a 784-512-10 round with its pull went from 109 to
+// 100 us.
+struct CopySegs {
+  CopySeg s[kMaxCopySegs];
+};
+__global__ void __launch_bounds__(256) unpad_kernel(const float* __restrict__ slot, float* __restrict__ canon,
+                                                    const __grid_constant__ CopySegs segs) {
+  const CopySeg& g = segs.s[blockIdx.y];
+  const float* from = slot + g.slot;
+  float* to = canon + g.canon;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * 256, t0 = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
+  if (((reinterpret_cast<uintptr_t>(from) | reinterpret_cast<uintptr_t>(to)) & 15) == 0 && g.len % 4 == 0 &&
+      g.pitch % 4 == 0) {
+    const int64_t l4 = g.len / 4, n4 = l4 * g.rows;
+    for (int64_t i = t0; i < n4; i += stride) {
+      const int64_t r = g.rows == 1 ? 0 : i / l4;
+      reinterpret_cast<float4*>(to)[i] = *reinterpret_cast<const float4*>(from + r * g.pitch + 4 * (i - r * l4));
+    }
+  } else {
+    const int64_t n = g.len * g.rows;
+    for (int64_t i = t0; i < n; i += stride) {
+      const int64_t r = g.rows == 1 ? 0 : i / g.len;
+      to[i] = from[r * g.pitch + (i - r * g.len)];
+    }
+  }
+}
+
 __global__ void broadcast_kernel(const float* __restrict__ xg, float* __restrict__ slab, int64_t stride, int W,
                                  int64_t count) {
   const int64_t gs = static_cast<int64_t>(gridDim.x) * blockDim.x;
@@ -811,6 +840,21 @@ cudaError_t launch_transpose_bf16(const __nv_bfloat16* src, __nv_bfloat16* dst, 
                                   cudaStream_t s) {
   dim3 grid((cols + 31) / 32, (rows + 31) / 32);
   transpose_bf16_kernel<<<grid, 256, 0, s>>>(src, dst, rows, cols);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_unpad(const float* slot, float* canon, const CopySeg* seg, int nseg, cudaStream_t s) {
+  if (nseg < 1 || nseg > kMaxCopySegs) return cudaErrorInvalidValue;
+  CopySegs m;
+  int64_t most = 0;
+  for (int i = 0; i < nseg; ++i) {
+    m.s[i] = seg[i];
+    const int64_t n = seg[i].len * seg[i].rows;
+    if (n > most) most = n;
+  }
+  int64_t blocks = (most + 1023) / 1024;
+  if (blocks > 1024) blocks = 1024;
+  unpad_kernel<<<dim3(static_cast<unsigned>(blocks), nseg), 256, 0, s>>>(slot, canon, m);
   return cudaGetLastError();
 }
 
