@@ -2173,18 +2173,22 @@ oscars_status oscars_gemm_bf16_nt(const void* A, const void* B, float* C, int32_
                                   void* stream) {
   if (!A || !B || !C || M < 128 || M % 128 != 0 || N < 1 || K < 8 || K % 8 != 0) return OSCARS_EINVAL;
   if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) return OSCARS_EINVAL;
-  CUtensorMap mA, mB;
+  const RowsPlan p = gemm_rows_plan(kRowsStore, M, N, K);
+  const int tma = N % 4 == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
+  CUtensorMap mA, mB, mC;
   if (!make_map(&mA, A, K, M, 1, K * 2ull, static_cast<uint64_t>(M) * K * 2ull, 128) ||
-      !make_map(&mB, B, K, N, 1, K * 2ull, static_cast<uint64_t>(N) * K * 2ull, 128))
+      !make_map(&mB, B, K, N, 1, K * 2ull, static_cast<uint64_t>(N) * K * 2ull, p.BN / p.cl))
     return OSCARS_ECUDA;
-  GemmArgs g;
-  std::memset(&g, 0, sizeof(g));
+  if (!tma) mC = mA;   // not used: plain stores
+  else if (!make_map_f32(&mC, C, N, M, 1, N * 4ull, static_cast<uint64_t>(M) * N * 4ull, 32)) return OSCARS_ECUDA;
+  RowsArgs g{};
   g.M = M;
   g.N = N;
   g.K = K;
-  g.c_out = C;
-  return launch_gemm(kEpiStore, mA, mB, g, 1, static_cast<cudaStream_t>(stream)) == cudaSuccess ? OSCARS_OK
-                                                                                               : OSCARS_ECUDA;
+  g.C = C;
+  g.tma_store = tma;
+  return launch_gemm_rows(kRowsStore, p, mA, mB, mC, g, static_cast<cudaStream_t>(stream)) == cudaSuccess ? OSCARS_OK
+                                                                                                         : OSCARS_ECUDA;
 }
 
 int32_t oscars_phase_times(oscars_ctx* c, int32_t cap, double* us) {

@@ -22,8 +22,6 @@
 //           W[dst] = fmaf(-lr, acc, W[src]) (fp32 master), bf16 shadow,
 //           optional bf16 transposed shadow; column-tile 0 also updates the
 //           bias b[dst] = fmaf(-lr, gb[m], b[src]).
-//  kEpiStore plain C[m][n] = acc in fp32 (a library GEMM for tests and
-//           callers that need one).
 //
 // All waits are bounded (see common.cuh) and report through a device word.
 #include <cstdio>
@@ -161,19 +159,6 @@ __device__ __forceinline__ void epi_dw_load(const GemmArgs& a, int src, int m_ba
     const int r = 4 * i + (lane >> 3);
     old[i] = nok ? *reinterpret_cast<const float4*>(a.master + so + static_cast<int64_t>(m_base + r) * a.N)
                  : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-}
-
-__device__ __forceinline__ void epi_store(const GemmArgs& a, int m, int n0, const float (&v)[32]) {
-  float* c = a.c_out + static_cast<int64_t>(m) * a.N + n0;
-  if (n0 + 32 <= a.N && (a.N & 3) == 0) {
-    float4* c4 = reinterpret_cast<float4*>(c);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) c4[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-  } else {
-#pragma unroll
-    for (int j = 0; j < 32; ++j)
-      if (n0 + j < a.N) c[j] = v[j];
   }
 }
 
@@ -421,11 +406,7 @@ __global__ void __launch_bounds__(warps_for<EPI>() * 32) gemm_tc_kernel(const __
       for (int c0 = 0; c0 < BN; c0 += 32) {
         float v[32];
         tmem_ld_32x32b_x32(trow + c0, v);
-        if (EPI == kEpiFwd) {
-          epi_fwd<EPI>(a, wid, src, m, n0 + c0, v);
-        } else if (EPI == kEpiStore) {
-          if (n0 + c0 < a.N) epi_store(a, m, n0 + c0, v);
-        }
+        epi_fwd<EPI>(a, wid, src, m, n0 + c0, v);
       }
     }
   }
@@ -522,7 +503,7 @@ int split_for(int M, int N, int BN, int K, int n_active) {
 }  // namespace
 
 int gemm_bn_for(int epi, int N) {
-  if (epi == kEpiDw || epi == kEpiStore) return 128;
+  if (epi == kEpiDw) return 128;
   return N;  // forward / input gradient: the whole batch in one tile
 }
 
@@ -530,7 +511,6 @@ cudaError_t launch_gemm(int epi, const CUtensorMap& mA, const CUtensorMap& mB, c
                         int n_active, cudaStream_t s) {
   if (a.M % BM != 0) return cudaErrorInvalidValue;
   if (epi == kEpiDw) return launch_tile<128, kEpiDw>(mA, mB, a, n_active, s);
-  if (epi == kEpiStore) return launch_tile<128, kEpiStore>(mA, mB, a, n_active, s);
   const int bn = gemm_bn_for(epi, a.N);
   const int split = bn == 128 ? split_for(a.M, a.N, bn, a.K, n_active) : 1;
   if (epi == kEpiFwd) {

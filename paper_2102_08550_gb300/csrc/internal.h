@@ -136,7 +136,7 @@ cudaError_t launch_stage_round_strided(const StageArgs& a, const int32_t* tau, i
 cudaError_t launch_stage_round_priority(const StageArgs& a, const int32_t* tau, int W, int max_tau, int priority,
                                         cudaStream_t s);
 
-enum GemmEpi { kEpiFwd = 0, kEpiDh = 1, kEpiDw = 2, kEpiStore = 3 };
+enum GemmEpi { kEpiFwd = 0, kEpiDh = 1, kEpiDw = 2 };
 
 struct GemmArgs {
   const int* wid;     // [n_active]
@@ -160,10 +160,32 @@ struct GemmArgs {
   __nv_bfloat16* out;       // [lanes][N][M]
   __nv_bfloat16* outT;      // [lanes][M][N]
   float* gb_out;            // [lanes][M] (kEpiDh)
-  float* c_out;             // kEpiStore: C [M][N] fp32 row-major (lane 0 only)
 };
 cudaError_t launch_gemm(int epi, const CUtensorMap& mapA, const CUtensorMap& mapB,
                         const GemmArgs& a, int n_active, cudaStream_t s);
+
+// One large product D[m][n] = sum_k A[m][k] B[n][k] (csrc/gemm_rows.cu).
+enum RowsEpi { kRowsStore = 0, kRowsRelu = 1, kRowsLoss = 2 };
+struct RowsPlan {
+  int BN, cl;              // columns per tile, CTAs per tile (row tiles of 128 each)
+};
+struct RowsArgs {
+  int M, N, K;
+  int BN, stages, mt, nt;  // set by the launcher
+  float* C;                // kRowsStore: [M][N] (when tma_store is 0)
+  int tma_store;           // kRowsStore: 1 = through mD (N % 4 == 0 and C 16-byte aligned)
+  const float* bias;       // kRowsRelu, kRowsLoss: [N]
+  const int32_t* labels;   // kRowsLoss: [M]
+  float* loss_part;        // kRowsLoss: [4 ceil(M / 128)] sums over 32 rows
+  int* err;
+};
+// kRowsRelu: N a multiple of 64, bias 16-byte aligned; kRowsLoss: N <= 32
+RowsPlan gemm_rows_plan(int epi, int M, int N, int K);
+// mA: [M][K] bf16, box {64, 128}; mB: [N][K] bf16, box {64, BN / cl}; mD: the
+// result, boxes of 32 rows x 128 bytes (kRowsStore fp32, kRowsRelu bf16); all
+// with 128-byte swizzle
+cudaError_t launch_gemm_rows(int epi, const RowsPlan& p, const CUtensorMap& mA, const CUtensorMap& mB,
+                             const CUtensorMap& mD, RowsArgs a, cudaStream_t s);
 
 // Weight gradient + SGD of one layer, persistent (csrc/gemm_dw.cu):
 // W[wid] = W[src] - lr * G^T X over the batch, its bf16 copy, and the bias

@@ -1,0 +1,31 @@
+"""The persistent GEMM at the edges of its tiles: one column, a column past a
+tile, C rows that are not 16-byte aligned (plain stores), an odd and an even
+number of row tiles (alone and in pairs that share their columns), more tiles
+than SMs, one to many K-blocks.  Bound as for the other GEMM cases: fp32
+accumulation of K <= 3072 products, 1e-5 of the largest value."""
+import pytest
+import torch
+
+import paper_2102_08550_gb300 as P
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,N,K,shift", [
+    (128, 1, 8, 0), (256, 1, 8, 0), (128, 33, 72, 0), (256, 33, 72, 0), (384, 257, 136, 0), (512, 260, 520, 1),
+    (256, 2049, 64, 0), (1024, 8192, 192, 0), (1024, 4100, 3072, 0), (4096, 30, 3072, 0), (2176, 1000, 1000, 0),
+])
+def test_gemm_tile_edges(cuda_device, M, N, K, shift):
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A = torch.randn(M, K, generator=g, device=cuda_device).to(torch.bfloat16)
+    B = torch.randn(N, K, generator=g, device=cuda_device).to(torch.bfloat16)
+    buf = torch.full((M * N + shift + 64,), float("nan"), device=cuda_device)   # C `shift` floats past an aligned start
+    C = buf[shift:shift + M * N]
+    for _ in range(2):
+        P.oscars_gemm_bf16_nt(A.data_ptr(), B.data_ptr(), C.data_ptr(), M, N, K,
+                              torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    ref = A.double() @ B.double().T
+    err = (C.double().reshape(M, N) - ref).abs().max().item()
+    assert err <= 1e-5 * ref.abs().max().item() + 1e-6, err
+    assert torch.isnan(buf[:shift]).all() and torch.isnan(buf[shift + M * N:]).all()
