@@ -164,14 +164,15 @@ struct oscars_ctx {
   const int32_t** dy_tab = nullptr;
   int64_t* dn_tab = nullptr;
   int* err = nullptr;
-  // eval scratch
-  const float** ex_tab = nullptr;
-  const int32_t** ey_tab = nullptr;
-  int64_t* en_tab = nullptr;
-  int64_t* estart = nullptr;
-  int64_t estart_cap = 0;
+  // evaluation: loss partials, the result in mapped host memory, and for the
+  // MLP the bf16 samples and two activation buffers of up to eval_rows samples
   float* eval_part = nullptr;
   int64_t eval_part_cap = 0;
+  EvalResult* eval_res = nullptr;       // pinned host
+  EvalResult* eval_res_dev = nullptr;   // its device address
+  __nv_bfloat16* eval_x = nullptr;
+  __nv_bfloat16* eval_h[2] = {};
+  int64_t eval_rows = 0;
   // tensor maps per layer
   std::vector<CUtensorMap> mShadow, mShadowMN, mA, mG, mGT, mAT;
   // G^T [lane][out][B] in boxes of 64 x 64: the MN-major B operand of the input
@@ -368,6 +369,15 @@ bool dev_alloc(oscars_ctx* c, T** p, size_t count) {
   return true;
 }
 
+// give a buffer of dev_alloc back before the context ends (a larger one follows)
+template <typename T>
+void dev_release(oscars_ctx* c, T** p) {
+  if (!*p) return;
+  c->allocs.erase(std::remove(c->allocs.begin(), c->allocs.end(), static_cast<void*>(*p)), c->allocs.end());
+  cudaFree(*p);
+  *p = nullptr;
+}
+
 void free_all(oscars_ctx* c) {
   for (auto& p : c->prof_pending)
     if (!p.graph_owned) {
@@ -392,6 +402,8 @@ void free_all(oscars_ctx* c) {
   }
   if (c->train_loss_host) cudaFreeHost(c->train_loss_host);
   c->train_loss_host = nullptr;
+  if (c->eval_res) cudaFreeHost(c->eval_res);
+  c->eval_res = nullptr;
   if (c->round_exec) cudaGraphExecDestroy(c->round_exec);
   c->round_exec = nullptr;
   for (auto& g : c->ahead_exec) {
@@ -486,12 +498,6 @@ oscars_status ensure_stage_buffers(oscars_ctx* c) {
                       CU_TENSOR_MAP_SWIZZLE_NONE))
       return fail(c, OSCARS_ECUDA, "cuTensorMapEncodeTiled failed (fused round model)");
   }
-  // step 0 doubles as the single-step buffers (evaluation)
-  c->A[0] = c->A0all;
-  c->AT[0] = c->A0Tall;
-  c->labels = c->labels_all;
-  c->mA[0] = c->mA0s[0];
-  c->mAT[0] = c->mAT0s[0];
   c->stage_cap = cap;
   return OSCARS_OK;
 }
@@ -1297,8 +1303,7 @@ oscars_status allocate_common(oscars_ctx* c) {
   cudaMemset(c->slab + slots * c->P_pad, kGuardByte, kGuardWords * sizeof(float));
   if (!dev_alloc(c, &c->cursor, W) || !dev_alloc(c, &c->tau_dev, W) || !dev_alloc(c, &c->loss_dev, std::max(W, 1)) ||
       !dev_alloc(c, &c->dx_tab, W) || !dev_alloc(c, &c->dy_tab, W) || !dev_alloc(c, &c->dn_tab, W) ||
-      !dev_alloc(c, &c->err, 1) || !dev_alloc(c, &c->lane_ids, W) || !dev_alloc(c, &c->global_src, W) ||
-      !dev_alloc(c, &c->ex_tab, W) || !dev_alloc(c, &c->ey_tab, W) || !dev_alloc(c, &c->en_tab, W))
+      !dev_alloc(c, &c->err, 1) || !dev_alloc(c, &c->lane_ids, W) || !dev_alloc(c, &c->global_src, W))
     return fail(c, OSCARS_ENOMEM, "device allocation failed (tables)");
   cudaMemset(c->cursor, 0, W * sizeof(int64_t));
   cudaMemset(c->err, 0, sizeof(int));
@@ -1953,151 +1958,194 @@ oscars_status oscars_set_iteration_ticks(oscars_ctx* c, const int64_t* t_iter) {
   return OSCARS_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+constexpr int64_t kEvalRows = 16384;   // samples of one pass over the layers
+
+oscars_status eval_parts(oscars_ctx* c, int64_t count) {
+  if (c->eval_part_cap >= count) return OSCARS_OK;
+  c->eval_part_cap = 0;
+  dev_release(c, &c->eval_part);
+  if (!dev_alloc(c, &c->eval_part, count)) return fail(c, OSCARS_ENOMEM, "eval scratch");
+  c->eval_part_cap = count;
+  return OSCARS_OK;
+}
+
+// MLP: the samples cast to bf16 once, then each hidden layer and the last one
+// with its loss as one product over all samples (csrc/gemm_rows.cu), with the
+// global model's bf16 copy.  Batches of W lanes through the training kernels
+// took eight times three launches and five blocking copies for 8192 samples
+// of the 784-512-10 model, 277 us; four launches and one synchronisation, 37.
+oscars_status eval_mlp(oscars_ctx* c, const float* x, const int32_t* y, int64_t n, int64_t* parts) {
+  const int L = c->L, D = c->dims[0];
+  const int64_t rows = std::min(n, kEvalRows);
+  if (c->eval_rows < rows) {
+    int widest = 0;
+    for (int l = 1; l < L; ++l) widest = std::max(widest, c->dims[l]);
+    c->eval_rows = 0;
+    dev_release(c, &c->eval_x);
+    for (auto& h : c->eval_h) dev_release(c, &h);
+    if (!dev_alloc(c, &c->eval_x, static_cast<size_t>(rows) * D) ||
+        !dev_alloc(c, &c->eval_h[0], static_cast<size_t>(rows) * widest) ||
+        (L > 2 && !dev_alloc(c, &c->eval_h[1], static_cast<size_t>(rows) * widest)))
+      return fail(c, OSCARS_ENOMEM, "eval scratch");
+    c->eval_rows = rows;
+  }
+  const int64_t per = (rows + 127) / 128 * 4;   // loss partials of a pass
+  const oscars_status st = eval_parts(c, (n + kEvalRows - 1) / kEvalRows * per);
+  if (st != OSCARS_OK) return st;
+  const int64_t g = static_cast<int64_t>(c->W) * c->P_pad;
+  *parts = 0;
+  for (int64_t base = 0; base < n; base += kEvalRows) {
+    const int m = static_cast<int>(std::min(kEvalRows, n - base));
+    cudaError_t e = launch_cast_rows(x + base * D, c->eval_x, static_cast<int64_t>(m) * D, c->sms, c->stream);
+    for (int l = 0; e == cudaSuccess && l < L; ++l) {
+      const Layer& ly = c->layers[l];
+      const bool last = l + 1 == L;
+      const __nv_bfloat16* in = l == 0 ? c->eval_x : c->eval_h[(l - 1) & 1];
+      __nv_bfloat16* out = c->eval_h[l & 1];
+      RowsArgs a{};
+      a.M = m;
+      a.N = ly.out;
+      a.K = ly.in;
+      a.bias = c->slab + g + ly.offB;
+      a.labels = y + base;
+      a.loss_part = c->eval_part + *parts;
+      a.err = c->err;
+      a.pdl = 1;
+      const int epi = last ? kRowsLoss : kRowsRelu;
+      const RowsPlan p = gemm_rows_plan(epi, a.M, a.N, a.K);
+      CUtensorMap mA, mB, mD;
+      bool ok = make_map(&mA, in, ly.in, m, 1, ly.in * 2ull, static_cast<uint64_t>(m) * ly.in * 2ull, 128) &&
+                make_map(&mB, c->shadow + g + ly.offW, ly.in, ly.out, 1, ly.in * 2ull,
+                         static_cast<uint64_t>(ly.in) * ly.out * 2ull, p.BN / p.cl);
+      if (last) mD = mA;   // no stores
+      else ok = ok && make_map(&mD, out, ly.out, m, 1, ly.out * 2ull, static_cast<uint64_t>(m) * ly.out * 2ull, 32);
+      if (!ok) return fail(c, OSCARS_ECUDA, "cuTensorMapEncodeTiled failed (evaluation)");
+      e = launch_gemm_rows(epi, p, mA, mB, mD, a, c->stream);
+    }
+    if (e != cudaSuccess) return cuda_fail(c, e, "eval");
+    *parts += (m + 127) / 128 * 4;
+  }
+  return OSCARS_OK;
+}
+
+// CNN: W lanes of B images at a time with the global model's weights (1024
+// images, 16 workers, batch 32: 2035 us one lane at a time with a
+// synchronisation each, 434 now)
+oscars_status eval_cnn(oscars_ctx* c, const float* x, const int32_t* y, int64_t n, int64_t* parts) {
+  const int W = c->W, B = c->B;
+  const int64_t g = static_cast<int64_t>(W) * c->P_pad;
+  *parts = (n + B - 1) / B;
+  const oscars_status st = eval_parts(c, *parts);
+  if (st != OSCARS_OK) return st;
+  for (int64_t lane0 = 0; lane0 < *parts; lane0 += W) {
+    const int na = static_cast<int>(std::min<int64_t>(W, *parts - lane0));
+    CnnStageArgs a{};
+    a.x1 = x;
+    a.y1 = y;
+    a.n1 = n;
+    a.eval_base = lane0 * B;
+    a.wid = c->lane_ids;
+    a.B = B;
+    a.Cin = c->dims[2];
+    a.im2col = c->cnn_im2col ? 1 : 0;
+    a.out = c->cnn_buf[0];
+    a.labels = c->labels;
+    cudaError_t e = launch_cnn_stage(a, na, c->stream);
+    auto conv = [&](int layer, int in, int add, int out) -> cudaError_t {
+      ConvArgs ca;
+      std::memset(&ca, 0, sizeof(ca));
+      ca.wid = c->lane_ids;
+      ca.src = c->global_src;
+      ca.B = B;
+      ca.bias = c->slab;
+      ca.slot_stride = c->P_pad;
+      ca.off_bias = c->cnn_offB[layer];
+      ca.add = add >= 0 ? c->cnn_buf[add] : nullptr;
+      ca.out = c->cnn_buf[out];
+      ca.err = c->err;
+      ca.im2col = layer == 0 && c->cnn_im2col ? 1 : 0;
+      return launch_conv_igemm(0, ca.im2col ? c->cnn_m4[in] : c->cnn_m6[in], c->cnn_mw[layer], ca, na,
+                               conv_ctas_per_worker(B, na, c->sms), c->stream);
+    };
+    if (e == cudaSuccess) e = conv(0, 0, -1, 1);
+    for (int k = 0; e == cudaSuccess && k < c->cnn_blocks; ++k) {
+      const int h = k == 0 ? 1 : 3 + 2 * (k - 1);
+      e = conv(1 + 2 * k, h, -1, 2 + 2 * k);
+      if (e == cudaSuccess) e = conv(2 + 2 * k, 2 + 2 * k, h, 3 + 2 * k);
+    }
+    if (e == cudaSuccess)
+      e = launch_cnn_pool(c->cnn_buf[3 + 2 * (c->cnn_blocks - 1)], c->lane_ids, B, c->cnn_g, na, c->stream);
+    if (e == cudaSuccess)
+      e = launch_cnn_head_loss(c->cnn_g, c->labels, na, B, n - lane0 * B, c->C, c->slab + g, c->cnn_offWf, c->cnn_offBf,
+                               c->eval_part + lane0, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "eval");
+  }
+  return OSCARS_OK;
+}
+
+oscars_status eval_softreg(oscars_ctx* c, const float* x, const int32_t* y, int64_t n, int64_t* parts) {
+  const int blocks = softreg_eval_blocks(n, c->sms);
+  const oscars_status st = eval_parts(c, blocks);
+  if (st != OSCARS_OK) return st;
+  SoftregEvalArgs a;
+  a.master = c->slab + static_cast<int64_t>(c->W) * c->P_pad;
+  a.offW = c->layers[0].offW;
+  a.offB = c->layers[0].offB;
+  a.D = c->dims[0];
+  a.C = c->C;
+  a.x = x;
+  a.y = y;
+  a.n = n;
+  a.loss_sum = c->eval_part;
+  const cudaError_t e = launch_softreg_eval(a, blocks, c->stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "eval");
+  *parts = blocks;
+  return OSCARS_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 oscars_status oscars_eval_loss(oscars_ctx* c, const float* x, const int32_t* y, int64_t n, float* loss) {
   if (!c || !x || !y || !loss || n < 1) return OSCARS_EINVAL;
   if (!slotted(c)) return fail(c, OSCARS_ESTATE, "eval needs an MLP or CNN context");
-  cudaError_t e = cudaSuccess;
-  const int64_t g = static_cast<int64_t>(c->W) * c->P_pad;
-  if (c->model == OSCARS_MODEL_CNN) {
-    // chunks of up to B images through lane 0 with the global model's weights
-    const int64_t chunks = (n + c->B - 1) / c->B;
-    if (c->eval_part_cap < chunks) {
-      if (!dev_alloc(c, &c->eval_part, chunks)) return fail(c, OSCARS_ENOMEM, "eval scratch");
-      c->eval_part_cap = chunks;
-    }
-    if (c->estart_cap < 1) {
-      if (!dev_alloc(c, &c->estart, 1)) return fail(c, OSCARS_ENOMEM, "eval scratch");
-      c->estart_cap = 1;
-    }
-    const int64_t zero = 0;
-    const int64_t img = static_cast<int64_t>(c->dims[0]) * c->dims[1] * c->dims[2];
-    e = cudaMemcpyAsync(c->estart, &zero, sizeof(int64_t), cudaMemcpyHostToDevice, c->stream);
-    for (int64_t ch = 0; e == cudaSuccess && ch < chunks; ++ch) {
-      const int Bc = static_cast<int>(std::min<int64_t>(c->B, n - ch * c->B));
-      const float* xc = x + ch * c->B * img;
-      const int32_t* yc = y + ch * c->B;
-      const int64_t nc = Bc;
-      e = cudaMemcpyAsync(c->ex_tab, &xc, sizeof(float*), cudaMemcpyHostToDevice, c->stream);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(c->ey_tab, &yc, sizeof(int32_t*), cudaMemcpyHostToDevice, c->stream);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(c->en_tab, &nc, sizeof(int64_t), cudaMemcpyHostToDevice, c->stream);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);   // the host values above must not go out of scope early
-      if (e != cudaSuccess) break;
-      CnnStageArgs a{};
-      a.x = c->ex_tab;
-      a.y = c->ey_tab;
-      a.n = c->en_tab;
-      a.start = c->estart;
-      a.wid = c->lane_ids;
-      a.step = 0;
-      a.B = Bc;
-      a.Cin = c->dims[2];
-      a.im2col = c->cnn_im2col ? 1 : 0;
-      a.out = c->cnn_buf[0];
-      a.labels = c->labels;
-      e = launch_cnn_stage(a, 1, c->stream);
-      auto conv = [&](int layer, int in, int add, int out) -> cudaError_t {
-        ConvArgs ca;
-        std::memset(&ca, 0, sizeof(ca));
-        ca.wid = c->lane_ids;
-        ca.src = c->global_src;
-        ca.B = Bc;
-        ca.bias = c->slab;
-        ca.slot_stride = c->P_pad;
-        ca.off_bias = c->cnn_offB[layer];
-        ca.add = add >= 0 ? c->cnn_buf[add] : nullptr;
-        ca.out = c->cnn_buf[out];
-        ca.err = c->err;
-        ca.im2col = layer == 0 && c->cnn_im2col ? 1 : 0;
-        return launch_conv_igemm(0, ca.im2col ? c->cnn_m4[in] : c->cnn_m6[in], c->cnn_mw[layer], ca, 1,
-                                 conv_ctas_per_worker(Bc, 1, c->sms), c->stream);
-      };
-      if (e == cudaSuccess) e = conv(0, 0, -1, 1);
-      for (int k = 0; e == cudaSuccess && k < c->cnn_blocks; ++k) {
-        const int h = k == 0 ? 1 : 3 + 2 * (k - 1);
-        e = conv(1 + 2 * k, h, -1, 2 + 2 * k);
-        if (e == cudaSuccess) e = conv(2 + 2 * k, 2 + 2 * k, h, 3 + 2 * k);
+  const bool mlp = c->model == OSCARS_MODEL_MLP && c->L >= 2;
+  if (mlp && n % c->B != 0) return fail(c, OSCARS_ENOTSUP, "MLP eval: n must be a multiple of the batch size");
+  try {
+    cudaError_t e = cudaSuccess;
+    if (!c->eval_res) {
+      e = cudaHostAlloc(&c->eval_res, sizeof(EvalResult), cudaHostAllocMapped);
+      if (e != cudaSuccess) {
+        c->eval_res = nullptr;
+        return cuda_fail(c, e, "eval result buffer");
       }
-      if (e == cudaSuccess)
-        e = launch_cnn_pool(c->cnn_buf[3 + 2 * (c->cnn_blocks - 1)], c->lane_ids, Bc, c->cnn_g, 1, c->stream);
-      if (e == cudaSuccess)
-        e = launch_cnn_head_loss(c->cnn_g, c->labels, Bc, c->C, c->slab + g, c->cnn_offWf, c->cnn_offBf,
-                                 c->eval_part + ch, c->stream);
+      if ((e = cudaHostGetDevicePointer(&c->eval_res_dev, c->eval_res, 0)) != cudaSuccess)
+        return cuda_fail(c, e, "eval result buffer");
     }
-    if (e == cudaSuccess) e = launch_sum_scaled(c->eval_part, chunks, 1.0 / static_cast<double>(n), c->loss_dev, c->stream);
-  } else if (c->L == 1 && !c->bf16) {
-    const int blocks = static_cast<int>(std::min<int64_t>(1024, (n + 7) / 8));
-    if (c->eval_part_cap < blocks) {
-      if (!dev_alloc(c, &c->eval_part, blocks)) return fail(c, OSCARS_ENOMEM, "eval scratch");
-      c->eval_part_cap = blocks;
-    }
-    SoftregEvalArgs a;
-    a.master = c->slab + g;
-    a.offW = c->layers[0].offW;
-    a.offB = c->layers[0].offB;
-    a.D = c->dims[0];
-    a.C = c->C;
-    a.x = x;
-    a.y = y;
-    a.n = n;
-    a.loss_sum = c->eval_part;
-    e = launch_softreg_eval(a, blocks, c->stream);
-    if (e == cudaSuccess) e = launch_sum_scaled(c->eval_part, blocks, 1.0 / static_cast<double>(n), c->loss_dev, c->stream);
-  } else {
-    if (n % c->B != 0) return fail(c, OSCARS_ENOTSUP, "MLP eval: n must be a multiple of the batch size");
-    const int64_t chunks = n / c->B;
-    const int nc = c->B / kRowsPerLossChunk;
-    if (c->estart_cap < chunks) {
-      if (!dev_alloc(c, &c->estart, chunks)) return fail(c, OSCARS_ENOMEM, "eval scratch");
-      c->estart_cap = chunks;
-    }
-    if (c->eval_part_cap < chunks * nc) {
-      if (!dev_alloc(c, &c->eval_part, chunks * nc)) return fail(c, OSCARS_ENOMEM, "eval scratch");
-      c->eval_part_cap = chunks * nc;
-    }
-    std::vector<int64_t> starts(chunks), ns(c->W, n);
-    for (int64_t i = 0; i < chunks; ++i) starts[i] = i * c->B;
-    std::vector<const float*> xs(c->W, x);
-    std::vector<const int32_t*> ys(c->W, y);
-    e = cudaStreamSynchronize(c->stream);
-    if (e == cudaSuccess) e = cudaMemcpy(c->estart, starts.data(), chunks * sizeof(int64_t), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(c->ex_tab, xs.data(), c->W * sizeof(float*), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(c->ey_tab, ys.data(), c->W * sizeof(int32_t*), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(c->en_tab, ns.data(), c->W * sizeof(int64_t), cudaMemcpyHostToDevice);
-    for (int64_t base = 0; e == cudaSuccess && base < chunks; base += c->W) {
-      const int na = static_cast<int>(std::min<int64_t>(c->W, chunks - base));
-      StageArgs sa{};
-      sa.x = c->ex_tab;
-      sa.y = c->ey_tab;
-      sa.n = c->en_tab;
-      sa.start = c->estart + base;
-      sa.row_add = 0;
-      sa.wid = c->lane_ids;
-      sa.D = c->dims[0];
-      sa.B = c->B;
-      sa.A0 = c->A[0];
-      sa.A0T = c->AT[0];
-      sa.labels = c->labels;
-      e = launch_stage(sa, na, c->stream);
-      c->cur_buf = 0;   // the evaluation stages its rows into the first input buffer
-      if (e == cudaSuccess) e = enqueue_forward(c, c->lane_ids, c->global_src, na, c->stream);
-      if (e == cudaSuccess) {
-        HeadArgs h = head_base(c);
-        h.wid = c->lane_ids;
-        h.src = c->global_src;
-        h.loss_part = c->eval_part;
-        h.part_mul = 1;
-        h.part_add = static_cast<int>(base);
-        e = launch_head_fwd(h, na, c->stream);
-      }
-    }
-    if (e == cudaSuccess)
-      e = launch_sum_scaled(c->eval_part, chunks * nc, 1.0 / static_cast<double>(n), c->loss_dev, c->stream);
+    int64_t parts = 0;
+    const oscars_status st = c->model == OSCARS_MODEL_CNN ? eval_cnn(c, x, y, n, &parts)
+                             : mlp                        ? eval_mlp(c, x, y, n, &parts)
+                                                          : eval_softreg(c, x, y, n, &parts);
+    if (st != OSCARS_OK) return st;
+    // the loss and the error word in one write to mapped host memory, read
+    // after one synchronisation (the two blocking copies they took each waited
+    // for a round trip of their own)
+    e = launch_eval_result(c->eval_part, parts, 1.0 / static_cast<double>(n), c->err, c->eval_res_dev, mlp ? 1 : 0,
+                           c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "eval");
+    *loss = c->eval_res->loss;
+    if (c->eval_res->err != 0)
+      return fail(c, OSCARS_ETIMEOUT, "a kernel's bounded wait ran out (code " + std::to_string(c->eval_res->err) + ")");
+    return OSCARS_OK;
+  } catch (const std::bad_alloc&) {
+    return fail(c, OSCARS_ENOMEM, "host allocation failed");
   }
-  if (c->model == OSCARS_MODEL_MLP && c->L >= 2) c->staged = false;   // eval used the first input buffer
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  if (e == cudaSuccess) e = cudaMemcpy(loss, c->loss_dev, sizeof(float), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(c, e, "eval");
-  return check_err_word(c);
 }
 
 oscars_status oscars_debug_slab(const oscars_ctx* c, float** slab, int64_t* slot_stride) {

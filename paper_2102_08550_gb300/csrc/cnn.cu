@@ -502,14 +502,16 @@ __global__ void __launch_bounds__(kCT) cnn_stage_kernel(const __grid_constant__ 
   const int tile = blockIdx.x, e = blockIdx.y;
   const int lane = a.wid[e];
   const int b = tile / kTilesPerImg, pix0 = (tile % kTilesPerImg) * kTilePix;
-  const int64_t n = a.n[lane];
-  const int64_t row = (a.start[lane] + static_cast<int64_t>(a.step) * a.B + b) % n;
-  const float* src = a.x[lane] + row * static_cast<int64_t>(kPix) * a.Cin;
+  const bool eval = a.x == nullptr;
+  const int64_t n = eval ? a.n1 : a.n[lane];
+  const int64_t row = (eval ? a.eval_base + static_cast<int64_t>(lane) * a.B + b
+                            : a.start[lane] + static_cast<int64_t>(a.step) * a.B + b) % n;
+  const float* src = (eval ? a.x1 : a.x[lane]) + row * static_cast<int64_t>(kPix) * a.Cin;
   __nv_bfloat16* dst = a.out + ((static_cast<int64_t>(lane) * a.B + b) * kPix + pix0) * kCC;
   const int K = a.im2col ? kTaps * a.Cin : a.Cin;
   const int chunks = (K + 7) / 8;
   if (a.labels && tile % kTilesPerImg == 0 && threadIdx.x == 0)
-    a.labels[static_cast<int64_t>(lane) * a.B + b] = a.y[lane][row];
+    a.labels[static_cast<int64_t>(lane) * a.B + b] = (eval ? a.y1 : a.y[lane])[row];
   if (a.im2col) {
     const int Cin = a.Cin, rowel = kImg * Cin, y0 = pix0 / kImg;
     if (threadIdx.x < kCC) {
@@ -670,36 +672,58 @@ __global__ void __launch_bounds__(256) cnn_head_kernel(const __grid_constant__ C
   }
 }
 
-// loss of the global model on labelled pooled features (evaluation): grid 1, 256 threads
-__global__ void __launch_bounds__(256) cnn_head_loss_kernel(const float* g, const int32_t* labels, int B, int K,
-                                                            const float* master, int64_t offWf, int64_t offBf,
+// loss of the global model on labelled pooled features (evaluation): grid =
+// lanes, 256 threads, one image of the lane's (B <= 256) per thread
+__global__ void __launch_bounds__(256) cnn_head_loss_kernel(const float* g, const int32_t* labels, int B, int64_t n_img,
+                                                            int K, const float* master, int64_t offWf, int64_t offBf,
                                                             float* out) {
   __shared__ float wf[32 * kCC];
   __shared__ float bfm[32];
-  __shared__ float rl[256];
-  const int t = threadIdx.x;
+  __shared__ float rl[8];
+  const int t = threadIdx.x, lane = blockIdx.x;
+  const int64_t left = n_img - static_cast<int64_t>(lane) * B;
+  const int mine = left < B ? static_cast<int>(left) : B;
   for (int q = t; q < K * kCC; q += 256) wf[q] = bf16_round(master[offWf + q]);
   if (t < K) bfm[t] = master[offBf + t];
   __syncthreads();
   float l = 0.f;
-  for (int b = t; b < B; b += 256) {
-    float z[32], mx = -INFINITY;
-    for (int k = 0; k < K; ++k) {
+  if (t < mine) {
+    const float4* gr = reinterpret_cast<const float4*>(g + (static_cast<int64_t>(lane) * B + t) * kCC);
+    float gb[kCC];
+#pragma unroll
+    for (int q = 0; q < kCC / 4; ++q) {
+      const float4 v = gr[q];
+      gb[4 * q] = bf16_round(v.x);
+      gb[4 * q + 1] = bf16_round(v.y);
+      gb[4 * q + 2] = bf16_round(v.z);
+      gb[4 * q + 3] = bf16_round(v.w);
+    }
+    const int y = labels[static_cast<int64_t>(lane) * B + t];
+    float z[32], mx = -INFINITY, zy = 0.f;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+      if (k >= K) continue;
       float acc = 0.f;
-      for (int c = 0; c < kCC; ++c) acc = fmaf(bf16_round(g[static_cast<int64_t>(b) * kCC + c]), wf[k * kCC + c], acc);
+#pragma unroll
+      for (int c = 0; c < kCC; ++c) acc = fmaf(gb[c], wf[k * kCC + c], acc);
       z[k] = acc + bfm[k];
       mx = fmaxf(mx, z[k]);
+      if (k == y) zy = z[k];
     }
     float se = 0.f;
-    for (int k = 0; k < K; ++k) se += expf(z[k] - mx);
-    l += mx + logf(se) - z[labels[b]];
+#pragma unroll
+    for (int k = 0; k < 32; ++k)
+      if (k < K) se += expf(z[k] - mx);
+    l = mx + logf(se) - zy;
   }
-  rl[t] = l;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+  if ((t & 31) == 0) rl[t >> 5] = l;
   __syncthreads();
   if (t == 0) {
     float s = 0.f;
-    for (int i = 0; i < 256; ++i) s += rl[i];
-    out[0] = s;
+    for (int i = 0; i < 8; ++i) s += rl[i];
+    out[lane] = s;
   }
 }
 
@@ -825,9 +849,9 @@ cudaError_t launch_cnn_head(const CnnHeadArgs& a, int n_active, cudaStream_t s) 
   return cudaGetLastError();
 }
 
-cudaError_t launch_cnn_head_loss(const float* g, const int32_t* labels, int B, int K, const float* master,
-                                 int64_t offWf, int64_t offBf, float* out, cudaStream_t s) {
-  cnn_head_loss_kernel<<<1, 256, 0, s>>>(g, labels, B, K, master, offWf, offBf, out);
+cudaError_t launch_cnn_head_loss(const float* g, const int32_t* labels, int lanes, int B, int64_t n_img, int K,
+                                 const float* master, int64_t offWf, int64_t offBf, float* out, cudaStream_t s) {
+  cnn_head_loss_kernel<<<lanes, 256, 0, s>>>(g, labels, B, n_img, K, master, offWf, offBf, out);
   return cudaGetLastError();
 }
 

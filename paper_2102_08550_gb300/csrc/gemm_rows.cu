@@ -413,8 +413,13 @@ cudaError_t launch_rows_t(const CUtensorMap& mA, const CUtensorMap& mB, const CU
   cudaError_t e = cudaFuncSetAttribute(gemm_rows_kernel<EPI, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = rows_config<EPI, CL>(attr, grid, smem, s);
+  if (a.pdl) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+    ++cfg.numAttrs;
+  }
   return cudaLaunchKernelEx(&cfg, gemm_rows_kernel<EPI, CL>, mA, mB, mD, a);
 }
 

@@ -104,6 +104,7 @@ struct SoftregEvalArgs {
   int64_t n;
   float* loss_sum;      // [blocks] partial sums
 };
+int softreg_eval_blocks(int64_t n, int sms);   // loss_sum entries
 cudaError_t launch_softreg_eval(const SoftregEvalArgs& a, int blocks, cudaStream_t s);
 
 // ---------------------------------------------------------------- MLP (bf16 GEMMs)
@@ -125,7 +126,8 @@ struct StageArgs {
   const int32_t* slots;    // stage_round: the n_slots active slots s * W + w (s < tau[w]), or null (all)
   int n_slots;
 };
-cudaError_t launch_stage(const StageArgs& a, int n_active, cudaStream_t s);
+// out[i] = bf16(x[i]), count a multiple of 8
+cudaError_t launch_cast_rows(const float* x, __nv_bfloat16* out, int64_t count, int sms, cudaStream_t s);
 // all mini-batches of a round: step s of worker w (s < tau[w]) at slot s * W + w
 // (grid z over a.slots when given, else over all max_tau * W slots)
 cudaError_t launch_stage_round(const StageArgs& a, const int32_t* tau, int W, int max_tau, cudaStream_t s);
@@ -178,6 +180,7 @@ struct RowsArgs {
   const int32_t* labels;   // kRowsLoss: [M]
   float* loss_part;        // kRowsLoss: [4 ceil(M / 128)] sums over 32 rows
   int* err;
+  int pdl;                 // launch as a programmatic dependent of the previous kernel on the stream
 };
 // kRowsRelu: N a multiple of 64, bias 16-byte aligned; kRowsLoss: N <= 32
 RowsPlan gemm_rows_plan(int epi, int M, int N, int K);
@@ -291,9 +294,15 @@ cudaError_t launch_fused_round(const CUtensorMap& mX, const CUtensorMap& mXT, co
 // loss[w] = sum_{s < tau[w]} sum_c part[(w*max_tau + s)*nc + c] / (B * tau[w])
 cudaError_t launch_loss_finalize(const float* part, const int32_t* tau, int W, int max_tau,
                                  int nc, int B, float* loss, cudaStream_t s);
-// out[0] = sum_i part[i] / n (fixed order)
-cudaError_t launch_sum_scaled(const float* part, int64_t count, double scale, float* out,
-                              cudaStream_t s);
+// the result of an evaluation: loss = scale * sum_i part[i] (fixed order), err
+// = the device error word, which is cleared; `out` in mapped host memory.
+// pdl: as a programmatic dependent of the launch before it.
+struct EvalResult {
+  float loss;
+  int err;
+};
+cudaError_t launch_eval_result(const float* part, int64_t count, double scale, int* err, EvalResult* out, int pdl,
+                               cudaStream_t s);
 // cursor[w] = (cursor[w] + tau[w] * B) % n[w]
 cudaError_t launch_cursor_advance(int64_t* cursor, const int32_t* tau, const int64_t* n, int B,
                                   int W, cudaStream_t s);
@@ -347,10 +356,13 @@ struct ConvSgdArgs {
   float lr;
 };
 struct CnnStageArgs {
-  const float* const* x;       // [W] fp32 NHWC shards
+  const float* const* x;       // [W] fp32 NHWC shards; null: the evaluation set below
   const int32_t* const* y;
   const int64_t* n;
   const int64_t* start;        // [W] cursors
+  const float* x1;             // evaluation: images from eval_base + lane * B (mod n1)
+  const int32_t* y1;
+  int64_t n1, eval_base;
   const int* wid;
   int step, B, Cin;
   int im2col;                  // 1: channel k = tap * Cin + i holds x[y + dy - 1][x + dx - 1][i], tap = 3 dy + dx
@@ -386,8 +398,9 @@ cudaError_t launch_cnn_stage(const CnnStageArgs& a, int n_active, cudaStream_t s
 cudaError_t launch_cnn_pool(const __nv_bfloat16* v, const int* wid, int B, float* g, int n_active, cudaStream_t s);
 size_t cnn_head_smem(int B, int K);
 cudaError_t launch_cnn_head(const CnnHeadArgs& a, int n_active, cudaStream_t s);
-cudaError_t launch_cnn_head_loss(const float* g, const int32_t* labels, int B, int K, const float* master,
-                                 int64_t offWf, int64_t offBf, float* out, cudaStream_t s);
+// out[lane] = loss sum of the lane's first min(B, n_img - lane * B) images, lane < lanes
+cudaError_t launch_cnn_head_loss(const float* g, const int32_t* labels, int lanes, int B, int64_t n_img, int K,
+                                 const float* master, int64_t offWf, int64_t offBf, float* out, cudaStream_t s);
 cudaError_t launch_cnn_dzb(const __nv_bfloat16* v, const float* dg, const int* wid, int B, __nv_bfloat16* dz,
                            float* bias_part, int n_active, cudaStream_t s);
 

@@ -25,42 +25,25 @@ __device__ __forceinline__ float warp_max(float v) {
 }
 
 // ---------------------------------------------------------------- stage
-// Mini-batch of lane w: rows (start[w] + row_add + b) mod n[w] of its sample
-// matrix, rounded to bf16 as A0 [B][D] and transposed A0T [D][B] (the
-// K-major operand of the first layer's weight-gradient GEMM).  32 x 32
-// tiles through shared memory so both writes are coalesced.
-__device__ __forceinline__ void stage_tile(const StageArgs& a, int w, int64_t base, __nv_bfloat16* A0,
-                                           __nv_bfloat16* A0T, int32_t* labels) {
-  __shared__ __nv_bfloat16 tile[32][34];
-  const int k0 = blockIdx.x * 32, b0 = blockIdx.y * 32;
-  const float* X = a.x[w];
-  const int64_t n = a.n[w];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
-  for (int r = ty; r < 32; r += 8) {
-    const int b = b0 + r, k = k0 + tx;
-    __nv_bfloat16 v = __float2bfloat16_rn(0.f);
-    if (b < a.B && k < a.D) {
-      const int64_t row = (base + b) % n;
-      v = __float2bfloat16_rn(X[row * a.D + k]);
-      A0[static_cast<int64_t>(b) * a.D + k] = v;
+// Evaluation: samples [n][D] fp32 to bf16, nothing else changed.  16-byte
+// loads where x is aligned (count is a multiple of 8 either way).
+__global__ void __launch_bounds__(256) cast_rows_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ out,
+                                                        int64_t count8, int vec) {
+  pdl_trigger();
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * 256;
+  for (int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; i < count8; i += stride) {
+    float v[8];
+    if (vec) {
+      const float4 a = __ldcs(reinterpret_cast<const float4*>(x) + 2 * i), b = __ldcs(reinterpret_cast<const float4*>(x) + 2 * i + 1);
+      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+      v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = x[8 * i + j];
     }
-    tile[r][tx] = v;
+    reinterpret_cast<uint4*>(out)[i] =
+        make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
   }
-  __syncthreads();
-  for (int r = ty; r < 32; r += 8) {
-    const int k = k0 + r, b = b0 + tx;
-    if (k < a.D && b < a.B) A0T[static_cast<int64_t>(k) * a.B + b] = tile[tx][r];
-  }
-  if (blockIdx.x == 0 && threadIdx.x < 32) {
-    const int b = b0 + threadIdx.x;
-    if (b < a.B) labels[b] = a.y[w][(base + b) % n];
-  }
-}
-
-__global__ void __launch_bounds__(256) stage_kernel(const __grid_constant__ StageArgs a) {
-  const int w = a.wid[blockIdx.z];
-  const int64_t off = static_cast<int64_t>(w) * a.B * a.D;
-  stage_tile(a, w, a.start[w] + a.row_add, a.A0 + off, a.A0T + off, a.labels + static_cast<int64_t>(w) * a.B);
 }
 
 // Every mini-batch of a round at once: grid z = step * W + worker (or the
@@ -640,8 +623,11 @@ __global__ void loss_finalize_kernel(const float* part, const int32_t* tau, int 
   loss[w] = static_cast<float>(s / (static_cast<double>(B) * t));
 }
 
-__global__ void sum_scaled_kernel(const float* part, int64_t count, double scale, float* out) {
+// out[0] = scale * sum of part in a fixed order, out[1] = the error word
+// (cleared): the result of an evaluation, in host memory the device can write
+__global__ void eval_result_kernel(const float* part, int64_t count, double scale, int* err, EvalResult* out) {
   __shared__ double red[256];
+  pdl_wait();
   double s = 0.0;
   for (int64_t i = threadIdx.x; i < count; i += blockDim.x) s += part[i];
   red[threadIdx.x] = s;
@@ -650,7 +636,11 @@ __global__ void sum_scaled_kernel(const float* part, int64_t count, double scale
     if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
     __syncthreads();
   }
-  if (threadIdx.x == 0) out[0] = static_cast<float>(red[0] * scale);
+  if (threadIdx.x == 0) {
+    out->loss = static_cast<float>(red[0] * scale);
+    out->err = *err;
+    *err = 0;
+  }
 }
 
 __global__ void cursor_advance_kernel(int64_t* cursor, const int32_t* tau, const int64_t* n, int B, int W) {
@@ -717,9 +707,13 @@ __global__ void broadcast_kernel(const float* __restrict__ xg, float* __restrict
 
 }  // namespace
 
-cudaError_t launch_stage(const StageArgs& a, int n_active, cudaStream_t s) {
-  dim3 grid((a.D + 31) / 32, (a.B + 31) / 32, n_active);
-  stage_kernel<<<grid, 256, 0, s>>>(a);
+cudaError_t launch_cast_rows(const float* x, __nv_bfloat16* out, int64_t count, int sms, cudaStream_t s) {
+  if (count % 8 != 0) return cudaErrorInvalidValue;
+  const int64_t c8 = count / 8;
+  int64_t blocks = (c8 + 255) / 256;
+  if (blocks > 8LL * sms) blocks = 8LL * sms;
+  cast_rows_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(x, out, c8,
+                                                                 (reinterpret_cast<uintptr_t>(x) & 15) == 0 ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -817,9 +811,18 @@ cudaError_t launch_loss_finalize(const float* part, const int32_t* tau, int W, i
   return cudaGetLastError();
 }
 
-cudaError_t launch_sum_scaled(const float* part, int64_t count, double scale, float* out, cudaStream_t s) {
-  sum_scaled_kernel<<<1, 256, 0, s>>>(part, count, scale, out);
-  return cudaGetLastError();
+cudaError_t launch_eval_result(const float* part, int64_t count, double scale, int* err, EvalResult* out, int pdl,
+                               cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1, 1, 1);
+  cfg.blockDim = dim3(256, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, eval_result_kernel, part, count, scale, err, out);
 }
 
 cudaError_t launch_cursor_advance(int64_t* cursor, const int32_t* tau, const int64_t* n, int B, int W,

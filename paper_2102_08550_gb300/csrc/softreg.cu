@@ -672,32 +672,91 @@ __global__ void __launch_bounds__(NT + NT / 4, 1) softreg_cluster_round_kernel(c
   }
 }
 
-// Mean cross-entropy of the global model: one warp per sample, partial sums
-// per block (summed afterwards in a fixed order).
-__global__ void __launch_bounds__(256) softreg_eval_kernel(const __grid_constant__ SoftregEvalArgs a) {
-  __shared__ float part[8];
+// Mean cross-entropy of the global model, partial sums per block (summed
+// afterwards in a fixed order).  The weights sit in shared memory; a warp
+// takes 4 samples at a time, lane = every 32nd input, so that a weight read
+// from shared memory serves 4 products (with one sample a warp each weight
+// read served one: 8192 samples of 784 inputs, 10 classes, took 106 us a
+// call, 28 now).  Classes come in G groups of CC; the 4 x CC sums are reduced over the lanes by two
+// exchange steps (a lane keeps one sample) and three butterfly steps.
+constexpr int kEvalThreads = 512;
+template <int CC, int G>
+__global__ void __launch_bounds__(kEvalThreads) softreg_eval_kernel(const __grid_constant__ SoftregEvalArgs a) {
+  extern __shared__ __align__(16) float Wsm[];   // [C][D]; a group's classes past C read the last row and are ignored
+  __shared__ float part[kEvalThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int D = a.D, C = a.C;
+  for (int i = threadIdx.x; i < C * D; i += kEvalThreads) Wsm[i] = a.master[a.offW + i];
+  __syncthreads();
   float mine = 0.f;
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * 8 + warp; i < a.n; i += static_cast<int64_t>(gridDim.x) * 8) {
-    const float* xr = a.x + i * a.D;
-    float z[kMaxClasses];
-    for (int c = 0; c < a.C; ++c) {
-      const float* wr = a.master + a.offW + static_cast<int64_t>(c) * a.D;
-      float acc = 0.f;
-      for (int k = lane; k < a.D; k += 32) acc = fmaf(xr[k], wr[k], acc);
-      z[c] = warp_sum(acc) + a.master[a.offB + c];
+  const int64_t step = static_cast<int64_t>(gridDim.x) * (kEvalThreads / 32) * 4;
+  for (int64_t i0 = (static_cast<int64_t>(blockIdx.x) * (kEvalThreads / 32) + warp) * 4; i0 < a.n; i0 += step) {
+    const float* xr[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) xr[r] = a.x + (i0 + r < a.n ? i0 + r : a.n - 1) * D;
+    float z[G][CC];   // of sample i0 + lane / 8
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      float acc[4][CC];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < CC; ++c) acc[r][c] = 0.f;
+      int woff[CC];
+#pragma unroll
+      for (int c = 0; c < CC; ++c) woff[c] = (g * CC + c < C ? g * CC + c : C - 1) * D;
+#pragma unroll 4
+      for (int k = lane; k < D; k += 32) {
+        float xv[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) xv[r] = xr[r][k];
+#pragma unroll
+        for (int c = 0; c < CC; ++c) {
+          const float w = Wsm[woff[c] + k];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) acc[r][c] = fmaf(xv[r], w, acc[r][c]);
+        }
+      }
+      const bool up = lane & 16, odd = lane & 8;
+#pragma unroll
+      for (int c = 0; c < CC; ++c) {
+        const float k0 = up ? acc[2][c] : acc[0][c], k1 = up ? acc[3][c] : acc[1][c];
+        const float g0 = up ? acc[0][c] : acc[2][c], g1 = up ? acc[1][c] : acc[3][c];
+        const float h0 = k0 + __shfl_xor_sync(0xffffffffu, g0, 16), h1 = k1 + __shfl_xor_sync(0xffffffffu, g1, 16);
+        float v = (odd ? h1 : h0) + __shfl_xor_sync(0xffffffffu, odd ? h0 : h1, 8);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        z[g][c] = v;
+      }
     }
-    float m = z[0];
-    for (int c = 1; c < a.C; ++c) m = fmaxf(m, z[c]);
-    float se = 0.f;
-    for (int c = 0; c < a.C; ++c) se += expf(z[c] - m);
-    mine += m + logf(se) - z[a.y[i]];
+    const int64_t i = i0 + (lane >> 3);
+    if (i < a.n && (lane & 7) == 0) {
+      const int y = a.y[i];
+      float m = -INFINITY, zy = 0.f, se = 0.f;
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int c = 0; c < CC; ++c) {
+          const int k = g * CC + c;
+          if (k >= C) continue;
+          z[g][c] += a.master[a.offB + k];
+          m = fmaxf(m, z[g][c]);
+          if (k == y) zy = z[g][c];
+        }
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int c = 0; c < CC; ++c)
+          if (g * CC + c < C) se += expf(z[g][c] - m);
+      mine += m + logf(se) - zy;
+    }
   }
+  mine = warp_sum(mine);
   if (lane == 0) part[warp] = mine;
   __syncthreads();
   if (threadIdx.x == 0) {
     float s = 0.f;
-    for (int i = 0; i < 8; ++i) s += part[i];
+    for (int i = 0; i < kEvalThreads / 32; ++i) s += part[i];
     a.loss_sum[blockIdx.x] = s;
   }
 }
@@ -771,9 +830,30 @@ cudaError_t launch_softreg_cluster_round(const SoftregArgs& a, int W, cudaStream
   }
 }
 
-cudaError_t launch_softreg_eval(const SoftregEvalArgs& a, int blocks, cudaStream_t s) {
-  softreg_eval_kernel<<<blocks, 256, 0, s>>>(a);
+int softreg_eval_blocks(int64_t n, int sms) {
+  const int64_t need = (n + kEvalThreads / 8 - 1) / (kEvalThreads / 8);   // 4 samples a warp
+  return static_cast<int>(need < sms ? need : sms);
+}
+
+namespace {
+template <int CC, int G>
+cudaError_t launch_eval(const SoftregEvalArgs& a, int blocks, cudaStream_t s) {
+  const size_t smem = sizeof(float) * a.C * static_cast<size_t>(a.D);
+  cudaError_t e = cudaFuncSetAttribute(softreg_eval_kernel<CC, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  softreg_eval_kernel<CC, G><<<blocks, kEvalThreads, smem, s>>>(a);
   return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_softreg_eval(const SoftregEvalArgs& a, int blocks, cudaStream_t s) {
+  if (a.C <= 4) return launch_eval<4, 1>(a, blocks, s);
+  if (a.C <= 8) return launch_eval<8, 1>(a, blocks, s);
+  if (a.C <= 12) return launch_eval<12, 1>(a, blocks, s);
+  if (a.C <= 16) return launch_eval<16, 1>(a, blocks, s);
+  if (a.C <= 24) return launch_eval<12, 2>(a, blocks, s);
+  return launch_eval<16, 2>(a, blocks, s);
 }
 
 }  // namespace oscars
