@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
   uint64_t* acce = accf + 2;         // [2] 128 arrivals
   uint32_t* tslot = reinterpret_cast<uint32_t*>(acce + 2);
   float* bias_s = reinterpret_cast<float*>(tslot + 4);   // [64] this worker's bias (forward)
-  const int t = threadIdx.x, warp = t >> 5, lane_id = t & 31;
+  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane_id = t & 31;
   const int c0 = blockIdx.x, cpw = gridDim.x, e = blockIdx.y;
   const int lane = a.wid[e], slot = a.src[e];
   const int ntiles = a.B * kTilesPerImg;
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
         }
       }
     }
-  } else if (t == 32) {
+  } else if (warp == 1) {   // converged, one elected lane issues: see elect_one
     constexpr uint32_t idesc = idesc_bf16_f32(128, kCC);
     bool ok = mbar_wait(wfull, 0, a.err, kDevTimeoutFull);
     tc_fence_after();
@@ -160,28 +160,29 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
           break;
         }
         tc_fence_after();
-        const uint32_t sa = smem_u32(slots + sl * kGBox);
-        if (one_tap) {
+        // descriptors count 16 bytes: 2 for the 32 bytes of a K slice
+        const uint64_t sa = smem_desc_k128(smem_u32(slots + sl * kGBox)), wb = smem_desc_k128(smem_u32(wts));
+        if (elect_one()) {
+          if (one_tap) {
 #pragma unroll
-          for (int j = 0; j < kCC / 16; ++j)
-            umma_bf16(tmem + buf * kCC, smem_desc_k128(sa + j * 32), smem_desc_k128(smem_u32(wts) + j * 32), idesc,
-                      j != 0 ? 1u : 0u);
+            for (int j = 0; j < kCC / 16; ++j)
+              umma_bf16(tmem + buf * kCC, sa + 2 * j, wb + 2 * j, idesc, j != 0 ? 1u : 0u);
+          } else {
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy) {
+              const int rowoff = MODE == 0 ? dy : 2 - dy;   // sub-tile of the 6-row box
+              const uint64_t aa = sa + rowoff * (kImg * kCC * 2 / 16), bb = wb + (dy * 3 + dx) * (kCB / 16);
+#pragma unroll
+              for (int j = 0; j < kCC / 16; ++j)
+                umma_bf16(tmem + buf * kCC, aa + 2 * j, bb + 2 * j, idesc, (dx | dy | j) != 0 ? 1u : 0u);
+            }
+          }
           umma_commit(&empty[sl]);
-          continue;
         }
-#pragma unroll
-        for (int dy = 0; dy < 3; ++dy) {
-          const int rowoff = MODE == 0 ? dy : 2 - dy;   // sub-tile of the 6-row box
-          const uint32_t aa = sa + rowoff * kImg * kCC * 2;
-          const uint32_t bb = smem_u32(wts + (dy * 3 + dx) * kCB);
-#pragma unroll
-          for (int j = 0; j < kCC / 16; ++j)
-            umma_bf16(tmem + buf * kCC, smem_desc_k128(aa + j * 32), smem_desc_k128(bb + j * 32), idesc,
-                      (dx | dy | j) != 0 ? 1u : 0u);
-        }
-        umma_commit(&empty[sl]);
+        __syncwarp();
       }
-      if (ok) umma_commit(&accf[buf]);
+      if (ok && elect_one()) umma_commit(&accf[buf]);
+      __syncwarp();
     }
   } else if (warp >= 2) {
     // epilogue: thread = output pixel (TMEM lane of its warp's quarter), 64 channels
@@ -320,7 +321,7 @@ __global__ void __launch_bounds__(kWT, 1) conv_wgrad_kernel(const __grid_constan
   uint64_t* empty = full + kWStages2;
   uint64_t* accb = empty + kWStages2;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(accb + 1);
-  const int t = threadIdx.x, warp = t >> 5;
+  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0);
   const int chunk = blockIdx.x, e = blockIdx.y;
   const int lane = a.wid[e];
   const int i0 = chunk * a.img_per_chunk;
@@ -362,35 +363,37 @@ __global__ void __launch_bounds__(kWT, 1) conv_wgrad_kernel(const __grid_constan
       }
       tma_load_4d(sa + 3 * kWBox, &mDz, 0, 0, yr, img, &full[st]);
     }
-  } else if (t == 32) {
+  } else if (warp == 1) {   // converged, one elected lane issues: see elect_one
     constexpr uint32_t idesc = idesc_bf16_f32_mn(128, kCC);
     for (int kb = 0; kb < nk; ++kb) {
       const int st = kb % kWStages2;
       if (!mbar_wait(&full[st], (kb / kWStages2) & 1, a.err, kDevTimeoutFull)) break;
       tc_fence_after();
       const uint32_t sa = smem_u32(sm + st * kWStage2);
-      const uint32_t sb = sa + 3 * kWBox;
-      if (a.im2col) {
-        // A = the 2-row box (in-channels k); its upper atom (the next row) is not read back
+      const uint64_t sb = smem_desc_mn128(sa + 3 * kWBox, kWTile);
+      if (elect_one()) {
+        if (a.im2col) {
+          // A = the 2-row box (in-channels k); its upper atom (the next row) is not read back
+          const uint64_t aa = smem_desc_mn128(sa, kWRow);
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          umma_bf16(tmem, smem_desc_mn128(sa + j * 2048, kWRow), smem_desc_mn128(sb + j * 2048, kWTile), idesc,
-                    (kb | j) != 0 ? 1u : 0u);
+          for (int j = 0; j < 4; ++j) umma_bf16(tmem, aa + 128 * j, sb + 128 * j, idesc, (kb | j) != 0 ? 1u : 0u);
+        } else {
+#pragma unroll
+          for (int pr = 0; pr < kWPairs; ++pr) {
+            int start, lbo, tap0, tap1;
+            wgrad_pair(pr, start, lbo, tap0, tap1);
+            const uint64_t aa = smem_desc_mn128(sa + start, lbo);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)   // K = 16 pixels per MMA: two 8-row groups, 2048 bytes
+              umma_bf16(tmem + pr * kCC, aa + 128 * j, sb + 128 * j, idesc, (kb | j) != 0 ? 1u : 0u);
+          }
+        }
         umma_commit(&empty[st]);
-        continue;
       }
-#pragma unroll
-      for (int pr = 0; pr < kWPairs; ++pr) {
-        int start, lbo, tap0, tap1;
-        wgrad_pair(pr, start, lbo, tap0, tap1);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)   // K = 16 pixels per MMA: two 8-row groups
-          umma_bf16(tmem + pr * kCC, smem_desc_mn128(sa + start + j * 2048, lbo), smem_desc_mn128(sb + j * 2048, kWTile),
-                    idesc, (kb | j) != 0 ? 1u : 0u);
-      }
-      umma_commit(&empty[st]);
+      __syncwarp();
     }
-    umma_commit(accb);
+    if (elect_one()) umma_commit(accb);
+    __syncwarp();
   }
   int ok = mbar_wait(accb, 0, a.err, kDevTimeoutAccum) ? 1 : 0;
   ok = __all_sync(0xffffffffu, ok);

@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(kFT, 1) fused_mlp2_round_kernel(const __grid_c
   const int grp = rank / S, half = rank % S;    // unit group, column half
   const int g0 = grp * kFU;                     // first unit of the group
   const int ku0 = half * UPC;                   // first kept unit within the group
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane = t & 31;
   const int D = a.D, H = a.H;
   const int nkF = (D + kFBK - 1) / kFBK;
   const int kb_split = S > 1 ? nkF / 2 : nkF;
@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(kFT, 1) fused_mlp2_round_kernel(const __grid_c
       if (warp == 0 && lane == 0) {
         if (producer_ok) producer_ok = issue_f(s, pre_f, nkf);   // the rest of this step's X tiles
         if (producer_ok) producer_ok = issue_d(s, 0, pre_d);     // the first X^T tiles of step D
-      } else if (warp == 1 && lane == 0) {
+      } else if (warp == 1) {   // converged, one elected lane issues: see elect_one
         constexpr uint32_t idesc = idesc_bf16_f32(128, B);
         for (int kb = 0; kb < nkf; ++kb) {
           const int c = sg * nkf + kb, st = c % Cfg::kStagesF;
@@ -492,14 +492,17 @@ __global__ void __launch_bounds__(kFT, 1) fused_mlp2_round_kernel(const __grid_c
           // K slices of 16 wholly past the input's end (zero in both
           // operands) are not issued
           const int kleft = D - (kb_begin + kb) * kFBK;
+          const uint64_t ad = smem_desc_k128(wa), bd = smem_desc_k128(xb);
+          if (elect_one()) {
 #pragma unroll
-          for (int j = 0; j < kFBK / 16; ++j)
-            if (j * 16 < kleft)
-              umma_bf16(tmem + kTAcc, smem_desc_k128(wa + j * 32), smem_desc_k128(xb + j * 32), idesc,
-                        (kb | j) != 0 ? 1u : 0u);
-          umma_commit(&emptyF[st]);
+            for (int j = 0; j < kFBK / 16; ++j)   // 32 bytes along K: 2 in the descriptor's address field
+              if (j * 16 < kleft) umma_bf16(tmem + kTAcc, ad + 2 * j, bd + 2 * j, idesc, (kb | j) != 0 ? 1u : 0u);
+            umma_commit(&emptyF[st]);
+          }
+          __syncwarp();
         }
-        umma_commit(accF);
+        if (elect_one()) umma_commit(accF);
+        __syncwarp();
       }
       for (int b = t; b < B; b += kFT) labs[b] = a.labels[(static_cast<int64_t>(s) * a.W + w) * B + b];
       if (warp >= 4) {   // epilogue F: thread = unit of the group, columns = samples
@@ -626,14 +629,17 @@ __global__ void __launch_bounds__(kFT, 1) fused_mlp2_round_kernel(const __grid_c
       if constexpr (Cfg::kTCH) {
         // partial logits plb[b][c] = sum over this CTA's units of h[b][u] W1[c][u]:
         // M = 128 (rows b < 64 used), N = 16 (classes < 10 used), K = 64 units
-        if (warp == 1 && lane == 0) {
+        if (warp == 1) {
           tc_fence_after();
           constexpr uint32_t idesc = idesc_bf16_f32(128, 16);
-          const uint32_t ha = smem_u32(fring + Cfg::tH), wb = smem_u32(fring + Cfg::tW1);
+          const uint64_t ha = smem_desc_k128(smem_u32(fring + Cfg::tH)), wb = smem_desc_k128(smem_u32(fring + Cfg::tW1));
+          if (elect_one()) {
 #pragma unroll
-          for (int j = 0; j < kFBK / 16; ++j)
-            umma_bf16(tmem + kTAcc + 64, smem_desc_k128(ha + j * 32), smem_desc_k128(wb + j * 32), idesc, j != 0 ? 1u : 0u);
-          umma_commit(accH1);
+            for (int j = 0; j < kFBK / 16; ++j)
+              umma_bf16(tmem + kTAcc + 64, ha + 2 * j, wb + 2 * j, idesc, j != 0 ? 1u : 0u);
+            umma_commit(accH1);
+          }
+          __syncwarp();
         } else if (warp == 4 || warp == 5) {   // lanes 0..63: one sample each
           int ok = mbar_wait(accH1, sg & 1, a.err, kDevTimeoutAccum) ? 1 : 0;
           ok = __all_sync(0xffffffffu, ok);
@@ -765,15 +771,18 @@ __global__ void __launch_bounds__(kFT, 1) fused_mlp2_round_kernel(const __grid_c
         // with rows u < 64 used, N = 64 samples, K = 16 classes) and the
         // head-weight gradient dW1^T[u][c] = sum_b h^T[u][b] dz1^T[c][b]
         // (N = 16 with classes < 10 used, K = 64 samples), one commit
-        if (warp == 1 && lane == 0) {
-          umma_bf16(tmem + kTAcc, smem_desc_k128(smem_u32(fring + Cfg::tW1T)), smem_desc_k128(smem_u32(fring + Cfg::tDz)),
-                    idesc_bf16_f32(128, B), 0u);
+        if (warp == 1) {
           constexpr uint32_t idesc = idesc_bf16_f32(128, 16);
-          const uint32_t ha = smem_u32(fring + Cfg::tHT), gb = smem_u32(fring + Cfg::tDzT);
+          const uint64_t wt = smem_desc_k128(smem_u32(fring + Cfg::tW1T)), dd = smem_desc_k128(smem_u32(fring + Cfg::tDz));
+          const uint64_t ha = smem_desc_k128(smem_u32(fring + Cfg::tHT)), gb = smem_desc_k128(smem_u32(fring + Cfg::tDzT));
+          if (elect_one()) {
+            umma_bf16(tmem + kTAcc, wt, dd, idesc_bf16_f32(128, B), 0u);
 #pragma unroll
-          for (int j = 0; j < kFBK / 16; ++j)
-            umma_bf16(tmem + kTAcc + 64, smem_desc_k128(ha + j * 32), smem_desc_k128(gb + j * 32), idesc, j != 0 ? 1u : 0u);
-          umma_commit(accH2);
+            for (int j = 0; j < kFBK / 16; ++j)
+              umma_bf16(tmem + kTAcc + 64, ha + 2 * j, gb + 2 * j, idesc, j != 0 ? 1u : 0u);
+            umma_commit(accH2);
+          }
+          __syncwarp();
         } else if (warp == 4 || warp == 5) {
           // unit u = (warp & 3) * 32 + lane: its masked dz0 row (bf16 into the
           // K-major dz0^T tile, the A operand of step D) and its b0 (the sum
@@ -966,14 +975,12 @@ __global__ void __launch_bounds__(kFT, 1) fused_mlp2_round_kernel(const __grid_c
           if (chain_ok) chain_ok = mbar_wait(&fullD[xb], (c / kNXD) & 1, a.err, kDevTimeoutFull);
           if (use >= 1) bar_named(1 + e, 128 + 32);   // the previous use of the buffer has been read
           tc_fence_after();
-          if (lane == 0) {
+          const uint64_t xd = smem_desc_k128(smem_u32(dring + xb * Cfg::kXtBytes)), dd = smem_desc_k128(smem_u32(dzT));
+          const uint32_t dcol = tmem + static_cast<uint32_t>(kTAcc + buf * kDT);
+          if (elect_one()) {
             if (chain_ok) {
-              const uint32_t xa = smem_u32(dring + xb * Cfg::kXtBytes);
-              const uint32_t da = smem_u32(dzT);
-              const uint32_t dcol = tmem + static_cast<uint32_t>(kTAcc + buf * kDT);
 #pragma unroll
-              for (int j = 0; j < kFBK / 16; ++j)
-                umma_bf16(dcol, smem_desc_k128(da + j * 32), smem_desc_k128(xa + j * 32), idesc, j != 0 ? 1u : 0u);
+              for (int j = 0; j < kFBK / 16; ++j) umma_bf16(dcol, dd + 2 * j, xd + 2 * j, idesc, j != 0 ? 1u : 0u);
             }
             umma_commit(&accD[buf]);
             umma_commit(&xfreeD[xb]);

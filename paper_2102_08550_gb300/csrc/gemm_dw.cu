@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
   uint8_t* sShadow = smem + kDwOffShadow;      // [2 boxes][128 rows][128 B]
   DwBars* bars = reinterpret_cast<DwBars*>(smem + kDwOffBar);
 
-  const int warp = threadIdx.x >> 5, lane_id = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane_id = threadIdx.x & 31;
   const int mt = a.M / kDwTile, nt = (a.N + kDwTile - 1) / kDwTile;
   const int tiles = a.n_active * mt * nt;
   const int nk = (a.K + kDwBK - 1) / kDwBK;
@@ -140,8 +140,8 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
       if (armed_ops[i]) mbar_wait(&bars->full[i], (armed_ops[i] - 1) & 1, a.err, kDevTimeoutFull);
       if (armed_master[i]) mbar_wait(&bars->mfull[i], (armed_master[i] - 1) & 1, a.err, kDevTimeoutFull);
     }
-  } else if (warp == 1 && lane_id == 0) {
-    // ---- MMA issuer
+  } else if (warp == 1) {
+    // ---- MMA issuer: the warp converged, one elected lane issues (see elect_one)
     constexpr uint32_t idesc = idesc_bf16_f32(kDwTile, kDwTile);
     int kc = 0, it = 0;
     bool ok = true;
@@ -154,16 +154,20 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
         const int s = kc & 1;
         if (!(ok = mbar_wait(&bars->full[s], (kc >> 1) & 1, a.err, kDevTimeoutFull))) break;
         tc_fence_after();
-        const uint32_t a_base = smem_u32(sOps + s * kDwOpBytes);
-        const uint32_t b_base = a_base + kDwOpBytes / 2;
+        const uint64_t ad = smem_desc_k128(smem_u32(sOps + s * kDwOpBytes));
+        const uint64_t bd = smem_desc_k128(smem_u32(sOps + s * kDwOpBytes + kDwOpBytes / 2));
+        if (elect_one()) {
 #pragma unroll
-        for (int j = 0; j < kDwBK / 16; ++j)
-          umma_bf16(acc, smem_desc_k128(a_base + j * 32), smem_desc_k128(b_base + j * 32), idesc, (kb | j) != 0 ? 1u : 0u);
-        umma_commit(&bars->empty[s]);
+          for (int j = 0; j < kDwBK / 16; ++j) umma_bf16(acc, ad + 2 * j, bd + 2 * j, idesc, (kb | j) != 0 ? 1u : 0u);
+          umma_commit(&bars->empty[s]);
+        }
+        __syncwarp();
       }
-      if (ok) umma_commit(&bars->afull[b]);
+      if (ok && elect_one()) umma_commit(&bars->afull[b]);
+      __syncwarp();
     }
-    umma_commit(&bars->mma_done);      // every product issued above has landed before TMEM is released
+    if (elect_one()) umma_commit(&bars->mma_done);   // every product issued above has landed before TMEM is released
+    __syncwarp();
     mbar_wait(&bars->mma_done, 0, a.err, kDevTimeoutAccum);
   } else if (warp >= 4) {
     // ---- epilogue: warp quarter q owns TMEM lanes [32 q, 32 q + 32) (tile rows),

@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(warps_for<EPI>() * 32) gemm_tc_kernel(const __
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(accum + 1);
   float* epi_tiles = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(full) + kBarrierBytes);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int li = blockIdx.z / SPLIT;
   const int rank = SPLIT > 1 ? static_cast<int>(cluster_ctarank()) : 0;
   const int wid = a.wid ? a.wid[li] : li, src = a.src ? a.src[li] : li;
@@ -252,8 +252,8 @@ __global__ void __launch_bounds__(warps_for<EPI>() * 32) gemm_tc_kernel(const __
         tma_load_3d(sB + s * Cfg::kBBytes, &mapB, k, n0, zb, &full[s]);
       }
     }
-  } else if (warp == 1 && lane == 0) {
-    // MMA issuer
+  } else if (warp == 1) {
+    // MMA issuer: the warp converged, one elected lane issues (see elect_one)
     // A MN-major (transpose-A bit 15) for the input gradient, K-major otherwise;
     // B MN-major (bit 16) when the input gradient reads G^T
     const bool bmn = EPI == kEpiDh && a.b_mn;
@@ -264,17 +264,21 @@ __global__ void __launch_bounds__(warps_for<EPI>() * 32) gemm_tc_kernel(const __
       tc_fence_after();
       const uint32_t a_base = smem_u32(sA + s * kABytes);
       const uint32_t b_base = smem_u32(sB + s * Cfg::kBBytes);
+      // K-major: 16 K-elements are 32 bytes along a row; MN-major: 16 rows of
+      // 128 bytes (the descriptor's address field counts 16 bytes)
+      const uint64_t ad = EPI == kEpiDh ? smem_desc_mn128(a_base, kABytes / 2) : smem_desc_k128(a_base);
+      const uint64_t bd = bmn ? smem_desc_mn128(b_base, 8192) : smem_desc_k128(b_base);
+      const uint32_t astep = EPI == kEpiDh ? 128 : 2, bstep = bmn ? 128 : 2;
+      if (elect_one()) {
 #pragma unroll
-      for (int j = 0; j < BK / 16; ++j) {
-        // K-major: 16 K-elements are 32 bytes along a row; MN-major: 16 rows of 128 bytes
-        const uint64_t adesc = EPI == kEpiDh ? smem_desc_mn128(a_base + j * 2048, kABytes / 2)
-                                             : smem_desc_k128(a_base + j * 32);
-        const uint64_t bdesc = bmn ? smem_desc_mn128(b_base + j * 2048, 8192) : smem_desc_k128(b_base + j * 32);
-        umma_bf16(tmem, adesc, bdesc, idesc, (kb | j) != 0 ? 1u : 0u);
+        for (int j = 0; j < BK / 16; ++j)
+          umma_bf16(tmem, ad + j * astep, bd + j * bstep, idesc, (kb | j) != 0 ? 1u : 0u);
+        umma_commit(&empty[s]);
       }
-      umma_commit(&empty[s]);
+      __syncwarp();
     }
-    umma_commit(accum);  // arrives once every issued MMA has completed
+    if (elect_one()) umma_commit(accum);  // arrives once every issued MMA has completed
+    __syncwarp();
   }
   __syncwarp();
 

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
   const uint32_t rank = cluster_ctarank();
   const int ncl = static_cast<int>(gridDim.y);
   const int k0 = blockIdx.y * F;
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane = t & 31;
   const int64_t so = static_cast<int64_t>(src) * a.slot_stride;
   const int64_t dof = static_cast<int64_t>(w) * a.slot_stride;
 
@@ -185,18 +185,22 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
   pdl_trigger();
 
   // ---- 1. partial logits
-  if (t == 0) {
-    if (mbar_wait(tma_bar, 0, a.err, kDevTimeoutFull)) {
-      tc_fence_after();
-      constexpr uint32_t idesc = idesc_bf16_f32(kHTRows, kHTN);
+  if (warp == 0) {   // converged, one elected lane issues: see elect_one
+    const bool landed = mbar_wait(tma_bar, 0, a.err, kDevTimeoutFull);
+    tc_fence_after();
+    constexpr uint32_t idesc = idesc_bf16_f32(kHTRows, kHTN);
+    const uint64_t hd = smem_desc_k128(smem_u32(hT)), wd = smem_desc_k128(smem_u32(w2));   // addresses in 16 bytes
+    if (elect_one()) {
+      if (landed)
 #pragma unroll
-      for (int kb = 0; kb < F / 64; ++kb)
+        for (int kb = 0; kb < F / 64; ++kb)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          umma_bf16(tmem, smem_desc_k128(smem_u32(hT + kb * kHTRows * 128) + j * 32),
-                    smem_desc_k128(smem_u32(w2 + kb * kHTN * 128) + j * 32), idesc, (kb | j) != 0 ? 1u : 0u);
+          for (int j = 0; j < 4; ++j)
+            umma_bf16(tmem, hd + kb * (kHTRows * 128 / 16) + 2 * j, wd + kb * (kHTN * 128 / 16) + 2 * j, idesc,
+                      (kb | j) != 0 ? 1u : 0u);
+      umma_commit(mma_bar);   // arrives even with nothing issued, so the waits below end
     }
-    umma_commit(mma_bar);   // arrives even with nothing issued, so the waits below end
+    __syncwarp();
   }
   bool ok = mbar_wait(mma_bar, 0, a.err, kDevTimeoutAccum);
   tc_fence_after();
@@ -276,16 +280,19 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
   tc_fence_after();
 
   // ---- 3. head weight gradient (M = features, N = classes, K = rows) + SGD
-  if (t == 0) {
-    if (ok) {
-      constexpr uint32_t idesc = idesc_bf16_f32(kHT, kHTN) | (1u << 15);   // A (h^T) MN-major
+  if (warp == 0) {
+    constexpr uint32_t idesc = idesc_bf16_f32(kHT, kHTN) | (1u << 15);   // A (h^T) MN-major
+    const uint64_t hd = smem_desc_mn128(smem_u32(hT), kHTRows * 128), zd = smem_desc_k128(smem_u32(dzT));
+    if (elect_one()) {
+      if (ok)
 #pragma unroll
-      for (int mh = 0; mh < NH; ++mh)   // half mh: features [128 mh, 128 mh + 128) into columns [16 mh, 16 mh + 16)
-        for (int j = 0; j < B / 16; ++j)
-          umma_bf16(tmem + 16 * mh, smem_desc_mn128(smem_u32(hT + mh * 2 * kHTRows * 128) + j * 2048, kHTRows * 128),
-                    smem_desc_k128(smem_u32(dzT + (j >> 2) * (kHTN * 128)) + (j & 3) * 32), idesc, j != 0 ? 1u : 0u);
+        for (int mh = 0; mh < NH; ++mh)   // half mh: features [128 mh, 128 mh + 128) into columns [16 mh, 16 mh + 16)
+          for (int j = 0; j < B / 16; ++j)
+            umma_bf16(tmem + 16 * mh, hd + mh * (2 * kHTRows * 128 / 16) + 128 * j,
+                      zd + (j >> 2) * (kHTN * 128 / 16) + 2 * (j & 3), idesc, j != 0 ? 1u : 0u);
+      umma_commit(mma_bar);
     }
-    umma_commit(mma_bar);
+    __syncwarp();
   }
   if (rank == 0 && warp >= 4) {   // loss partials and the head bias (CUDA cores, meanwhile)
     const int u = t - 128;
@@ -334,15 +341,17 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
   tc_fence_after();
 
   // ---- 4. input gradient, transposed (M = features, N = rows, K = 16 classes)
-  if (t == 0) {
-    if (ok) {
-      const uint32_t idesc = idesc_bf16_f32(kHT, B) | (1u << 15);   // A (W2^T) MN-major
+  if (warp == 0) {
+    const uint32_t idesc = idesc_bf16_f32(kHT, B) | (1u << 15);   // A (W2^T) MN-major
+    const uint64_t wd = smem_desc_mn128(smem_u32(w2), kHTN * 128), kd = smem_desc_none(smem_u32(dzK), 128, 256);
+    if (elect_one()) {
+      if (ok)
 #pragma unroll
-      for (int mh = 0; mh < NH; ++mh)   // half mh into columns [B mh, B mh + B)
-        umma_bf16(tmem + B * mh, smem_desc_mn128(smem_u32(w2 + mh * 2 * kHTN * 128), kHTN * 128),
-                  smem_desc_none(smem_u32(dzK), 128, 256), idesc, 0u);
+        for (int mh = 0; mh < NH; ++mh)   // half mh into columns [B mh, B mh + B)
+          umma_bf16(tmem + B * mh, wd + mh * (2 * kHTN * 128 / 16), kd, idesc, 0u);
+      umma_commit(mma_bar);
     }
-    umma_commit(mma_bar);
+    __syncwarp();
   }
   ok = mbar_wait(mma_bar, 0, a.err, kDevTimeoutAccum) && ok;
   tc_fence_after();
