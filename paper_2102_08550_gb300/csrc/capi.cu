@@ -217,11 +217,11 @@ struct oscars_ctx {
   bool cnn_im2col = false;                   // stem over the im2col input (9 Cin <= 64): weights [64 out][64 k]
   __nv_bfloat16* cnn_wt = nullptr;           // [slot][2 * blocks][9][64 in][64 out]
   std::vector<__nv_bfloat16*> cnn_buf;       // x, s, (u_k, v_k) per block, dz0, dz1, dz2: [W][B][1024][64]
-  std::vector<CUtensorMap> cnn_m6, cnn_m4, cnn_m2;   // per buffer: boxes of 6, 4 and 2 image rows
+  std::vector<CUtensorMap> cnn_m6, cnn_m4, cnn_m2, cnn_m1;   // per buffer: boxes of 6, 4, 2 and 1 image rows
   int sms = 0;                               // multiprocessors of the device
   std::vector<CUtensorMap> cnn_mw, cnn_mwt;  // weights per conv layer: forward layout, transposed (blocks)
-  float* cnn_g = nullptr;                    // [W][B][64] pooled features
-  float* cnn_dg = nullptr;                   // [W][B][64] their gradient
+  float* cnn_pool = nullptr;                 // [W][B][32][64] channel sums of the last activation's image rows
+  float* cnn_dg = nullptr;                   // [W][B][64] gradient of the pooled features
   float* cnn_wpart = nullptr;                // [layer][W][chunks][9][64][64]
   float* cnn_bpart = nullptr;                // [layer][W][B * 8][64]
   // streams / graph
@@ -1020,8 +1020,7 @@ cudaError_t enqueue_step_cnn(oscars_ctx* c, int s, int na, const int* wid, const
   const int X = 0, S = 1, dzbase = 2 + 2 * nb;
   auto U = [&](int k) { return 2 + 2 * k; };
   auto V = [&](int k) { return 3 + 2 * k; };
-  const int ipc = conv_wgrad_images_per_chunk(B, na, c->sms);
-  const int chunks = (B + ipc - 1) / ipc;
+  const int chunks = conv_wgrad_chunks(B, na, c->sms);
   const size_t wpl = static_cast<size_t>(c->W) * chunks * 9 * 64 * 64;          // weight partials per layer
   const size_t bpl = static_cast<size_t>(c->W) * tiles * 64;                    // bias partials per layer
   {
@@ -1040,7 +1039,8 @@ cudaError_t enqueue_step_cnn(oscars_ctx* c, int s, int na, const int* wid, const
     ProfScope ps(c, "cnn_stage", st);
     if ((e = launch_cnn_stage(a, na, st)) != cudaSuccess) return e;
   }
-  auto conv = [&](int mode, int layer, int in, int add, int mask, int out, float* bpart) -> cudaError_t {
+  auto conv = [&](int mode, int layer, int in, int add, int mask, int out, float* bpart,
+                  float* pool = nullptr) -> cudaError_t {
     ConvArgs a;
     std::memset(&a, 0, sizeof(a));
     a.wid = wid;
@@ -1049,15 +1049,15 @@ cudaError_t enqueue_step_cnn(oscars_ctx* c, int s, int na, const int* wid, const
     a.bias = c->slab;
     a.slot_stride = c->P_pad;
     a.off_bias = c->cnn_offB[layer];
-    a.add = add >= 0 ? c->cnn_buf[add] : nullptr;
-    a.mask = mask >= 0 ? c->cnn_buf[mask] : nullptr;
-    a.out = c->cnn_buf[out];
+    a.has_add = add >= 0;
+    a.pool_part = pool;
     a.bias_part = bpart;
     a.err = c->err;
     a.im2col = layer == 0 && c->cnn_im2col ? 1 : 0;
     ProfScope ps(c, mode == 0 ? "conv_fwd" : "conv_dgrad", st);
     return launch_conv_igemm(mode, a.im2col ? c->cnn_m4[in] : c->cnn_m6[in],
-                             mode == 0 ? c->cnn_mw[layer] : c->cnn_mwt[layer - 1], a, na,
+                             mode == 0 ? c->cnn_mw[layer] : c->cnn_mwt[layer - 1],
+                             ConvMaps{c->cnn_m4[add >= 0 ? add : out], c->cnn_m4[mask >= 0 ? mask : out], c->cnn_m1[out]}, a, na,
                              conv_ctas_per_worker(B, na, c->sms), st);
   };
   auto wgrad = [&](int layer, int in, int dz) -> cudaError_t {
@@ -1065,7 +1065,6 @@ cudaError_t enqueue_step_cnn(oscars_ctx* c, int s, int na, const int* wid, const
     a.wid = wid;
     a.B = B;
     a.n_chunks = chunks;
-    a.img_per_chunk = ipc;
     a.part = c->cnn_wpart + layer * wpl;
     a.err = c->err;
     a.im2col = layer == 0 && c->cnn_im2col ? 1 : 0;
@@ -1077,12 +1076,11 @@ cudaError_t enqueue_step_cnn(oscars_ctx* c, int s, int na, const int* wid, const
   for (int k = 0; k < nb; ++k) {
     const int h = k == 0 ? S : V(k - 1);
     if ((e = conv(0, 1 + 2 * k, h, -1, -1, U(k), nullptr)) != cudaSuccess) return e;
-    if ((e = conv(0, 2 + 2 * k, U(k), h, -1, V(k), nullptr)) != cudaSuccess) return e;
+    if ((e = conv(0, 2 + 2 * k, U(k), h, -1, V(k), nullptr, k == nb - 1 ? c->cnn_pool : nullptr)) != cudaSuccess) return e;
   }
   // head: pooling, FC, softmax cross-entropy, its backward and SGD
   {
     ProfScope ps(c, "cnn_head", st);
-    if ((e = launch_cnn_pool(c->cnn_buf[V(nb - 1)], wid, B, c->cnn_g, na, st)) != cudaSuccess) return e;
     CnnHeadArgs h;
     h.wid = wid;
     h.src = src;
@@ -1091,7 +1089,7 @@ cudaError_t enqueue_step_cnn(oscars_ctx* c, int s, int na, const int* wid, const
     h.step = s;
     h.max_tau = c->max_tau;
     h.n_loss_chunks = B / kRowsPerLossChunk;
-    h.g = c->cnn_g;
+    h.pool_part = c->cnn_pool;
     h.labels = c->labels;
     h.dg = c->cnn_dg;
     h.loss_part = c->loss_part;
@@ -1338,7 +1336,7 @@ oscars_status allocate_cnn(oscars_ctx* c) {
   if (cudaMemset(c->cnn_buf[0], 0, act * sizeof(__nv_bfloat16)) != cudaSuccess)
     return fail(c, OSCARS_ECUDA, "clearing the input buffer failed");
   const size_t tiles = static_cast<size_t>(B) * cnn_tiles_per_image();
-  if (!dev_alloc(c, &c->cnn_g, static_cast<size_t>(W) * B * 64) ||
+  if (!dev_alloc(c, &c->cnn_pool, static_cast<size_t>(W) * B * 32 * 64) ||
       !dev_alloc(c, &c->cnn_dg, static_cast<size_t>(W) * B * 64) ||
       !dev_alloc(c, &c->labels, static_cast<size_t>(W) * B) ||
       !dev_alloc(c, &c->cnn_wpart, static_cast<size_t>(layers) * W * c->cnn_chunks * 9 * 64 * 64) ||
@@ -1348,6 +1346,7 @@ oscars_status allocate_cnn(oscars_ctx* c) {
   c->cnn_m6.resize(nbuf);
   c->cnn_m4.resize(nbuf);
   c->cnn_m2.resize(nbuf);
+  c->cnn_m1.resize(nbuf);
   const uint64_t imgs = static_cast<uint64_t>(W) * B;
   bool ok = true;
   for (int i = 0; i < nbuf; ++i) {
@@ -1356,6 +1355,7 @@ oscars_status allocate_cnn(oscars_ctx* c) {
     ok &= make_map_box4(&c->cnn_m6[i], c->cnn_buf[i], d, stv, {64, 32, 6, 1});
     ok &= make_map_box4(&c->cnn_m4[i], c->cnn_buf[i], d, stv, {64, 32, 4, 1});
     ok &= make_map_box4(&c->cnn_m2[i], c->cnn_buf[i], d, stv, {64, 32, 2, 1});
+    ok &= make_map_box4(&c->cnn_m1[i], c->cnn_buf[i], d, stv, {64, 32, 1, 1});
   }
   c->cnn_mw.resize(layers);
   c->cnn_mwt.resize(layers > 1 ? layers - 1 : 1);
@@ -2055,7 +2055,7 @@ oscars_status eval_cnn(oscars_ctx* c, const float* x, const int32_t* y, int64_t 
     a.out = c->cnn_buf[0];
     a.labels = c->labels;
     cudaError_t e = launch_cnn_stage(a, na, c->stream);
-    auto conv = [&](int layer, int in, int add, int out) -> cudaError_t {
+    auto conv = [&](int layer, int in, int add, int out, float* pool) -> cudaError_t {
       ConvArgs ca;
       std::memset(&ca, 0, sizeof(ca));
       ca.wid = c->lane_ids;
@@ -2064,23 +2064,22 @@ oscars_status eval_cnn(oscars_ctx* c, const float* x, const int32_t* y, int64_t 
       ca.bias = c->slab;
       ca.slot_stride = c->P_pad;
       ca.off_bias = c->cnn_offB[layer];
-      ca.add = add >= 0 ? c->cnn_buf[add] : nullptr;
-      ca.out = c->cnn_buf[out];
+      ca.has_add = add >= 0;
+      ca.pool_part = pool;
       ca.err = c->err;
       ca.im2col = layer == 0 && c->cnn_im2col ? 1 : 0;
-      return launch_conv_igemm(0, ca.im2col ? c->cnn_m4[in] : c->cnn_m6[in], c->cnn_mw[layer], ca, na,
+      return launch_conv_igemm(0, ca.im2col ? c->cnn_m4[in] : c->cnn_m6[in], c->cnn_mw[layer],
+                               ConvMaps{c->cnn_m4[add >= 0 ? add : out], c->cnn_m4[out], c->cnn_m1[out]}, ca, na,
                                conv_ctas_per_worker(B, na, c->sms), c->stream);
     };
-    if (e == cudaSuccess) e = conv(0, 0, -1, 1);
+    if (e == cudaSuccess) e = conv(0, 0, -1, 1, nullptr);
     for (int k = 0; e == cudaSuccess && k < c->cnn_blocks; ++k) {
       const int h = k == 0 ? 1 : 3 + 2 * (k - 1);
-      e = conv(1 + 2 * k, h, -1, 2 + 2 * k);
-      if (e == cudaSuccess) e = conv(2 + 2 * k, 2 + 2 * k, h, 3 + 2 * k);
+      e = conv(1 + 2 * k, h, -1, 2 + 2 * k, nullptr);
+      if (e == cudaSuccess) e = conv(2 + 2 * k, 2 + 2 * k, h, 3 + 2 * k, k == c->cnn_blocks - 1 ? c->cnn_pool : nullptr);
     }
     if (e == cudaSuccess)
-      e = launch_cnn_pool(c->cnn_buf[3 + 2 * (c->cnn_blocks - 1)], c->lane_ids, B, c->cnn_g, na, c->stream);
-    if (e == cudaSuccess)
-      e = launch_cnn_head_loss(c->cnn_g, c->labels, na, B, n - lane0 * B, c->C, c->slab + g, c->cnn_offWf, c->cnn_offBf,
+      e = launch_cnn_head_loss(c->cnn_pool, c->labels, na, B, n - lane0 * B, c->C, c->slab + g, c->cnn_offWf, c->cnn_offBf,
                                c->eval_part + lane0, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "eval");
   }

@@ -23,14 +23,14 @@
 //    gradient.
 //  * conv_wgrad_kernel: dW[o][tap][i] = sum_p dz[p][o] x[p + off(tap)][i] on
 //    tcgen05 with both operands MN-major straight from the NHWC tensors: the
-//    K dimension is the pixels, taps are stacked in pairs to make M = 128
-//    (in-channels of two taps), N = 64 out-channels; one 4-row input box per
-//    x-offset serves the three y-offsets.  Split over chunks of images (one
-//    wave of CTAs); partial sums go to global memory.
+//    K dimension is the pixels, M = 128 (in-channels of two taps), N = 192
+//    (out-channels of three x-offsets).  Split over chunks of the worker's
+//    pixels (one wave of CTAs); partial sums go to global memory.
 //  * conv_sgd_kernel: sums the chunks in order, SGD of the fp32 master and
 //    its bf16 copies (the forward layout and the transposed one), bias from
 //    the per-tile sums.
-//  * pool, head, and output-gradient kernels on CUDA cores; input staging.
+//  * head (pooling of the last convolution's row sums, FC, softmax) and
+//    output-gradient kernels on CUDA cores; input staging.
 #include "common.cuh"
 #include "internal.h"
 
@@ -49,7 +49,6 @@ constexpr int kCB = kCC * kCC * 2;          // 8 KB: one tap of the weights
 // weight gradient
 constexpr int kWT = 128;
 constexpr int kWTile = 2 * kImg * kCC * 2;  // 8 KB: 64 pixels (2 rows) x 64 channels
-constexpr int kWPairs = 5;                  // accumulators of stacked tap pairs
 
 __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
   return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~uintptr_t(1023));
@@ -61,29 +60,47 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 // in shared memory.  Per tile and x-offset dx one TMA box of 6 image rows
 // (rows y0 - 1 .. y0 + 4, shifted by the x-offset) is loaded; the three
 // y-offsets are its 4-row sub-tiles at row offsets 0, 1, 2 (multiples of 8
-// pixel rows of 128 bytes, so the 128-byte swizzle phase is unchanged).  Two
-// TMEM accumulators: the epilogue of one tile overlaps the MMAs of the next.
-constexpr int kGT = 192;                    // warp 0 TMA, warp 1 MMA, warps 2-5 epilogue
-constexpr int kGSlots = 6;                  // input boxes in flight (two tiles)
+// pixel rows of 128 bytes, so the 128-byte swizzle phase is unchanged).
+//
+// Two TMEM accumulators and two epilogue warpgroups, tile k with accumulator
+// and group k % 2: the epilogues of two tiles overlap the MMAs of a third.
+// What an epilogue reads beside the accumulator (the residual, the mask, the
+// skip gradient) comes by TMA into a tile buffer of its group, laid out like
+// the output; a thread (one pixel) updates its 128-byte row there in place,
+// and a warp (one image row) sends it out with one TMA store.  Loads and
+// stores of a pixel's row by its thread touched 32 lines an instruction: they
+// took the load/store unit about 2000 clocks a tile, four times the MMAs, and
+// the kernels ran at 41 us (forward) and 60 us (input gradient) a launch of
+// up to 16 workers; 36 and 48 us with this epilogue.
+constexpr int kGT = 320;                    // warp 0 TMA, warp 1 MMA, warps 2-5 and 6-9 epilogue
+constexpr int kGSlots = 4;                  // input boxes in flight
 constexpr int kGBox = 6 * kImg * kCC * 2;   // 24 KB: 6 rows x 32 pixels x 64 channels
 constexpr int kGW = kTaps * kCB;            // 72 KB of resident weights
-constexpr int kGSmem = kGW + kGSlots * kGBox + 512 + 1024;   // + barriers, TMEM slot, bias
-static_assert(kTilePix * (kCC + 1) * 4 <= kGSlots * kGBox, "the bias reduction reuses the input slots");
+constexpr int kGTile = kTilePix * kCC * 2;  // 16 KB: an output tile
+constexpr int kGOffE = kGW + kGSlots * kGBox;      // [2] tile buffer of a group: residual or mask, then the output
+constexpr int kGOffS = kGOffE + 2 * kGTile;        // skip gradient (input gradient)
+constexpr int kGOffBar = kGOffS + kGTile;
+constexpr int kGSmem = kGOffBar + 512 + 1024;      // + barriers, TMEM slot, bias
+static_assert(2 * kTilePix * (kCC + 1) * 4 <= kGSlots * kGBox, "the bias reduction reuses the input slots");
 
 template <int MODE>   // 0 forward, 1 input gradient
 __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constant__ CUtensorMap mIn,
                                                             const __grid_constant__ CUtensorMap mW,
+                                                            const __grid_constant__ ConvMaps mm,
                                                             const __grid_constant__ ConvArgs a) {
   extern __shared__ uint8_t cs_raw[];
   uint8_t* sm = align1024(cs_raw);
   uint8_t* wts = sm;                 // [9][64][64] bf16, 128-byte swizzled K-major
   uint8_t* slots = sm + kGW;         // [kGSlots][6 rows][32][64]
-  uint64_t* wfull = reinterpret_cast<uint64_t*>(slots + kGSlots * kGBox);
+  uint64_t* wfull = reinterpret_cast<uint64_t*>(sm + kGOffBar);
   uint64_t* full = wfull + 1;
   uint64_t* empty = full + kGSlots;
   uint64_t* accf = empty + kGSlots;  // [2]
   uint64_t* acce = accf + 2;         // [2] 128 arrivals
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(acce + 2);
+  uint64_t* auxf = acce + 2;         // [2] the tile buffer (and skip gradient) has landed
+  uint64_t* auxe = auxf + 2;         // [2] the tile buffer has been stored: 4 arrivals
+  uint64_t* skipe = auxe + 2;        // the skip gradient has been read: 4 arrivals
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(skipe + 1);
   float* bias_s = reinterpret_cast<float*>(tslot + 4);   // [64] this worker's bias (forward)
   const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane_id = t & 31;
   const int c0 = blockIdx.x, cpw = gridDim.x, e = blockIdx.y;
@@ -93,6 +110,7 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
   if (t == 0) {
     prefetch_tmap(&mIn);
     prefetch_tmap(&mW);
+    prefetch_tmap(&mm.out1);
     mbar_init(wfull, 1);
     for (int i = 0; i < kGSlots; ++i) {
       mbar_init(&full[i], 1);
@@ -101,7 +119,10 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
     for (int i = 0; i < 2; ++i) {
       mbar_init(&accf[i], 1);
       mbar_init(&acce[i], 128);
+      mbar_init(&auxf[i], 1);
+      mbar_init(&auxe[i], 4);
     }
+    mbar_init(skipe, 4);
     fence_barrier_init();
   }
   if (warp == 0) {
@@ -119,6 +140,9 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
   // box is {64, 32, 4, 1}), four MMAs
   const bool one_tap = MODE == 0 && a.im2col;
   const int nbox = one_tap ? 1 : 3;
+  // forward: the residual (if any) in the tile buffer; input gradient: the
+  // mask there and the skip gradient (if any) in its own buffer
+  const bool aux = MODE == 1 || a.has_add, skip = MODE == 1 && a.has_add;
   if (t == 0) {
     mbar_arrive_expect_tx(wfull, one_tap ? kCB : kGW);
     for (int tap = 0; tap < (one_tap ? 1 : kTaps); ++tap) {
@@ -142,6 +166,15 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
           mbar_arrive_expect_tx(&full[sl], kGBox);
           tma_load_4d(slots + sl * kGBox, &mIn, 0, sgn * (dx - 1), y0 - 1, img, &full[sl]);
         }
+      }
+      if (aux && k < my_tiles) {
+        const int p = k & 1, use = k >> 1;
+        // the group's previous output has left the tile buffer; the previous tile has read the skip gradient
+        if (use >= 1 && !mbar_wait(&auxe[p], (use - 1) & 1, a.err, kDevTimeoutEmpty)) break;
+        if (skip && k >= 1 && !mbar_wait(skipe, (k - 1) & 1, a.err, kDevTimeoutEmpty)) break;
+        mbar_arrive_expect_tx(&auxf[p], skip ? 2 * kGTile : kGTile);
+        tma_load_4d(sm + kGOffE + p * kGTile, MODE == 1 ? &mm.mask4 : &mm.add4, 0, 0, y0, img, &auxf[p]);
+        if (skip) tma_load_4d(sm + kGOffS, &mm.add4, 0, 0, y0, img, &auxf[p]);
       }
     }
   } else if (warp == 1) {   // converged, one elected lane issues: see elect_one
@@ -185,24 +218,28 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
       __syncwarp();
     }
   } else if (warp >= 2) {
-    // epilogue: thread = output pixel (TMEM lane of its warp's quarter), 64 channels
-    const int quarter = warp & 3;
+    // epilogue: thread = output pixel (TMEM lane of its warp's quarter), 64
+    // channels; warp = image row y0 + quarter
+    const int grp = (warp - 2) >> 2, quarter = warp & 3;
     const int p = quarter * 32 + lane_id;
-    const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+    const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + grp * kCC;
+    uint8_t* row = sm + kGOffE + grp * kGTile + p * 128;          // 16-byte chunk q at (q ^ (p & 7))
+    const uint8_t* srow = sm + kGOffS + p * 128;
+    const uint32_t sw = static_cast<uint32_t>(p & 7);
     float bsum[kCC];
 #pragma unroll
     for (int c = 0; c < kCC; ++c) bsum[c] = 0.f;
-    for (int k = 0; k < my_tiles; ++k) {
+    for (int k = grp; k < my_tiles; k += 2) {
       const int tile = c0 + k * cpw;
       const int img = lane * a.B + tile / kTilesPerImg, y0 = (tile % kTilesPerImg) * kTileRows;
-      const int buf = k & 1, use = k >> 1;
-      int ok = mbar_wait(&accf[buf], use & 1, a.err, kDevTimeoutAccum) ? 1 : 0;
+      const int use = k >> 1;
+      int ok = mbar_wait(&accf[grp], use & 1, a.err, kDevTimeoutAccum) ? 1 : 0;
       ok = __all_sync(0xffffffffu, ok);
       tc_fence_after();
       float v[kCC];
       {
         float lo[32], hi[32];
-        tmem_ld_32x32b_x32_pair(trow + buf * kCC, lo, trow + buf * kCC + 32, hi);
+        tmem_ld_32x32b_x32_pair(trow, lo, trow + 32, hi);
 #pragma unroll
         for (int c = 0; c < 32; ++c) {
           v[c] = ok ? lo[c] : 0.f;
@@ -210,16 +247,21 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
         }
       }
       tc_fence_before();
-      mbar_arrive(&acce[buf]);   // the accumulator has been read: the next tile may use it
-      const int64_t base = (static_cast<int64_t>(img) * kPix + y0 * kImg + p) * kCC;
+      mbar_arrive(&acce[grp]);   // the accumulator has been read: the next tile may use it
       if (MODE == 0) {
 #pragma unroll
         for (int c = 0; c < kCC; ++c) v[c] += bias_s[c];
       }
-      if (a.add) {
+      if (aux) {
+        mbar_wait(&auxf[grp], use & 1, a.err, kDevTimeoutFull);
+      } else {   // this warp's previous output has left its rows
+        if (lane_id == 0) bulk_wait_read_all();
+        __syncwarp();
+      }
+      if (a.has_add) {
 #pragma unroll
         for (int q = 0; q < kCC / 8; ++q) {
-          const uint4 r = *reinterpret_cast<const uint4*>(a.add + base + 8 * q);
+          const uint4 r = *reinterpret_cast<const uint4*>((MODE == 0 ? row : srow) + ((q ^ sw) << 4));
           const __nv_bfloat162* r2 = reinterpret_cast<const __nv_bfloat162*>(&r);
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
@@ -228,6 +270,10 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
             v[8 * q + 2 * j + 1] += f.y;
           }
         }
+        if (skip) {
+          __syncwarp();
+          if (lane_id == 0) mbar_arrive(skipe);
+        }
       }
       if (MODE == 0) {
 #pragma unroll
@@ -235,7 +281,7 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
       } else {
 #pragma unroll
         for (int q = 0; q < kCC / 8; ++q) {
-          const uint4 r = *reinterpret_cast<const uint4*>(a.mask + base + 8 * q);
+          const uint4 r = *reinterpret_cast<const uint4*>(row + ((q ^ sw) << 4));
           const __nv_bfloat162* r2 = reinterpret_cast<const __nv_bfloat162*>(&r);
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
@@ -248,27 +294,72 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
         for (int c = 0; c < kCC; ++c) bsum[c] += v[c];
       }
 #pragma unroll
-      for (int q = 0; q < kCC / 8; ++q)
-        *reinterpret_cast<uint4*>(a.out + base + 8 * q) =
-            make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
-                       pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
+      for (int q = 0; q < kCC / 8; ++q) {
+        const uint4 o = make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
+                                   pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
+        *reinterpret_cast<uint4*>(row + ((q ^ sw) << 4)) = o;
+        if (MODE == 0 && a.pool_part) {   // the pooling sums the stored values
+          const __nv_bfloat162* o2 = reinterpret_cast<const __nv_bfloat162*>(&o);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float2 f = __bfloat1622float2(o2[j]);
+            v[8 * q + 2 * j] = f.x;
+            v[8 * q + 2 * j + 1] = f.y;
+          }
+        }
+      }
+      fence_proxy_async_smem();   // the rows are read by the TMA store
+      __syncwarp();
+      if (lane_id == 0) {
+        tma_store_4d(&mm.out1, sm + kGOffE + grp * kGTile + quarter * 32 * 128, 0, 0, y0 + quarter, img);
+        bulk_commit_group();
+      }
+      if (MODE == 0 && a.pool_part) {
+        // channel sums over the image row's 32 pixels: halves exchanged over
+        // the lanes until a lane holds two channels
+#pragma unroll
+        for (int w = 32, o = 16; o > 0; w >>= 1, o >>= 1) {
+          const bool up = lane_id & o;
+#pragma unroll
+          for (int c = 0; c < 32; ++c)
+            if (c < w) {
+              const float keep = up ? v[c + w] : v[c], give = up ? v[c] : v[c + w];
+              v[c] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+        }
+        // the lane's bits chose halves of 32, 16, 8, 4, 2 channels: channels 2 lane', 2 lane' + 1
+        const int ch = ((lane_id & 16) ? 32 : 0) + ((lane_id & 8) ? 16 : 0) + ((lane_id & 4) ? 8 : 0) +
+                       ((lane_id & 2) ? 4 : 0) + ((lane_id & 1) ? 2 : 0);
+        *reinterpret_cast<float2*>(a.pool_part + (static_cast<int64_t>(img) * kImg + y0 + quarter) * kCC + ch) =
+            make_float2(v[0], v[1]);
+      }
+      if (aux && lane_id == 0) {   // the tile buffer may take the next tile's inputs
+        bulk_wait_read_all();
+        mbar_arrive(&auxe[grp]);
+      }
     }
+    if (lane_id == 0) bulk_wait_all();
     if (MODE == 1 && a.bias_part) {
+      bar_named(1, 256);   // both groups have seen their last product: the input slots are idle
       // this CTA's channel sums: per thread over its tiles in order, then over
-      // the 128 pixels of the tile in pixel order (the input slots are idle now)
+      // the two groups' 128 pixels in order
       float* T = reinterpret_cast<float*>(slots);
 #pragma unroll
-      for (int c = 0; c < kCC; ++c) T[p * (kCC + 1) + c] = bsum[c];
+      for (int c = 0; c < kCC; ++c) T[(grp * kTilePix + p) * (kCC + 1) + c] = bsum[c];
     }
   }
   if (MODE == 1 && a.bias_part) {
     __syncthreads();
-    if (t < kCC) {
-      const float* T = reinterpret_cast<const float*>(slots);
+    float* T = reinterpret_cast<float*>(slots);
+    float* part = reinterpret_cast<float*>(sm + kGOffE);   // [4][64]: every store has left the tile buffers
+    if (t < 256) {
       float s = 0.f;
-      for (int q = 0; q < kTilePix; ++q) s += T[q * (kCC + 1) + t];
-      a.bias_part[(static_cast<int64_t>(lane) * cpw + c0) * kCC + t] = s;
+      for (int q = (t >> 6) * 64; q < (t >> 6) * 64 + 64; ++q) s += T[q * (kCC + 1) + (t & 63)];
+      part[t] = s;
     }
+    __syncthreads();
+    if (t < kCC)
+      a.bias_part[(static_cast<int64_t>(lane) * cpw + c0) * kCC + t] = part[t] + part[64 + t] + part[128 + t] + part[192 + t];
   }
   tc_fence_before();
   __syncthreads();
@@ -279,38 +370,28 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
 }
 
 // ------------------------------------------------------------------ weight gradient
-// K-block = 64 pixels (2 image rows yr, yr + 1).  Per K-block TMA loads the
-// output-gradient tile (2 rows) and, per x-offset dx, one 4-row box of the
-// input (rows yr - 1 .. yr + 2, shifted by dx - 1); tap (dy, dx)'s operand is
-// the box's 2-row sub-tile at row offset dy.  The A operand (M = 128) stacks
-// two taps as two 64-channel atoms `lbo` bytes apart:
-//   pair 0..2: (dy 0, dy 1) of box dx = pair      (atoms 4 KB apart)
-//   pair 3:    dy 2 of box 0 and of box 1         (atoms one box apart)
-//   pair 4:    dy 2 of box 2                      (upper half unused)
+// K-block = 64 pixels (2 image rows yr, yr + 1).  Per K-block TMA loads one
+// 4-row box of the input (rows yr - 1 .. yr + 2) and the two output-gradient
+// rows three times, shifted by 1 - dx pixels: sum_p dz[p] x[p + off] over the
+// pixels p equals the sum over q = p + (0, dx - 1) of dz[q - (0, dx - 1)]
+// x[q + (dy - 1, 0)], and TMA's zero fill drops the terms outside the image.
+// So every tap of one dx has the same B, and one MMA covers
+//   M = 128: two 64-channel atoms of the input 4 KB apart (dy 0 and dy 1; for
+//            dy 2 the upper half is not used)
+//   N = 192: the three shifted output gradients, 64 channels each, 8 KB apart
+// - 8 MMAs a K-block for the nine taps.  What bounds the kernel is the shared
+// memory that the operands are read from (about 128 bytes a clock) and TMA
+// writes: 80 + 40 KB a K-block; with the input shifted instead (three boxes,
+// 20 MMAs of N = 64) it was 120 + 56 KB and 1350 clocks a K-block: 43 us a
+// launch of up to 16 workers, 32 now (nine chunks a worker instead of eight
+// whole-image ones and coalesced partial rows included).
 constexpr int kWRow = kImg * kCC * 2;           // 4 KB: one image row, 64 channels
 constexpr int kWBox = 4 * kWRow;                // 16 KB
-constexpr int kWStage2 = 3 * kWBox + kWTile;    // 56 KB: three input boxes + the output-gradient tile
-constexpr int kWStages2 = 3;
+constexpr int kWStage2 = kWBox + 3 * kWTile;    // 40 KB: the input box and three output-gradient tiles
+constexpr int kWStages2 = 5;
 constexpr int kWSmem2 = kWStages2 * kWStage2 + 256 + 1024;
-
-__device__ __forceinline__ void wgrad_pair(int pr, int& start, int& lbo, int& tap0, int& tap1) {
-  if (pr < 3) {
-    start = pr * kWBox;
-    lbo = kWRow;
-    tap0 = pr;            // (dy 0, dx pr)
-    tap1 = 3 + pr;        // (dy 1, dx pr)
-  } else if (pr == 3) {
-    start = 2 * kWRow;
-    lbo = kWBox;
-    tap0 = 6;             // (dy 2, dx 0)
-    tap1 = 7;             // (dy 2, dx 1)
-  } else {
-    start = 2 * kWBox + 2 * kWRow;
-    lbo = kWRow;
-    tap0 = 8;             // (dy 2, dx 2)
-    tap1 = -1;
-  }
-}
+constexpr int kWLd = kCC + 4;                   // row stride of the epilogue's staging (floats): conflict-free both ways
+static_assert(kWT / 32 * 32 * kWLd * 4 <= kWStages2 * kWStage2, "the epilogue stages in the operand ring");
 
 __global__ void __launch_bounds__(kWT, 1) conv_wgrad_kernel(const __grid_constant__ CUtensorMap mIn,
                                                             const __grid_constant__ CUtensorMap mDz,
@@ -321,12 +402,12 @@ __global__ void __launch_bounds__(kWT, 1) conv_wgrad_kernel(const __grid_constan
   uint64_t* empty = full + kWStages2;
   uint64_t* accb = empty + kWStages2;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(accb + 1);
-  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0);
+  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane_id = t & 31;
   const int chunk = blockIdx.x, e = blockIdx.y;
   const int lane = a.wid[e];
-  const int i0 = chunk * a.img_per_chunk;
-  const int n_img = min(a.img_per_chunk, a.B - i0);
-  const int nk = n_img * (kImg / 2);             // K-blocks: 64 pixels = 2 image rows
+  const int all = a.B * (kImg / 2);              // the worker's K-blocks; this chunk's [kb0, kb0 + nk)
+  const int kb0 = static_cast<int>(static_cast<int64_t>(chunk) * all / a.n_chunks);
+  const int nk = static_cast<int>(static_cast<int64_t>(chunk + 1) * all / a.n_chunks) - kb0;
   if (t == 0) {
     prefetch_tmap(&mIn);
     prefetch_tmap(&mDz);
@@ -345,48 +426,43 @@ __global__ void __launch_bounds__(kWT, 1) conv_wgrad_kernel(const __grid_constan
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
-  // im2col stem: one 2-row input box per K-block (mIn's box is {64, 32, 2, 1})
-  // and one accumulator, tap 0 in its lower half
-  const int npairs = a.im2col ? 1 : kWPairs;
+  // im2col stem: one 2-row input box per K-block (mIn's box is {64, 32, 2, 1}),
+  // one unshifted output-gradient tile and one accumulator, tap 0 in its lower half
   if (t == 0) {
     for (int kb = 0; kb < nk; ++kb) {
       const int st = kb % kWStages2;
       if (kb >= kWStages2 && !mbar_wait(&empty[st], ((kb / kWStages2) + 1) & 1, a.err, kDevTimeoutEmpty)) break;
       uint8_t* sa = sm + st * kWStage2;
-      const int img = lane * a.B + i0 + kb / (kImg / 2), yr = (kb % (kImg / 2)) * 2;
+      const int img = lane * a.B + (kb0 + kb) / (kImg / 2), yr = ((kb0 + kb) % (kImg / 2)) * 2;
       if (a.im2col) {
         mbar_arrive_expect_tx(&full[st], 2 * kWRow + kWTile);
         tma_load_4d(sa, &mIn, 0, 0, yr, img, &full[st]);
+        tma_load_4d(sa + kWBox, &mDz, 0, 0, yr, img, &full[st]);
       } else {
         mbar_arrive_expect_tx(&full[st], kWStage2);
-        for (int dx = 0; dx < 3; ++dx) tma_load_4d(sa + dx * kWBox, &mIn, 0, dx - 1, yr - 1, img, &full[st]);
+        tma_load_4d(sa, &mIn, 0, 0, yr - 1, img, &full[st]);
+        for (int dx = 0; dx < 3; ++dx) tma_load_4d(sa + kWBox + dx * kWTile, &mDz, 0, 1 - dx, yr, img, &full[st]);
       }
-      tma_load_4d(sa + 3 * kWBox, &mDz, 0, 0, yr, img, &full[st]);
     }
   } else if (warp == 1) {   // converged, one elected lane issues: see elect_one
-    constexpr uint32_t idesc = idesc_bf16_f32_mn(128, kCC);
+    constexpr uint32_t idesc1 = idesc_bf16_f32_mn(128, kCC), idesc3 = idesc_bf16_f32_mn(128, 3 * kCC);
     for (int kb = 0; kb < nk; ++kb) {
       const int st = kb % kWStages2;
       if (!mbar_wait(&full[st], (kb / kWStages2) & 1, a.err, kDevTimeoutFull)) break;
       tc_fence_after();
       const uint32_t sa = smem_u32(sm + st * kWStage2);
-      const uint64_t sb = smem_desc_mn128(sa + 3 * kWBox, kWTile);
+      const uint64_t ad = smem_desc_mn128(sa, kWRow), bd = smem_desc_mn128(sa + kWBox, kWTile);
       if (elect_one()) {
-        if (a.im2col) {
-          // A = the 2-row box (in-channels k); its upper atom (the next row) is not read back
-          const uint64_t aa = smem_desc_mn128(sa, kWRow);
+        // K = 16 pixels per MMA: two 8-row groups, 2048 bytes (descriptors count 16)
+        if (a.im2col) {   // A's upper atom (the next row) is not read back
 #pragma unroll
-          for (int j = 0; j < 4; ++j) umma_bf16(tmem, aa + 128 * j, sb + 128 * j, idesc, (kb | j) != 0 ? 1u : 0u);
+          for (int j = 0; j < 4; ++j) umma_bf16(tmem, ad + 128 * j, bd + 128 * j, idesc1, (kb | j) != 0 ? 1u : 0u);
         } else {
 #pragma unroll
-          for (int pr = 0; pr < kWPairs; ++pr) {
-            int start, lbo, tap0, tap1;
-            wgrad_pair(pr, start, lbo, tap0, tap1);
-            const uint64_t aa = smem_desc_mn128(sa + start, lbo);
+          for (int j = 0; j < 4; ++j) umma_bf16(tmem, ad + 128 * j, bd + 128 * j, idesc3, (kb | j) != 0 ? 1u : 0u);
 #pragma unroll
-            for (int j = 0; j < 4; ++j)   // K = 16 pixels per MMA: two 8-row groups, 2048 bytes
-              umma_bf16(tmem + pr * kCC, aa + 128 * j, sb + 128 * j, idesc, (kb | j) != 0 ? 1u : 0u);
-          }
+          for (int j = 0; j < 4; ++j)   // dy 2: two image rows further
+            umma_bf16(tmem + 3 * kCC, ad + 2 * kWRow / 16 + 128 * j, bd + 128 * j, idesc3, (kb | j) != 0 ? 1u : 0u);
         }
         umma_commit(&empty[st]);
       }
@@ -398,24 +474,33 @@ __global__ void __launch_bounds__(kWT, 1) conv_wgrad_kernel(const __grid_constan
   int ok = mbar_wait(accb, 0, a.err, kDevTimeoutAccum) ? 1 : 0;
   ok = __all_sync(0xffffffffu, ok);
   tc_fence_after();
-  // TMEM lane r: row r of each pair's accumulator = (tap of atom r / 64, in-channel r % 64)
-  const int r = t;
-  const int ci = r & (kCC - 1);
-  for (int pr = 0; pr < npairs; ++pr) {
-    int start, lbo, tap0, tap1;
-    wgrad_pair(pr, start, lbo, tap0, tap1);
-    if (a.im2col) tap1 = -1;
-    const int tap = r < 64 ? tap0 : tap1;
+  // TMEM lane r: in-channel r % 64 of dy 0 (r < 64) and dy 1 in columns [0,
+  // 192), of dy 2 (r < 64) in [192, 384); columns dx * 64 + out-channel.  Rows
+  // of 64 go through shared memory (the ring is idle: every product is done)
+  // so that a warp writes whole 256-byte rows, two an instruction.
+  float* T = reinterpret_cast<float*>(sm) + warp * 32 * kWLd;
+  const uint32_t trow = tmem + (static_cast<uint32_t>(warp * 32) << 16);
+  const int ci0 = (warp & 1) * 32;
+  float* part = a.part + (static_cast<int64_t>(lane) * a.n_chunks + chunk) * kTaps * kCC * kCC;
+  for (int i = 0; i < 6; ++i) {
+    const int dy = i < 3 ? warp >> 1 : 2, dx = i % 3;
+    if (i >= 3 && warp >= 2) break;            // dy 2: lanes 0..63
+    if (a.im2col && (i > 0 || warp >= 2)) break;
     float lo[32], hi[32];
-    tmem_ld_32x32b_x32_pair(tmem + (static_cast<uint32_t>(warp * 32) << 16) + pr * kCC, lo,
-                            tmem + (static_cast<uint32_t>(warp * 32) << 16) + pr * kCC + 32, hi);
-    if (tap >= 0 && ok) {
-      float* dst = a.part + ((static_cast<int64_t>(lane) * a.n_chunks + chunk) * kTaps + tap) * kCC * kCC + ci * kCC;
+    tmem_ld_32x32b_x32_pair(trow + i * kCC, lo, trow + i * kCC + 32, hi);
+    if (!ok) continue;
+    __syncwarp();
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        reinterpret_cast<float4*>(dst)[q] = make_float4(lo[4 * q], lo[4 * q + 1], lo[4 * q + 2], lo[4 * q + 3]);
-        reinterpret_cast<float4*>(dst + 32)[q] = make_float4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
-      }
+    for (int q = 0; q < 8; ++q) {
+      *reinterpret_cast<float4*>(T + lane_id * kWLd + 4 * q) = make_float4(lo[4 * q], lo[4 * q + 1], lo[4 * q + 2], lo[4 * q + 3]);
+      *reinterpret_cast<float4*>(T + lane_id * kWLd + 32 + 4 * q) = make_float4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
+    }
+    __syncwarp();
+    float* dst = part + ((a.im2col ? 0 : dy * 3 + dx) * kCC + ci0) * kCC;
+#pragma unroll 4
+    for (int r = 0; r < 32; r += 2) {
+      const int rr = r + (lane_id >> 4), q = lane_id & 15;
+      *reinterpret_cast<float4*>(dst + rr * kCC + 4 * q) = *reinterpret_cast<const float4*>(T + rr * kWLd + 4 * q);
     }
   }
   tc_fence_before();
@@ -429,6 +514,9 @@ __global__ void __launch_bounds__(kWT, 1) conv_wgrad_kernel(const __grid_constan
 // ------------------------------------------------------------------ reduce + SGD of the convolution layers
 // grid (taps * 4, active workers, layers), 256 threads: one tap's 16 in-channel
 // rows x 64 out-channels of one layer; the chunks are summed in chunk order.
+// Latency of the loads is what bounds it: 56 MB for 16 workers took 33 us a
+// launch with one load after the other in the bias sums (256 of them), 21
+// now.
 // The im2col stem has one tap (its blocks of taps 1..8 return at once).
 constexpr int kSgdRows = 16;
 __global__ void __launch_bounds__(256) conv_sgd_kernel(const __grid_constant__ ConvSgdArgs a) {
@@ -441,11 +529,22 @@ __global__ void __launch_bounds__(256) conv_sgd_kernel(const __grid_constant__ C
   if (tap >= ntap) return;
   const float* part = a.part[layer] + (static_cast<int64_t>(lane) * a.n_chunks * kTaps + tap) * kCC * kCC + r0 * kCC;
   const int64_t chunk_stride = static_cast<int64_t>(kTaps) * kCC * kCC;
-  for (int q = t; q < kSgdRows * kCC; q += 256) {
-    float s = 0.f;
-#pragma unroll 4
-    for (int c = 0; c < a.n_chunks; ++c) s += part[c * chunk_stride + q];
-    T[q / kCC][q % kCC] = s;
+  static_assert(kSgdRows * kCC == 4 * 256, "four values a thread");
+  {   // eight 16-byte loads in flight a thread
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+    for (int c = 0; c < a.n_chunks; ++c) {
+      const float4 v = *reinterpret_cast<const float4*>(part + c * chunk_stride + 4 * t);
+      s.x += v.x;
+      s.y += v.y;
+      s.z += v.z;
+      s.w += v.w;
+    }
+    float* d = &T[t / (kCC / 4)][t % (kCC / 4) * 4];
+    d[0] = s.x;
+    d[1] = s.y;
+    d[2] = s.z;
+    d[3] = s.w;
   }
   __syncthreads();
   const int64_t so = static_cast<int64_t>(src) * a.slot_stride, dof = static_cast<int64_t>(lane) * a.slot_stride;
@@ -466,11 +565,20 @@ __global__ void __launch_bounds__(256) conv_sgd_kernel(const __grid_constant__ C
                         (static_cast<int64_t>(tap) * kCC + r0) * kCC;
     for (int q = t; q < kSgdRows * kCC; q += 256) wt[q] = __float2bfloat16_rn(T[q / kCC][q % kCC]);
   }
-  if (blockIdx.x == 0 && t < kCC) {   // bias: per-tile sums in tile order
-    const float* bp = a.bias_part[layer] + static_cast<int64_t>(lane) * a.n_tiles[layer] * kCC;
+  if (blockIdx.x == 0) {   // bias: four threads a channel over the per-tile sums, 16 loads in flight each
+    __syncthreads();
+    float* P = &T[0][0];   // [4][64]
+    const int n = a.n_tiles[layer], c = t & (kCC - 1), g = t / kCC;
+    const float* bp = a.bias_part[layer] + static_cast<int64_t>(lane) * n * kCC + c;
     float s = 0.f;
-    for (int i = 0; i < a.n_tiles[layer]; ++i) s += bp[static_cast<int64_t>(i) * kCC + t];
-    a.master_w[dof + a.offB[layer] + t] = fmaf(-a.lr, s, a.master[so + a.offB[layer] + t]);
+#pragma unroll 16
+    for (int i = g; i < n; i += 4) s += bp[static_cast<int64_t>(i) * kCC];
+    P[t] = s;
+    __syncthreads();
+    if (t < kCC) {
+      s = P[t] + P[kCC + t] + P[2 * kCC + t] + P[3 * kCC + t];
+      a.master_w[dof + a.offB[layer] + t] = fmaf(-a.lr, s, a.master[so + a.offB[layer] + t]);
+    }
   }
 }
 
@@ -494,14 +602,14 @@ __global__ void conv_refresh_wt_kernel(const float* master, __nv_bfloat16* wt, i
 // k = tap * Cin + i of pixel (y, x) is x[y + dy - 1][x + dx - 1][i] for
 // tap = 3 dy + dx (zero outside the image): the stem becomes one 64 x 64
 // product per pixel.
-// im2col: the tile's 6 source rows (y0 - 1 .. y0 + 4, zero outside the
-// image) are first copied to shared memory with coalesced loads; a table
-// gives each channel k its offset from the centre pixel and its x-offset.
+// im2col: the tile's 6 source rows (y0 - 1 .. y0 + 4) are first copied to
+// shared memory with coalesced loads, with a zero pixel on either side; a
+// thread always has the same 16-byte chunk, so that its 8 channels' offsets
+// from the centre pixel stay in registers.
 constexpr int kStageMaxCin = kCC / kTaps;   // 7: the largest input with an im2col stem
-constexpr int kNoTap = 1 << 20;
 __global__ void __launch_bounds__(kCT) cnn_stage_kernel(const __grid_constant__ CnnStageArgs a) {
-  __shared__ float rows[(kTileRows + 2) * kImg * kStageMaxCin];
-  __shared__ int koff[kCC], kdx[kCC];
+  __shared__ float rows[(kTileRows + 2) * (kImg + 2) * kStageMaxCin + 1];
+  __shared__ int koff_s[kCC];
   const int tile = blockIdx.x, e = blockIdx.y;
   const int lane = a.wid[e];
   const int b = tile / kTilesPerImg, pix0 = (tile % kTilesPerImg) * kTilePix;
@@ -516,36 +624,37 @@ __global__ void __launch_bounds__(kCT) cnn_stage_kernel(const __grid_constant__ 
   if (a.labels && tile % kTilesPerImg == 0 && threadIdx.x == 0)
     a.labels[static_cast<int64_t>(lane) * a.B + b] = (eval ? a.y1 : a.y[lane])[row];
   if (a.im2col) {
-    const int Cin = a.Cin, rowel = kImg * Cin, y0 = pix0 / kImg;
+    const int Cin = a.Cin, rowel = kImg * Cin, pitch = rowel + 2 * Cin, y0 = pix0 / kImg;
+    // chunk of this thread: chunks rounded up to a power of two lanes a pixel
+    const int csh = chunks <= 1 ? 0 : 32 - __clz(chunks - 1);
+    const int q = threadIdx.x & ((1 << csh) - 1);
+    const int zero = (kTileRows + 2) * pitch;   // an element that stays zero: channels past K
     if (threadIdx.x < kCC) {
-      const int k = threadIdx.x;
-      if (k < K) {
-        const int tap = k / Cin, i = k - tap * Cin, dy = tap / 3, dx = tap % 3;
-        koff[k] = (dy - 1) * rowel + (dx - 1) * Cin + i;
-        kdx[k] = dx - 1;
-      } else {
-        koff[k] = 0;
-        kdx[k] = kNoTap;
-      }
+      const int k = threadIdx.x, tap = k / Cin, i = k - tap * Cin;
+      koff_s[k] = k < K ? (tap / 3) * pitch + (tap % 3) * Cin + i : -1;
     }
     for (int i = threadIdx.x; i < (kTileRows + 2) * rowel; i += kCT) {
-      const int yy = y0 - 1 + i / rowel;
-      rows[i] = yy >= 0 && yy < kImg ? src[static_cast<int64_t>(y0 - 1) * rowel + i] : 0.f;
+      const int r = i / rowel, x = i - r * rowel, yy = y0 - 1 + r;
+      rows[r * pitch + Cin + x] = yy >= 0 && yy < kImg ? src[static_cast<int64_t>(y0 - 1) * rowel + i] : 0.f;
     }
+    for (int i = threadIdx.x; i < (kTileRows + 2) * 2 * Cin; i += kCT) {   // the pixels beside the image
+      const int r = i / (2 * Cin), x = i - r * 2 * Cin;
+      rows[r * pitch + (x < Cin ? x : rowel + x)] = 0.f;
+    }
+    if (threadIdx.x == 0) rows[zero] = 0.f;
     __syncthreads();
-    for (int it = threadIdx.x; it < kTilePix * chunks; it += kCT) {
-      const int px = it / chunks, q = it - px * chunks;
-      const int x = px % kImg;
-      const int centre = (px / kImg + 1) * rowel + x * Cin;
-      float v[8];
+    int koff[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int k = 8 * q + j, xx = x + kdx[k];
-        v[j] = xx >= 0 && xx < kImg ? rows[centre + koff[k]] : 0.f;
+    for (int j = 0; j < 8; ++j) koff[j] = koff_s[8 * q + j];
+    if (q < chunks)
+      for (int px = threadIdx.x >> csh; px < kTilePix; px += kCT >> csh) {
+        const int centre = (px / kImg) * pitch + (px % kImg) * Cin;   // its upper left neighbour
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = rows[koff[j] >= 0 ? centre + koff[j] : zero];
+        *reinterpret_cast<uint4*>(dst + static_cast<int64_t>(px) * kCC + 8 * q) =
+            make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
       }
-      *reinterpret_cast<uint4*>(dst + static_cast<int64_t>(px) * kCC + 8 * q) =
-          make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
-    }
     return;
   }
   for (int it = threadIdx.x; it < kTilePix * chunks; it += kCT) {
@@ -561,75 +670,74 @@ __global__ void __launch_bounds__(kCT) cnn_stage_kernel(const __grid_constant__ 
   }
 }
 
-// ------------------------------------------------------------------ pooling
-// grid (B, active), 256 threads: g[lane][b][c] = sum over the 1024 pixels / 1024.
-// Thread t sums channels 8 (t % 8) .. + 8 over pixels t / 8 + 32 i (16-byte
-// loads, a warp reading 512 contiguous bytes), then the 32 partials of each
-// channel group are summed in order.
-__global__ void __launch_bounds__(256) cnn_pool_kernel(const __nv_bfloat16* v, const int* wid, int B, float* g) {
-  __shared__ float part[32][kCC + 1];
-  const int b = blockIdx.x, lane = wid[blockIdx.y];
-  const int q = threadIdx.x & 7, p0 = threadIdx.x >> 3;
-  const __nv_bfloat16* src = v + (static_cast<int64_t>(lane) * B + b) * kPix * kCC + 8 * q;
-  float s[8];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) s[j] = 0.f;
-#pragma unroll 4
-  for (int p = p0; p < kPix; p += 32) {
-    const uint4 r = *reinterpret_cast<const uint4*>(src + static_cast<int64_t>(p) * kCC);
-    const __nv_bfloat162* r2 = reinterpret_cast<const __nv_bfloat162*>(&r);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float2 f = __bfloat1622float2(r2[j]);
-      s[2 * j] += f.x;
-      s[2 * j + 1] += f.y;
+// ------------------------------------------------------------------ head: pooling, FC, softmax CE, backward, SGD of the FC
+// The last convolution leaves the channel sums of every image row
+// (pool_part [image][32 rows][64]); g[b][c] = their sum / 1024.  A row of 64
+// features is kept kGld floats apart in shared memory: with 64 the threads of
+// a warp, one sample each, all read one bank (the logits then took 10 us).
+constexpr int kGld = kCC + 1;
+
+// rounded pooled features of `n` images of a lane into gb [n][kGld]
+__device__ __forceinline__ void gather_pooled(const float* pool, int n, float* gb, int threads) {
+  for (int i = threadIdx.x; i < n * (kCC / 4); i += threads) {
+    const int b = i >> 4, c = (i & 15) * 4;
+    const float4* src = reinterpret_cast<const float4*>(pool + static_cast<int64_t>(b) * kImg * kCC + c);
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 16
+    for (int y = 0; y < kImg; ++y) {
+      const float4 v = src[y * (kCC / 4)];
+      s.x += v.x;
+      s.y += v.y;
+      s.z += v.z;
+      s.w += v.w;
     }
-  }
-#pragma unroll
-  for (int j = 0; j < 8; ++j) part[p0][8 * q + j] = s[j];
-  __syncthreads();
-  if (threadIdx.x < kCC) {
-    float t = 0.f;
-    for (int r = 0; r < 32; ++r) t += part[r][threadIdx.x];
-    g[(static_cast<int64_t>(lane) * B + b) * kCC + threadIdx.x] = t / static_cast<float>(kPix);
+    float* d = gb + b * kGld + c;
+    d[0] = bf16_round(s.x / static_cast<float>(kPix));
+    d[1] = bf16_round(s.y / static_cast<float>(kPix));
+    d[2] = bf16_round(s.z / static_cast<float>(kPix));
+    d[3] = bf16_round(s.w / static_cast<float>(kPix));
   }
 }
 
-// ------------------------------------------------------------------ head: FC, softmax CE, backward, SGD of the FC
-// grid (active), 256 threads; B <= 256, K <= 32
-__global__ void __launch_bounds__(256) cnn_head_kernel(const __grid_constant__ CnnHeadArgs a) {
+// grid (active), 512 threads; B <= 256, K <= 32
+constexpr int kHeadT = 512;
+__global__ void __launch_bounds__(kHeadT) cnn_head_kernel(const __grid_constant__ CnnHeadArgs a) {
   extern __shared__ float hsm[];
   const int K = a.K, B = a.B;
-  float* gb = hsm;                    // [B][64] bf16-rounded pooled features
-  float* wf = gb + B * kCC;           // [K][64] bf16-rounded head weights
+  float* gb = hsm;                    // [B][kGld] bf16-rounded pooled features
+  float* wf = gb + B * kGld;          // [K][64] bf16-rounded head weights
   float* wm = wf + K * kCC;           // [K][64] fp32 master
-  float* dl = wm + K * kCC;           // [B][K] fp32 logit gradient
+  float* dl = wm + K * kCC;           // [B][K] logits, then their fp32 gradient
   float* dlb = dl + B * K;            // [B][K] bf16-rounded
   float* rl = dlb + B * K;            // [B] per-sample loss
   float* bfm = rl + B;                // [32]
   const int e = blockIdx.x, lane = a.wid[e], src = a.src[e];
   const int t = threadIdx.x;
   const int64_t so = static_cast<int64_t>(src) * a.slot_stride, dof = static_cast<int64_t>(lane) * a.slot_stride;
-  for (int q = t; q < B * kCC; q += 256) gb[q] = bf16_round(a.g[static_cast<int64_t>(lane) * B * kCC + q]);
-  for (int q = t; q < K * kCC; q += 256) {
+  gather_pooled(a.pool_part + static_cast<int64_t>(lane) * B * kImg * kCC, B, gb, kHeadT);
+  for (int q = t; q < K * kCC; q += kHeadT) {
     const float m = a.master[so + a.offWf + q];
     wm[q] = m;
     wf[q] = bf16_round(m);
   }
   if (t < K) bfm[t] = a.master[so + a.offBf + t];
   __syncthreads();
-  for (int b = t; b < B; b += 256) {
+  // logits: item = (class, sample), samples fastest (the class weights broadcast)
+  for (int q = t; q < B * K; q += kHeadT) {
+    const int k = q / B, b = q - k * B;
+    float acc = 0.f;
+#pragma unroll 16
+    for (int c = 0; c < kCC; ++c) acc = fmaf(gb[b * kGld + c], wf[k * kCC + c], acc);
+    dl[b * K + k] = acc + bfm[k];
+  }
+  __syncthreads();
+  for (int b = t; b < B; b += kHeadT) {
     const int y = a.labels[static_cast<int64_t>(lane) * B + b];
-    float z[32];
-    float mx = -INFINITY, zy = 0.f;
-    for (int k = 0; k < K; ++k) {
-      float acc = 0.f;
-      for (int c = 0; c < kCC; ++c) acc = fmaf(gb[b * kCC + c], wf[k * kCC + c], acc);
-      z[k] = acc + bfm[k];
-      if (k == y) zy = z[k];
-      mx = fmaxf(mx, z[k]);
-    }
+    float* z = dl + b * K;
+    float mx = -INFINITY;
+    for (int k = 0; k < K; ++k) mx = fmaxf(mx, z[k]);
     float se = 0.f, so_ = 0.f;
+    const float zy = z[y];
     for (int k = 0; k < K; ++k) {
       const float ev = expf(z[k] - mx);
       z[k] = ev;
@@ -639,8 +747,8 @@ __global__ void __launch_bounds__(256) cnn_head_kernel(const __grid_constant__ C
     rl[b] = mx + logf(se) - zy;
     const float inv = 1.0f / static_cast<float>(B);
     for (int k = 0; k < K; ++k) {
-      const float gk = (k == y ? -(so_ / se) : z[k] / se) * inv;
-      dl[b * K + k] = gk;
+      const float gk = (k == y ? -so_ : z[k]) / se * inv;
+      z[k] = gk;
       dlb[b * K + k] = bf16_round(gk);
     }
   }
@@ -651,17 +759,18 @@ __global__ void __launch_bounds__(256) cnn_head_kernel(const __grid_constant__ C
     a.loss_part[(static_cast<int64_t>(lane) * a.max_tau + a.step) * a.n_loss_chunks + t] = l;
   }
   // dg[b][c] = sum_k dlb[b][k] wf[k][c] (old weights)
-  for (int q = t; q < B * kCC; q += 256) {
+  for (int q = t; q < B * kCC; q += kHeadT) {
     const int b = q / kCC, c = q % kCC;
     float acc = 0.f;
     for (int k = 0; k < K; ++k) acc = fmaf(dlb[b * K + k], wf[k * kCC + c], acc);
     a.dg[static_cast<int64_t>(lane) * B * kCC + q] = acc;
   }
   // head weights and bias
-  for (int q = t; q < K * kCC; q += 256) {
+  for (int q = t; q < K * kCC; q += kHeadT) {
     const int k = q / kCC, c = q % kCC;
     float acc = 0.f;
-    for (int b = 0; b < B; ++b) acc = fmaf(dlb[b * K + k], gb[b * kCC + c], acc);
+#pragma unroll 4
+    for (int b = 0; b < B; ++b) acc = fmaf(dlb[b * K + k], gb[b * kGld + c], acc);
     const float nw = fmaf(-a.lr, acc, wm[q]);
     a.master_w[dof + a.offWf + q] = nw;
     a.shadow[dof + a.offWf + q] = __float2bfloat16_rn(nw);
@@ -675,40 +784,33 @@ __global__ void __launch_bounds__(256) cnn_head_kernel(const __grid_constant__ C
   }
 }
 
-// loss of the global model on labelled pooled features (evaluation): grid =
-// lanes, 256 threads, one image of the lane's (B <= 256) per thread
-__global__ void __launch_bounds__(256) cnn_head_loss_kernel(const float* g, const int32_t* labels, int B, int64_t n_img,
+// loss of the global model on labelled images (evaluation): grid = lanes, 256
+// threads, one image of the lane's (B <= 256) per thread
+__global__ void __launch_bounds__(256) cnn_head_loss_kernel(const float* pool, const int32_t* labels, int B, int64_t n_img,
                                                             int K, const float* master, int64_t offWf, int64_t offBf,
                                                             float* out) {
-  __shared__ float wf[32 * kCC];
+  extern __shared__ float hsm[];
+  float* gb = hsm;                    // [B][kGld]
+  float* wf = gb + B * kGld;          // [K][64]
   __shared__ float bfm[32];
   __shared__ float rl[8];
   const int t = threadIdx.x, lane = blockIdx.x;
   const int64_t left = n_img - static_cast<int64_t>(lane) * B;
   const int mine = left < B ? static_cast<int>(left) : B;
+  gather_pooled(pool + static_cast<int64_t>(lane) * B * kImg * kCC, mine, gb, 256);
   for (int q = t; q < K * kCC; q += 256) wf[q] = bf16_round(master[offWf + q]);
   if (t < K) bfm[t] = master[offBf + t];
   __syncthreads();
   float l = 0.f;
   if (t < mine) {
-    const float4* gr = reinterpret_cast<const float4*>(g + (static_cast<int64_t>(lane) * B + t) * kCC);
-    float gb[kCC];
-#pragma unroll
-    for (int q = 0; q < kCC / 4; ++q) {
-      const float4 v = gr[q];
-      gb[4 * q] = bf16_round(v.x);
-      gb[4 * q + 1] = bf16_round(v.y);
-      gb[4 * q + 2] = bf16_round(v.z);
-      gb[4 * q + 3] = bf16_round(v.w);
-    }
     const int y = labels[static_cast<int64_t>(lane) * B + t];
     float z[32], mx = -INFINITY, zy = 0.f;
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
       if (k >= K) continue;
       float acc = 0.f;
-#pragma unroll
-      for (int c = 0; c < kCC; ++c) acc = fmaf(gb[c], wf[k * kCC + c], acc);
+#pragma unroll 16
+      for (int c = 0; c < kCC; ++c) acc = fmaf(gb[t * kGld + c], wf[k * kCC + c], acc);
       z[k] = acc + bfm[k];
       mx = fmaxf(mx, z[k]);
       if (k == y) zy = z[k];
@@ -792,25 +894,25 @@ int conv_ctas_per_worker(int B, int n_active, int sms) {
   return cpw;
 }
 
-cudaError_t launch_conv_igemm(int mode, const CUtensorMap& mIn, const CUtensorMap& mW, const ConvArgs& a, int n_active,
-                              int cpw, cudaStream_t s) {
+cudaError_t launch_conv_igemm(int mode, const CUtensorMap& mIn, const CUtensorMap& mW, const ConvMaps& mm,
+                              const ConvArgs& a, int n_active, int cpw, cudaStream_t s) {
   const dim3 grid(cpw, n_active);
   if (mode == 0) {
     cudaError_t e = cudaFuncSetAttribute(conv_igemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGSmem);
     if (e != cudaSuccess) return e;
-    conv_igemm_kernel<0><<<grid, kGT, kGSmem, s>>>(mIn, mW, a);
+    conv_igemm_kernel<0><<<grid, kGT, kGSmem, s>>>(mIn, mW, mm, a);
   } else {
     cudaError_t e = cudaFuncSetAttribute(conv_igemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGSmem);
     if (e != cudaSuccess) return e;
-    conv_igemm_kernel<1><<<grid, kGT, kGSmem, s>>>(mIn, mW, a);
+    conv_igemm_kernel<1><<<grid, kGT, kGSmem, s>>>(mIn, mW, mm, a);
   }
   return cudaGetLastError();
 }
 
-int conv_wgrad_images_per_chunk(int B, int n_active, int sms) {
+int conv_wgrad_chunks(int B, int n_active, int sms) {
   int per_worker = sms / (n_active > 0 ? n_active : 1);   // CTAs per worker in one wave
   if (per_worker < 1) per_worker = 1;
-  return (B + per_worker - 1) / per_worker;
+  return per_worker < B ? per_worker : B;
 }
 
 cudaError_t launch_conv_wgrad(const CUtensorMap& mIn, const CUtensorMap& mDz, const WgradArgs& a, int n_active,
@@ -837,24 +939,25 @@ cudaError_t launch_cnn_stage(const CnnStageArgs& a, int n_active, cudaStream_t s
   return cudaGetLastError();
 }
 
-cudaError_t launch_cnn_pool(const __nv_bfloat16* v, const int* wid, int B, float* g, int n_active, cudaStream_t s) {
-  cnn_pool_kernel<<<dim3(B, n_active), 256, 0, s>>>(v, wid, B, g);
-  return cudaGetLastError();
+static size_t cnn_head_smem(int B, int K) {
+  return sizeof(float) * (static_cast<size_t>(B) * kGld + 2 * K * kCC + 2 * B * K + B + 32);
 }
-
-size_t cnn_head_smem(int B, int K) { return sizeof(float) * (static_cast<size_t>(B) * kCC + 2 * K * kCC + 2 * B * K + B + 32); }
 
 cudaError_t launch_cnn_head(const CnnHeadArgs& a, int n_active, cudaStream_t s) {
   const size_t smem = cnn_head_smem(a.B, a.K);
   cudaError_t e = cudaFuncSetAttribute(cnn_head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  cnn_head_kernel<<<n_active, 256, smem, s>>>(a);
+  cnn_head_kernel<<<n_active, kHeadT, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_cnn_head_loss(const float* g, const int32_t* labels, int lanes, int B, int64_t n_img, int K,
+cudaError_t launch_cnn_head_loss(const float* pool_part, const int32_t* labels, int lanes, int B, int64_t n_img, int K,
                                  const float* master, int64_t offWf, int64_t offBf, float* out, cudaStream_t s) {
-  cnn_head_loss_kernel<<<lanes, 256, 0, s>>>(g, labels, B, n_img, K, master, offWf, offBf, out);
+  const size_t smem = sizeof(float) * (static_cast<size_t>(B) * kGld + K * kCC);
+  cudaError_t e = cudaFuncSetAttribute(cnn_head_loss_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  cnn_head_loss_kernel<<<lanes, 256, smem, s>>>(pool_part, labels, B, n_img, K, master, offWf, offBf, out);
   return cudaGetLastError();
 }
 

@@ -324,16 +324,21 @@ struct ConvArgs {
   int B;                       // images per lane
   const float* bias;           // forward: fp32 slab; bias of slot s at bias + s * slot_stride + off_bias
   int64_t slot_stride, off_bias;
-  const __nv_bfloat16* add;    // [lane][B][1024][64] added before the activation / mask, or null
-  const __nv_bfloat16* mask;   // input gradient: stored activation of the layer input (> 0 keeps)
-  __nv_bfloat16* out;          // [lane][B][1024][64]
+  int has_add;                 // a tensor is added before the activation / mask (ConvMaps::add4)
+  float* pool_part;            // forward: [lane * B + image][32 image rows][64] channel sums of the output, or null
   float* bias_part;            // input gradient: [lane][cpw][64] per-CTA channel sums, or null
   int* err;
   int im2col;                  // forward only: 1 = the stem as one 64 x 64 product over the im2col input
 };
+// tensors an implicit GEMM's epilogue reads and writes, [lane * B + image][32][32][64] bf16
+struct ConvMaps {
+  CUtensorMap add4;            // added before the activation / mask, box of 4 image rows (has_add)
+  CUtensorMap mask4;           // input gradient: stored activation of the layer input (> 0 keeps), 4 image rows
+  CUtensorMap out1;            // the output, box of one image row
+};
 struct WgradArgs {
   const int* wid;
-  int B, n_chunks, img_per_chunk;
+  int B, n_chunks;             // chunk c: K-blocks (2 image rows) [c n / n_chunks, (c + 1) n / n_chunks) of n = 16 B
   float* part;                 // [lane][n_chunks][9][64 in][64 out]
   int* err;
   int im2col;                  // 1 = the stem over the im2col input: tap 0 of `part` only
@@ -373,7 +378,7 @@ struct CnnHeadArgs {
   const int* wid;
   const int* src;
   int B, K, step, max_tau, n_loss_chunks;
-  const float* g;              // [lane][B][64]
+  const float* pool_part;      // [lane * B + image][32][64] channel sums of the image rows
   const int32_t* labels;       // [lane][B]
   float* dg;                   // [lane][B][64]
   float* loss_part;            // [(lane * max_tau + step) * n_loss_chunks + chunk]
@@ -384,22 +389,20 @@ struct CnnHeadArgs {
   float lr;
 };
 int cnn_tiles_per_image();
-// images per split-K chunk of the weight gradient (one wave of CTAs over the active workers)
-int conv_wgrad_images_per_chunk(int B, int n_active, int sms);
+// split-K chunks of the weight gradient per worker (one wave of CTAs over the active workers, at most B)
+int conv_wgrad_chunks(int B, int n_active, int sms);
 // CTAs per worker of the implicit-GEMM kernel (one per SM over the active workers)
 int conv_ctas_per_worker(int B, int n_active, int sms);
-cudaError_t launch_conv_igemm(int mode, const CUtensorMap& mIn, const CUtensorMap& mW, const ConvArgs& a, int n_active,
-                              int cpw, cudaStream_t s);
+cudaError_t launch_conv_igemm(int mode, const CUtensorMap& mIn, const CUtensorMap& mW, const ConvMaps& mm,
+                              const ConvArgs& a, int n_active, int cpw, cudaStream_t s);
 cudaError_t launch_conv_wgrad(const CUtensorMap& mIn, const CUtensorMap& mDz, const WgradArgs& a, int n_active,
                               cudaStream_t s);
 cudaError_t launch_conv_sgd(const ConvSgdArgs& a, int n_active, cudaStream_t s);
 cudaError_t launch_conv_refresh_wt(const float* master, __nv_bfloat16* wt, int64_t offW, cudaStream_t s);
 cudaError_t launch_cnn_stage(const CnnStageArgs& a, int n_active, cudaStream_t s);
-cudaError_t launch_cnn_pool(const __nv_bfloat16* v, const int* wid, int B, float* g, int n_active, cudaStream_t s);
-size_t cnn_head_smem(int B, int K);
 cudaError_t launch_cnn_head(const CnnHeadArgs& a, int n_active, cudaStream_t s);
 // out[lane] = loss sum of the lane's first min(B, n_img - lane * B) images, lane < lanes
-cudaError_t launch_cnn_head_loss(const float* g, const int32_t* labels, int lanes, int B, int64_t n_img, int K,
+cudaError_t launch_cnn_head_loss(const float* pool_part, const int32_t* labels, int lanes, int B, int64_t n_img, int K,
                                  const float* master, int64_t offWf, int64_t offBf, float* out, cudaStream_t s);
 cudaError_t launch_cnn_dzb(const __nv_bfloat16* v, const float* dg, const int* wid, int B, __nv_bfloat16* dz,
                            float* bias_part, int n_active, cudaStream_t s);
