@@ -12,10 +12,10 @@
 // Kernels (all workers of a local step in one launch, grid y = active worker):
 //  * conv_igemm_kernel: implicit GEMM on tcgen05.  An output tile is 128
 //    pixels (4 image rows) x 64 channels, the sum over the 9 taps of
-//    [128 pixels x 64 in-channels] x [64 x 64] products; the input boxes are
-//    loaded by TMA shifted by the tap offsets (the zero padding is TMA's
-//    out-of-bounds fill), one 6-row box per x-offset serving the three
-//    y-offsets, and a CTA keeps its worker's weights resident across its
+//    [128 pixels x 64 in-channels] x [64 x 64] products; one TMA box of 6 rows
+//    serves the three y-offsets (the zero padding is TMA's out-of-bounds
+//    fill), the three x-offsets are 192 columns of one product whose sum is
+//    taken in the epilogue, and a CTA keeps its worker's weights resident across its
 //    tiles.  Forward epilogue: bias, optional residual, ReLU, bf16.
 //    Input-gradient mode: the boxes are shifted the other way and the weights
 //    are the transposed copy; epilogue: optional skip-path gradient, the ReLU
@@ -57,10 +57,20 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 // ------------------------------------------------------------------ implicit GEMM (forward / input gradient)
 // A CTA works through tiles c, c + cpw, c + 2 cpw, ... of one worker (grid x
 // = c < cpw, grid y = active worker) with that worker's 9 weight taps resident
-// in shared memory.  Per tile and x-offset dx one TMA box of 6 image rows
-// (rows y0 - 1 .. y0 + 4, shifted by the x-offset) is loaded; the three
-// y-offsets are its 4-row sub-tiles at row offsets 0, 1, 2 (multiples of 8
-// pixel rows of 128 bytes, so the 128-byte swizzle phase is unchanged).
+// in shared memory.  Per tile TMA loads one box of 6 image rows (y0 - 1 .. y0
+// + 4); the three y-offsets are its 4-row sub-tiles at row offsets 0, 1, 2
+// (multiples of 8 pixel rows of 128 bytes, so the 128-byte swizzle phase is
+// unchanged).  The x-offsets are not shifts of the input but columns of the
+// product: with N = 192 the three taps of one dy multiply the same sub-tile,
+//   E[q][dx][o] = sum_dy x[q + (dy - 1, 0)] W[dy][dx][o],
+//   out[p][o] = sum_dx E[p + (0, dx - 1)][dx][o],
+// and a row of the image is the 32 lanes of a warp, so the sum over dx is two
+// shuffles a channel with zero at the image's edges.  What bounds the kernel
+// is the shared memory bandwidth (128 bytes a clock): operands 120 KB, TMA
+// writes 24 KB, shuffles and epilogue about 100 KB a tile; with three shifted
+// boxes and N = 64 it was 216 + 72 KB and 2900 to 3400 clocks a tile (36 us a
+// forward launch of up to 16 workers, 48 an input gradient), 33 and 49:
+// at 16 workers a launch moves 128 to 256 MB of activations, 19 to 38 us of HBM.
 //
 // Two TMEM accumulators and two epilogue warpgroups, tile k with accumulator
 // and group k % 2: the epilogues of two tiles overlap the MMAs of a third.
@@ -73,7 +83,8 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 // the kernels ran at 41 us (forward) and 60 us (input gradient) a launch of
 // up to 16 workers; 36 and 48 us with this epilogue.
 constexpr int kGT = 320;                    // warp 0 TMA, warp 1 MMA, warps 2-5 and 6-9 epilogue
-constexpr int kGSlots = 4;                  // input boxes in flight
+constexpr int kGSlots = 4;                  // input boxes in flight (one a tile)
+constexpr int kGAcc = 256;                  // TMEM columns of an accumulator (192 used)
 constexpr int kGBox = 6 * kImg * kCC * 2;   // 24 KB: 6 rows x 32 pixels x 64 channels
 constexpr int kGW = kTaps * kCB;            // 72 KB of resident weights
 constexpr int kGTile = kTilePix * kCC * 2;  // 16 KB: an output tile
@@ -126,7 +137,7 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
     fence_barrier_init();
   }
   if (warp == 0) {
-    tmem_alloc(tslot, 128);
+    tmem_alloc(tslot, 512);
     tmem_relinquish();
   }
   if (MODE == 0 && t >= 64 && t < 64 + kCC)
@@ -135,11 +146,9 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
-  constexpr int sgn = MODE == 0 ? 1 : -1;   // the input gradient reads the output gradient at p - off(tap)
   // im2col stem (forward): one tap of weights, one 4-row box per tile (mIn's
   // box is {64, 32, 4, 1}), four MMAs
   const bool one_tap = MODE == 0 && a.im2col;
-  const int nbox = one_tap ? 1 : 3;
   // forward: the residual (if any) in the tile buffer; input gradient: the
   // mask there and the skip gradient (if any) in its own buffer
   const bool aux = MODE == 1 || a.has_add, skip = MODE == 1 && a.has_add;
@@ -149,25 +158,14 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
       if (MODE == 0) tma_load_4d(wts + tap * kCB, &mW, 0, tap, 0, slot, wfull);   // {in, tap, out, slot}
       else tma_load_4d(wts + tap * kCB, &mW, 0, 0, tap, slot, wfull);             // {out, in, tap, slot}
     }
-    int it = 0;
     for (int k = 0; k < my_tiles; ++k) {
       const int tile = c0 + k * cpw;
       const int img = lane * a.B + tile / kTilesPerImg, y0 = (tile % kTilesPerImg) * kTileRows;
-      for (int dx = 0; dx < nbox; ++dx, ++it) {
-        const int sl = it % kGSlots;
-        if (it >= kGSlots && !mbar_wait(&empty[sl], ((it / kGSlots) + 1) & 1, a.err, kDevTimeoutEmpty)) {
-          k = my_tiles;
-          break;
-        }
-        if (one_tap) {
-          mbar_arrive_expect_tx(&full[sl], kTilePix * kCC * 2);
-          tma_load_4d(slots + sl * kGBox, &mIn, 0, 0, y0, img, &full[sl]);
-        } else {
-          mbar_arrive_expect_tx(&full[sl], kGBox);
-          tma_load_4d(slots + sl * kGBox, &mIn, 0, sgn * (dx - 1), y0 - 1, img, &full[sl]);
-        }
-      }
-      if (aux && k < my_tiles) {
+      const int sl = k % kGSlots;
+      if (k >= kGSlots && !mbar_wait(&empty[sl], ((k / kGSlots) + 1) & 1, a.err, kDevTimeoutEmpty)) break;
+      mbar_arrive_expect_tx(&full[sl], one_tap ? kGTile : kGBox);
+      tma_load_4d(slots + sl * kGBox, &mIn, 0, 0, one_tap ? y0 : y0 - 1, img, &full[sl]);
+      if (aux) {
         const int p = k & 1, use = k >> 1;
         // the group's previous output has left the tile buffer; the previous tile has read the skip gradient
         if (use >= 1 && !mbar_wait(&auxe[p], (use - 1) & 1, a.err, kDevTimeoutEmpty)) break;
@@ -178,43 +176,36 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
       }
     }
   } else if (warp == 1) {   // converged, one elected lane issues: see elect_one
-    constexpr uint32_t idesc = idesc_bf16_f32(128, kCC);
-    bool ok = mbar_wait(wfull, 0, a.err, kDevTimeoutFull);
+    constexpr uint32_t idesc = idesc_bf16_f32(128, kCC), idesc3 = idesc_bf16_f32(128, 3 * kCC);
+    const bool ok = mbar_wait(wfull, 0, a.err, kDevTimeoutFull);
     tc_fence_after();
-    int it = 0;
+    const uint64_t wb = smem_desc_k128(smem_u32(wts));
     for (int k = 0; ok && k < my_tiles; ++k) {
-      const int buf = k & 1, use = k >> 1;
+      const int buf = k & 1, use = k >> 1, sl = k % kGSlots;
       if (use >= 1 && !mbar_wait(&acce[buf], (use - 1) & 1, a.err, kDevTimeoutAccum)) break;
+      if (!mbar_wait(&full[sl], (k / kGSlots) & 1, a.err, kDevTimeoutFull)) break;
       tc_fence_after();
-      for (int dx = 0; dx < nbox; ++dx, ++it) {
-        const int sl = it % kGSlots;
-        if (!mbar_wait(&full[sl], (it / kGSlots) & 1, a.err, kDevTimeoutFull)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        // descriptors count 16 bytes: 2 for the 32 bytes of a K slice
-        const uint64_t sa = smem_desc_k128(smem_u32(slots + sl * kGBox)), wb = smem_desc_k128(smem_u32(wts));
-        if (elect_one()) {
-          if (one_tap) {
+      // descriptors count 16 bytes: 2 for the 32 bytes of a K slice
+      const uint64_t sa = smem_desc_k128(smem_u32(slots + sl * kGBox));
+      const uint32_t acc = tmem + buf * kGAcc;
+      if (elect_one()) {
+        if (one_tap) {
+#pragma unroll
+          for (int j = 0; j < kCC / 16; ++j) umma_bf16(acc, sa + 2 * j, wb + 2 * j, idesc, j != 0 ? 1u : 0u);
+        } else {
+#pragma unroll
+          for (int dy = 0; dy < 3; ++dy) {
+            // sub-tile of the 6-row box; the input gradient reads the output gradient at p - off(tap)
+            const int rowoff = MODE == 0 ? dy : 2 - dy;
+            const uint64_t aa = sa + rowoff * (kImg * kCC * 2 / 16), bb = wb + dy * (3 * kCB / 16);
 #pragma unroll
             for (int j = 0; j < kCC / 16; ++j)
-              umma_bf16(tmem + buf * kCC, sa + 2 * j, wb + 2 * j, idesc, j != 0 ? 1u : 0u);
-          } else {
-#pragma unroll
-            for (int dy = 0; dy < 3; ++dy) {
-              const int rowoff = MODE == 0 ? dy : 2 - dy;   // sub-tile of the 6-row box
-              const uint64_t aa = sa + rowoff * (kImg * kCC * 2 / 16), bb = wb + (dy * 3 + dx) * (kCB / 16);
-#pragma unroll
-              for (int j = 0; j < kCC / 16; ++j)
-                umma_bf16(tmem + buf * kCC, aa + 2 * j, bb + 2 * j, idesc, (dx | dy | j) != 0 ? 1u : 0u);
-            }
+              umma_bf16(acc, aa + 2 * j, bb + 2 * j, idesc3, (dy | j) != 0 ? 1u : 0u);
           }
-          umma_commit(&empty[sl]);
         }
-        __syncwarp();
+        umma_commit(&empty[sl]);
+        umma_commit(&accf[buf]);
       }
-      if (ok && elect_one()) umma_commit(&accf[buf]);
       __syncwarp();
     }
   } else if (warp >= 2) {
@@ -222,7 +213,7 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
     // channels; warp = image row y0 + quarter
     const int grp = (warp - 2) >> 2, quarter = warp & 3;
     const int p = quarter * 32 + lane_id;
-    const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + grp * kCC;
+    const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + grp * kGAcc;
     uint8_t* row = sm + kGOffE + grp * kGTile + p * 128;          // 16-byte chunk q at (q ^ (p & 7))
     const uint8_t* srow = sm + kGOffS + p * 128;
     const uint32_t sw = static_cast<uint32_t>(p & 7);
@@ -236,76 +227,102 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
       int ok = mbar_wait(&accf[grp], use & 1, a.err, kDevTimeoutAccum) ? 1 : 0;
       ok = __all_sync(0xffffffffu, ok);
       tc_fence_after();
-      float v[kCC];
-      {
-        float lo[32], hi[32];
-        tmem_ld_32x32b_x32_pair(trow, lo, trow + 32, hi);
-#pragma unroll
-        for (int c = 0; c < 32; ++c) {
-          v[c] = ok ? lo[c] : 0.f;
-          v[32 + c] = ok ? hi[c] : 0.f;
-        }
-      }
-      tc_fence_before();
-      mbar_arrive(&acce[grp]);   // the accumulator has been read: the next tile may use it
-      if (MODE == 0) {
-#pragma unroll
-        for (int c = 0; c < kCC; ++c) v[c] += bias_s[c];
-      }
       if (aux) {
         mbar_wait(&auxf[grp], use & 1, a.err, kDevTimeoutFull);
       } else {   // this warp's previous output has left its rows
         if (lane_id == 0) bulk_wait_read_all();
         __syncwarp();
       }
-      if (a.has_add) {
 #pragma unroll
-        for (int q = 0; q < kCC / 8; ++q) {
-          const uint4 r = *reinterpret_cast<const uint4*>((MODE == 0 ? row : srow) + ((q ^ sw) << 4));
-          const __nv_bfloat162* r2 = reinterpret_cast<const __nv_bfloat162*>(&r);
+      for (int h = 0; h < 2; ++h) {   // 32 channels at a time
+        float v[32];
+        // forward: dx 0 from the pixel before, dx 2 from the one after; the input gradient the other way round
+        const uint32_t before = trow + (MODE == 0 ? 0 : 2 * kCC) + 32 * h, after = trow + (MODE == 0 ? 2 * kCC : 0) + 32 * h;
+        if (one_tap) {
+          tmem_ld_32x32b_x32(trow + 32 * h, v);
+        } else {
+          float l[32];
+          tmem_ld_32x32b_x32_pair(trow + kCC + 32 * h, v, before, l);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float2 f = __bfloat1622float2(r2[j]);
-            v[8 * q + 2 * j] += f.x;
-            v[8 * q + 2 * j + 1] += f.y;
+          for (int c = 0; c < 32; ++c) {
+            const float x = __shfl_up_sync(0xffffffffu, l[c], 1);
+            v[c] += lane_id == 0 ? 0.f : x;
+          }
+          tmem_ld_32x32b_x32(after, l);
+#pragma unroll
+          for (int c = 0; c < 32; ++c) {
+            const float x = __shfl_down_sync(0xffffffffu, l[c], 1);
+            v[c] += lane_id == 31 ? 0.f : x;
           }
         }
-        if (skip) {
-          __syncwarp();
-          if (lane_id == 0) mbar_arrive(skipe);
+        if (h == 1) {
+          tc_fence_before();
+          mbar_arrive(&acce[grp]);   // the accumulator has been read: the next tile may use it
         }
-      }
-      if (MODE == 0) {
 #pragma unroll
-        for (int c = 0; c < kCC; ++c) v[c] = fmaxf(v[c], 0.f);
-      } else {
+        for (int c = 0; c < 32; ++c) v[c] = ok ? v[c] + (MODE == 0 ? bias_s[32 * h + c] : 0.f) : 0.f;
+        if (a.has_add) {
 #pragma unroll
-        for (int q = 0; q < kCC / 8; ++q) {
-          const uint4 r = *reinterpret_cast<const uint4*>(row + ((q ^ sw) << 4));
-          const __nv_bfloat162* r2 = reinterpret_cast<const __nv_bfloat162*>(&r);
+          for (int q = 0; q < 4; ++q) {
+            const uint4 r = *reinterpret_cast<const uint4*>((MODE == 0 ? row : srow) + (((4 * h + q) ^ sw) << 4));
+            const __nv_bfloat162* r2 = reinterpret_cast<const __nv_bfloat162*>(&r);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float2 f = __bfloat1622float2(r2[j]);
-            if (!(f.x > 0.f)) v[8 * q + 2 * j] = 0.f;
-            if (!(f.y > 0.f)) v[8 * q + 2 * j + 1] = 0.f;
+            for (int j = 0; j < 4; ++j) {
+              const float2 f = __bfloat1622float2(r2[j]);
+              v[8 * q + 2 * j] += f.x;
+              v[8 * q + 2 * j + 1] += f.y;
+            }
+          }
+          if (skip && h == 1) {
+            __syncwarp();
+            if (lane_id == 0) mbar_arrive(skipe);
           }
         }
 #pragma unroll
-        for (int c = 0; c < kCC; ++c) bsum[c] += v[c];
-      }
+        for (int q = 0; q < 4; ++q) {
+          uint4* chunk = reinterpret_cast<uint4*>(row + (((4 * h + q) ^ sw) << 4));
+          if (MODE == 0) {
 #pragma unroll
-      for (int q = 0; q < kCC / 8; ++q) {
-        const uint4 o = make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
-                                   pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
-        *reinterpret_cast<uint4*>(row + ((q ^ sw) << 4)) = o;
-        if (MODE == 0 && a.pool_part) {   // the pooling sums the stored values
-          const __nv_bfloat162* o2 = reinterpret_cast<const __nv_bfloat162*>(&o);
+            for (int j = 0; j < 8; ++j) v[8 * q + j] = fmaxf(v[8 * q + j], 0.f);
+          } else {
+            const uint4 r = *chunk;   // the mask
+            const __nv_bfloat162* r2 = reinterpret_cast<const __nv_bfloat162*>(&r);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float2 f = __bfloat1622float2(o2[j]);
-            v[8 * q + 2 * j] = f.x;
-            v[8 * q + 2 * j + 1] = f.y;
+            for (int j = 0; j < 4; ++j) {
+              const float2 f = __bfloat1622float2(r2[j]);
+              if (!(f.x > 0.f)) v[8 * q + 2 * j] = 0.f;
+              if (!(f.y > 0.f)) v[8 * q + 2 * j + 1] = 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) bsum[32 * h + 8 * q + j] += v[8 * q + j];
           }
+          const uint4 o = make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
+                                     pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
+          *chunk = o;
+          if (MODE == 0) {   // the pooling sums the stored values
+            const __nv_bfloat162* o2 = reinterpret_cast<const __nv_bfloat162*>(&o);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float2 f = __bfloat1622float2(o2[j]);
+              v[8 * q + 2 * j] = f.x;
+              v[8 * q + 2 * j + 1] = f.y;
+            }
+          }
+        }
+        if (MODE == 0 && a.pool_part) {
+          // channel sums over the image row's 32 pixels: halves exchanged over
+          // the lanes until a lane holds one channel (its own index of the 32)
+#pragma unroll
+          for (int w = 16; w > 0; w >>= 1) {
+            const bool up = lane_id & w;
+#pragma unroll
+            for (int c = 0; c < 16; ++c)
+              if (c < w) {
+                const float keep = up ? v[c + w] : v[c], give = up ? v[c] : v[c + w];
+                v[c] = keep + __shfl_xor_sync(0xffffffffu, give, w);
+              }
+          }
+          a.pool_part[(static_cast<int64_t>(img) * kImg + y0 + quarter) * kCC + 32 * h + lane_id] = v[0];
         }
       }
       fence_proxy_async_smem();   // the rows are read by the TMA store
@@ -313,25 +330,6 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
       if (lane_id == 0) {
         tma_store_4d(&mm.out1, sm + kGOffE + grp * kGTile + quarter * 32 * 128, 0, 0, y0 + quarter, img);
         bulk_commit_group();
-      }
-      if (MODE == 0 && a.pool_part) {
-        // channel sums over the image row's 32 pixels: halves exchanged over
-        // the lanes until a lane holds two channels
-#pragma unroll
-        for (int w = 32, o = 16; o > 0; w >>= 1, o >>= 1) {
-          const bool up = lane_id & o;
-#pragma unroll
-          for (int c = 0; c < 32; ++c)
-            if (c < w) {
-              const float keep = up ? v[c + w] : v[c], give = up ? v[c] : v[c + w];
-              v[c] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-            }
-        }
-        // the lane's bits chose halves of 32, 16, 8, 4, 2 channels: channels 2 lane', 2 lane' + 1
-        const int ch = ((lane_id & 16) ? 32 : 0) + ((lane_id & 8) ? 16 : 0) + ((lane_id & 4) ? 8 : 0) +
-                       ((lane_id & 2) ? 4 : 0) + ((lane_id & 1) ? 2 : 0);
-        *reinterpret_cast<float2*>(a.pool_part + (static_cast<int64_t>(img) * kImg + y0 + quarter) * kCC + ch) =
-            make_float2(v[0], v[1]);
       }
       if (aux && lane_id == 0) {   // the tile buffer may take the next tile's inputs
         bulk_wait_read_all();
@@ -365,7 +363,7 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem, 128);
+    tmem_dealloc(tmem, 512);
   }
 }
 
