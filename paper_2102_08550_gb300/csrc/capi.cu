@@ -1454,7 +1454,8 @@ oscars_status allocate_mlp(oscars_ctx* c) {
   {
     const Layer& hl = c->layers.back();
     if (!make_map(&c->mHeadIn, c->A[L - 1], hl.in, B, W, hl.in * 2ull, static_cast<uint64_t>(B) * hl.in * 2ull, 128) ||
-        !make_map(&c->mHeadW, c->shadow + hl.offW, hl.in, hl.out, slots64, hl.in * 2ull, c->P_pad * 2ull, 16))
+        !make_map(&c->mHeadW, c->shadow + hl.offW, hl.in, hl.out, slots64, hl.in * 2ull, c->P_pad * 2ull,
+                  head_tc_class_rows(hl.out)))
       return fail(c, OSCARS_ECUDA, "cuTensorMapEncodeTiled failed (head)");
   }
   return OSCARS_OK;

@@ -1,4 +1,4 @@
-// Forward and backward of the last layer (10 classes) of the per-layer path
+// Forward and backward of the last layer (2 to 32 classes) of the per-layer path
 // on the tensor cores (Eq. 4, "otherwise" branch: one SGD step of the
 // worker's head).  A cluster of H/F CTAs serves one active worker; CTA r owns
 // hidden features [F r, F r + F), F = 128 NH with NH = 1 or 2 halves of 128
@@ -7,17 +7,17 @@
 // [B][H]) and W2 the head weights ([C][H]):
 //
 //  1. partial logits of the CTA's features, P[b][c] = sum_f h[b][f] W2[c][f]:
-//     tcgen05.mma M = 128 rows, N = 16 classes (rows >= B and classes >= C
+//     tcgen05.mma M = 128 rows, N = NC = 16 or 32 classes (rows >= B and classes >= C
 //     are zero-filled by the TMA loads), K = F features;
 //  2. cluster barrier; the logits are the partials of ranks 0..n-1 summed in
 //     that order from distributed shared memory, plus the bias; softmax
 //     cross-entropy per row (one thread per row); dz (fp32) and its bf16
 //     copy, written into two shared tiles laid out as tensor-core operands;
 //  3. head weight gradient dW2^T[f][c] = sum_b h[b][f] dz[b][c] (per half
-//     M = 128 features, N = 16, K = B: the h tile read MN-major) and SGD of
+//     M = 128 features, N = NC, K = B: the h tile read MN-major) and SGD of
 //     the CTA's head columns;
 //  4. input gradient of the layer below, transposed: dh^T[f][b] = sum_c
-//     W2[c][f] dz[b][c] (per half M = 128 features, N = B, K = 16: the W2
+//     W2[c][f] dz[b][c] (per half M = 128 features, N = B, K = NC: the W2
 //     tile read MN-major); masked by h > 0; G^T rows from registers, the fp32 bias
 //     gradient per feature, and G rows through the h tile (overwritten in
 //     place with the bf16 input gradient, then written as full 16-byte
@@ -27,6 +27,13 @@
 // TMEM columns (the phases run one after another).  All mbarrier waits are
 // bounded; the cluster barriers are unconditional, so a timeout cannot leave
 // a CTA of the cluster behind at one.
+//
+// NC is C rounded up to 16 or 32; C = 10 is also a template argument (CT), which
+// keeps the row softmax in as few registers and instructions as it needs.
+// Latency-bound: one launch here against a forward and a backward launch on
+// the CUDA cores for other class counts (17 and 12 us each with 17 classes,
+// 256 features, batch 32): a round of the 1000-384-256-17 model, 5 workers,
+// 534 -> 440 us.
 #include "common.cuh"
 #include "internal.h"
 
@@ -37,25 +44,23 @@ namespace {
 constexpr int kHT = 128;                 // hidden features per half (tensor-core rows)
 constexpr int kHTThreads = 256;
 constexpr int kHTMaxCluster = 8;
-constexpr int kHTC = 10;                 // classes
-constexpr int kHTN = 16;                 // classes padded to the MMA's N
 constexpr int kHTRows = 128;             // rows of the h tile (B <= 128; the rest zero)
 
 // shared memory carve-up (bytes from a 1024-aligned base) for NH halves
-template <int NH>
+template <int NH, int NC>
 struct HTCfg {
   static constexpr int F = kHT * NH;                     // features per CTA
   static constexpr int oH = 0;                           // h tile: F/64 boxes [128 rows][64 features] bf16, 128-B swizzle
-  static constexpr int oW2 = oH + (F / 64) * kHTRows * 128;   // W2 tile: F/64 boxes [16 classes][64 features]
-  static constexpr int oDzT = oW2 + (F / 64) * kHTN * 128;    // dz^T: [16 classes][B rows] K-major (K = rows), 2 atoms
-  static constexpr int oDzK = oDzT + 2 * kHTN * 128;     // dz: [B rows][16 classes] K-major, no swizzle
-  static constexpr int oPl = oDzK + kHTRows * 32;        // [128][16] fp32 partial logits (read by the cluster)
-  static constexpr int oDz = oPl + kHTRows * kHTN * 4;   // [128][16] fp32 dlogits
-  static constexpr int oLoss = oDz + kHTRows * kHTN * 4; // [128]
+  static constexpr int oW2 = oH + (F / 64) * kHTRows * 128;   // W2 tile: F/64 boxes [NC classes][64 features]
+  static constexpr int oDzT = oW2 + (F / 64) * NC * 128;    // dz^T: [16 classes][B rows] K-major (K = rows), 2 atoms
+  static constexpr int oDzK = oDzT + 2 * NC * 128;       // dz: [B rows][NC classes] K-major, no swizzle
+  static constexpr int oPl = oDzK + kHTRows * NC * 2;    // [128][NC] fp32 partial logits (read by the cluster)
+  static constexpr int oDz = oPl + kHTRows * NC * 4;   // [128][16] fp32 dlogits
+  static constexpr int oLoss = oDz + kHTRows * NC * 4; // [128]
   static constexpr int oGbp = oLoss + kHTRows * 4;       // [2][F]
   static constexpr int oLab = oGbp + 2 * F * 4;          // [128] int
   static constexpr int oB2 = oLab + kHTRows * 4;         // [16]
-  static constexpr int oBar = oB2 + kHTN * 4;            // tma, mma barriers, TMEM slot
+  static constexpr int oBar = oB2 + NC * 4;            // tma, mma barriers, TMEM slot
   static constexpr int kSmem = oBar + 64 + 1024;
   static constexpr uint32_t kTmemCols = 128 * NH;
 };
@@ -120,11 +125,11 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16x2(uint32_t taddr, float (&v)[
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-template <int NH>
+template <int NH, int NC, int CT>
 __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_constant__ CUtensorMap mH,
                                                               const __grid_constant__ CUtensorMap mW2,
                                                               const __grid_constant__ HeadArgs a) {
-  using Cfg = HTCfg<NH>;
+  using Cfg = HTCfg<NH, NC>;
   constexpr int F = Cfg::F;
   extern __shared__ uint8_t ht_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(ht_raw) + 1023) & ~uintptr_t(1023));
@@ -142,7 +147,8 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
   uint64_t* mma_bar = tma_bar + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_bar + 1);
 
-  const int H = a.H, B = a.B;
+  const int H = a.H, B = a.B, C = CT > 0 ? CT : a.C;
+  constexpr int CL = CT > 0 ? CT : NC;   // class loops: compile-time bound, `c < C` inside
   const int i = blockIdx.x;
   const int w = a.wid[i], src = a.src[i];
   const uint32_t rank = cluster_ctarank();
@@ -162,11 +168,11 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
   pdl_wait();      // the layer input (the previous kernel's output) is complete
   if (t == 0) {
     // the h and W2 tiles, requested first: the rest of the prologue overlaps them
-    mbar_arrive_expect_tx(tma_bar, (F / 64) * (kHTRows * 128 + kHTN * 128));
+    mbar_arrive_expect_tx(tma_bar, (F / 64) * (kHTRows * 128 + NC * 128));
 #pragma unroll
     for (int q = 0; q < F / 64; ++q) {
       tma_load_3d(hT + q * kHTRows * 128, &mH, k0 + 64 * q, 0, w, tma_bar);
-      tma_load_3d(w2 + q * kHTN * 128, &mW2, k0 + 64 * q, 0, src, tma_bar);
+      tma_load_3d(w2 + q * NC * 128, &mW2, k0 + 64 * q, 0, src, tma_bar);
     }
   }
   if (warp == 0) {
@@ -174,10 +180,10 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
     tmem_relinquish();
   }
   // the dz tiles' padding (classes >= C, rows >= B) stays zero
-  for (int q = t; q < (2 * kHTN * 128 + kHTRows * 32) / 16; q += kHTThreads)
+  for (int q = t; q < (2 * NC * 128 + kHTRows * NC * 2) / 16; q += kHTThreads)
     reinterpret_cast<uint4*>(dzT)[q] = make_uint4(0, 0, 0, 0);
   for (int b = t; b < B; b += kHTThreads) labs[b] = a.labels[static_cast<int64_t>(w) * B + b];
-  if (t < kHTN) b2[t] = t < kHTC ? a.master[so + a.offB + t] : 0.f;
+  if (t < NC) b2[t] = t < C ? a.master[so + a.offB + t] : 0.f;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -188,7 +194,7 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
   if (warp == 0) {   // converged, one elected lane issues: see elect_one
     const bool landed = mbar_wait(tma_bar, 0, a.err, kDevTimeoutFull);
     tc_fence_after();
-    constexpr uint32_t idesc = idesc_bf16_f32(kHTRows, kHTN);
+    constexpr uint32_t idesc = idesc_bf16_f32(kHTRows, NC);
     const uint64_t hd = smem_desc_k128(smem_u32(hT)), wd = smem_desc_k128(smem_u32(w2));   // addresses in 16 bytes
     if (elect_one()) {
       if (landed)
@@ -196,7 +202,7 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
         for (int kb = 0; kb < F / 64; ++kb)
 #pragma unroll
           for (int j = 0; j < 4; ++j)
-            umma_bf16(tmem, hd + kb * (kHTRows * 128 / 16) + 2 * j, wd + kb * (kHTN * 128 / 16) + 2 * j, idesc,
+            umma_bf16(tmem, hd + kb * (kHTRows * 128 / 16) + 2 * j, wd + kb * (NC * 128 / 16) + 2 * j, idesc,
                       (kb | j) != 0 ? 1u : 0u);
       umma_commit(mma_bar);   // arrives even with nothing issued, so the waits below end
     }
@@ -205,11 +211,12 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
   bool ok = mbar_wait(mma_bar, 0, a.err, kDevTimeoutAccum);
   tc_fence_after();
   if (warp < 4) {
-    float v[16];
-    tmem_ld_32x32b_x16(tmem + (static_cast<uint32_t>(32 * warp) << 16), v);
-    float4* row = reinterpret_cast<float4*>(pl + (32 * warp + lane) * kHTN);
+    float v[NC];
+    if constexpr (NC == 16) tmem_ld_32x32b_x16(tmem + (static_cast<uint32_t>(32 * warp) << 16), v);
+    else tmem_ld_32x32b_x32(tmem + (static_cast<uint32_t>(32 * warp) << 16), v);
+    float4* row = reinterpret_cast<float4*>(pl + (32 * warp + lane) * NC);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) row[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    for (int q = 0; q < NC / 4; ++q) row[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
   }
   tc_fence_before();
   cluster_sync();
@@ -218,61 +225,74 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
   // ---- 2. logits (cluster sum in rank order), softmax cross-entropy, dz tiles
   if (t < B) {
     const int b = t;
-    float z[kHTC];
+    constexpr int QN = (CL + 3) / 4;                 // 16-byte chunks of a row of partial logits
+    constexpr int RG = QN <= 4 ? kHTMaxCluster : 2;  // ranks whose partials are in flight at once
+    float z[4 * QN];
 #pragma unroll
-    for (int c = 0; c < kHTC; ++c) z[c] = 0.f;
-    // every rank's partials are requested before the first is added (a
-    // remote load waits a round trip across the cluster)
-    float4 p[kHTMaxCluster][3];
+    for (int c = 0; c < 4 * QN; ++c) z[c] = 0.f;
+    // the ranks' partials are requested before the first is added (a remote
+    // load waits a round trip across the cluster)
 #pragma unroll
-    for (int r = 0; r < kHTMaxCluster; ++r)
-      if (r < ncl) {
-        p[r][0] = ld_dsmem_f32x4(pl + b * kHTN, r);
-        p[r][1] = ld_dsmem_f32x4(pl + b * kHTN + 4, r);
-        p[r][2] = ld_dsmem_f32x4(pl + b * kHTN + 8, r);
-      }
+    for (int r0 = 0; r0 < kHTMaxCluster; r0 += RG) {
+      if (r0 >= ncl) continue;
+      float4 p[RG][QN];
 #pragma unroll
-    for (int r = 0; r < kHTMaxCluster; ++r)
-      if (r < ncl) {
-        z[0] += p[r][0].x; z[1] += p[r][0].y; z[2] += p[r][0].z; z[3] += p[r][0].w;
-        z[4] += p[r][1].x; z[5] += p[r][1].y; z[6] += p[r][1].z; z[7] += p[r][1].w;
-        z[8] += p[r][2].x; z[9] += p[r][2].y;
-      }
+      for (int r = 0; r < RG; ++r)
+        if (r0 + r < ncl)
 #pragma unroll
-    for (int c = 0; c < kHTC; ++c) z[c] += b2[c];
-    float m = z[0];
+          for (int q = 0; q < QN; ++q) p[r][q] = ld_dsmem_f32x4(pl + b * NC + 4 * q, r0 + r);
 #pragma unroll
-    for (int c = 1; c < kHTC; ++c) m = fmaxf(m, z[c]);
-    const int y = labs[b];
-    float e[kHTC], s = 0.f, so_ = 0.f, zy = 0.f;
+      for (int r = 0; r < RG; ++r)
+        if (r0 + r < ncl)
 #pragma unroll
-    for (int c = 0; c < kHTC; ++c) {
-      e[c] = expf(z[c] - m);
-      s += e[c];
-      if (c != y) so_ += e[c];
-      else zy = z[c];
+          for (int q = 0; q < QN; ++q) {
+            z[4 * q] += p[r][q].x;
+            z[4 * q + 1] += p[r][q].y;
+            z[4 * q + 2] += p[r][q].z;
+            z[4 * q + 3] += p[r][q].w;
+          }
     }
+    const int y = labs[b];
+    float m = -INFINITY, zy = 0.f;
+#pragma unroll
+    for (int c = 0; c < CL; ++c)
+      if (c < C) {
+        z[c] += b2[c];
+        m = fmaxf(m, z[c]);
+        if (c == y) zy = z[c];
+      }
+    float s = 0.f, so_ = 0.f;
+#pragma unroll
+    for (int c = 0; c < CL; ++c)
+      if (c < C) {
+        z[c] = expf(z[c] - m);
+        s += z[c];
+        if (c != y) so_ += z[c];
+      }
     rowloss[b] = m + logf(s) - zy;
     const float inv = 1.0f / static_cast<float>(B);
-    float g[kHTC];
+    float g[NC];
 #pragma unroll
-    for (int c = 0; c < kHTC; ++c) {
-      g[c] = (c == y ? -(so_ / s) : e[c] / s) * inv;
-      dz[b * kHTN + c] = g[c];
+    for (int c = 0; c < NC; ++c) {
+      g[c] = c < CL && c < C ? (c == y ? -so_ : z[c < CL ? c : 0]) / s * inv : 0.f;
+      if (c < CL && c < C) dz[b * NC + c] = g[c];
     }
-    // dz as the K-major [rows][16 classes] operand: classes 0-7 one 16-byte
-    // chunk of core matrix (b / 8, 0), classes 8-9 the start of core matrix (b / 8, 1)
-    uint8_t* ck = dzK + (b >> 3) * 256 + (b & 7) * 16;
-    *reinterpret_cast<uint4*>(ck) = make_uint4(pack_bf16x2(g[0], g[1]), pack_bf16x2(g[2], g[3]),
-                                               pack_bf16x2(g[4], g[5]), pack_bf16x2(g[6], g[7]));
-    *reinterpret_cast<uint32_t*>(ck + 128) = pack_bf16x2(g[8], g[9]);
-    // dz^T as the K-major [16 classes][rows] operand (K = rows, atoms of 64 rows)
-    uint8_t* at = dzT + (b >> 6) * (kHTN * 128);
+    // dz as the K-major [rows][NC classes] operand: classes 8 k .. 8 k + 7 one
+    // 16-byte chunk of core matrix (b / 8, k)
+    uint8_t* ck = dzK + (b >> 3) * (NC / 8 * 128) + (b & 7) * 16;
+#pragma unroll
+    for (int k = 0; k < NC / 8; ++k)
+      *reinterpret_cast<uint4*>(ck + 128 * k) =
+          make_uint4(pack_bf16x2(g[8 * k], g[8 * k + 1]), pack_bf16x2(g[8 * k + 2], g[8 * k + 3]),
+                     pack_bf16x2(g[8 * k + 4], g[8 * k + 5]), pack_bf16x2(g[8 * k + 6], g[8 * k + 7]));
+    // dz^T as the K-major [NC classes][rows] operand (K = rows, atoms of 64 rows)
+    uint8_t* at = dzT + (b >> 6) * (NC * 128);
     const int e64 = b & 63;
 #pragma unroll
-    for (int c = 0; c < kHTC; ++c)
-      *reinterpret_cast<__nv_bfloat16*>(at + c * 128 + ((((e64 >> 3) ^ (c & 7)) & 7) << 4) + (e64 & 7) * 2) =
-          __float2bfloat16_rn(g[c]);
+    for (int c = 0; c < CL; ++c)
+      if (c < C)
+        *reinterpret_cast<__nv_bfloat16*>(at + c * 128 + ((((e64 >> 3) ^ (c & 7)) & 7) << 4) + (e64 & 7) * 2) =
+            __float2bfloat16_rn(g[c]);
   }
   fence_proxy_async_smem();   // the dz tiles are read by the tensor core
   tc_fence_before();
@@ -281,15 +301,15 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
 
   // ---- 3. head weight gradient (M = features, N = classes, K = rows) + SGD
   if (warp == 0) {
-    constexpr uint32_t idesc = idesc_bf16_f32(kHT, kHTN) | (1u << 15);   // A (h^T) MN-major
+    constexpr uint32_t idesc = idesc_bf16_f32(kHT, NC) | (1u << 15);   // A (h^T) MN-major
     const uint64_t hd = smem_desc_mn128(smem_u32(hT), kHTRows * 128), zd = smem_desc_k128(smem_u32(dzT));
     if (elect_one()) {
       if (ok)
 #pragma unroll
-        for (int mh = 0; mh < NH; ++mh)   // half mh: features [128 mh, 128 mh + 128) into columns [16 mh, 16 mh + 16)
+        for (int mh = 0; mh < NH; ++mh)   // half mh: features [128 mh, 128 mh + 128) into columns [NC mh, NC mh + NC)
           for (int j = 0; j < B / 16; ++j)
-            umma_bf16(tmem + 16 * mh, hd + mh * (2 * kHTRows * 128 / 16) + 128 * j,
-                      zd + (j >> 2) * (kHTN * 128 / 16) + 2 * (j & 3), idesc, j != 0 ? 1u : 0u);
+            umma_bf16(tmem + NC * mh, hd + mh * (2 * kHTRows * 128 / 16) + 128 * j,
+                      zd + (j >> 2) * (NC * 128 / 16) + 2 * (j & 3), idesc, j != 0 ? 1u : 0u);
       umma_commit(mma_bar);
     }
     __syncwarp();
@@ -302,34 +322,40 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
       const int64_t row = static_cast<int64_t>(w) * a.part_mul + a.part_add;
       a.loss_part[row * (B / kRowsPerLossChunk) + u] = l;
     }
-    if (u >= 32) {   // warps 5-7: 8 lanes per class, then shuffles within each group of 8 (whole warps)
-      const int c = (u - 32) >> 3, j = u & 7;
-      float g = 0.f;
-      if (c < kHTC)
-        for (int b = j; b < B; b += 8) g += dz[b * kHTN + c];
+    if (u >= 32) {   // warps 5-7: 8 lanes per class (12 classes a pass), then shuffles within each group of 8
+      const int j = u & 7;
+      for (int c0 = 0; c0 < C; c0 += 12) {
+        const int c = c0 + ((u - 32) >> 3);
+        float g = 0.f;
+        if (c < C)
+          for (int b = j; b < B; b += 8) g += dz[b * NC + c];
 #pragma unroll
-      for (int o = 4; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o, 8);
-      if (c < kHTC && j == 0) a.master_w[dof + a.offB + c] = fmaf(-a.lr, g, a.master[so + a.offB + c]);
+        for (int o = 4; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o, 8);
+        if (c < C && j == 0) a.master_w[dof + a.offB + c] = fmaf(-a.lr, g, a.master[so + a.offB + c]);
+      }
     }
   }
   // the old master values of this thread's head column, requested while the
   // MMAs run and before any new value is stored (source and destination
   // slots may be the same slab)
-  float old[kHTC];
+  float old[CL];
   if (warp < 4 * NH) {
     const int f = kHT * (warp >> 2) + 32 * (warp & 3) + lane;
 #pragma unroll
-    for (int c = 0; c < kHTC; ++c) old[c] = a.master[so + a.offW + static_cast<int64_t>(c) * H + k0 + f];
+    for (int c = 0; c < CL; ++c)
+      if (c < C) old[c] = a.master[so + a.offW + static_cast<int64_t>(c) * H + k0 + f];
   }
   ok = mbar_wait(mma_bar, 1, a.err, kDevTimeoutAccum) && ok;
   tc_fence_after();
   if (warp < 4 * NH && ok) {
     const int mh = warp >> 2, q = warp & 3;
     const int f = kHT * mh + 32 * q + lane;
-    float v[16];
-    tmem_ld_32x32b_x16(tmem + 16 * mh + (static_cast<uint32_t>(32 * q) << 16), v);
+    float v[NC];
+    if constexpr (NC == 16) tmem_ld_32x32b_x16(tmem + NC * mh + (static_cast<uint32_t>(32 * q) << 16), v);
+    else tmem_ld_32x32b_x32(tmem + NC * mh + (static_cast<uint32_t>(32 * q) << 16), v);
 #pragma unroll
-    for (int c = 0; c < kHTC; ++c) {
+    for (int c = 0; c < CL; ++c) {
+      if (c >= C) continue;
       const int64_t e = a.offW + static_cast<int64_t>(c) * H + k0 + f;
       const float nw = fmaf(-a.lr, v[c], old[c]);
       a.master_w[dof + e] = nw;
@@ -340,15 +366,17 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
   __syncthreads();
   tc_fence_after();
 
-  // ---- 4. input gradient, transposed (M = features, N = rows, K = 16 classes)
+  // ---- 4. input gradient, transposed (M = features, N = rows, K = NC classes)
   if (warp == 0) {
     const uint32_t idesc = idesc_bf16_f32(kHT, B) | (1u << 15);   // A (W2^T) MN-major
-    const uint64_t wd = smem_desc_mn128(smem_u32(w2), kHTN * 128), kd = smem_desc_none(smem_u32(dzK), 128, 256);
+    const uint64_t wd = smem_desc_mn128(smem_u32(w2), NC * 128), kd = smem_desc_none(smem_u32(dzK), 128, NC / 8 * 128);
     if (elect_one()) {
       if (ok)
 #pragma unroll
         for (int mh = 0; mh < NH; ++mh)   // half mh into columns [B mh, B mh + B)
-          umma_bf16(tmem + B * mh, wd + mh * (2 * kHTN * 128 / 16), kd, idesc, 0u);
+#pragma unroll
+          for (int j = 0; j < NC / 16; ++j)   // 16 classes: 16 rows of the W2 tile, two core matrices of dz
+            umma_bf16(tmem + B * mh, wd + mh * (2 * NC * 128 / 16) + 128 * j, kd + 16 * j, idesc, j != 0 ? 1u : 0u);
       umma_commit(mma_bar);
     }
     __syncwarp();
@@ -429,16 +457,19 @@ int head_tc_halves(int H) { return H / kHT > 4 ? 2 : 1; }
 }  // namespace
 
 bool head_tc_supported(int H, int B, int C) {
-  if (C != kHTC || B % 32 != 0 || B < 32 || B > kHTRows || H % kHT != 0) return false;
+  if (C < 2 || C > 32 || B % 32 != 0 || B < 32 || B > kHTRows || H % kHT != 0) return false;
   const int F = kHT * head_tc_halves(H);
   return H % F == 0 && H / F <= kHTMaxCluster;
 }
 
-template <int NH>
+int head_tc_class_rows(int C) { return C <= 16 ? 16 : 32; }
+
+namespace {
+template <int NH, int NC, int CT>
 cudaError_t launch_head_tc_nh(const CUtensorMap& mH, const CUtensorMap& mW2, const HeadArgs& a, int n_active,
                               cudaStream_t s) {
-  using Cfg = HTCfg<NH>;
-  cudaError_t e = cudaFuncSetAttribute(head_tc_kernel<NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem);
+  using Cfg = HTCfg<NH, NC>;
+  cudaError_t e = cudaFuncSetAttribute(head_tc_kernel<NH, NC, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_active, a.H / Cfg::F, 1);
@@ -454,14 +485,23 @@ cudaError_t launch_head_tc_nh(const CUtensorMap& mH, const CUtensorMap& mW2, con
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = a.pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, head_tc_kernel<NH>, mH, mW2, a);
+  return cudaLaunchKernelEx(&cfg, head_tc_kernel<NH, NC, CT>, mH, mW2, a);
 }
+
+template <int NH>
+cudaError_t launch_head_tc_c(const CUtensorMap& mH, const CUtensorMap& mW2, const HeadArgs& a, int n_active,
+                             cudaStream_t s) {
+  return a.C == 10   ? launch_head_tc_nh<NH, 16, 10>(mH, mW2, a, n_active, s)
+         : a.C <= 16 ? launch_head_tc_nh<NH, 16, 0>(mH, mW2, a, n_active, s)
+                     : launch_head_tc_nh<NH, 32, 0>(mH, mW2, a, n_active, s);
+}
+}  // namespace
 
 cudaError_t launch_head_tc(const CUtensorMap& mH, const CUtensorMap& mW2, const HeadArgs& a, int n_active,
                            cudaStream_t s) {
   if (!head_tc_supported(a.H, a.B, a.C)) return cudaErrorInvalidValue;
-  return head_tc_halves(a.H) == 2 ? launch_head_tc_nh<2>(mH, mW2, a, n_active, s)
-                                  : launch_head_tc_nh<1>(mH, mW2, a, n_active, s);
+  return head_tc_halves(a.H) == 2 ? launch_head_tc_c<2>(mH, mW2, a, n_active, s)
+                                  : launch_head_tc_c<1>(mH, mW2, a, n_active, s);
 }
 
 }  // namespace oscars

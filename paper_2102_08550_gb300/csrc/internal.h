@@ -242,9 +242,11 @@ struct HeadArgs {
 };
 cudaError_t launch_head_fwd(const HeadArgs& a, int n_active, cudaStream_t s);
 // forward + backward of the last layer on the tensor cores (csrc/head_tc.cu):
-// one cluster of H/128 CTAs per active lane; C = 10, 32 <= B <= 128.  mH: the
-// layer input [lane][B][H] bf16, box {64, 128}; mW2: the head weights of every
-// slot [slot][C][H] bf16, box {64, 16}; both with 128-byte swizzle.
+// one cluster of H/128 CTAs per active lane; 2 <= C <= 32, 32 <= B <= 128.
+// mH: the layer input [lane][B][H] bf16, box {64, 128}; mW2: the head weights
+// of every slot [slot][C][H] bf16, box {64, head_tc_class_rows(C)}; both with
+// 128-byte swizzle.
+int head_tc_class_rows(int C);
 bool head_tc_supported(int H, int B, int C);
 cudaError_t launch_head_tc(const CUtensorMap& mH, const CUtensorMap& mW2, const HeadArgs& a, int n_active,
                            cudaStream_t s);
