@@ -652,10 +652,7 @@ GemmArgs gemm_base(oscars_ctx* c, const int* wid, const int* src) {
   g.src = src;
   g.err = c->err;
   g.master = c->slab;
-  g.master_w = c->slab;
-  g.shadow = c->shadow;
   g.slot_stride = c->P_pad;
-  g.lr = c->lr;
   return g;
 }
 
@@ -706,7 +703,6 @@ cudaError_t enqueue_forward(oscars_ctx* c, const int* wid, const int* src, int n
     g.K = ly.in;
     g.a_z_src = 1;
     g.b_z_src = 0;
-    g.offW = ly.offW;
     g.offB = ly.offB;
     g.out = c->A[l + 1];
     g.outT = c->AT[l + 1];
@@ -745,59 +741,47 @@ cudaError_t enqueue_step(oscars_ctx* c, int s, int na, const int* wid, const int
     ProfScope ps(c, "head_bwd", st);
     if ((e = launch_head_bwd(h, na, st)) != cudaSuccess) return e;
   }
-  for (int l = c->L - 2; l >= 0; --l) {
+  for (int l = c->L - 2; l >= 1; --l) {   // input gradient of layer l -> gradient of layer l-1's output
     const Layer& ly = c->layers[l];
-    if (l >= 1) {  // input gradient of layer l -> gradient of layer l-1's output
-      GemmArgs g = gemm_base(c, wid, src);
-      g.M = ly.in;
-      g.N = c->B;
-      g.K = ly.out;
-      g.a_z_src = 1;
-      g.b_z_src = 0;
-      g.hmask = c->A[l];
-      g.out = c->g_rows ? c->G[l - 1] : nullptr;
-      g.b_mn = c->g_rows ? 0 : 1;
-      g.pdl = c->profiling ? 0 : 1;
-      g.outT = c->GT[l - 1];
-      g.gb_out = c->gb[l - 1];
-      ProfScope ps(c, "gemm_dh", st);
-      if ((e = launch_gemm(kEpiDh, c->mShadowMN[l], c->g_rows ? c->mG[l] : c->mGTmn[l], g, na, st)) != cudaSuccess)
-        return e;
-    }
-    const CUtensorMap& mX = l == 0 ? step_inputs_t(c, s) : c->mAT[l];
-    if (gemm_dw_supported(ly.out, ly.in, c->B)) {
-      DwArgs d{};
-      d.wid = wid;
-      d.src = src;
-      d.n_active = na;
-      d.M = ly.out;
-      d.N = ly.in;
-      d.K = c->B;
-      d.lr = c->lr;
-      d.master = c->slab;
-      d.master_w = c->slab;
-      d.slot_stride = c->P_pad;
-      d.offB = ly.offB;
-      d.gb = c->gb[l];
-      d.err = c->err;
-      d.pdl = c->profiling ? 0 : 1;
-      ProfScope ps(c, "gemm_dw_sgd", st);
-      if ((e = launch_gemm_dw(c->mGT[l], mX, c->mMaster[l], c->mMasterSt[l], c->mShadowSt[l], d, c->sms, st)) !=
-          cudaSuccess)
-        return e;
-      continue;
-    }
     GemmArgs g = gemm_base(c, wid, src);
-    g.M = ly.out;
-    g.N = ly.in;
-    g.K = c->B;
-    g.a_z_src = 0;
+    g.M = ly.in;
+    g.N = c->B;
+    g.K = ly.out;
+    g.a_z_src = 1;
     g.b_z_src = 0;
-    g.offW = ly.offW;
-    g.offB = ly.offB;
-    g.gb_in = c->gb[l];
+    g.hmask = c->A[l];
+    g.out = c->g_rows ? c->G[l - 1] : nullptr;
+    g.b_mn = c->g_rows ? 0 : 1;
+    g.pdl = c->profiling ? 0 : 1;
+    g.outT = c->GT[l - 1];
+    g.gb_out = c->gb[l - 1];
+    ProfScope ps(c, "gemm_dh", st);
+    if ((e = launch_gemm(kEpiDh, c->mShadowMN[l], c->g_rows ? c->mG[l] : c->mGTmn[l], g, na, st)) != cudaSuccess)
+      return e;
+  }
+  // the weight gradients of all hidden layers, after the last input gradient
+  // has read the old weights
+  for (int l0 = 0; l0 + 1 < c->L; l0 += kDwMaxLayers) {
+    DwArgs d{};
+    DwMaps m;
+    d.wid = wid;
+    d.src = src;
+    d.n_active = na;
+    d.K = c->B;
+    d.lr = c->lr;
+    d.master = c->slab;
+    d.master_w = c->slab;
+    d.slot_stride = c->P_pad;
+    d.err = c->err;
+    d.pdl = c->profiling ? 0 : 1;
+    for (int l = l0; l + 1 < c->L && l < l0 + kDwMaxLayers; ++l) {
+      const Layer& ly = c->layers[l];
+      d.layer[d.n_layers] = DwLayer{ly.out, ly.in, ly.offB, c->gb[l]};
+      m.l[d.n_layers] = {c->mGT[l], l == 0 ? step_inputs_t(c, s) : c->mAT[l], c->mMaster[l], c->mMasterSt[l], c->mShadowSt[l]};
+      ++d.n_layers;
+    }
     ProfScope ps(c, "gemm_dw_sgd", st);
-    if ((e = launch_gemm(kEpiDw, c->mGT[l], mX, g, na, st)) != cudaSuccess) return e;
+    if ((e = launch_gemm_dw(m, d, c->sms, st)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }

@@ -1,4 +1,4 @@
-// Weight gradient + SGD of one dense layer for every active worker in one
+// Weight gradient + SGD of every hidden layer for every active worker in one
 // persistent launch (Eq. 4, "otherwise" branch: x <- x - lr g(x)):
 //
 //   dW[m][n] = sum_b G[b][m] X[b][n]        bf16 operands, fp32 sums in TMEM
@@ -9,8 +9,11 @@
 // batch).  The work is the stream of the fp32 master (read once, written
 // once) and its bf16 copy, so the kernel is built around moving those bytes
 // asynchronously:
-//  * tiles of 128 x 128 outputs, tile t = (lane, m-tile, n-tile) with n
-//    fastest, CTAs striding over the tiles (one CTA per SM);
+//  * tiles of 128 x 128 outputs, tile t = (layer, lane, m-tile, n-tile) with n
+//    fastest, CTAs striding over the tiles (one CTA per SM).  The layers of a
+//    step share the launch (their input gradients have all run before): with
+//    a launch per layer each paid its own start and last wave (1000-384-256-17,
+//    5 workers, a round: 440 -> 386 us; 3072-1024-1024-10, 32: 1625 -> 1594);
 //  * warp 0 lane 0 (TMA producer) loads each tile's fp32 master block into
 //    one of two buffers (four 32-column boxes, 128-byte swizzle) as soon as
 //    that buffer is free, and the operand k-blocks through a 2-slot ring;
@@ -55,18 +58,19 @@ struct DwBars {
   uint32_t tmem;
 };
 
-__device__ __forceinline__ void dw_tile_coords(const DwArgs& a, int t, int mt, int nt, int& lane, int& m0, int& n0) {
-  lane = t / (mt * nt);
-  const int r = t - lane * mt * nt;
+// the layer, lane and corner of tile t
+__device__ __forceinline__ void dw_tile_coords(const DwArgs& a, int t, int& layer, int& lane, int& m0, int& n0) {
+  layer = 0;
+  while (layer + 1 < a.n_layers && t >= a.first_tile[layer + 1]) ++layer;
+  const DwLayer& ly = a.layer[layer];
+  const int mt = ly.M / kDwTile, nt = (ly.N + kDwTile - 1) / kDwTile, u = t - a.first_tile[layer];
+  lane = u / (mt * nt);
+  const int r = u - lane * mt * nt;
   m0 = (r / nt) * kDwTile;
   n0 = (r % nt) * kDwTile;
 }
 
-__global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_constant__ CUtensorMap mapA,
-                                                                 const __grid_constant__ CUtensorMap mapB,
-                                                                 const __grid_constant__ CUtensorMap mapMaster,
-                                                                 const __grid_constant__ CUtensorMap mapMasterSt,
-                                                                 const __grid_constant__ CUtensorMap mapShadowSt,
+__global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_constant__ DwMaps maps,
                                                                  const __grid_constant__ DwArgs a) {
   extern __shared__ uint8_t dw_smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dw_smem_raw) + 1023) & ~uintptr_t(1023));
@@ -76,16 +80,17 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
   DwBars* bars = reinterpret_cast<DwBars*>(smem + kDwOffBar);
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane_id = threadIdx.x & 31;
-  const int mt = a.M / kDwTile, nt = (a.N + kDwTile - 1) / kDwTile;
-  const int tiles = a.n_active * mt * nt;
+  const int tiles = a.first_tile[a.n_layers];
   const int nk = (a.K + kDwBK - 1) / kDwBK;
 
   if (threadIdx.x == 0) {
-    prefetch_tmap(&mapA);
-    prefetch_tmap(&mapB);
-    prefetch_tmap(&mapMaster);
-    prefetch_tmap(&mapMasterSt);
-    prefetch_tmap(&mapShadowSt);
+    for (int l = 0; l < a.n_layers; ++l) {
+      prefetch_tmap(&maps.l[l].gt);
+      prefetch_tmap(&maps.l[l].xt);
+      prefetch_tmap(&maps.l[l].master);
+      prefetch_tmap(&maps.l[l].master_st);
+      prefetch_tmap(&maps.l[l].shadow_st);
+    }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bars->full[i], 1);
       mbar_init(&bars->empty[i], 1);
@@ -115,8 +120,8 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
     int armed_ops[2] = {0, 0}, armed_master[2] = {0, 0};
     bool ok = true;
     for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x, ++it) {
-      int li, m0, n0;
-      dw_tile_coords(a, t, mt, nt, li, m0, n0);
+      int ly, li, m0, n0;
+      dw_tile_coords(a, t, ly, li, m0, n0);
       const int wid = a.wid ? a.wid[li] : li, src = a.src ? a.src[li] : li;
       const int b = it & 1;
       if (it >= 2 && !(ok = mbar_wait(&bars->mempty[b], ((it >> 1) + 1) & 1, a.err, kDevTimeoutEmpty))) break;
@@ -124,14 +129,14 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
       ++armed_master[b];
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        tma_load_3d(sMaster + b * kDwMasterBytes + q * kDwBoxF32, &mapMaster, n0 + 32 * q, m0, src, &bars->mfull[b]);
+        tma_load_3d(sMaster + b * kDwMasterBytes + q * kDwBoxF32, &maps.l[ly].master, n0 + 32 * q, m0, src, &bars->mfull[b]);
       for (int kb = 0; kb < nk; ++kb, ++kc) {
         const int s = kc & 1;
         if (kc >= 2 && !(ok = mbar_wait(&bars->empty[s], ((kc >> 1) + 1) & 1, a.err, kDevTimeoutEmpty))) break;
         mbar_arrive_expect_tx(&bars->full[s], kDwOpBytes);
         ++armed_ops[s];
-        tma_load_3d(sOps + s * kDwOpBytes, &mapA, kb * kDwBK, m0, wid, &bars->full[s]);
-        tma_load_3d(sOps + s * kDwOpBytes + kDwOpBytes / 2, &mapB, kb * kDwBK, n0, wid, &bars->full[s]);
+        tma_load_3d(sOps + s * kDwOpBytes, &maps.l[ly].gt, kb * kDwBK, m0, wid, &bars->full[s]);
+        tma_load_3d(sOps + s * kDwOpBytes + kDwOpBytes / 2, &maps.l[ly].xt, kb * kDwBK, n0, wid, &bars->full[s]);
       }
     }
     // no copy may still be landing in shared memory when the CTA ends (all
@@ -177,8 +182,8 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
     const uint32_t rsw = static_cast<uint32_t>(r & 7);      // 128-byte swizzle phase of this row
     int it = 0;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {
-      int li, m0, n0;
-      dw_tile_coords(a, t, mt, nt, li, m0, n0);
+      int ly, li, m0, n0;
+      dw_tile_coords(a, t, ly, li, m0, n0);
       const int wid = a.wid ? a.wid[li] : li, src = a.src ? a.src[li] : li;
       const int b = it & 1;
       const bool ok = mbar_wait(&bars->afull[b], (it >> 1) & 1, a.err, kDevTimeoutAccum) &&
@@ -231,19 +236,20 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
           const int col0 = 64 * h + 32 * c;
-          if (n0 + col0 < a.N)
-            tma_store_3d(&mapMasterSt, mblk + (col0 / 32) * kDwBoxF32 + 32 * q * 128, n0 + col0, m0 + 32 * q, wid);
+          if (n0 + col0 < a.layer[ly].N)
+            tma_store_3d(&maps.l[ly].master_st, mblk + (col0 / 32) * kDwBoxF32 + 32 * q * 128, n0 + col0, m0 + 32 * q, wid);
         }
-        if (n0 + 64 * h < a.N)
-          tma_store_3d(&mapShadowSt, sShadow + h * kDwBoxBf16 + 32 * q * 128, n0 + 64 * h, m0 + 32 * q, wid);
+        if (n0 + 64 * h < a.layer[ly].N)
+          tma_store_3d(&maps.l[ly].shadow_st, sShadow + h * kDwBoxBf16 + 32 * q * 128, n0 + 64 * h, m0 + 32 * q, wid);
         bulk_commit_group();
       }
       // bias with the first column tile
       if (h == 0 && n0 == 0) {
         const int m = m0 + r;
-        a.master_w[static_cast<int64_t>(wid) * a.slot_stride + a.offB + m] =
-            fmaf(-a.lr, a.gb[static_cast<int64_t>(wid) * a.M + m],
-                 a.master[static_cast<int64_t>(src) * a.slot_stride + a.offB + m]);
+        const int64_t offB = a.layer[ly].offB;
+        a.master_w[static_cast<int64_t>(wid) * a.slot_stride + offB + m] =
+            fmaf(-a.lr, a.layer[ly].gb[static_cast<int64_t>(wid) * a.layer[ly].M + m],
+                 a.master[static_cast<int64_t>(src) * a.slot_stride + offB + m]);
       }
     }
     if (lane_id == 0) bulk_wait_all();
@@ -258,18 +264,19 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
 
 }  // namespace
 
-bool gemm_dw_supported(int M, int N, int K) { return M % kDwTile == 0 && N % 8 == 0 && K >= 1; }
-
-cudaError_t launch_gemm_dw(const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mMaster,
-                           const CUtensorMap& mMasterSt, const CUtensorMap& mShadowSt, const DwArgs& a, int sms,
-                           cudaStream_t s) {
-  if (!gemm_dw_supported(a.M, a.N, a.K) || a.n_active < 1 || sms < 1) return cudaErrorInvalidValue;
+cudaError_t launch_gemm_dw(const DwMaps& maps, DwArgs a, int sms, cudaStream_t s) {
+  if (a.n_layers < 1 || a.n_layers > kDwMaxLayers || a.n_active < 1 || sms < 1 || a.K < 1) return cudaErrorInvalidValue;
+  a.first_tile[0] = 0;
+  for (int l = 0; l < a.n_layers; ++l) {
+    const DwLayer& ly = a.layer[l];
+    if (ly.M % kDwTile != 0 || ly.N % 8 != 0) return cudaErrorInvalidValue;
+    a.first_tile[l + 1] = a.first_tile[l] + a.n_active * (ly.M / kDwTile) * ((ly.N + kDwTile - 1) / kDwTile);
+  }
   cudaError_t e = cudaFuncSetAttribute(gemm_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDwSmem);
   if (e != cudaSuccess) return e;
-  const int tiles = a.n_active * (a.M / kDwTile) * ((a.N + kDwTile - 1) / kDwTile);
-  const int grid = tiles < sms ? tiles : sms;
+  const int tiles = a.first_tile[a.n_layers];
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.gridDim = dim3(tiles < sms ? tiles : sms, 1, 1);
   cfg.blockDim = dim3(kDwThreads, 1, 1);
   cfg.dynamicSmemBytes = kDwSmem;
   cfg.stream = s;
@@ -278,7 +285,7 @@ cudaError_t launch_gemm_dw(const CUtensorMap& mA, const CUtensorMap& mB, const C
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = a.pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, gemm_dw_kernel, mA, mB, mMaster, mMasterSt, mShadowSt, a);
+  return cudaLaunchKernelEx(&cfg, gemm_dw_kernel, maps, a);
 }
 
 }  // namespace oscars

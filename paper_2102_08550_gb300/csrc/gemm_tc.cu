@@ -18,10 +18,6 @@
 //  kEpiDh   input gradient of a hidden layer, m = input feature, n = sample:
 //           g = acc * (Hmask[n][m] > 0) -> bf16 G[n][m], G^T[m][n] and the
 //           bias gradient gb[m] = sum_n g (fp32, whole batch in one tile).
-//  kEpiDw   weight gradient + SGD, m = output feature, n = input feature:
-//           W[dst] = fmaf(-lr, acc, W[src]) (fp32 master), bf16 shadow,
-//           optional bf16 transposed shadow; column-tile 0 also updates the
-//           bias b[dst] = fmaf(-lr, gb[m], b[src]).
 //
 // All waits are bounded (see common.cuh) and report through a device word.
 #include <cstdio>
@@ -37,13 +33,7 @@ constexpr int BM = 128;
 constexpr int BK = 64;
 constexpr int kABytes = BM * BK * 2;
 constexpr int kBarrierBytes = 256;          // mbarriers + TMEM address slot
-constexpr int kEpiTileFloats = 32 * 36;     // per-warp staging tile (row stride 36: conflict-free 16-byte accesses)
-
-// Warps per CTA: the weight-gradient epilogue streams the fp32 master and
-// runs two warpgroups (each warp owns its TMEM lane quarter, the two groups
-// split the columns); the others use one warpgroup.
-template <int EPI>
-constexpr int warps_for() { return EPI == kEpiDw ? 8 : 4; }
+constexpr int kWarps = 4;
 
 template <int BN>
 struct TileCfg {
@@ -110,58 +100,6 @@ __device__ __forceinline__ float epi_dh(const GemmArgs& a, int wid, int m, int n
   return gsum;
 }
 
-// Weight gradient + SGD for one 32 x 32 block: rows m_base .. m_base + 31
-// (thread `lane` holds row m_base + lane in v), columns n_base .. n_base + 31.
-// `old` holds the block's fp32 master values in the column layout of the
-// store pass: old[i] (i < 8) = 4 columns (n_base + 4 (lane % 8) ..) of row
-// m_base + 4 i + lane / 8.  The accumulators go through a shared-memory tile
-// (row stride 36: 16-byte accesses of 8 lanes hit distinct banks both along
-// rows and along columns) so that the fp32 master and bf16 shadow writes move
-// full lines, 4 rows per instruction.  (The persistent kernel of gemm_dw.cu
-// serves every layer whose input count is a multiple of 8; this epilogue is
-// the general fallback.)
-__device__ __forceinline__ void epi_dw_block(const GemmArgs& a, int wid, int m_base, int n_base,
-                                             const float (&v)[32], const float4 (&old)[8], float* T, int lane) {
-#pragma unroll
-  for (int q = 0; q < 8; ++q)
-    *reinterpret_cast<float4*>(T + lane * 36 + 4 * q) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-  __syncwarp();
-  const int cq = (lane & 7) * 4;
-  const bool nok = n_base + cq < a.N;     // N % 8 == 0: a 4-column group is all in or all out
-  const int64_t dof = static_cast<int64_t>(wid) * a.slot_stride + a.offW + n_base + cq;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int r = 4 * i + (lane >> 3);
-    const float4 g = *reinterpret_cast<const float4*>(T + r * 36 + cq);
-    float4 nw;
-    nw.x = fmaf(-a.lr, g.x, old[i].x);
-    nw.y = fmaf(-a.lr, g.y, old[i].y);
-    nw.z = fmaf(-a.lr, g.z, old[i].z);
-    nw.w = fmaf(-a.lr, g.w, old[i].w);
-    if (nok) {
-      const int64_t e = dof + static_cast<int64_t>(m_base + r) * a.N;
-      *reinterpret_cast<float4*>(a.master_w + e) = nw;
-      *reinterpret_cast<uint2*>(a.shadow + e) = make_uint2(pack_bf16x2(nw.x, nw.y), pack_bf16x2(nw.z, nw.w));
-    }
-  }
-  __syncwarp();
-}
-
-// old[i] = master[src][m_base + 4 i + lane / 8][n_base + 4 (lane % 8) ..] as
-// float4 (0 outside N): all 8 loads issued before any is used
-__device__ __forceinline__ void epi_dw_load(const GemmArgs& a, int src, int m_base, int n_base, int lane,
-                                            float4 (&old)[8]) {
-  const int cq = (lane & 7) * 4;
-  const bool nok = n_base + cq < a.N;
-  const int64_t so = static_cast<int64_t>(src) * a.slot_stride + a.offW + n_base + cq;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int r = 4 * i + (lane >> 3);
-    old[i] = nok ? *reinterpret_cast<const float4*>(a.master + so + static_cast<int64_t>(m_base + r) * a.N)
-                 : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-}
-
 // Split-K (SPLIT > 1, forward and input-gradient epilogues): a cluster of
 // SPLIT CTAs shares one output tile, CTA r multiplying K-blocks [r nk / SPLIT,
 // (r + 1) nk / SPLIT).  Each CTA pushes its fp32 partial rows into the CTA
@@ -180,7 +118,7 @@ __device__ __forceinline__ void st_dsmem_f32x4(float* local, uint32_t rank, floa
 }
 
 template <int BN, int EPI, int SPLIT = 1>
-__global__ void __launch_bounds__(warps_for<EPI>() * 32) gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA,
+__global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA,
                                                            const __grid_constant__ CUtensorMap mapB,
                                                            const __grid_constant__ GemmArgs a,
                                                            int stages) {
@@ -312,7 +250,7 @@ __global__ void __launch_bounds__(warps_for<EPI>() * 32) gemm_tc_kernel(const __
     cluster_sync();   // every partial has landed in its owner
     // own rows: item = (row, 32-column chunk); partials summed in rank order
     float* gpart = red + SPLIT * R * ld;            // [R][BN / 32] bias-gradient partials (input gradient)
-    for (int it = threadIdx.x; it < R * (BN / 32); it += warps_for<EPI>() * 32) {
+    for (int it = threadIdx.x; it < R * (BN / 32); it += kWarps * 32) {
       const int rl = it / (BN / 32), c0 = (it % (BN / 32)) * 32;
       float v[32];
 #pragma unroll
@@ -340,7 +278,7 @@ __global__ void __launch_bounds__(warps_for<EPI>() * 32) gemm_tc_kernel(const __
     }
     if constexpr (EPI == kEpiDh) {
       __syncthreads();
-      for (int rl = threadIdx.x; rl < R; rl += warps_for<EPI>() * 32) {
+      for (int rl = threadIdx.x; rl < R; rl += kWarps * 32) {
         float g = 0.f;
         for (int c = 0; c < BN / 32; ++c) g += gpart[rl * (BN / 32) + c];
         a.gb_out[static_cast<int64_t>(wid) * a.M + m0 + rank * R + rl] = g;
@@ -358,13 +296,6 @@ __global__ void __launch_bounds__(warps_for<EPI>() * 32) gemm_tc_kernel(const __
   // epilogue: thread = one accumulator row
   unsigned short mk[32];   // input-gradient mask of the next 32 columns, read while the MMAs run
   if constexpr (EPI == kEpiDh) epi_dh_mask(a, wid, m0 + (warp & 3) * 32 + lane, n0, mk);
-  float4 old0[8], old1[8];  // weight-gradient epilogue: the fp32 master block, read while the MMAs run
-  if constexpr (EPI == kEpiDw) {
-    const int c_begin = (warp >> 2) * (BN / 2);
-    const int mb = m0 + (warp & 3) * 32;
-    epi_dw_load(a, src, mb, n0 + c_begin, lane, old0);
-    epi_dw_load(a, src, mb, n0 + c_begin + 32, lane, old1);
-  }
   int acc_ok = mbar_wait(accum, 0, a.err, kDevTimeoutAccum) ? 1 : 0;
   acc_ok = __all_sync(0xffffffffu, acc_ok);
   tc_fence_after();
@@ -372,27 +303,7 @@ __global__ void __launch_bounds__(warps_for<EPI>() * 32) gemm_tc_kernel(const __
     const int quarter = warp & 3;
     const int m = m0 + quarter * 32 + lane;
     const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
-    if constexpr (EPI == kEpiDw) {
-      static_assert(BN == 128, "the weight-gradient epilogue covers 2 x 32 columns per warp");
-      const int c_begin = (warp >> 2) * (BN / 2);
-      const int mb = m0 + quarter * 32;
-      float* T = epi_tiles + warp * kEpiTileFloats;
-      if (n0 + c_begin < a.N) {
-        float v[32];
-        tmem_ld_32x32b_x32(trow + c_begin, v);
-        epi_dw_block(a, wid, mb, n0 + c_begin, v, old0, T, lane);
-      }
-      if (n0 + c_begin + 32 < a.N) {
-        float v[32];
-        tmem_ld_32x32b_x32(trow + c_begin + 32, v);
-        epi_dw_block(a, wid, mb, n0 + c_begin + 32, v, old1, T, lane);
-      }
-      if (warp < 4 && blockIdx.y == 0) {
-        const int64_t bo = a.offB + m;
-        a.master_w[static_cast<int64_t>(wid) * a.slot_stride + bo] =
-            fmaf(-a.lr, a.gb_in[static_cast<int64_t>(wid) * a.M + m], a.master[static_cast<int64_t>(src) * a.slot_stride + bo]);
-      }
-    } else if constexpr (EPI == kEpiDh) {
+    if constexpr (EPI == kEpiDh) {
       float gsum = 0.f;
 #pragma unroll
       for (int c0 = 0; c0 < BN; c0 += 32) {
@@ -457,12 +368,10 @@ cudaError_t launch_tile(const CUtensorMap& mA, const CUtensorMap& mB, const Gemm
   const size_t red_bytes = SPLIT > 1 ? sizeof(float) * (static_cast<size_t>(BM) * (BN + kRedLd) + BM / SPLIT * (BN / 32))
                                      : 0;
   const int budget = SPLIT > 1 ? 150 * 1024 : ctas > sms ? 100 * 1024 : 200 * 1024;
-  const int max_stages = static_cast<int>((budget - (EPI == kEpiDw ? 8 * 32 * 33 * 4 : 0)) / Cfg::kStageBytes);
+  const int max_stages = budget / Cfg::kStageBytes;
   int stages = nk < max_stages ? nk : (max_stages < 8 ? max_stages : 8);
   if (stages < 2) stages = nk < 2 ? nk : 2;
-  constexpr int kWarps = warps_for<EPI>();
-  size_t smem = 1024 + static_cast<size_t>(stages) * Cfg::kStageBytes + kBarrierBytes +
-                (EPI == kEpiDw ? sizeof(float) * kWarps * kEpiTileFloats : 0) + red_bytes;
+  size_t smem = 1024 + static_cast<size_t>(stages) * Cfg::kStageBytes + kBarrierBytes + red_bytes;
   const size_t floor_b = smem_floor_for_tmem(Cfg::kTmemCols);
   if (smem < floor_b) smem = floor_b;
   cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -507,14 +416,12 @@ int split_for(int M, int N, int BN, int K, int n_active) {
 }  // namespace
 
 int gemm_bn_for(int epi, int N) {
-  if (epi == kEpiDw) return 128;
   return N;  // forward / input gradient: the whole batch in one tile
 }
 
 cudaError_t launch_gemm(int epi, const CUtensorMap& mA, const CUtensorMap& mB, const GemmArgs& a,
                         int n_active, cudaStream_t s) {
   if (a.M % BM != 0) return cudaErrorInvalidValue;
-  if (epi == kEpiDw) return launch_tile<128, kEpiDw>(mA, mB, a, n_active, s);
   const int bn = gemm_bn_for(epi, a.N);
   const int split = bn == 128 ? split_for(a.M, a.N, bn, a.K, n_active) : 1;
   if (epi == kEpiFwd) {

@@ -138,7 +138,7 @@ cudaError_t launch_stage_round_strided(const StageArgs& a, const int32_t* tau, i
 cudaError_t launch_stage_round_priority(const StageArgs& a, const int32_t* tau, int W, int max_tau, int priority,
                                         cudaStream_t s);
 
-enum GemmEpi { kEpiFwd = 0, kEpiDh = 1, kEpiDw = 2 };
+enum GemmEpi { kEpiFwd = 0, kEpiDh = 1 };
 
 struct GemmArgs {
   const int* wid;     // [n_active]
@@ -150,14 +150,9 @@ struct GemmArgs {
   int* err;
   // kEpiFwd: out = relu(acc + bias[m]) -> H [lane][N][M], HT [lane][M][N]
   // kEpiDh : out = acc * (Hmask[lane][n][m] > 0) -> G (if out), GT, gb[lane][m]
-  // kEpiDw : W[dst] = W[src] - lr * acc (rows m, cols n < N), shadows, bias
   const float* master;      // fp32 slab base
-  float* master_w;          // same slab (written)
-  __nv_bfloat16* shadow;    // bf16 slab (same layout as master)
   int64_t slot_stride;      // P_pad
-  int64_t offW, offB;       // element offsets of W_l, b_l in a slot
-  float lr;
-  const float* gb_in;       // [lanes][M] bias gradient (kEpiDw)
+  int64_t offB;             // element offset of b_l in a slot
   const __nv_bfloat16* hmask;  // [lanes][N][M] (kEpiDh)
   __nv_bfloat16* out;       // [lanes][N][M]
   __nv_bfloat16* outT;      // [lanes][M][N]
@@ -190,32 +185,41 @@ RowsPlan gemm_rows_plan(int epi, int M, int N, int K);
 cudaError_t launch_gemm_rows(int epi, const RowsPlan& p, const CUtensorMap& mA, const CUtensorMap& mB,
                              const CUtensorMap& mD, RowsArgs a, cudaStream_t s);
 
-// Weight gradient + SGD of one layer, persistent (csrc/gemm_dw.cu):
-// W[wid] = W[src] - lr * G^T X over the batch, its bf16 copy, and the bias
-// b[wid] = b[src] - lr * gb[wid] (outputs m < M, inputs n < N, batch K).
+// Weight gradient + SGD of up to kDwMaxLayers hidden layers, persistent
+// (csrc/gemm_dw.cu): W[wid] = W[src] - lr * G^T X over the batch, its bf16
+// copy, and the bias b[wid] = b[src] - lr * gb[wid] (outputs m < M, inputs n <
+// N, batch K; M a multiple of 128, N of 8).
+constexpr int kDwMaxLayers = 4;
+struct DwLayer {
+  int M, N;
+  int64_t offB;             // element offset of b_l in a slot
+  const float* gb;          // [W][M] bias gradient
+};
 struct DwArgs {
   const int* wid;           // [n_active] destination slots (device), or null = lane id
   const int* src;           // [n_active] source slots (device), or null = lane id
-  int n_active;
-  int M, N, K;
+  int n_active, n_layers;
+  int K;
   float lr;
   const float* master;      // fp32 slab (bias read)
   float* master_w;          // fp32 slab (bias written)
   int64_t slot_stride;      // P_pad
-  int64_t offB;             // element offset of b_l in a slot
-  const float* gb;          // [W][M] bias gradient
+  DwLayer layer[kDwMaxLayers];
+  int first_tile[kDwMaxLayers + 1];   // set by the launcher
   int* err;
   int pdl;                  // launch as a programmatic dependent of the previous kernel on the stream
 };
-bool gemm_dw_supported(int M, int N, int K);
-// mA: G^T [lane][M][K] bf16, box {64, 128}; mB: X^T [lane][N][K] bf16, box
-// {64, 128}; mMaster: W_l fp32 [slot][M][N], box {32, 128} (loads);
-// mMasterSt: the same with box {32, 32} (stores); mShadowSt: W_l bf16
-// [slot][M][N], box {64, 32} (stores); all with 128-byte swizzle.  `sms`:
-// the device's multiprocessors (one CTA each at most).
-cudaError_t launch_gemm_dw(const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mMaster,
-                           const CUtensorMap& mMasterSt, const CUtensorMap& mShadowSt, const DwArgs& a, int sms,
-                           cudaStream_t s);
+// gt: G^T [lane][M][K] bf16, box {64, 128}; xt: X^T [lane][N][K] bf16, box
+// {64, 128}; master: W_l fp32 [slot][M][N], box {32, 128} (loads); master_st:
+// the same with box {32, 32} (stores); shadow_st: W_l bf16 [slot][M][N], box
+// {64, 32} (stores); all with 128-byte swizzle
+struct DwMaps {
+  struct Layer {
+    CUtensorMap gt, xt, master, master_st, shadow_st;
+  } l[kDwMaxLayers];
+};
+// `sms`: the device's multiprocessors (one CTA each at most)
+cudaError_t launch_gemm_dw(const DwMaps& maps, DwArgs a, int sms, cudaStream_t s);
 int gemm_bn_for(int epi, int N);
 
 struct HeadArgs {
