@@ -11,8 +11,11 @@
 //     are zero-filled by the TMA loads), K = F features;
 //  2. cluster barrier; the logits are the partials of ranks 0..n-1 summed in
 //     that order from distributed shared memory, plus the bias; softmax
-//     cross-entropy per row (one thread per row); dz (fp32) and its bf16
-//     copy, written into two shared tiles laid out as tensor-core operands;
+//     cross-entropy on 2, 4 or 8 threads per row, four classes at a time
+//     (with one thread a row its divisions and bank conflicts took 8800 of
+//     the kernel's 22500 clocks with 17 classes, 4500 with 10); dz (fp32) and
+//     its bf16 copy, written into two shared tiles laid out as tensor-core
+//     operands;
 //  3. head weight gradient dW2^T[f][c] = sum_b h[b][f] dz[b][c] (per half
 //     M = 128 features, N = NC, K = B: the h tile read MN-major) and SGD of
 //     the CTA's head columns;
@@ -55,8 +58,9 @@ struct HTCfg {
   static constexpr int oDzT = oW2 + (F / 64) * NC * 128;    // dz^T: [16 classes][B rows] K-major (K = rows), 2 atoms
   static constexpr int oDzK = oDzT + 2 * NC * 128;       // dz: [B rows][NC classes] K-major, no swizzle
   static constexpr int oPl = oDzK + kHTRows * NC * 2;    // [128][NC] fp32 partial logits (read by the cluster)
-  static constexpr int oDz = oPl + kHTRows * NC * 4;   // [128][16] fp32 dlogits
-  static constexpr int oLoss = oDz + kHTRows * NC * 4; // [128]
+  static constexpr int oDz = oPl + kHTRows * NC * 4;   // [128][kLdz] fp32 dlogits
+  static constexpr int kLdz = NC + 4;                    // row stride of dz: rows of neighbouring threads in other banks
+  static constexpr int oLoss = oDz + kHTRows * kLdz * 4; // [128]
   static constexpr int oGbp = oLoss + kHTRows * 4;       // [2][F]
   static constexpr int oLab = oGbp + 2 * F * 4;          // [128] int
   static constexpr int oB2 = oLab + kHTRows * 4;         // [16]
@@ -179,6 +183,16 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
     tmem_alloc(tmem_slot, Cfg::kTmemCols);
     tmem_relinquish();
   }
+  // the old master values of this thread's head column, requested long before
+  // the update needs them (and before any new value is stored: source and
+  // destination slots may be the same slab)
+  float old[CL];
+  if (warp < 4 * NH) {
+    const int f = kHT * (warp >> 2) + 32 * (warp & 3) + lane;
+#pragma unroll
+    for (int c = 0; c < CL; ++c)
+      if (c < C) old[c] = a.master[so + a.offW + static_cast<int64_t>(c) * H + k0 + f];
+  }
   // the dz tiles' padding (classes >= C, rows >= B) stays zero
   for (int q = t; q < (2 * NC * 128 + kHTRows * NC * 2) / 16; q += kHTThreads)
     reinterpret_cast<uint4*>(dzT)[q] = make_uint4(0, 0, 0, 0);
@@ -222,77 +236,89 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
   cluster_sync();
   tc_fence_after();
 
-  // ---- 2. logits (cluster sum in rank order), softmax cross-entropy, dz tiles
-  if (t < B) {
-    const int b = t;
-    constexpr int QN = (CL + 3) / 4;                 // 16-byte chunks of a row of partial logits
-    constexpr int RG = QN <= 4 ? kHTMaxCluster : 2;  // ranks whose partials are in flight at once
-    float z[4 * QN];
+  // ---- 2. logits (cluster sum in rank order), softmax cross-entropy, dz tiles.
+  // TPR threads per row (the whole block for B = 32, 64 and 128), thread q
+  // takes the 4-class chunks q, q + TPR, ...
+  {
+    const int tsh = B <= 32 ? 3 : B <= 64 ? 2 : 1, tpr = 1 << tsh;   // 8, 4 or 2
+    const int b = t >> tsh, q = t & (tpr - 1);
+    constexpr int QN = (CL + 3) / 4;      // chunks with classes
+    constexpr int QT = (QN + 1) / 2;      // chunks of a thread at most (two threads a row)
+    const bool row = b < B;
+    float z[4 * QT];
 #pragma unroll
-    for (int c = 0; c < 4 * QN; ++c) z[c] = 0.f;
-    // the ranks' partials are requested before the first is added (a remote
-    // load waits a round trip across the cluster)
+    for (int i = 0; i < 4 * QT; ++i) z[i] = 0.f;
+    if (row) {
+      // the ranks' partials are requested before the first is added (a remote
+      // load waits a round trip across the cluster)
+      float4 p[kHTMaxCluster][QT];
 #pragma unroll
-    for (int r0 = 0; r0 < kHTMaxCluster; r0 += RG) {
-      if (r0 >= ncl) continue;
-      float4 p[RG][QN];
+      for (int r = 0; r < kHTMaxCluster; ++r)
 #pragma unroll
-      for (int r = 0; r < RG; ++r)
-        if (r0 + r < ncl)
+        for (int i = 0; i < QT; ++i)
+          if (r < ncl && q + i * tpr < QN) p[r][i] = ld_dsmem_f32x4(pl + b * NC + 4 * (q + i * tpr), r);
 #pragma unroll
-          for (int q = 0; q < QN; ++q) p[r][q] = ld_dsmem_f32x4(pl + b * NC + 4 * q, r0 + r);
+      for (int r = 0; r < kHTMaxCluster; ++r)
 #pragma unroll
-      for (int r = 0; r < RG; ++r)
-        if (r0 + r < ncl)
-#pragma unroll
-          for (int q = 0; q < QN; ++q) {
-            z[4 * q] += p[r][q].x;
-            z[4 * q + 1] += p[r][q].y;
-            z[4 * q + 2] += p[r][q].z;
-            z[4 * q + 3] += p[r][q].w;
+        for (int i = 0; i < QT; ++i)
+          if (r < ncl && q + i * tpr < QN) {
+            z[4 * i] += p[r][i].x;
+            z[4 * i + 1] += p[r][i].y;
+            z[4 * i + 2] += p[r][i].z;
+            z[4 * i + 3] += p[r][i].w;
           }
     }
-    const int y = labs[b];
-    float m = -INFINITY, zy = 0.f;
+    const int y = row ? labs[b] : 0;
+    float m = -INFINITY, zy = -INFINITY;
 #pragma unroll
-    for (int c = 0; c < CL; ++c)
-      if (c < C) {
-        z[c] += b2[c];
-        m = fmaxf(m, z[c]);
-        if (c == y) zy = z[c];
-      }
+    for (int i = 0; i < 4 * QT; ++i) {
+      const int c = 4 * (q + i / 4 * tpr) + i % 4;
+      z[i] = c < C ? z[i] + b2[c < NC ? c : 0] : -INFINITY;
+      m = fmaxf(m, z[i]);
+      if (c == y) zy = z[i];
+    }
+    for (int o = tpr >> 1; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     float s = 0.f, so_ = 0.f;
 #pragma unroll
-    for (int c = 0; c < CL; ++c)
-      if (c < C) {
-        z[c] = expf(z[c] - m);
-        s += z[c];
-        if (c != y) so_ += z[c];
-      }
-    rowloss[b] = m + logf(s) - zy;
-    const float inv = 1.0f / static_cast<float>(B);
-    float g[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      g[c] = c < CL && c < C ? (c == y ? -so_ : z[c < CL ? c : 0]) / s * inv : 0.f;
-      if (c < CL && c < C) dz[b * NC + c] = g[c];
+    for (int i = 0; i < 4 * QT; ++i) {
+      const int c = 4 * (q + i / 4 * tpr) + i % 4;
+      z[i] = c < C ? expf(z[i] - m) : 0.f;
+      s += z[i];
+      if (c != y) so_ += z[i];
     }
-    // dz as the K-major [rows][NC classes] operand: classes 8 k .. 8 k + 7 one
-    // 16-byte chunk of core matrix (b / 8, k)
-    uint8_t* ck = dzK + (b >> 3) * (NC / 8 * 128) + (b & 7) * 16;
+    for (int o = tpr >> 1; o > 0; o >>= 1) {
+      s += __shfl_xor_sync(0xffffffffu, s, o);
+      so_ += __shfl_xor_sync(0xffffffffu, so_, o);
+    }
+    const float inv = 1.0f / static_cast<float>(B);
+    if (row) {
+      if (q == ((y >> 2) & (tpr - 1))) rowloss[b] = m + logf(s) - zy;   // the thread that has class y
+      uint8_t* ck = dzK + (b >> 3) * (NC / 8 * 128) + (b & 7) * 16;
+      uint8_t* at = dzT + (b >> 6) * (NC * 128);
+      const int e64 = b & 63;
 #pragma unroll
-    for (int k = 0; k < NC / 8; ++k)
-      *reinterpret_cast<uint4*>(ck + 128 * k) =
-          make_uint4(pack_bf16x2(g[8 * k], g[8 * k + 1]), pack_bf16x2(g[8 * k + 2], g[8 * k + 3]),
-                     pack_bf16x2(g[8 * k + 4], g[8 * k + 5]), pack_bf16x2(g[8 * k + 6], g[8 * k + 7]));
-    // dz^T as the K-major [NC classes][rows] operand (K = rows, atoms of 64 rows)
-    uint8_t* at = dzT + (b >> 6) * (NC * 128);
-    const int e64 = b & 63;
+      for (int i = 0; i < QT; ++i) {
+        const int k = q + i * tpr;
+        if (k >= QN) continue;
+        float g[4];
 #pragma unroll
-    for (int c = 0; c < CL; ++c)
-      if (c < C)
-        *reinterpret_cast<__nv_bfloat16*>(at + c * 128 + ((((e64 >> 3) ^ (c & 7)) & 7) << 4) + (e64 & 7) * 2) =
-            __float2bfloat16_rn(g[c]);
+        for (int j = 0; j < 4; ++j) {
+          const int c = 4 * k + j;
+          g[j] = c < C ? (c == y ? -so_ : z[4 * i + j]) / s * inv : 0.f;
+        }
+        *reinterpret_cast<float4*>(dz + b * Cfg::kLdz + 4 * k) = make_float4(g[0], g[1], g[2], g[3]);
+        // dz as the K-major [rows][NC classes] operand: classes 8 j .. 8 j + 7
+        // one 16-byte chunk of core matrix (b / 8, j)
+        *reinterpret_cast<uint2*>(ck + 128 * (k >> 1) + 8 * (k & 1)) = make_uint2(pack_bf16x2(g[0], g[1]), pack_bf16x2(g[2], g[3]));
+        // dz^T as the K-major [NC classes][rows] operand (K = rows, atoms of 64 rows)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int c = 4 * k + j;
+          *reinterpret_cast<__nv_bfloat16*>(at + c * 128 + ((((e64 >> 3) ^ (c & 7)) & 7) << 4) + (e64 & 7) * 2) =
+              __float2bfloat16_rn(g[j]);
+        }
+      }
+    }
   }
   fence_proxy_async_smem();   // the dz tiles are read by the tensor core
   tc_fence_before();
@@ -328,22 +354,12 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
         const int c = c0 + ((u - 32) >> 3);
         float g = 0.f;
         if (c < C)
-          for (int b = j; b < B; b += 8) g += dz[b * NC + c];
+          for (int b = j; b < B; b += 8) g += dz[b * Cfg::kLdz + c];
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o, 8);
         if (c < C && j == 0) a.master_w[dof + a.offB + c] = fmaf(-a.lr, g, a.master[so + a.offB + c]);
       }
     }
-  }
-  // the old master values of this thread's head column, requested while the
-  // MMAs run and before any new value is stored (source and destination
-  // slots may be the same slab)
-  float old[CL];
-  if (warp < 4 * NH) {
-    const int f = kHT * (warp >> 2) + 32 * (warp & 3) + lane;
-#pragma unroll
-    for (int c = 0; c < CL; ++c)
-      if (c < C) old[c] = a.master[so + a.offW + static_cast<int64_t>(c) * H + k0 + f];
   }
   ok = mbar_wait(mma_bar, 1, a.err, kDevTimeoutAccum) && ok;
   tc_fence_after();
