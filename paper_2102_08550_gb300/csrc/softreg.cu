@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(kThreads) softreg_round_kernel(const __grid_co
 //     summed in shared memory;
 //  2. the partials of a row go to the CTA that owns it with asynchronous
 //     16-byte stores (st.async) that complete on the owner's mbarrier; the
-//     owner adds the kCl partials in rank order and one warp per row (lane =
+//     owner adds the kCl partials in a fixed order and one warp per row (lane =
 //     class) computes the softmax cross-entropy;
 //  3. the row of dz goes to every CTA the same way;
 //  4. weight update of the CTA's columns: a thread sums CC classes x 4
@@ -245,7 +245,9 @@ __global__ void __launch_bounds__(kThreads) softreg_round_kernel(const __grid_co
 //     memory.
 // Four more warps fetch: the rows of step s + 1 come by cp.async into the
 // other of two buffers (and the labels of the CTA's rows beside them) while
-// step s runs; they meet the others once a step.  Classes are kept in rows of "slots": groups of CC classes,
+// step s runs; they meet the others once a step.
+//
+// Classes are kept in rows of "slots": groups of CC classes,
 // each padded to CCp = a multiple of 4 slots (at most 32 slots in all).
 // Every index a thread needs in a step is worked out before the first one or
 // by shifts: an integer division by a run-time value costs as much as a
@@ -261,17 +263,17 @@ __global__ void __launch_bounds__(kThreads) softreg_round_kernel(const __grid_co
 //
 // What bounds it: the latency of the chain (issue slots 39% busy, 0.3% of
 // DRAM).  Eight steps of one 784 x 10 worker, batch 32: 203 us on one CTA,
-// 35 us here (about 3.9 us a step).  A round of 333 x 26, batch 100, 12
+// 35 us here (about 3.3 us a step).  A round of 333 x 26, batch 100, 12
 // workers, with its merge and pull: 373 us with the earlier cluster kernel
-// (cluster barrier, remote reads, one-thread row loops), 134 us now.
-// 784 x 10, 4 workers, at most 4 steps: 49 and 37 us.
+// (cluster barrier, remote reads, one-thread row loops), 128 us now.
+// 784 x 10, 4 workers, at most 4 steps: 49 and 35 us.
 constexpr int kCl = 8;
 // A CTA has NT computing threads and NT / 4 fetching ones.  NT = 512 fills the
 // SM's registers, so 17 to 19 workers run at once; a step of few products
 // leaves most of its warps without work, and NT = 128 lets four CTAs share an
 // SM.  The line: 16 x 2, batch 1, 32 workers, a round: 50 us with the earlier
 // kernel, 62 with NT = 512, 40 with 128; 333 x 26, batch
-// 100, 24 workers: 140 us with 512, 392 with the earlier 256-thread kernel.
+// 100, 24 workers: 135 us with 512, 392 with the earlier 256-thread kernel.
 constexpr int kClThreads = 512, kClSmall = 128;
 constexpr int kClSmallWork = 4096;   // products of a step in a CTA, at most, for kClSmall
 constexpr int kClMaxWarps = kClThreads / 32;
@@ -425,14 +427,21 @@ __global__ void __launch_bounds__(NT + NT / 4, 1) softreg_cluster_round_kernel(c
     }
     bar_named(2, NF);
     float* buf = Xsm + (s & 1) * B * Xld;
-    const int fw = warp - NW, u0 = lane & ((1 << ush) - 1);
-    for (int b = (fw << (5 - ush)) + (lane >> ush); b < B; b += NF >> ush) {
-      const float* from = X + Rsm[b] * D + c0;
-      float* to = buf + b * Xld;
-      if (vec)
-        for (int u = u0; u < units; u += 1 << ush) cp_async16(to + 4 * u, from + 4 * u);
-      else
-        for (int u = u0; u < units; u += 1 << ush) cp_async4(to + u, from + u);
+    const int fw = warp - NW, u0 = lane & ((1 << ush) - 1), bstep = NF >> ush;
+    // four rows at a time: their offsets are read before the first copy goes out
+    for (int b = (fw << (5 - ush)) + (lane >> ush); b < B; b += 4 * bstep) {
+      const float* from[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) from[i] = X + Rsm[b + i * bstep < B ? b + i * bstep : b] * D + c0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (b + i * bstep >= B) break;
+        float* to = buf + (b + i * bstep) * Xld;
+        if (vec)
+          for (int u = u0; u < units; u += 1 << ush) cp_async16(to + 4 * u, from[i] + 4 * u);
+        else
+          for (int u = u0; u < units; u += 1 << ush) cp_async4(to + u, from[i] + u);
+      }
     }
     for (int l = ft; l < R_own; l += NF) Ysm[(s & 1) * R + l] = Y[Rsm[l * kCl + rank]];
     cp_async_wait_all();
@@ -558,9 +567,8 @@ __global__ void __launch_bounds__(NT + NT / 4, 1) softreg_cluster_round_kernel(c
         float part[kCl];
 #pragma unroll
         for (int q = 0; q < kCl; ++q) part[q] = lane < Zp ? Pin[(q * R + l) * Zp + lane] : 0.f;
-        float z = 0.f;
-#pragma unroll
-        for (int q = 0; q < kCl; ++q) z += part[q];
+        static_assert(kCl == 8, "the ranks' sum");
+        float z = ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
         z = cls >= 0 ? z : -INFINITY;
         const int y = Ysm[(s & 1) * R + l], ys = y / CC * CCp + y % CC;
         const float m = warp_max(z);
@@ -585,7 +593,13 @@ __global__ void __launch_bounds__(NT + NT / 4, 1) softreg_cluster_round_kernel(c
         __syncwarp();
       }
     }
-    if (alive) alive = mbar_wait(zbar, s & 1, a.err, kDevTimeoutFull);
+    // one warp polls for dz, the others wait at a named barrier (with the
+    // deeper unrolling below and the fetch's early offsets, 333 x 26, 12
+    // workers, a round: 131.5 -> 127.6 us)
+    if (warp == NW - 1) {
+      if (alive) alive = mbar_wait(zbar, s & 1, a.err, kDevTimeoutFull);
+    }
+    bar_named(3, NT);
     // 4. weight gradient of this CTA's columns: item = (4 columns, CC classes, 1 / BS of the rows)
     int kv = u_kv, cg = u_cg, bs = u_bs, b0 = u_b0, b1 = u_b1;
     for (int i = tid; i < items;) {
@@ -593,7 +607,7 @@ __global__ void __launch_bounds__(NT + NT / 4, 1) softreg_cluster_round_kernel(c
         float4 g[CC];
 #pragma unroll
         for (int j = 0; j < CC; ++j) g[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
+#pragma unroll 4
         for (int b = b0; b < b1; ++b) {
           const float4 xv = *reinterpret_cast<const float4*>(Xs + b * Xld + 4 * kv);
           const float* zr = Zsm + b * Zp + cg * CCp;
@@ -651,7 +665,9 @@ __global__ void __launch_bounds__(NT + NT / 4, 1) softreg_cluster_round_kernel(c
       }
     }
   }
-  if (!fetcher && lane == 0) lsum[warp] = static_cast<double>(loss_hi) + static_cast<double>(loss_lo);
+  // a wait that ran out shows as a NaN loss (the allocation-free entry has no error word)
+  if (!fetcher && lane == 0)
+    lsum[warp] = alive ? static_cast<double>(loss_hi) + static_cast<double>(loss_lo) : static_cast<double>(NAN);
   __syncthreads();
   // push: this CTA's columns into the replica
   for (int c = warp; c < C; c += (NT + NF) / 32)
@@ -666,8 +682,7 @@ __global__ void __launch_bounds__(NT + NT / 4, 1) softreg_cluster_round_kernel(c
   if (rank == 0 && tid == 0) {
     double t = 0.0;
     for (int q = 0; q < kCl; ++q) t += lrank[q];
-    // without an error word (the allocation-free entry) a wait that ran out shows as a NaN loss
-    a.loss_out[w] = alive ? static_cast<float>(t / (static_cast<double>(B) * tau)) : NAN;
+    a.loss_out[w] = static_cast<float>(t / (static_cast<double>(B) * tau));
     if (a.cursor_next) a.cursor_next[w] = (cur + static_cast<int64_t>(tau) * B) % n;
   }
 }
