@@ -729,7 +729,7 @@ cudaError_t enqueue_step(oscars_ctx* c, int s, int na, const int* wid, const int
   if (head_tc_supported(h.H, h.B, h.C)) {
     h.pdl = c->profiling ? 0 : 1;
     ProfScope ps(c, "head_fused", st);
-    if ((e = launch_head_tc(c->mHeadIn, c->mHeadW, h, na, st)) != cudaSuccess) return e;
+    if ((e = launch_head_tc(c->mHeadIn, c->mHeadW, c->mGT[c->L - 2], h, na, st)) != cudaSuccess) return e;
   } else if (head_fused_supported(h.H, h.B, h.C)) {
     ProfScope ps(c, "head_fused", st);
     if ((e = launch_head_fused(h, na, st)) != cudaSuccess) return e;
@@ -1437,7 +1437,10 @@ oscars_status allocate_mlp(oscars_ctx* c) {
   }
   {
     const Layer& hl = c->layers.back();
-    if (!make_map(&c->mHeadIn, c->A[L - 1], hl.in, B, W, hl.in * 2ull, static_cast<uint64_t>(B) * hl.in * 2ull, 128) ||
+    // the head's input: h [lane][B][in], or h^T [lane][in][B] where G^T alone is written
+    const bool ht = !c->g_rows;
+    if (!make_map(&c->mHeadIn, ht ? c->AT[L - 1] : c->A[L - 1], ht ? B : hl.in, ht ? hl.in : B, W,
+                  (ht ? B : hl.in) * 2ull, static_cast<uint64_t>(B) * hl.in * 2ull, 128) ||
         !make_map(&c->mHeadW, c->shadow + hl.offW, hl.in, hl.out, slots64, hl.in * 2ull, c->P_pad * 2ull,
                   head_tc_class_rows(hl.out)))
       return fail(c, OSCARS_ECUDA, "cuTensorMapEncodeTiled failed (head)");

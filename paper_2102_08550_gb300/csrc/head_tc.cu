@@ -21,10 +21,17 @@
 //     the CTA's head columns;
 //  4. input gradient of the layer below, transposed: dh^T[f][b] = sum_c
 //     W2[c][f] dz[b][c] (per half M = 128 features, N = B, K = NC: the W2
-//     tile read MN-major); masked by h > 0; G^T rows from registers, the fp32 bias
-//     gradient per feature, and G rows through the h tile (overwritten in
-//     place with the bf16 input gradient, then written as full 16-byte
-//     chunks of each row).
+//     tile read MN-major); masked by h > 0; the fp32
+//     bias gradient per feature, and the bf16 gradient.
+// For B a multiple of 64, where the next kernels read only G^T, the tile in
+// shared memory is h^T (as in memory, [H][B]): the products read it MN-major
+// in 1 and K-major in 3, a thread finds the masks of 16 rows in two of its own
+// 16-byte chunks and leaves the gradient there, and TMA stores write G^T (with
+// the h tile, a thread reads 2-byte elements and stores 16-byte chunks of its
+// own row, 32 lines an instruction; mask bits read beforehand from the h tile
+// took 2700 clocks: 3072-1024-1024-10, a round: 1584 -> 1573 us).  For other B it is
+// the h tile [B][H]; G^T rows are written from registers, G rows through the
+// tile (overwritten in place, then written as full 16-byte chunks).
 // Rank 0 also writes the loss partials and updates the head bias.  One
 // thread issues the TMA loads and the MMAs; the accumulators share 128 NH
 // TMEM columns (the phases run one after another).  All mbarrier waits are
@@ -33,10 +40,15 @@
 //
 // NC is C rounded up to 16 or 32; C = 10 is also a template argument (CT), which
 // keeps the row softmax in as few registers and instructions as it needs.
-// Latency-bound: one launch here against a forward and a backward launch on
-// the CUDA cores for other class counts (17 and 12 us each with 17 classes,
-// 256 features, batch 32): a round of the 1000-384-256-17 model, 5 workers,
-// 534 -> 440 us.
+// Bound by latency and by instruction fetch: each launch runs its code once,
+// so the phases are short loops, not unrolled ones (a first pass over 32 rows
+// in phase 4 took 4500 clocks, the next ones 720), and one warp brings the
+// code in early (below).  One launch replaces a forward and a backward launch
+// on the CUDA cores for other class counts (17 and 12 us each with 17 classes,
+// 256 features, batch 32).  A round of the 1000-384-256-17 model, 5 workers:
+// 534 us with those, 440 with this kernel's first form, 335 now (374 before
+// the loops, the early code and the h^T tile); 3072-1024-1024-10, 32 workers:
+// 1579 -> 1573.
 #include "common.cuh"
 #include "internal.h"
 
@@ -110,28 +122,108 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, float (&v)[16
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// columns [c, c + 32) of the warp's 32 lanes as two 16-column loads under one wait
-__device__ __forceinline__ void tmem_ld_32x32b_x16x2(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%33];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=&r"(r[0]), "=&r"(r[1]), "=&r"(r[2]), "=&r"(r[3]), "=&r"(r[4]), "=&r"(r[5]), "=&r"(r[6]), "=&r"(r[7]),
-        "=&r"(r[8]), "=&r"(r[9]), "=&r"(r[10]), "=&r"(r[11]), "=&r"(r[12]), "=&r"(r[13]), "=&r"(r[14]), "=&r"(r[15]),
-        "=&r"(r[16]), "=&r"(r[17]), "=&r"(r[18]), "=&r"(r[19]), "=&r"(r[20]), "=&r"(r[21]), "=&r"(r[22]), "=&r"(r[23]),
-        "=&r"(r[24]), "=&r"(r[25]), "=&r"(r[26]), "=&r"(r[27]), "=&r"(r[28]), "=&r"(r[29]), "=&r"(r[30]), "=&r"(r[31])
-      : "r"(taddr), "r"(taddr + 16u)
-      : "memory");
+// Phase 2 with TPR = 1 << TSH threads per row (the whole block for B = 32, 64
+// and 128): thread q takes the 4-class chunks q, q + TPR, ...
+template <int NH, int NC, int CT, int TSH>
+__device__ __forceinline__ void head_softmax(const HeadArgs& a, uint8_t* sm, int t, int ncl) {
+  using Cfg = HTCfg<NH, NC>;
+  const float* pl = reinterpret_cast<const float*>(sm + Cfg::oPl);
+  const float* b2 = reinterpret_cast<const float*>(sm + Cfg::oB2);
+  const int* labs = reinterpret_cast<const int*>(sm + Cfg::oLab);
+  float* dz = reinterpret_cast<float*>(sm + Cfg::oDz);
+  float* rowloss = reinterpret_cast<float*>(sm + Cfg::oLoss);
+  uint8_t* dzT = sm + Cfg::oDzT;
+  uint8_t* dzK = sm + Cfg::oDzK;
+  const int B = a.B, C = CT > 0 ? CT : a.C;
+  constexpr int CL = CT > 0 ? CT : NC;   // class loops: compile-time bound, `c < C` inside
+  constexpr int tpr = 1 << TSH;
+  const int b = t >> TSH, q = t & (tpr - 1);
+  constexpr int QN = (CL + 3) / 4;      // chunks with classes
+  constexpr int QT = (QN + tpr - 1) / tpr;   // chunks of a thread at most
+  const bool row = b < B;
+  float z[4 * QT];
 #pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 4 * QT; ++i) z[i] = 0.f;
+  if (row) {
+    // four ranks' partials are requested before the first is added (a remote
+    // load waits a round trip across the cluster); NH = 1 has at most four
+#pragma unroll
+    for (int r0 = 0; r0 < (NH == 1 ? 4 : kHTMaxCluster); r0 += 4) {
+      float4 p[4][QT];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int i = 0; i < QT; ++i)
+          if (r0 + r < ncl && q + i * tpr < QN) p[r][i] = ld_dsmem_f32x4(pl + b * NC + 4 * (q + i * tpr), r0 + r);
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int i = 0; i < QT; ++i)
+          if (r0 + r < ncl && q + i * tpr < QN) {
+            z[4 * i] += p[r][i].x;
+            z[4 * i + 1] += p[r][i].y;
+            z[4 * i + 2] += p[r][i].z;
+            z[4 * i + 3] += p[r][i].w;
+          }
+    }
+  }
+  const int y = row ? labs[b] : 0;
+  float m = -INFINITY, zy = -INFINITY;
+#pragma unroll
+  for (int i = 0; i < 4 * QT; ++i) {
+    const int c = 4 * (q + i / 4 * tpr) + i % 4;
+    z[i] = c < C ? z[i] + b2[c < NC ? c : 0] : -INFINITY;
+    m = fmaxf(m, z[i]);
+    if (c == y) zy = z[i];
+  }
+  for (int o = tpr >> 1; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  float s = 0.f, so_ = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4 * QT; ++i) {
+    const int c = 4 * (q + i / 4 * tpr) + i % 4;
+    z[i] = c < C ? expf(z[i] - m) : 0.f;
+    s += z[i];
+    if (c != y) so_ += z[i];
+  }
+  for (int o = tpr >> 1; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    so_ += __shfl_xor_sync(0xffffffffu, so_, o);
+  }
+  const float inv = 1.0f / static_cast<float>(B);
+  if (row) {
+    if (q == ((y >> 2) & (tpr - 1))) rowloss[b] = m + logf(s) - zy;   // the thread that has class y
+    uint8_t* ck = dzK + (b >> 3) * (NC / 8 * 128) + (b & 7) * 16;
+    uint8_t* at = dzT + (b >> 6) * (NC * 128);
+    const int e64 = b & 63;
+#pragma unroll
+    for (int i = 0; i < QT; ++i) {
+      const int k = q + i * tpr;
+      if (k >= QN) continue;
+      float g[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = 4 * k + j;
+        g[j] = c < C ? (c == y ? -so_ : z[4 * i + j]) / s * inv : 0.f;
+      }
+      *reinterpret_cast<float4*>(dz + b * Cfg::kLdz + 4 * k) = make_float4(g[0], g[1], g[2], g[3]);
+      // dz as the K-major [rows][NC classes] operand: classes 8 j .. 8 j + 7
+      // one 16-byte chunk of core matrix (b / 8, j)
+      *reinterpret_cast<uint2*>(ck + 128 * (k >> 1) + 8 * (k & 1)) = make_uint2(pack_bf16x2(g[0], g[1]), pack_bf16x2(g[2], g[3]));
+      // dz^T as the K-major [NC classes][rows] operand (K = rows, atoms of 64 rows)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = 4 * k + j;
+        *reinterpret_cast<__nv_bfloat16*>(at + c * 128 + ((((e64 >> 3) ^ (c & 7)) & 7) << 4) + (e64 & 7) * 2) =
+            __float2bfloat16_rn(g[j]);
+      }
+    }
+  }
 }
 
 template <int NH, int NC, int CT>
 __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_constant__ CUtensorMap mH,
                                                               const __grid_constant__ CUtensorMap mW2,
+                                                              const __grid_constant__ CUtensorMap mGT,
                                                               const __grid_constant__ HeadArgs a) {
   using Cfg = HTCfg<NH, NC>;
   constexpr int F = Cfg::F;
@@ -169,286 +261,268 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
     mbar_init(mma_bar, 1);
     fence_barrier_init();
   }
-  pdl_wait();      // the layer input (the previous kernel's output) is complete
-  if (t == 0) {
-    // the h and W2 tiles, requested first: the rest of the prologue overlaps them
-    mbar_arrive_expect_tx(tma_bar, (F / 64) * (kHTRows * 128 + NC * 128));
-#pragma unroll
-    for (int q = 0; q < F / 64; ++q) {
-      tma_load_3d(hT + q * kHTRows * 128, &mH, k0 + 64 * q, 0, w, tma_bar);
-      tma_load_3d(w2 + q * NC * 128, &mW2, k0 + 64 * q, 0, src, tma_bar);
-    }
-  }
-  if (warp == 0) {
-    tmem_alloc(tmem_slot, Cfg::kTmemCols);
-    tmem_relinquish();
-  }
-  // the old master values of this thread's head column, requested long before
-  // the update needs them (and before any new value is stored: source and
-  // destination slots may be the same slab)
+  // B a multiple of 64: the tile is h^T [features][rows], boxes (half, 64 rows)
+  // of 128 features; otherwise h [rows][features], boxes of 64 features
+  const bool ht = !a.G;
+  const int hb = B >> 6;                 // h^T: boxes per half
+  bool ok = false;
+  uint32_t tmem = 0;
   float old[CL];
-  if (warp < 4 * NH) {
-    const int f = kHT * (warp >> 2) + 32 * (warp & 3) + lane;
+  const int e_mh = NH == 2 ? warp >> 2 : 0;                    // phases 3 and 4: this thread's half, feature and rows
+  const int e_fl = 32 * (warp & 3) + lane, e_f = kHT * e_mh + e_fl;
+  const int e_rows = NH == 2 ? B : B / 2, e_r0 = NH == 2 ? 0 : (warp >> 2) * e_rows;
+  // rows e_r0, e_r0 + 1, ... of the h tile (e_r0 is a multiple of 16) at this feature: see h_off
+  uint8_t* const h_col = hT + (e_f >> 6) * (kHTRows * 128) + e_r0 * 128 + (e_f & 7) * 2;
+  const int h_chunk = (e_f & 63) >> 3;
+  // While the previous kernel still runs, the last warp goes through the code
+  // of phases 2 to 4 once on whatever shared memory holds, without touching
+  // other memory, the cluster or the tensor core: it brings the instructions
+  // to the SM.  Each launch runs them once, and the weights that stream
+  // through L2 between two launches evict them (a round of
+  // 1000-384-256-17, 5 workers: 346 -> 338 us; 3072-1024-1024-10, 32: 1592 -> 1584).
+#pragma unroll 1
+  for (int dry = a.pdl && warp == kHTThreads / 32 - 1 ? 1 : 0; dry >= 0; --dry) {
+    if (!dry) {
+      __syncthreads();   // the dry pass has left the tiles
+      pdl_wait();      // the layer input (the previous kernel's output) is complete
+      if (t == 0) {
+        // the h and W2 tiles, requested first: the rest of the prologue overlaps them
+        mbar_arrive_expect_tx(tma_bar, (ht ? NH * hb : F / 64) * (kHTRows * 128) + (F / 64) * (NC * 128));
+        if (ht)
+          for (int q = 0; q < NH * hb; ++q)
+            tma_load_3d(hT + q * (kHT * 128), &mH, 64 * (q & (hb - 1)), k0 + kHT * (q / hb), w, tma_bar);
 #pragma unroll
-    for (int c = 0; c < CL; ++c)
-      if (c < C) old[c] = a.master[so + a.offW + static_cast<int64_t>(c) * H + k0 + f];
-  }
-  // the dz tiles' padding (classes >= C, rows >= B) stays zero
-  for (int q = t; q < (2 * NC * 128 + kHTRows * NC * 2) / 16; q += kHTThreads)
-    reinterpret_cast<uint4*>(dzT)[q] = make_uint4(0, 0, 0, 0);
-  for (int b = t; b < B; b += kHTThreads) labs[b] = a.labels[static_cast<int64_t>(w) * B + b];
-  if (t < NC) b2[t] = t < C ? a.master[so + a.offB + t] : 0.f;
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  pdl_trigger();
+        for (int q = 0; q < F / 64; ++q) {
+          if (!ht) tma_load_3d(hT + q * kHTRows * 128, &mH, k0 + 64 * q, 0, w, tma_bar);
+          tma_load_3d(w2 + q * NC * 128, &mW2, k0 + 64 * q, 0, src, tma_bar);
+        }
+      }
+      if (warp == 0) {
+        tmem_alloc(tmem_slot, Cfg::kTmemCols);
+        tmem_relinquish();
+      }
+      // the old master values of this thread's head column, requested long before
+      // the update needs them (and before any new value is stored: source and
+      // destination slots may be the same slab)
+      if (warp < 4 * NH) {
+        const int f = kHT * (warp >> 2) + 32 * (warp & 3) + lane;
+#pragma unroll
+        for (int c = 0; c < CL; ++c)
+          if (c < C) old[c] = a.master[so + a.offW + static_cast<int64_t>(c) * H + k0 + f];
+      }
+      // the dz tiles' padding (classes >= C, rows >= B) stays zero
+      for (int q = t; q < (2 * NC * 128 + kHTRows * NC * 2) / 16; q += kHTThreads)
+        reinterpret_cast<uint4*>(dzT)[q] = make_uint4(0, 0, 0, 0);
+      for (int b = t; b < B; b += kHTThreads) labs[b] = a.labels[static_cast<int64_t>(w) * B + b];
+      if (t < NC) b2[t] = t < C ? a.master[so + a.offB + t] : 0.f;
+      tc_fence_before();
+      __syncthreads();
+      tc_fence_after();
+      tmem = *tmem_slot;
+      pdl_trigger();
 
-  // ---- 1. partial logits
-  if (warp == 0) {   // converged, one elected lane issues: see elect_one
-    const bool landed = mbar_wait(tma_bar, 0, a.err, kDevTimeoutFull);
-    tc_fence_after();
-    constexpr uint32_t idesc = idesc_bf16_f32(kHTRows, NC);
-    const uint64_t hd = smem_desc_k128(smem_u32(hT)), wd = smem_desc_k128(smem_u32(w2));   // addresses in 16 bytes
-    if (elect_one()) {
-      if (landed)
+      // ---- 1. partial logits
+      if (warp == 0) {   // converged, one elected lane issues: see elect_one
+        const bool landed = mbar_wait(tma_bar, 0, a.err, kDevTimeoutFull);
+        tc_fence_after();
+        // A = h: MN-major from the h^T tile (rows >= B are whatever follows it; their
+        // logits are not used), K-major from the h tile
+        const uint32_t idesc = idesc_bf16_f32(kHTRows, NC) | (ht ? 1u << 15 : 0u);
+        const uint64_t hd = ht ? smem_desc_mn128(smem_u32(hT), kHT * 128) : smem_desc_k128(smem_u32(hT));
+        const uint64_t wd = smem_desc_k128(smem_u32(w2));   // addresses in 16 bytes
+        const uint32_t jstep = ht ? 128 : 2, ostep = ht ? 512 : kHTRows * 128 / 16, hstep = ht ? hb * 1024 : 2 * 1024;
+        if (elect_one()) {
+          if (landed)
 #pragma unroll
-        for (int kb = 0; kb < F / 64; ++kb)
+            for (int kb = 0; kb < F / 64; ++kb)
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            umma_bf16(tmem, hd + kb * (kHTRows * 128 / 16) + 2 * j, wd + kb * (NC * 128 / 16) + 2 * j, idesc,
-                      (kb | j) != 0 ? 1u : 0u);
-      umma_commit(mma_bar);   // arrives even with nothing issued, so the waits below end
+              for (int j = 0; j < 4; ++j)
+                umma_bf16(tmem, hd + (kb >> 1) * hstep + (kb & 1) * ostep + j * jstep, wd + kb * (NC * 128 / 16) + 2 * j,
+                          idesc, (kb | j) != 0 ? 1u : 0u);
+          umma_commit(mma_bar);   // arrives even with nothing issued, so the waits below end
+        }
+        __syncwarp();
+      }
+      ok = mbar_wait(mma_bar, 0, a.err, kDevTimeoutAccum);
+      tc_fence_after();
+      if (warp < 4) {
+        float v[NC];
+        if constexpr (NC == 16) tmem_ld_32x32b_x16(tmem + (static_cast<uint32_t>(32 * warp) << 16), v);
+        else tmem_ld_32x32b_x32(tmem + (static_cast<uint32_t>(32 * warp) << 16), v);
+        float4* row = reinterpret_cast<float4*>(pl + (32 * warp + lane) * NC);
+#pragma unroll
+        for (int q = 0; q < NC / 4; ++q) row[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      }
+      tc_fence_before();
+      cluster_sync();
+      tc_fence_after();
+
     }
-    __syncwarp();
-  }
-  bool ok = mbar_wait(mma_bar, 0, a.err, kDevTimeoutAccum);
-  tc_fence_after();
-  if (warp < 4) {
-    float v[NC];
-    if constexpr (NC == 16) tmem_ld_32x32b_x16(tmem + (static_cast<uint32_t>(32 * warp) << 16), v);
-    else tmem_ld_32x32b_x32(tmem + (static_cast<uint32_t>(32 * warp) << 16), v);
-    float4* row = reinterpret_cast<float4*>(pl + (32 * warp + lane) * NC);
-#pragma unroll
-    for (int q = 0; q < NC / 4; ++q) row[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-  }
-  tc_fence_before();
-  cluster_sync();
-  tc_fence_after();
 
-  // ---- 2. logits (cluster sum in rank order), softmax cross-entropy, dz tiles.
-  // TPR threads per row (the whole block for B = 32, 64 and 128), thread q
-  // takes the 4-class chunks q, q + TPR, ...
-  {
-    const int tsh = B <= 32 ? 3 : B <= 64 ? 2 : 1, tpr = 1 << tsh;   // 8, 4 or 2
-    const int b = t >> tsh, q = t & (tpr - 1);
-    constexpr int QN = (CL + 3) / 4;      // chunks with classes
-    constexpr int QT = (QN + 1) / 2;      // chunks of a thread at most (two threads a row)
-    const bool row = b < B;
-    float z[4 * QT];
+    // ---- 2. logits (cluster sum in rank order), softmax cross-entropy, dz tiles.
+    // 8, 4 or 2 threads a row, each count its own code: chunks that no thread
+    // of a count has cost their instructions' fetch (17 classes,
+    // batch 32: this phase 5000 -> 2300 clocks)
+    if (B <= 32) head_softmax<NH, NC, CT, 3>(a, sm, dry ? lane : t, dry ? 0 : ncl);
+    else if (B <= 64) head_softmax<NH, NC, CT, 2>(a, sm, dry ? lane : t, dry ? 0 : ncl);
+    else head_softmax<NH, NC, CT, 1>(a, sm, dry ? lane : t, dry ? 0 : ncl);
+    if (!dry) {
+      fence_proxy_async_smem();   // the dz tiles are read by the tensor core
+      tc_fence_before();
+      __syncthreads();
+      tc_fence_after();
+
+      // ---- 3. head weight gradient (M = features, N = classes, K = rows) + SGD
+      if (warp == 0) {
+        // A = h^T: K-major from the h^T tile, MN-major from the h tile
+        const uint32_t idesc = idesc_bf16_f32(kHT, NC) | (ht ? 0u : 1u << 15);
+        const uint64_t hd = ht ? smem_desc_k128(smem_u32(hT)) : smem_desc_mn128(smem_u32(hT), kHTRows * 128);
+        const uint64_t zd = smem_desc_k128(smem_u32(dzT));
+        const uint32_t jstep = ht ? 2 : 128, qstep = ht ? 1024 : 512, hstep = ht ? hb * 1024 : 2 * 1024;
+        if (elect_one()) {
+          if (ok)
 #pragma unroll
-    for (int i = 0; i < 4 * QT; ++i) z[i] = 0.f;
-    if (row) {
-      // the ranks' partials are requested before the first is added (a remote
-      // load waits a round trip across the cluster)
-      float4 p[kHTMaxCluster][QT];
+            for (int mh = 0; mh < NH; ++mh)   // half mh: features [128 mh, 128 mh + 128) into columns [NC mh, NC mh + NC)
+              for (int j = 0; j < B / 16; ++j)
+                umma_bf16(tmem + NC * mh, hd + mh * hstep + (j >> 2) * qstep + (j & 3) * jstep,
+                          zd + (j >> 2) * (NC * 128 / 16) + 2 * (j & 3), idesc, j != 0 ? 1u : 0u);
+          umma_commit(mma_bar);
+        }
+        __syncwarp();
+      }
+      if (rank == 0 && warp >= 4) {   // loss partials and the head bias (CUDA cores, meanwhile)
+        const int u = t - 128;
+        if (u < B / kRowsPerLossChunk) {
+          float l = 0.f;
+          for (int r = 0; r < kRowsPerLossChunk; ++r) l += rowloss[u * kRowsPerLossChunk + r];
+          const int64_t row = static_cast<int64_t>(w) * a.part_mul + a.part_add;
+          a.loss_part[row * (B / kRowsPerLossChunk) + u] = l;
+        }
+        if (u >= 32) {   // warps 5-7: 8 lanes per class (12 classes a pass), then shuffles within each group of 8
+          const int j = u & 7;
+          for (int c0 = 0; c0 < C; c0 += 12) {
+            const int c = c0 + ((u - 32) >> 3);
+            float g = 0.f;
+            if (c < C)
+              for (int b = j; b < B; b += 8) g += dz[b * Cfg::kLdz + c];
 #pragma unroll
-      for (int r = 0; r < kHTMaxCluster; ++r)
-#pragma unroll
-        for (int i = 0; i < QT; ++i)
-          if (r < ncl && q + i * tpr < QN) p[r][i] = ld_dsmem_f32x4(pl + b * NC + 4 * (q + i * tpr), r);
-#pragma unroll
-      for (int r = 0; r < kHTMaxCluster; ++r)
-#pragma unroll
-        for (int i = 0; i < QT; ++i)
-          if (r < ncl && q + i * tpr < QN) {
-            z[4 * i] += p[r][i].x;
-            z[4 * i + 1] += p[r][i].y;
-            z[4 * i + 2] += p[r][i].z;
-            z[4 * i + 3] += p[r][i].w;
+            for (int o = 4; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o, 8);
+            if (c < C && j == 0) a.master_w[dof + a.offB + c] = fmaf(-a.lr, g, a.master[so + a.offB + c]);
           }
-    }
-    const int y = row ? labs[b] : 0;
-    float m = -INFINITY, zy = -INFINITY;
-#pragma unroll
-    for (int i = 0; i < 4 * QT; ++i) {
-      const int c = 4 * (q + i / 4 * tpr) + i % 4;
-      z[i] = c < C ? z[i] + b2[c < NC ? c : 0] : -INFINITY;
-      m = fmaxf(m, z[i]);
-      if (c == y) zy = z[i];
-    }
-    for (int o = tpr >> 1; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    float s = 0.f, so_ = 0.f;
-#pragma unroll
-    for (int i = 0; i < 4 * QT; ++i) {
-      const int c = 4 * (q + i / 4 * tpr) + i % 4;
-      z[i] = c < C ? expf(z[i] - m) : 0.f;
-      s += z[i];
-      if (c != y) so_ += z[i];
-    }
-    for (int o = tpr >> 1; o > 0; o >>= 1) {
-      s += __shfl_xor_sync(0xffffffffu, s, o);
-      so_ += __shfl_xor_sync(0xffffffffu, so_, o);
-    }
-    const float inv = 1.0f / static_cast<float>(B);
-    if (row) {
-      if (q == ((y >> 2) & (tpr - 1))) rowloss[b] = m + logf(s) - zy;   // the thread that has class y
-      uint8_t* ck = dzK + (b >> 3) * (NC / 8 * 128) + (b & 7) * 16;
-      uint8_t* at = dzT + (b >> 6) * (NC * 128);
-      const int e64 = b & 63;
-#pragma unroll
-      for (int i = 0; i < QT; ++i) {
-        const int k = q + i * tpr;
-        if (k >= QN) continue;
-        float g[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int c = 4 * k + j;
-          g[j] = c < C ? (c == y ? -so_ : z[4 * i + j]) / s * inv : 0.f;
-        }
-        *reinterpret_cast<float4*>(dz + b * Cfg::kLdz + 4 * k) = make_float4(g[0], g[1], g[2], g[3]);
-        // dz as the K-major [rows][NC classes] operand: classes 8 j .. 8 j + 7
-        // one 16-byte chunk of core matrix (b / 8, j)
-        *reinterpret_cast<uint2*>(ck + 128 * (k >> 1) + 8 * (k & 1)) = make_uint2(pack_bf16x2(g[0], g[1]), pack_bf16x2(g[2], g[3]));
-        // dz^T as the K-major [NC classes][rows] operand (K = rows, atoms of 64 rows)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int c = 4 * k + j;
-          *reinterpret_cast<__nv_bfloat16*>(at + c * 128 + ((((e64 >> 3) ^ (c & 7)) & 7) << 4) + (e64 & 7) * 2) =
-              __float2bfloat16_rn(g[j]);
         }
       }
-    }
-  }
-  fence_proxy_async_smem();   // the dz tiles are read by the tensor core
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-
-  // ---- 3. head weight gradient (M = features, N = classes, K = rows) + SGD
-  if (warp == 0) {
-    constexpr uint32_t idesc = idesc_bf16_f32(kHT, NC) | (1u << 15);   // A (h^T) MN-major
-    const uint64_t hd = smem_desc_mn128(smem_u32(hT), kHTRows * 128), zd = smem_desc_k128(smem_u32(dzT));
-    if (elect_one()) {
-      if (ok)
+      ok = mbar_wait(mma_bar, 1, a.err, kDevTimeoutAccum) && ok;
+      tc_fence_after();
+      if (warp < 4 * NH && ok) {
+        const int mh = warp >> 2, q = warp & 3;
+        const int f = kHT * mh + 32 * q + lane;
+        float v[NC];
+        if constexpr (NC == 16) tmem_ld_32x32b_x16(tmem + NC * mh + (static_cast<uint32_t>(32 * q) << 16), v);
+        else tmem_ld_32x32b_x32(tmem + NC * mh + (static_cast<uint32_t>(32 * q) << 16), v);
 #pragma unroll
-        for (int mh = 0; mh < NH; ++mh)   // half mh: features [128 mh, 128 mh + 128) into columns [NC mh, NC mh + NC)
-          for (int j = 0; j < B / 16; ++j)
-            umma_bf16(tmem + NC * mh, hd + mh * (2 * kHTRows * 128 / 16) + 128 * j,
-                      zd + (j >> 2) * (NC * 128 / 16) + 2 * (j & 3), idesc, j != 0 ? 1u : 0u);
-      umma_commit(mma_bar);
-    }
-    __syncwarp();
-  }
-  if (rank == 0 && warp >= 4) {   // loss partials and the head bias (CUDA cores, meanwhile)
-    const int u = t - 128;
-    if (u < B / kRowsPerLossChunk) {
-      float l = 0.f;
-      for (int r = 0; r < kRowsPerLossChunk; ++r) l += rowloss[u * kRowsPerLossChunk + r];
-      const int64_t row = static_cast<int64_t>(w) * a.part_mul + a.part_add;
-      a.loss_part[row * (B / kRowsPerLossChunk) + u] = l;
-    }
-    if (u >= 32) {   // warps 5-7: 8 lanes per class (12 classes a pass), then shuffles within each group of 8
-      const int j = u & 7;
-      for (int c0 = 0; c0 < C; c0 += 12) {
-        const int c = c0 + ((u - 32) >> 3);
-        float g = 0.f;
-        if (c < C)
-          for (int b = j; b < B; b += 8) g += dz[b * Cfg::kLdz + c];
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o, 8);
-        if (c < C && j == 0) a.master_w[dof + a.offB + c] = fmaf(-a.lr, g, a.master[so + a.offB + c]);
-      }
-    }
-  }
-  ok = mbar_wait(mma_bar, 1, a.err, kDevTimeoutAccum) && ok;
-  tc_fence_after();
-  if (warp < 4 * NH && ok) {
-    const int mh = warp >> 2, q = warp & 3;
-    const int f = kHT * mh + 32 * q + lane;
-    float v[NC];
-    if constexpr (NC == 16) tmem_ld_32x32b_x16(tmem + NC * mh + (static_cast<uint32_t>(32 * q) << 16), v);
-    else tmem_ld_32x32b_x32(tmem + NC * mh + (static_cast<uint32_t>(32 * q) << 16), v);
-#pragma unroll
-    for (int c = 0; c < CL; ++c) {
-      if (c >= C) continue;
-      const int64_t e = a.offW + static_cast<int64_t>(c) * H + k0 + f;
-      const float nw = fmaf(-a.lr, v[c], old[c]);
-      a.master_w[dof + e] = nw;
-      a.shadow_w[dof + e] = __float2bfloat16_rn(nw);
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-
-  // ---- 4. input gradient, transposed (M = features, N = rows, K = NC classes)
-  if (warp == 0) {
-    const uint32_t idesc = idesc_bf16_f32(kHT, B) | (1u << 15);   // A (W2^T) MN-major
-    const uint64_t wd = smem_desc_mn128(smem_u32(w2), NC * 128), kd = smem_desc_none(smem_u32(dzK), 128, NC / 8 * 128);
-    if (elect_one()) {
-      if (ok)
-#pragma unroll
-        for (int mh = 0; mh < NH; ++mh)   // half mh into columns [B mh, B mh + B)
-#pragma unroll
-          for (int j = 0; j < NC / 16; ++j)   // 16 classes: 16 rows of the W2 tile, two core matrices of dz
-            umma_bf16(tmem + B * mh, wd + mh * (2 * NC * 128 / 16) + 128 * j, kd + 16 * j, idesc, j != 0 ? 1u : 0u);
-      umma_commit(mma_bar);
-    }
-    __syncwarp();
-  }
-  ok = mbar_wait(mma_bar, 0, a.err, kDevTimeoutAccum) && ok;
-  tc_fence_after();
-  {
-    // warp quarter q: features 32 q .. of its half; NH = 1: the two warp
-    // groups split the rows; NH = 2: warp group g takes half g, all rows
-    const int q = warp & 3, g = warp >> 2;
-    const int mh = NH == 2 ? g : 0;
-    const int f = kHT * mh + 32 * q + lane;
-    const int rows = NH == 2 ? B : B / 2;
-    const int r0 = NH == 2 ? 0 : g * rows;
-    float gsum = 0.f;
-    if (ok) {
-      for (int c0 = 0; c0 < rows; c0 += 32) {   // rows is a multiple of 16; a 32-row pass when it fits
-        const int b0 = r0 + c0;
-        const int nr = rows - c0 >= 32 ? 32 : 16;
-        float v[32];
-        const uint32_t ta = tmem + static_cast<uint32_t>(B * mh + b0) + (static_cast<uint32_t>(32 * q) << 16);
-        if (nr == 32) {
-          tmem_ld_32x32b_x16x2(ta, v);
-        } else {
-          float h16[16];
-          tmem_ld_32x32b_x16(ta, h16);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] = h16[j];
+        for (int c = 0; c < CL; ++c) {
+          if (c >= C) continue;
+          const int64_t e = a.offW + static_cast<int64_t>(c) * H + k0 + f;
+          const float nw = fmaf(-a.lr, v[c], old[c]);
+          a.master_w[dof + e] = nw;
+          a.shadow_w[dof + e] = __float2bfloat16_rn(nw);
         }
-        uint32_t pk[16];
+      }
+      tc_fence_before();
+      __syncthreads();
+      tc_fence_after();
+
+      // ---- 4. input gradient, transposed (M = features, N = rows, K = NC classes)
+      if (warp == 0) {
+        const uint32_t idesc = idesc_bf16_f32(kHT, B) | (1u << 15);   // A (W2^T) MN-major
+        const uint64_t wd = smem_desc_mn128(smem_u32(w2), NC * 128), kd = smem_desc_none(smem_u32(dzK), 128, NC / 8 * 128);
+        if (elect_one()) {
+          if (ok)
 #pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-          if (j >= nr) break;
-          __nv_bfloat16* h0 = reinterpret_cast<__nv_bfloat16*>(hT + h_off(b0 + j, f));
-          __nv_bfloat16* h1 = reinterpret_cast<__nv_bfloat16*>(hT + h_off(b0 + j + 1, f));
-          const float d0 = __bfloat162float(*h0) > 0.f ? v[j] : 0.f;
-          const float d1 = __bfloat162float(*h1) > 0.f ? v[j + 1] : 0.f;
-          gsum += d0;
-          gsum += d1;
-          const __nv_bfloat162 p = __floats2bfloat162_rn(d0, d1);
-          if (a.G) {      // the h tile now holds the bf16 input gradient at (b, f), for the G rows below
-            *h0 = p.x;
-            *h1 = p.y;
+            for (int mh = 0; mh < NH; ++mh)   // half mh into columns [B mh, B mh + B)
+#pragma unroll
+              for (int j = 0; j < NC / 16; ++j)   // 16 classes: 16 rows of the W2 tile, two core matrices of dz
+                umma_bf16(tmem + B * mh, wd + mh * (2 * NC * 128 / 16) + 128 * j, kd + 16 * j, idesc, j != 0 ? 1u : 0u);
+          umma_commit(mma_bar);
+        }
+        __syncwarp();
+      }
+      ok = mbar_wait(mma_bar, 0, a.err, kDevTimeoutAccum) && ok;
+      mbar_wait(tma_bar, 0, a.err, kDevTimeoutFull);   // completed long ago: orders the tile reads below
+      tc_fence_after();
+    }
+    {
+      // warp quarter q: features 32 q .. of its half; NH = 1: the two warp
+      // groups split the rows; NH = 2: warp group g takes half g, all rows
+      const int g = warp >> 2;
+      const uint32_t tq = tmem + static_cast<uint32_t>(B * e_mh + e_r0) + (static_cast<uint32_t>(32 * (warp & 3)) << 16);
+      const int together = NH == 1 && B == 64 ? 256 : 128;   // threads that fill one tile
+      float gsum = 0.f;
+#pragma unroll 1
+      for (int r = 0; r < (dry ? 16 : e_rows); r += 16) {
+        const int b0 = e_r0 + r;
+        if (ok || dry) {
+          float v[16];
+          if (!dry) tmem_ld_32x32b_x16(tq + r, v);
+          else
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] = 0.f;
+          // the ReLU mask, and the bf16 gradient in its place: the thread's two
+          // 16-byte chunks of the h^T tile, or its 16 elements of the h tile
+          uint4* c0 = reinterpret_cast<uint4*>(hT + (e_mh * hb + (b0 >> 6)) * (kHT * 128) + e_fl * 128 +
+                                               ((((b0 & 63) >> 3) ^ (e_fl & 7)) << 4));
+          uint4* c1 = reinterpret_cast<uint4*>(reinterpret_cast<uintptr_t>(c0) ^ 16);
+          uint32_t pk[8];
+          if (ht) {
+            const uint4 x = *c0, y = *c1;
+            pk[0] = x.x; pk[1] = x.y; pk[2] = x.z; pk[3] = x.w;
+            pk[4] = y.x; pk[5] = y.y; pk[6] = y.z; pk[7] = y.w;
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; j += 2) {
+              const uint32_t lo = *reinterpret_cast<const unsigned short*>(h_col + (r + j) * 128 + ((h_chunk ^ (j & 7)) << 4));
+              const uint32_t hi =
+                  *reinterpret_cast<const unsigned short*>(h_col + (r + j + 1) * 128 + ((h_chunk ^ ((j + 1) & 7)) << 4));
+              pk[j >> 1] = lo | hi << 16;
+            }
           }
-          pk[j >> 1] = *reinterpret_cast<const uint32_t*>(&p);
+#pragma unroll
+          for (int j = 0; j < 16; j += 2) {
+            const uint32_t h2 = pk[j >> 1];
+            const float d0 = __uint_as_float(h2 << 16) > 0.f ? v[j] : 0.f;
+            const float d1 = __uint_as_float(h2 & 0xffff0000u) > 0.f ? v[j + 1] : 0.f;
+            gsum += d0;
+            gsum += d1;
+            pk[j >> 1] = pack_bf16x2(d0, d1);
+          }
+          if (ht) {
+            *c0 = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            *c1 = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+          } else {   // for the G rows below; the G^T rows from registers
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              *reinterpret_cast<unsigned short*>(h_col + (r + j) * 128 + ((h_chunk ^ (j & 7)) << 4)) =
+                  static_cast<unsigned short>(pk[j >> 1] >> (16 * (j & 1)));
+            if (dry) continue;
+            uint4* gt = reinterpret_cast<uint4*>(a.GT + (static_cast<int64_t>(w) * H + k0 + e_f) * B + b0);
+            gt[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            gt[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+          }
         }
-        uint4* gt = reinterpret_cast<uint4*>(a.GT + (static_cast<int64_t>(w) * H + k0 + f) * B + b0);
-        gt[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-        gt[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-        if (nr == 32) {
-          gt[2] = make_uint4(pk[8], pk[9], pk[10], pk[11]);
-          gt[3] = make_uint4(pk[12], pk[13], pk[14], pk[15]);
+        if (!dry && ht && (together == 256 ? r + 16 == e_rows : (b0 & 48) == 48)) {   // 64 rows are complete: one TMA store
+          fence_proxy_async_smem();
+          if (together == 256) bar_named(1, 256);
+          else if (g == 0) bar_named(1, 128);
+          else bar_named(2, 128);
+          if (ok && lane == 0 && warp == (together == 256 ? 0 : 4 * g)) {
+            tma_store_3d(&mGT, hT + (e_mh * hb + (b0 >> 6)) * (kHT * 128), b0 & ~63, k0 + kHT * e_mh, w);
+            bulk_commit_group();
+          }
         }
       }
+      gbp[(NH == 2 ? 0 : g) * F + e_f] = gsum;
     }
-    gbp[(NH == 2 ? 0 : g) * F + f] = gsum;
+    if (dry) fence_proxy_async_smem();   // its writes of the h tile's place, before the TMA load
   }
   tc_fence_before();
   __syncthreads();
@@ -460,6 +534,7 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
           *reinterpret_cast<const uint4*>(hT + h_off(b, 8 * j));
     }
   }
+  if (ht && lane == 0 && (warp & 3) == 0) bulk_wait_all();
   cluster_sync();   // no CTA leaves while another may still read its partial logits
   if (warp == 0) {
     tc_fence_after();
@@ -482,8 +557,8 @@ int head_tc_class_rows(int C) { return C <= 16 ? 16 : 32; }
 
 namespace {
 template <int NH, int NC, int CT>
-cudaError_t launch_head_tc_nh(const CUtensorMap& mH, const CUtensorMap& mW2, const HeadArgs& a, int n_active,
-                              cudaStream_t s) {
+cudaError_t launch_head_tc_nh(const CUtensorMap& mH, const CUtensorMap& mW2, const CUtensorMap& mGT,
+                              const HeadArgs& a, int n_active, cudaStream_t s) {
   using Cfg = HTCfg<NH, NC>;
   cudaError_t e = cudaFuncSetAttribute(head_tc_kernel<NH, NC, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem);
   if (e != cudaSuccess) return e;
@@ -501,23 +576,23 @@ cudaError_t launch_head_tc_nh(const CUtensorMap& mH, const CUtensorMap& mW2, con
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = a.pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, head_tc_kernel<NH, NC, CT>, mH, mW2, a);
+  return cudaLaunchKernelEx(&cfg, head_tc_kernel<NH, NC, CT>, mH, mW2, mGT, a);
 }
 
 template <int NH>
-cudaError_t launch_head_tc_c(const CUtensorMap& mH, const CUtensorMap& mW2, const HeadArgs& a, int n_active,
-                             cudaStream_t s) {
-  return a.C == 10   ? launch_head_tc_nh<NH, 16, 10>(mH, mW2, a, n_active, s)
-         : a.C <= 16 ? launch_head_tc_nh<NH, 16, 0>(mH, mW2, a, n_active, s)
-                     : launch_head_tc_nh<NH, 32, 0>(mH, mW2, a, n_active, s);
+cudaError_t launch_head_tc_c(const CUtensorMap& mH, const CUtensorMap& mW2, const CUtensorMap& mGT,
+                             const HeadArgs& a, int n_active, cudaStream_t s) {
+  return a.C == 10   ? launch_head_tc_nh<NH, 16, 10>(mH, mW2, mGT, a, n_active, s)
+         : a.C <= 16 ? launch_head_tc_nh<NH, 16, 0>(mH, mW2, mGT, a, n_active, s)
+                     : launch_head_tc_nh<NH, 32, 0>(mH, mW2, mGT, a, n_active, s);
 }
 }  // namespace
 
-cudaError_t launch_head_tc(const CUtensorMap& mH, const CUtensorMap& mW2, const HeadArgs& a, int n_active,
-                           cudaStream_t s) {
-  if (!head_tc_supported(a.H, a.B, a.C)) return cudaErrorInvalidValue;
-  return head_tc_halves(a.H) == 2 ? launch_head_tc_c<2>(mH, mW2, a, n_active, s)
-                                  : launch_head_tc_c<1>(mH, mW2, a, n_active, s);
+cudaError_t launch_head_tc(const CUtensorMap& mH, const CUtensorMap& mW2, const CUtensorMap& mGT,
+                           const HeadArgs& a, int n_active, cudaStream_t s) {
+  if (!head_tc_supported(a.H, a.B, a.C) || (!a.G && a.B % 64 != 0)) return cudaErrorInvalidValue;
+  return head_tc_halves(a.H) == 2 ? launch_head_tc_c<2>(mH, mW2, mGT, a, n_active, s)
+                                  : launch_head_tc_c<1>(mH, mW2, mGT, a, n_active, s);
 }
 
 }  // namespace oscars

@@ -247,13 +247,15 @@ struct HeadArgs {
 cudaError_t launch_head_fwd(const HeadArgs& a, int n_active, cudaStream_t s);
 // forward + backward of the last layer on the tensor cores (csrc/head_tc.cu):
 // one cluster of H/128 CTAs per active lane; 2 <= C <= 32, 32 <= B <= 128.
-// mH: the layer input [lane][B][H] bf16, box {64, 128}; mW2: the head weights
-// of every slot [slot][C][H] bf16, box {64, head_tc_class_rows(C)}; both with
-// 128-byte swizzle.
+// mH: the layer input [lane][B][H] bf16 (its transpose [lane][H][B] when a.G
+// is null), box {64, 128}; mW2: the head weights
+// of every slot [slot][C][H] bf16, box {64, head_tc_class_rows(C)}; mGT: the
+// input gradient^T [lane][H][B] bf16 (a.GT), box {64, 128}, written through
+// when a.G is null (B a multiple of 64); all with 128-byte swizzle.
 int head_tc_class_rows(int C);
 bool head_tc_supported(int H, int B, int C);
-cudaError_t launch_head_tc(const CUtensorMap& mH, const CUtensorMap& mW2, const HeadArgs& a, int n_active,
-                           cudaStream_t s);
+cudaError_t launch_head_tc(const CUtensorMap& mH, const CUtensorMap& mW2, const CUtensorMap& mGT,
+                           const HeadArgs& a, int n_active, cudaStream_t s);
 // forward + backward of the last layer in one launch: one cluster of H/128
 // CTAs per active lane (H <= 1024); false if the shape needs the two-kernel path
 bool head_fused_supported(int H, int B, int C);
