@@ -106,8 +106,9 @@ __device__ __forceinline__ float epi_dh(const GemmArgs& a, int wid, int m, int n
 // that owns them (rows [r 128 / SPLIT, (r + 1) 128 / SPLIT) belong to CTA r)
 // through distributed shared memory, one cluster barrier follows, and each
 // owner sums the SPLIT partials in rank order and runs the epilogue on its
-// rows.  Used when a launch has too few tiles to fill the GPU (the tail of a
-// round, where one worker with many local steps runs alone).
+// rows.  Used when a launch has too few tiles to fill the GPU: small layers,
+// and the tail of a round, where one worker with many local steps runs alone
+// (split_for).
 constexpr int kRedLd = 4;   // padding of a partial row (floats)
 
 __device__ __forceinline__ void st_dsmem_f32x4(float* local, uint32_t rank, float4 v) {
@@ -401,9 +402,15 @@ cudaError_t launch_tile(const CUtensorMap& mA, const CUtensorMap& mB, const Gemm
   return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, EPI, SPLIT>, mA, mB, a, stages);
 }
 
-// K split of a forward or input-gradient launch: 4 or 2 CTAs per tile when
-// the unsplit grid would leave most of the GPU idle and each CTA keeps at
-// least 4 K-blocks
+// K split of a forward or input-gradient launch of up to 128 samples: 4 or 2
+// CTAs per tile when the unsplit grid would leave most of the GPU idle (one SM
+// takes in about 60 bytes a clock: by that, K = 1000 at 32 samples is 5000
+// clocks) and each CTA keeps at least 4 K-blocks.  Rounds of
+// 1000-384-256-17, batch 32, 5 workers, and 3072-1024-1024-10, batch 128, 32
+// workers: 336.7 and 1574 us without a split below 128 samples, 316.9 and 1573
+// with this rule (one run); 318.5 and 1580 with this rule, 328.3 and 1581 with
+// 2 K-blocks a CTA, 327.4 and 1592 with that and 8 CTAs from 16 K-blocks
+// (another).
 int split_for(int M, int N, int BN, int K, int n_active) {
   const long long tiles = static_cast<long long>(M / BM) * ((N + BN - 1) / BN) * n_active;
   const int nk = (K + BK - 1) / BK;
@@ -411,6 +418,27 @@ int split_for(int M, int N, int BN, int K, int n_active) {
   if (tiles * 4 <= sms && nk >= 16) return 4;
   if (tiles * 2 <= sms && nk >= 8) return 2;
   return 1;
+}
+
+template <int BN, int EPI>
+cudaError_t launch_split(const CUtensorMap& mA, const CUtensorMap& mB, const GemmArgs& a, int n_active, cudaStream_t s) {
+  switch (split_for(a.M, a.N, BN, a.K, n_active)) {
+    case 4: return launch_tile<BN, EPI, 4>(mA, mB, a, n_active, s);
+    case 2: return launch_tile<BN, EPI, 2>(mA, mB, a, n_active, s);
+    default: return launch_tile<BN, EPI>(mA, mB, a, n_active, s);
+  }
+}
+
+template <int EPI>
+cudaError_t launch_epi(int bn, const CUtensorMap& mA, const CUtensorMap& mB, const GemmArgs& a, int n_active,
+                       cudaStream_t s) {
+  switch (bn) {
+    case 32: return launch_split<32, EPI>(mA, mB, a, n_active, s);
+    case 64: return launch_split<64, EPI>(mA, mB, a, n_active, s);
+    case 128: return launch_split<128, EPI>(mA, mB, a, n_active, s);
+    case 256: return launch_tile<256, EPI>(mA, mB, a, n_active, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 }  // namespace
@@ -423,27 +451,7 @@ cudaError_t launch_gemm(int epi, const CUtensorMap& mA, const CUtensorMap& mB, c
                         int n_active, cudaStream_t s) {
   if (a.M % BM != 0) return cudaErrorInvalidValue;
   const int bn = gemm_bn_for(epi, a.N);
-  const int split = bn == 128 ? split_for(a.M, a.N, bn, a.K, n_active) : 1;
-  if (epi == kEpiFwd) {
-    if (split == 4) return launch_tile<128, kEpiFwd, 4>(mA, mB, a, n_active, s);
-    if (split == 2) return launch_tile<128, kEpiFwd, 2>(mA, mB, a, n_active, s);
-    switch (bn) {
-      case 32: return launch_tile<32, kEpiFwd>(mA, mB, a, n_active, s);
-      case 64: return launch_tile<64, kEpiFwd>(mA, mB, a, n_active, s);
-      case 128: return launch_tile<128, kEpiFwd>(mA, mB, a, n_active, s);
-      case 256: return launch_tile<256, kEpiFwd>(mA, mB, a, n_active, s);
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  if (split == 4) return launch_tile<128, kEpiDh, 4>(mA, mB, a, n_active, s);
-  if (split == 2) return launch_tile<128, kEpiDh, 2>(mA, mB, a, n_active, s);
-  switch (bn) {
-    case 32: return launch_tile<32, kEpiDh>(mA, mB, a, n_active, s);
-    case 64: return launch_tile<64, kEpiDh>(mA, mB, a, n_active, s);
-    case 128: return launch_tile<128, kEpiDh>(mA, mB, a, n_active, s);
-    case 256: return launch_tile<256, kEpiDh>(mA, mB, a, n_active, s);
-    default: return cudaErrorInvalidValue;
-  }
+  return epi == kEpiFwd ? launch_epi<kEpiFwd>(bn, mA, mB, a, n_active, s) : launch_epi<kEpiDh>(bn, mA, mB, a, n_active, s);
 }
 
 }  // namespace oscars
