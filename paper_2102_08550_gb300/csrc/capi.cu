@@ -175,10 +175,11 @@ struct oscars_ctx {
   int64_t eval_rows = 0;
   // tensor maps per layer
   std::vector<CUtensorMap> mShadow, mShadowMN, mA, mG, mGT, mAT;
-  // G^T [lane][out][B] in boxes of 64 x 64: the MN-major B operand of the input
-  // gradient.  With it (g_rows false: B a multiple of 64 and the tensor-core
-  // head) the row-major output gradients G are neither kept nor written.
-  std::vector<CUtensorMap> mGTmn;
+  // G^T [lane][out][B] and H^T [lane][in][B] in boxes of 64 x 64: the MN-major B
+  // operands of the input gradient and the forward; in boxes of 64 x 32: stores
+  // of their tiles.  With them (g_rows false: B a multiple of 64 and the
+  // tensor-core head) the row-major G and H are neither kept nor written.
+  std::vector<CUtensorMap> mGTmn, mATmn, mGTst, mATst;
   bool g_rows = true;
   // fp32 W_l of every slot: boxes {32, 128} (loads) and {32, 32} (stores), and
   // the bf16 copy with boxes {64, 32} (stores): the persistent weight gradient
@@ -704,11 +705,13 @@ cudaError_t enqueue_forward(oscars_ctx* c, const int* wid, const int* src, int n
     g.a_z_src = 1;
     g.b_z_src = 0;
     g.offB = ly.offB;
-    g.out = c->A[l + 1];
+    g.out = c->A[l + 1];   // null without row-major activations
+    g.b_mn = l > 0 && !c->g_rows;
     g.outT = c->AT[l + 1];
     g.pdl = c->profiling ? 0 : 1;   // overlaps its prologue with the previous kernel's tail
     ProfScope ps(c, "gemm_fwd", st);
-    cudaError_t e = launch_gemm(kEpiFwd, c->mShadow[l], l == 0 ? step_inputs(c, step) : c->mA[l], g, na, st);
+    const CUtensorMap& in = l == 0 ? step_inputs(c, step) : c->g_rows ? c->mA[l] : c->mATmn[l];
+    cudaError_t e = launch_gemm(kEpiFwd, GemmMaps{&c->mShadow[l], &in, &c->mATst[l + 1], nullptr}, g, na, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -749,15 +752,15 @@ cudaError_t enqueue_step(oscars_ctx* c, int s, int na, const int* wid, const int
     g.K = ly.out;
     g.a_z_src = 1;
     g.b_z_src = 0;
-    g.hmask = c->A[l];
+    g.hmask = c->g_rows ? c->A[l] : c->AT[l];
     g.out = c->g_rows ? c->G[l - 1] : nullptr;
     g.b_mn = c->g_rows ? 0 : 1;
     g.pdl = c->profiling ? 0 : 1;
     g.outT = c->GT[l - 1];
     g.gb_out = c->gb[l - 1];
     ProfScope ps(c, "gemm_dh", st);
-    if ((e = launch_gemm(kEpiDh, c->mShadowMN[l], c->g_rows ? c->mG[l] : c->mGTmn[l], g, na, st)) != cudaSuccess)
-      return e;
+    const GemmMaps m{&c->mShadowMN[l], c->g_rows ? &c->mG[l] : &c->mGTmn[l], &c->mGTst[l - 1], &c->mAT[l]};
+    if ((e = launch_gemm(kEpiDh, m, g, na, st)) != cudaSuccess) return e;
   }
   // the weight gradients of all hidden layers, after the last input gradient
   // has read the old weights
@@ -1384,7 +1387,7 @@ oscars_status allocate_mlp(oscars_ctx* c) {
   c->gb.assign(L, nullptr);
   for (int l = 0; l < L; ++l) {
     const size_t act = static_cast<size_t>(W) * B * c->dims[l];
-    if (l > 0 && (!dev_alloc(c, &c->A[l], act) || !dev_alloc(c, &c->AT[l], act)))
+    if (l > 0 && ((c->g_rows && !dev_alloc(c, &c->A[l], act)) || !dev_alloc(c, &c->AT[l], act)))
       return fail(c, OSCARS_ENOMEM, "device allocation failed (activations)");
     if (l + 1 < L) {
       const size_t gsz = static_cast<size_t>(W) * B * c->dims[l + 1];
@@ -1405,6 +1408,9 @@ oscars_status allocate_mlp(oscars_ctx* c) {
   c->mA.resize(L);
   c->mG.resize(L);
   c->mGTmn.resize(L);
+  c->mATmn.resize(L);
+  c->mGTst.resize(L);
+  c->mATst.resize(L);
   c->mGT.resize(L);
   c->mAT.resize(L);
   const uint64_t slots64 = slots;
@@ -1418,7 +1424,14 @@ oscars_status allocate_mlp(oscars_ctx* c) {
     ok &= make_map_f32(&c->mMasterSt[l], c->slab + ly.offW, ly.in, ly.out, slots64, ly.in * 4ull, c->P_pad * 4ull, 32);
     ok &= make_map(&c->mShadowSt[l], c->shadow + ly.offW, ly.in, ly.out, slots64, ly.in * 2ull, c->P_pad * 2ull, 32);
     // layer input [lane][B][in]: B operand of the forward GEMM (layer 0: per step)
-    if (l > 0) ok &= make_map(&c->mA[l], c->A[l], ly.in, B, W, ly.in * 2ull, static_cast<uint64_t>(B) * ly.in * 2ull, B);
+    if (l > 0 && c->g_rows)
+      ok &= make_map(&c->mA[l], c->A[l], ly.in, B, W, ly.in * 2ull, static_cast<uint64_t>(B) * ly.in * 2ull, B);
+    if (!c->g_rows) {   // the transposes alone: MN-major operand and tile stores
+      const uint64_t lane_b = static_cast<uint64_t>(B) * 2ull;
+      if (l > 0) ok &= make_map(&c->mATmn[l], c->AT[l], B, ly.in, W, B * 2ull, lane_b * ly.in, 64);
+      ok &= make_map(&c->mATst[l + 1], c->AT[l + 1], B, ly.out, W, B * 2ull, lane_b * ly.out, 32);
+      ok &= make_map(&c->mGTst[l], c->GT[l], B, ly.out, W, B * 2ull, lane_b * ly.out, 32);
+    }
     // output gradient^T [lane][out][B]: A operand of the weight-gradient GEMM
     ok &= make_map(&c->mGT[l], c->GT[l], B, ly.out, W, B * 2ull, static_cast<uint64_t>(B) * ly.out * 2ull, 128);
     // layer input^T [lane][in][B]: B operand of the weight-gradient GEMM (layer 0: per step)

@@ -13,6 +13,15 @@
 // the TMEM allocation; then all four warps read their 32 TMEM lanes
 // (one output row per thread) and run the epilogue:
 //
+// Where the samples come in boxes of 64 and the head reads H^T (out null; TT
+// below), only the transposes H^T and G^T are kept: the next layer's forward
+// and the input gradient read them MN-major, the ReLU mask comes by TMA as one
+// ring entry more, and each warp stores its rows of a tile by TMA.  With both
+// layouts written, and the mask read, by the threads of a row, the epilogue
+// took 5000 to 9500 clocks of a forward (main loop 12000 for K = 1024) and
+// 7400 to 15000 of an input gradient (12000 to 16000): a round of
+// 3072-1024-1024-10, batch 128, 32 workers, 1576 -> 1524 us.
+//
 //  kEpiFwd  hidden layer forward, m = output feature, n = sample:
 //           h = relu(acc + bias[m]) -> bf16 H[n][m] and H^T[m][n].
 //  kEpiDh   input gradient of a hidden layer, m = input feature, n = sample:
@@ -41,6 +50,35 @@ struct TileCfg {
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr uint32_t kTmemCols = BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;
 };
+
+// 32 samples of a forward row: relu(acc + bias) as bf16 pairs
+__device__ __forceinline__ void fwd_pack(const float (&v)[32], float bias, uint32_t (&pk)[16]) {
+#pragma unroll
+  for (int c = 0; c < 32; c += 2) pk[c >> 1] = pack_bf16x2(fmaxf(v[c] + bias, 0.f), fmaxf(v[c + 1] + bias, 0.f));
+}
+
+// 32 samples of an input-gradient row, masked by h > 0 (pk: bf16 pairs of h,
+// replaced by the gradient's); returns their sum in sample order
+__device__ __forceinline__ float dh_mask_pack(const float (&v)[32], uint32_t (&pk)[16]) {
+  float gsum = 0.f;
+#pragma unroll
+  for (int c = 0; c < 32; c += 2) {
+    const uint32_t h = pk[c >> 1];
+    const float g0 = __uint_as_float(h << 16) > 0.f ? v[c] : 0.f;
+    const float g1 = __uint_as_float(h & 0xffff0000u) > 0.f ? v[c + 1] : 0.f;
+    gsum += g0;
+    gsum += g1;
+    pk[c >> 1] = pack_bf16x2(g0, g1);
+  }
+  return gsum;
+}
+
+__device__ __forceinline__ void lds128(uint32_t addr, uint32_t* r) {
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void sts128(uint32_t addr, const uint32_t* r) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
 
 template <int EPI>
 __device__ __forceinline__ void epi_fwd(const GemmArgs& a, int wid, int src, int m, int n0,
@@ -76,7 +114,7 @@ __device__ __forceinline__ void epi_dh_mask(const GemmArgs& a, int wid, int m, i
 
 __device__ __forceinline__ float epi_dh(const GemmArgs& a, int wid, int m, int n0, const float (&v)[32],
                                         const unsigned short (&mk)[32]) {
-  __nv_bfloat16* out = a.out ? a.out + static_cast<int64_t>(wid) * a.N * a.M : nullptr;
+  __nv_bfloat16* out = a.out + static_cast<int64_t>(wid) * a.N * a.M;
   uint32_t pk[16];
   float gsum = 0.f;
 #pragma unroll
@@ -88,10 +126,8 @@ __device__ __forceinline__ float epi_dh(const GemmArgs& a, int wid, int m, int n
     gsum += g0;
     gsum += g1;
     const __nv_bfloat162 p = __floats2bfloat162_rn(g0, g1);
-    if (out) {   // the row-major copy only when a consumer reads it K-major
-      out[e0] = p.x;
-      out[e1] = p.y;
-    }
+    out[e0] = p.x;
+    out[e1] = p.y;
     pk[c >> 1] = *reinterpret_cast<const uint32_t*>(&p);
   }
   uint4* outT = reinterpret_cast<uint4*>(a.outT + (static_cast<int64_t>(wid) * a.M + m) * a.N + n0);
@@ -118,12 +154,14 @@ __device__ __forceinline__ void st_dsmem_f32x4(float* local, uint32_t rank, floa
                : "memory");
 }
 
-template <int BN, int EPI, int SPLIT = 1>
+template <int BN, int EPI, int SPLIT, bool TT>
 __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA,
                                                            const __grid_constant__ CUtensorMap mapB,
+                                                           const __grid_constant__ CUtensorMap mapT,
+                                                           const __grid_constant__ CUtensorMap mapM,
                                                            const __grid_constant__ GemmArgs a,
                                                            int stages) {
-  static_assert(SPLIT == 1 || EPI == kEpiFwd || EPI == kEpiDh, "split-K serves the forward and input-gradient GEMMs");
+  static_assert(!TT || BN == 64 || BN == 128, "transposed results are stored in boxes of 64 samples");
   using Cfg = TileCfg<BN>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -147,6 +185,7 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
   if (threadIdx.x == 0) {
     prefetch_tmap(&mapA);
     prefetch_tmap(&mapB);
+    if (TT && SPLIT == 1) prefetch_tmap(&mapT);
     for (int s = 0; s < stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
@@ -183,19 +222,28 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
       } else {
         tma_load_3d(sA + s * kABytes, &mapA, k, m0, za, &full[s]);
       }
-      if (EPI == kEpiDh && a.b_mn) {
-        // B = G read MN-major from G^T [K = out][N = batch]: boxes of 64 N x 64 K, 8 KB apart
+      if (a.b_mn) {
+        // B (G, H) read MN-major from its transpose [K][N = batch]: boxes of 64 N x 64 K, 8 KB apart
         for (int nb = 0; nb < BN / 64; ++nb)
           tma_load_3d(sB + s * Cfg::kBBytes + nb * 8192, &mapB, n0 + 64 * nb, k, zb, &full[s]);
       } else {
         tma_load_3d(sB + s * Cfg::kBBytes, &mapB, k, n0, zb, &full[s]);
       }
     }
+    if constexpr (TT && SPLIT == 1 && EPI == kEpiDh) {
+      // the ReLU mask, one entry of the ring more: h^T tiles of 64 samples
+      const int s = nk % stages;
+      if (nk < stages || mbar_wait(&empty[s], ((nk / stages) + 1) & 1, a.err, kDevTimeoutEmpty)) {
+        mbar_arrive_expect_tx(&full[s], BN / 64 * kABytes);
+        tma_load_3d(sA + s * kABytes, &mapM, n0, m0, wid, &full[s]);
+        if (BN == 128) tma_load_3d(sB + s * Cfg::kBBytes, &mapM, n0 + 64, m0, wid, &full[s]);
+      }
+    }
   } else if (warp == 1) {
     // MMA issuer: the warp converged, one elected lane issues (see elect_one)
     // A MN-major (transpose-A bit 15) for the input gradient, K-major otherwise;
-    // B MN-major (bit 16) when the input gradient reads G^T
-    const bool bmn = EPI == kEpiDh && a.b_mn;
+    // B MN-major (bit 16) when it is read from its transpose
+    const bool bmn = a.b_mn;
     const uint32_t idesc = idesc_bf16_f32(BM, BN) | (EPI == kEpiDh ? (1u << 15) : 0u) | (bmn ? (1u << 16) : 0u);
     for (int kb = 0; kb < nk; ++kb) {
       const int s = kb % stages;
@@ -248,6 +296,15 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
       }
     }
     tc_fence_before();
+    // TT: the mask bits of this thread's (one) item, while the partials land
+    uint4 hm[4];
+    if constexpr (TT && EPI == kEpiDh) {
+      const int it = threadIdx.x < R * (BN / 32) ? threadIdx.x : 0;
+      const uint4* hrow = reinterpret_cast<const uint4*>(
+          a.hmask + (static_cast<int64_t>(wid) * a.M + m0 + rank * R + it / (BN / 32)) * a.N + n0 + it % (BN / 32) * 32);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) hm[q] = __ldg(hrow + q);
+    }
     cluster_sync();   // every partial has landed in its owner
     // own rows: item = (row, 32-column chunk); partials summed in rank order
     float* gpart = red + SPLIT * R * ld;            // [R][BN / 32] bias-gradient partials (input gradient)
@@ -269,7 +326,30 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
         }
       }
       const int m = m0 + rank * R + rl;
-      if constexpr (EPI == kEpiFwd) {
+      if constexpr (TT) {
+        uint32_t pk[16];
+        if constexpr (EPI == kEpiFwd) {
+          fwd_pack(v, a.master[static_cast<int64_t>(src) * a.slot_stride + a.offB + m], pk);
+        } else {
+          if (it != threadIdx.x) {   // SPLIT = 2 at 128 samples: a thread's second item
+            const uint4* hrow =
+                reinterpret_cast<const uint4*>(a.hmask + (static_cast<int64_t>(wid) * a.M + m) * a.N + n0 + c0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) hm[q] = __ldg(hrow + q);
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            pk[4 * q] = hm[q].x;
+            pk[4 * q + 1] = hm[q].y;
+            pk[4 * q + 2] = hm[q].z;
+            pk[4 * q + 3] = hm[q].w;
+          }
+          gpart[rl * (BN / 32) + c0 / 32] = dh_mask_pack(v, pk);
+        }
+        uint4* outT = reinterpret_cast<uint4*>(a.outT + (static_cast<int64_t>(wid) * a.M + m) * a.N + n0 + c0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) outT[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+      } else if constexpr (EPI == kEpiFwd) {
         epi_fwd<EPI>(a, wid, src, m, n0 + c0, v);
       } else {
         unsigned short mk[32];
@@ -284,6 +364,58 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
         for (int c = 0; c < BN / 32; ++c) g += gpart[rl * (BN / 32) + c];
         a.gb_out[static_cast<int64_t>(wid) * a.M + m0 + rank * R + rl] = g;
       }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 2) {
+      tc_fence_after();
+      tmem_dealloc(tmem, Cfg::kTmemCols);
+    }
+    return;
+  }
+
+  if constexpr (TT) {
+    // ---- epilogue with H^T / G^T alone: thread = one accumulator row, its
+    // 64-sample halves in tiles [128][64] (128-byte swizzle) in the ring: the
+    // mask's entry, overwritten in place, or the first one; each warp stores
+    // its 32 rows of a tile with one TMA store
+    const int m = m0 + 32 * warp + lane, row = 32 * warp + lane;
+    const float bias = EPI == kEpiFwd ? a.master[static_cast<int64_t>(src) * a.slot_stride + a.offB + m] : 0.f;
+    const int st = EPI == kEpiDh ? nk % stages : 0;
+    bool ok = mbar_wait(accum, 0, a.err, kDevTimeoutAccum);
+    if constexpr (EPI == kEpiDh) ok = mbar_wait(&full[st], (nk / stages) & 1, a.err, kDevTimeoutFull) && ok;
+    const int all_ok = __all_sync(0xffffffffu, ok);
+    tc_fence_after();
+    if (all_ok) {
+      const uint32_t trow = tmem + (static_cast<uint32_t>(warp * 32) << 16);
+      float gsum = 0.f;
+#pragma unroll 1
+      for (int c0 = 0; c0 < BN; c0 += 32) {
+        float v[32];
+        tmem_ld_32x32b_x32(trow + c0, v);
+        uint8_t* tile = c0 < 64 ? sA + st * kABytes : sB + st * Cfg::kBBytes;
+        const uint32_t at = smem_u32(tile) + row * 128, ch = (c0 & 63) >> 3;
+        uint32_t pk[16];
+        if constexpr (EPI == kEpiFwd) {
+          fwd_pack(v, bias, pk);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) lds128(at + (((ch + q) ^ (row & 7)) << 4), pk + 4 * q);
+          gsum += dh_mask_pack(v, pk);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sts128(at + (((ch + q) ^ (row & 7)) << 4), pk + 4 * q);
+        if (c0 & 32) {
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            tma_store_3d(&mapT, tile + 32 * warp * 128, n0 + (c0 & 64), m0 + 32 * warp, wid);
+            bulk_commit_group();
+          }
+        }
+      }
+      if constexpr (EPI == kEpiDh) a.gb_out[static_cast<int64_t>(wid) * a.M + m] = gsum;
+      if (lane == 0) bulk_wait_all();
     }
     tc_fence_before();
     __syncthreads();
@@ -352,11 +484,11 @@ int device_sms() {
   return sms;
 }
 
-template <int BN, int EPI, int SPLIT = 1>
-cudaError_t launch_tile(const CUtensorMap& mA, const CUtensorMap& mB, const GemmArgs& a, int n_active,
-                        cudaStream_t s) {
+template <int BN, int EPI, int SPLIT, bool TT>
+cudaError_t launch_tile(const GemmMaps& m, const GemmArgs& a, int n_active, cudaStream_t s) {
   using Cfg = TileCfg<BN>;
-  const int nk = ((a.K + BK - 1) / BK + SPLIT - 1) / SPLIT;   // K-blocks of the CTA with the most
+  // ring entries of the CTA with the most K-blocks, and the mask's
+  const int nk = ((a.K + BK - 1) / BK + SPLIT - 1) / SPLIT + (TT && SPLIT == 1 && EPI == kEpiDh ? 1 : 0);
   dim3 grid(a.M / BM, (a.N + BN - 1) / BN, n_active * SPLIT);
   // A grid that fits one CTA per SM gets as many stages as K-blocks, within
   // ~200 KB of shared memory: the whole K extent of these skinny GEMMs is
@@ -375,7 +507,7 @@ cudaError_t launch_tile(const CUtensorMap& mA, const CUtensorMap& mB, const Gemm
   size_t smem = 1024 + static_cast<size_t>(stages) * Cfg::kStageBytes + kBarrierBytes + red_bytes;
   const size_t floor_b = smem_floor_for_tmem(Cfg::kTmemCols);
   if (smem < floor_b) smem = floor_b;
-  cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, SPLIT, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -399,7 +531,7 @@ cudaError_t launch_tile(const CUtensorMap& mA, const CUtensorMap& mB, const Gemm
   }
   cfg.attrs = attr;
   cfg.numAttrs = n;
-  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, EPI, SPLIT>, mA, mB, a, stages);
+  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, EPI, SPLIT, TT>, *m.a, *m.b, TT ? *m.t : *m.a, TT && EPI == kEpiDh ? *m.mask : *m.a, a, stages);
 }
 
 // K split of a forward or input-gradient launch of up to 128 samples: 4 or 2
@@ -420,23 +552,23 @@ int split_for(int M, int N, int BN, int K, int n_active) {
   return 1;
 }
 
-template <int BN, int EPI>
-cudaError_t launch_split(const CUtensorMap& mA, const CUtensorMap& mB, const GemmArgs& a, int n_active, cudaStream_t s) {
+template <int BN, int EPI, bool TT>
+cudaError_t launch_split(const GemmMaps& m, const GemmArgs& a, int n_active, cudaStream_t s) {
   switch (split_for(a.M, a.N, BN, a.K, n_active)) {
-    case 4: return launch_tile<BN, EPI, 4>(mA, mB, a, n_active, s);
-    case 2: return launch_tile<BN, EPI, 2>(mA, mB, a, n_active, s);
-    default: return launch_tile<BN, EPI>(mA, mB, a, n_active, s);
+    case 4: return launch_tile<BN, EPI, 4, TT>(m, a, n_active, s);
+    case 2: return launch_tile<BN, EPI, 2, TT>(m, a, n_active, s);
+    default: return launch_tile<BN, EPI, 1, TT>(m, a, n_active, s);
   }
 }
 
 template <int EPI>
-cudaError_t launch_epi(int bn, const CUtensorMap& mA, const CUtensorMap& mB, const GemmArgs& a, int n_active,
-                       cudaStream_t s) {
+cudaError_t launch_epi(int bn, const GemmMaps& m, const GemmArgs& a, int n_active, cudaStream_t s) {
+  const bool tt = a.out == nullptr;
   switch (bn) {
-    case 32: return launch_split<32, EPI>(mA, mB, a, n_active, s);
-    case 64: return launch_split<64, EPI>(mA, mB, a, n_active, s);
-    case 128: return launch_split<128, EPI>(mA, mB, a, n_active, s);
-    case 256: return launch_tile<256, EPI>(mA, mB, a, n_active, s);
+    case 32: return tt ? cudaErrorInvalidValue : launch_split<32, EPI, false>(m, a, n_active, s);
+    case 64: return tt ? launch_split<64, EPI, true>(m, a, n_active, s) : launch_split<64, EPI, false>(m, a, n_active, s);
+    case 128: return tt ? launch_split<128, EPI, true>(m, a, n_active, s) : launch_split<128, EPI, false>(m, a, n_active, s);
+    case 256: return tt ? cudaErrorInvalidValue : launch_tile<256, EPI, 1, false>(m, a, n_active, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -447,11 +579,10 @@ int gemm_bn_for(int epi, int N) {
   return N;  // forward / input gradient: the whole batch in one tile
 }
 
-cudaError_t launch_gemm(int epi, const CUtensorMap& mA, const CUtensorMap& mB, const GemmArgs& a,
-                        int n_active, cudaStream_t s) {
+cudaError_t launch_gemm(int epi, const GemmMaps& m, const GemmArgs& a, int n_active, cudaStream_t s) {
   if (a.M % BM != 0) return cudaErrorInvalidValue;
   const int bn = gemm_bn_for(epi, a.N);
-  return epi == kEpiFwd ? launch_epi<kEpiFwd>(bn, mA, mB, a, n_active, s) : launch_epi<kEpiDh>(bn, mA, mB, a, n_active, s);
+  return epi == kEpiFwd ? launch_epi<kEpiFwd>(bn, m, a, n_active, s) : launch_epi<kEpiDh>(bn, m, a, n_active, s);
 }
 
 }  // namespace oscars

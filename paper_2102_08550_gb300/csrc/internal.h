@@ -145,21 +145,26 @@ struct GemmArgs {
   const int* src;     // [n_active]
   int M, N, K;
   int a_z_src, b_z_src;  // TMA z coordinate of A / B: 1 = src slot, 0 = lane id
-  int b_mn;              // kEpiDh: B read MN-major (G^T [lane][K][N] in boxes of 64 N x 64 K; N % 64 == 0)
+  int b_mn;              // B read MN-major (its transpose [lane][K][N] in boxes of 64 N x 64 K; N % 64 == 0)
   int pdl;               // launch as a programmatic dependent of the previous kernel on the stream
   int* err;
-  // kEpiFwd: out = relu(acc + bias[m]) -> H [lane][N][M], HT [lane][M][N]
-  // kEpiDh : out = acc * (Hmask[lane][n][m] > 0) -> G (if out), GT, gb[lane][m]
+  // kEpiFwd: relu(acc + bias[m]) -> H [lane][N][M], H^T [lane][M][N]
+  // kEpiDh : acc * (h > 0) -> G [lane][N][M], G^T [lane][M][N], gb[lane][m]
+  // With out null (N = 64 or 128) only the transposes are written.
   const float* master;      // fp32 slab base
   int64_t slot_stride;      // P_pad
   int64_t offB;             // element offset of b_l in a slot
-  const __nv_bfloat16* hmask;  // [lanes][N][M] (kEpiDh)
-  __nv_bfloat16* out;       // [lanes][N][M]
+  const __nv_bfloat16* hmask;  // kEpiDh: h [lanes][N][M]; h^T [lanes][M][N] with out null
+  __nv_bfloat16* out;       // [lanes][N][M], or null
   __nv_bfloat16* outT;      // [lanes][M][N]
   float* gb_out;            // [lanes][M] (kEpiDh)
 };
-cudaError_t launch_gemm(int epi, const CUtensorMap& mapA, const CUtensorMap& mapB,
-                        const GemmArgs& a, int n_active, cudaStream_t s);
+struct GemmMaps {
+  const CUtensorMap *a, *b;
+  const CUtensorMap* t;     // outT [lane][M][N], box {64, 32}: used when out is null
+  const CUtensorMap* mask;  // hmask [lane][M][N], box {64, 128}: kEpiDh, used when out is null
+};
+cudaError_t launch_gemm(int epi, const GemmMaps& m, const GemmArgs& a, int n_active, cudaStream_t s);
 
 // One large product D[m][n] = sum_k A[m][k] B[n][k] (csrc/gemm_rows.cu).
 enum RowsEpi { kRowsStore = 0, kRowsRelu = 1, kRowsLoss = 2 };
