@@ -148,8 +148,9 @@ __device__ __forceinline__ void bar_arrive_named(int id, int count) {
 // dependent may start while the previous kernel on its stream finishes;
 // pdl_wait() blocks until that kernel has completed and its memory is
 // visible (a no-op without a programmatic dependency), so a kernel calls it
-// after its prologue (barriers, TMEM, tensor-map prefetch) and before its
-// first global access.  pdl_trigger() lets this kernel's own dependent start
+// after its prologue (barriers, TMEM, tensor-map prefetch, and reads of what
+// was complete before the previous kernel's own pdl_wait) and before its
+// first other global access.  pdl_trigger() lets this kernel's own dependent start
 // its prologue (every CTA of this grid has started by then: no CTA of it can
 // be kept from starting by the dependent's).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

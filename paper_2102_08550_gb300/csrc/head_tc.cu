@@ -48,7 +48,8 @@
 // 256 features, batch 32).  A round of the 1000-384-256-17 model, 5 workers:
 // 534 us with those, 440 with this kernel's first form, 335 now (374 before
 // the loops, the early code and the h^T tile); 3072-1024-1024-10, 32 workers:
-// 1579 -> 1573.
+// 1579 -> 1573.  (Both models' rounds have become shorter by other kernels
+// since.)
 #include "common.cuh"
 #include "internal.h"
 
@@ -284,18 +285,14 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
   for (int dry = a.pdl && warp == kHTThreads / 32 - 1 ? 1 : 0; dry >= 0; --dry) {
     if (!dry) {
       __syncthreads();   // the dry pass has left the tiles
-      pdl_wait();      // the layer input (the previous kernel's output) is complete
+      // what the previous kernel does not write is requested while it runs (the
+      // weights of the previous step: every kernel of the chain waits for its
+      // predecessor before it lets its successor start); rounds as above: 318.9
+      // -> 313.9 us and 1526 -> 1521
       if (t == 0) {
-        // the h and W2 tiles, requested first: the rest of the prologue overlaps them
         mbar_arrive_expect_tx(tma_bar, (ht ? NH * hb : F / 64) * (kHTRows * 128) + (F / 64) * (NC * 128));
-        if (ht)
-          for (int q = 0; q < NH * hb; ++q)
-            tma_load_3d(hT + q * (kHT * 128), &mH, 64 * (q & (hb - 1)), k0 + kHT * (q / hb), w, tma_bar);
 #pragma unroll
-        for (int q = 0; q < F / 64; ++q) {
-          if (!ht) tma_load_3d(hT + q * kHTRows * 128, &mH, k0 + 64 * q, 0, w, tma_bar);
-          tma_load_3d(w2 + q * NC * 128, &mW2, k0 + 64 * q, 0, src, tma_bar);
-        }
+        for (int q = 0; q < F / 64; ++q) tma_load_3d(w2 + q * NC * 128, &mW2, k0 + 64 * q, 0, src, tma_bar);
       }
       if (warp == 0) {
         tmem_alloc(tmem_slot, Cfg::kTmemCols);
@@ -315,6 +312,16 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
         reinterpret_cast<uint4*>(dzT)[q] = make_uint4(0, 0, 0, 0);
       for (int b = t; b < B; b += kHTThreads) labs[b] = a.labels[static_cast<int64_t>(w) * B + b];
       if (t < NC) b2[t] = t < C ? a.master[so + a.offB + t] : 0.f;
+      pdl_wait();      // the layer input (the previous kernel's output) is complete
+      if (t == 0) {
+        if (ht) {
+          for (int q = 0; q < NH * hb; ++q)
+            tma_load_3d(hT + q * (kHT * 128), &mH, 64 * (q & (hb - 1)), k0 + kHT * (q / hb), w, tma_bar);
+        } else {
+#pragma unroll
+          for (int q = 0; q < F / 64; ++q) tma_load_3d(hT + q * kHTRows * 128, &mH, k0 + 64 * q, 0, w, tma_bar);
+        }
+      }
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
