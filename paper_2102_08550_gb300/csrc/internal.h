@@ -319,11 +319,9 @@ cudaError_t launch_eval_result(const float* part, int64_t count, double scale, i
 // cursor[w] = (cursor[w] + tau[w] * B) % n[w]
 cudaError_t launch_cursor_advance(int64_t* cursor, const int32_t* tau, const int64_t* n, int B,
                                   int W, cudaStream_t s);
-// shadow[p] = bf16(master[p]) for one slot; shadowT for layers with a transposed copy
+// shadow[p] = bf16(master[p]) for one slot
 cudaError_t launch_shadow_refresh(const float* master, __nv_bfloat16* shadow, int64_t count,
                                   cudaStream_t s);
-cudaError_t launch_transpose_bf16(const __nv_bfloat16* src, __nv_bfloat16* dst, int rows,
-                                  int cols, cudaStream_t s);
 // replicas[k] = x_g for k < W (fp32 and bf16 shadows)
 cudaError_t launch_broadcast(const float* xg, float* slab, int64_t stride, int W, int64_t count,
                              cudaStream_t s);

@@ -654,19 +654,6 @@ __global__ void shadow_refresh_kernel(const float* __restrict__ m, __nv_bfloat16
     s[i] = __float2bfloat16_rn(m[i]);
 }
 
-// dst[c][r] = src[r][c] for a rows x cols bf16 matrix
-__global__ void transpose_bf16_kernel(const __nv_bfloat16* __restrict__ src, __nv_bfloat16* __restrict__ dst,
-                                      int rows, int cols) {
-  __shared__ __nv_bfloat16 t[32][34];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int r = ty; r < 32; r += 8)
-    if (r0 + r < rows && c0 + tx < cols) t[r][tx] = src[static_cast<int64_t>(r0 + r) * cols + c0 + tx];
-  __syncthreads();
-  for (int c = ty; c < 32; c += 8)
-    if (c0 + c < cols && r0 + tx < rows) dst[static_cast<int64_t>(c0 + c) * rows + r0 + tx] = t[tx][c];
-}
-
 // Canonical vector <- padded slot, grid y = piece: 16-byte copies where both
 // sides of every row are 16-byte aligned.  One launch instead of a copy per
 // tensor (two per layer): a 784-512-10 round with its pull went from 109 to
@@ -836,13 +823,6 @@ cudaError_t launch_shadow_refresh(const float* master, __nv_bfloat16* shadow, in
   if (blocks > 4096) blocks = 4096;
   if (blocks < 1) return cudaSuccess;
   shadow_refresh_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(master, shadow, count);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_transpose_bf16(const __nv_bfloat16* src, __nv_bfloat16* dst, int rows, int cols,
-                                  cudaStream_t s) {
-  dim3 grid((cols + 31) / 32, (rows + 31) / 32);
-  transpose_bf16_kernel<<<grid, 256, 0, s>>>(src, dst, rows, cols);
   return cudaGetLastError();
 }
 
