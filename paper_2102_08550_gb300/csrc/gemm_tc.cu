@@ -140,7 +140,9 @@ __device__ __forceinline__ float epi_dh(const GemmArgs& a, int wid, int m, int n
 // SPLIT CTAs shares one output tile, CTA r multiplying K-blocks [r nk / SPLIT,
 // (r + 1) nk / SPLIT).  Each CTA pushes its fp32 partial rows into the CTA
 // that owns them (rows [r 128 / SPLIT, (r + 1) 128 / SPLIT) belong to CTA r)
-// through distributed shared memory, one cluster barrier follows, and each
+// through distributed shared memory, between two cluster barriers (every CTA
+// has started before the first store, arrived on in the prologue and so free;
+// every partial has landed before the first is read), and each
 // owner sums the SPLIT partials in rank order and runs the epilogue on its
 // rows.  Used when a launch has too few tiles to fill the GPU: small layers,
 // and the tail of a round, where one worker with many local steps runs alone
@@ -201,6 +203,7 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (SPLIT > 1) cluster_arrive();   // this CTA has started; the wait stands before the first store into a peer
   const uint32_t tmem = *tmem_slot;
   pdl_wait();      // the previous kernel's outputs (operands, masks, biases) are complete
   pdl_trigger();
@@ -281,6 +284,7 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
     const int owner = row / R;
     float* dst = red + (rank * R + (row - owner * R)) * ld;
     const uint32_t trow = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+    cluster_wait();   // every CTA of the cluster has started: its shared memory may be written
 #pragma unroll 1
     for (int c0 = 0; c0 < BN; c0 += 32) {
       float v[32];
