@@ -72,6 +72,20 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
   return false;
 }
 
+// A converged warp that issues through an elected lane (elect_one), or reads
+// tensor memory, must stay together even when a wait runs out, and it may run
+// out in some lanes only.  A loop that elects a lane is therefore never left on
+// a wait: a lane whose wait ran out goes through the rest of it without waiting
+// (mbar_wait_keep), and the elected lane issues nothing any more once its own
+// has.  A branch around a warp-wide instruction takes one answer for all lanes
+// (mbar_wait_warp; in the loops its vote cost 1 to 2% of a round).
+__device__ __forceinline__ void mbar_wait_keep(bool& ok, uint64_t* bar, uint32_t parity, int* err, int code) {
+  if (ok) ok = mbar_wait(bar, parity, err, code);
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err, int code) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, code));
+}
+
 // 3-D tiled TMA load of one box into shared memory, completing on `bar`.
 __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* map, int c0, int c1,
                                             int c2, uint64_t* bar) {
@@ -233,7 +247,7 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
 // together and lets one elected lane issue: the descriptors and addresses of
 // tcgen05 instructions then stay in uniform registers.  With a loop run by
 // lane 0 alone an issue cost about 60 clocks (a 4096 x 128 x 3072 product took
-// 24.8 us, 18.7 with an elected lane).
+// 24.8 us, 18.7 with an elected lane).  Its waits: see mbar_wait_keep.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));

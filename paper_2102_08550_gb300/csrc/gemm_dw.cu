@@ -168,25 +168,25 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
     constexpr uint32_t idesc = idesc_bf16_f32(kDwTile, kDwTile);
     int kc = 0, it = 0;
     bool ok = true;
-    for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x, ++it) {
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {
       const int b = it & 1;
-      if (it >= 2 && !(ok = mbar_wait(&bars->aempty[b], ((it >> 1) + 1) & 1, a.err, kDevTimeoutAccum))) break;
+      if (it >= 2) mbar_wait_keep(ok, &bars->aempty[b], ((it >> 1) + 1) & 1, a.err, kDevTimeoutAccum);
       tc_fence_after();
       const uint32_t acc = tmem + static_cast<uint32_t>(b * kDwTile);
       for (int kb = 0; kb < nk; ++kb, ++kc) {
         const int s = kc & 1;
-        if (!(ok = mbar_wait(&bars->full[s], (kc >> 1) & 1, a.err, kDevTimeoutFull))) break;
+        mbar_wait_keep(ok, &bars->full[s], (kc >> 1) & 1, a.err, kDevTimeoutFull);
         tc_fence_after();
         const uint64_t ad = smem_desc_k128(smem_u32(sOps + s * kDwOpBytes));
         const uint64_t bd = smem_desc_k128(smem_u32(sOps + s * kDwOpBytes + kDwOpBytes / 2));
-        if (elect_one()) {
+        if (elect_one() && ok) {
 #pragma unroll
           for (int j = 0; j < kDwBK / 16; ++j) umma_bf16(acc, ad + 2 * j, bd + 2 * j, idesc, (kb | j) != 0 ? 1u : 0u);
           umma_commit(&bars->empty[s]);
         }
         __syncwarp();
       }
-      if (ok && elect_one()) umma_commit(&bars->afull[b]);
+      if (elect_one() && ok) umma_commit(&bars->afull[b]);
       __syncwarp();
     }
     if (elect_one()) umma_commit(&bars->mma_done);   // every product issued above has landed before TMEM is released

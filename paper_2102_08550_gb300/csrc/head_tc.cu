@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
         }
         __syncwarp();
       }
-      ok = mbar_wait(mma_bar, 0, a.err, kDevTimeoutAccum);
+      ok = mbar_wait_warp(mma_bar, 0, a.err, kDevTimeoutAccum);
       tc_fence_after();
       if (warp < 4) {
         float v[NC];
@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
           }
         }
       }
-      ok = mbar_wait(mma_bar, 1, a.err, kDevTimeoutAccum) && ok;
+      ok = mbar_wait_warp(mma_bar, 1, a.err, kDevTimeoutAccum) && ok;
       tc_fence_after();
       if (warp < 4 * NH && ok) {
         const int mh = warp >> 2, q = warp & 3;
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_consta
         }
         __syncwarp();
       }
-      ok = mbar_wait(mma_bar, 0, a.err, kDevTimeoutAccum) && ok;
+      ok = mbar_wait_warp(mma_bar, 0, a.err, kDevTimeoutAccum) && ok;
       mbar_wait(tma_bar, 0, a.err, kDevTimeoutFull);   // completed long ago: orders the tile reads below
       tc_fence_after();
     }

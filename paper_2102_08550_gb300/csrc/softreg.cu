@@ -665,7 +665,8 @@ __global__ void __launch_bounds__(NT + NT / 4, 1) softreg_cluster_round_kernel(c
       }
     }
   }
-  // a wait that ran out shows as a NaN loss (the allocation-free entry has no error word)
+  // a wait that ran out, in any lane, shows as a NaN loss (the allocation-free entry has no error word)
+  alive = __all_sync(0xffffffffu, alive);
   if (!fetcher && lane == 0)
     lsum[warp] = alive ? static_cast<double>(loss_hi) + static_cast<double>(loss_lo) : static_cast<double>(NAN);
   __syncthreads();

@@ -3,7 +3,10 @@ missing one shows only as a fault or a hang, and only now and then, on a GPU).
 
 * A CTA's shared memory may be touched by a peer of its cluster only once that
   CTA is known to run: in every kernel a cluster barrier's wait comes before
-  the first remote load, store or arrival."""
+  the first remote load, store or arrival.
+* A warp that runs a loop together and elects a lane to issue (elect.sync with a
+  full mask) must stay together: such a loop is not left on a wait, which may run
+  out in some lanes and not in the others."""
 import os
 import re
 
@@ -86,3 +89,49 @@ def test_a_missing_start_barrier_is_caught():
     assert first_remote_access_without_start(kernel % "") == ["k"]
     assert first_remote_access_without_start(kernel % "cluster_arrive(); cluster_wait();") == []
     assert first_remote_access_without_start(kernel % "// cluster_wait();\n") == ["k"]
+
+
+def _loops(body):
+    """(start, end) of the braced for loops of a function body."""
+    out = []
+    for m in re.finditer(r"\bfor \(", body):
+        depth, i = 0, m.end() - 1
+        while True:
+            depth += {"(": 1, ")": -1}.get(body[i], 0)
+            i += 1
+            if depth == 0:
+                break
+        if body[i:].lstrip().startswith("{"):
+            at = body.index("{", i)
+            out.append((at, at + len(_block(body, at))))
+    return out
+
+
+def lanes_that_leave_alone(text):
+    """Kernels with a loop that elects an issuer and ends on a wait that each lane decides for itself."""
+    bad = []
+    for name, (kernel, body) in _functions(_clean(text)).items():
+        if not kernel:
+            continue
+        loops = _loops(body)
+        for m in re.finditer(r"if \([^;{}]*\bmbar_wait\([^;{}]*break;", body):
+            lo, hi = max(l for l in loops if l[0] < m.start() < l[1])
+            if _calls(body[lo:hi], ("elect_one",)):
+                bad.append(name)
+        for lo, hi in loops:
+            head = body[body.rindex("for (", 0, lo):lo]
+            if re.search(r"\bok\b", head) and _calls(body[lo:hi], ("elect_one",)):
+                bad.append(name)
+    return bad
+
+
+@pytest.mark.parametrize("f", _sources())
+def test_issuing_warps_leave_their_loops_together(f):
+    assert lanes_that_leave_alone(_read(f)) == []
+
+
+def test_a_lane_wise_wait_is_caught():
+    kernel = "__global__ void __launch_bounds__(32) k(int* p) {\n for (int i = 0; %si < 4; ++i) {\n %s;\n if (elect_one() && ok) { go(); }\n }\n}\n"
+    assert lanes_that_leave_alone(kernel % ("", "if (!(ok = mbar_wait(b, i))) break")) == ["k"]
+    assert lanes_that_leave_alone(kernel % ("ok && ", "ok = mbar_wait(b, i)")) == ["k"]
+    assert lanes_that_leave_alone(kernel % ("", "mbar_wait_keep(ok, b, i)")) == []
