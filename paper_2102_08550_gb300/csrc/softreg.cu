@@ -17,6 +17,8 @@
 // products), p = softmax(z), loss_b = logsumexp(z_b) - z_b[y_b],
 // dz = (p - onehot(y)) / B, dW[c][k] = sum_b dz[b][c] x[b][k],
 // db[c] = sum_b dz[b][c], W <- W - lr dW (fmaf), all fp32.
+#include <atomic>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -268,14 +270,13 @@ __global__ void __launch_bounds__(kThreads) softreg_round_kernel(const __grid_co
 // (cluster barrier, remote reads, one-thread row loops), 128 us now.
 // 784 x 10, 4 workers, at most 4 steps: 49 and 35 us.
 constexpr int kCl = 8;
-// A CTA has NT computing threads and NT / 4 fetching ones.  NT = 512 fills the
-// SM's registers, so 17 to 19 workers run at once; a step of few products
-// leaves most of its warps without work, and NT = 128 lets four CTAs share an
-// SM.  The line: 16 x 2, batch 1, 32 workers, a round: 50 us with the earlier
-// kernel, 62 with NT = 512, 40 with 128; 333 x 26, batch
-// 100, 24 workers: 135 us with 512, 392 with the earlier 256-thread kernel.
-constexpr int kClThreads = 512, kClSmall = 128;
-constexpr int kClSmallWork = 4096;   // products of a step in a CTA, at most, for kClSmall
+// A CTA has NT computing threads and NT / 4 fetching ones, and K CTAs share an
+// SM (launch bounds): 512 threads and one (96 registers a thread), 256 and two,
+// 128 and four; 128 and two (up to 177 registers) for steps of few products,
+// which leave most of 512 threads without work.  More workers than clusters
+// that run at once take several waves: see cluster_variant.
+constexpr int kClThreads = 512;
+constexpr int kClSmallWork = 4096;   // products of a step in a CTA, at most, for 128 threads whatever the workers
 constexpr int kClMaxWarps = kClThreads / 32;
 // columns per CTA: (D + the bias column) / kCl rounded up to a multiple of 4
 __host__ __device__ inline int cluster_cols(int D) { return ((D + 1 + kCl - 1) / kCl + 3) / 4 * 4; }
@@ -365,8 +366,8 @@ __device__ __forceinline__ void st_dsmem_f64(double* local, uint32_t rank, doubl
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(local, rank)), "d"(v) : "memory");
 }
 
-template <int CC, int NT>
-__global__ void __launch_bounds__(NT + NT / 4, 1) softreg_cluster_round_kernel(const __grid_constant__ SoftregArgs a) {
+template <int CC, int NT, int K>
+__global__ void __launch_bounds__(NT + NT / 4, K) softreg_cluster_round_kernel(const __grid_constant__ SoftregArgs a) {
   constexpr int NW = NT / 32, NF = NT / 4;   // computing warps, fetching threads
   extern __shared__ __align__(16) float sm[];
   constexpr int CCp = (CC + 3) / 4 * 4;
@@ -795,45 +796,120 @@ cudaError_t launch_softreg_round(const SoftregArgs& a, int W, cudaStream_t s) {
 }
 
 namespace {
-int cluster_threads(int D, int C, int B) {
-  return static_cast<int64_t>(B) * C * cluster_cols(D) <= kClSmallWork ? kClSmall : kClThreads;
-}
-
-size_t cluster_smem_bytes(int D, int C, int B) {
-  const ClPlan p = cluster_plan(D, C, B, cluster_cc(C), cluster_threads(D, C, B));
+size_t cluster_smem_bytes(int D, int C, int B, int NT) {
+  const ClPlan p = cluster_plan(D, C, B, cluster_cc(C), NT);
   return sizeof(float) * p.oEnd + cluster_tail_bytes(B);
 }
 
-template <int CC, int NT>
-cudaError_t launch_cluster_nt(const SoftregArgs& a, int W, cudaStream_t s) {
-  const size_t smem = cluster_smem_bytes(a.D, a.C, a.B);
-  cudaError_t e = cudaFuncSetAttribute(softreg_cluster_round_kernel<CC, NT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
+// computing threads where the workers need not share SMs
+int cluster_threads_alone(int D, int C, int B) {
+  return static_cast<int64_t>(B) * C * cluster_cols(D) <= kClSmallWork ? 128 : kClThreads;
+}
+
+template <int CC, int NT, int K>
+cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, int W, size_t smem, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kCl, W, 1);
   cfg.blockDim = dim3(NT + NT / 4, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = kCl;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = kCl;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, softreg_cluster_round_kernel<CC, NT>, a);
+  return cfg;
+}
+
+// Clusters that run at once with k CTAs an SM, k <= 4 (not k SMs / 8: the SMs of
+// a cluster share a processor cluster).  Queried once per device.
+constexpr int kMaxDevices = 64;
+constexpr size_t kSmSmem = 228 * 1024, kCtaSmem = 1024;   // shared memory of an SM; taken by each CTA beside its own
+std::atomic<int> g_room[kMaxDevices][4];
+template <int NT, int K>
+int query_room(size_t smem) {
+  int room = 0;
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t cfg = cluster_config<8, NT, K>(&attr, 1, smem, nullptr);
+  if (cudaOccupancyMaxActiveClusters(&room, softreg_cluster_round_kernel<8, NT, K>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    room = 0;
+  }
+  return room < 1 ? 1 : room;
+}
+int cluster_room(int k) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) dev = 0;
+  std::atomic<int>& r = g_room[dev][k - 1];
+  int room = r.load(std::memory_order_relaxed);
+  if (room > 0) return room;
+  // 3 CTAs an SM: what 2 and 4 leave between them
+  room = k == 1   ? query_room<512, 1>(0)
+         : k == 2 ? query_room<256, 2>(0)
+         : k == 4 ? query_room<128, 4>(0)
+                  : (cluster_room(2) + cluster_room(4)) / 2;
+  r.store(room, std::memory_order_relaxed);
+  return room;
+}
+
+// The variant for W workers: the fewest waves, then the most threads.  About 15
+// clusters run at once with one CTA an SM: with 512 threads whatever W, more
+// workers waited for a second and third wave, and the smaller shapes were slower
+// than on the 256-thread cluster kernel before this one, several of whose CTAs
+// share an SM.  Rounds of 4 steps with their merge, us, by workers (before /
+// 512 threads / this rule):
+//   784 x 10, batch 8      1: 27 / 25 / 25    16: 29 / 43 / 27    32: 33 / 60 / 29     64: 56 / 94 / 37
+//   64 x 10, batch 64      1: 35 / 25 / 25    16: 38 / 43 / 25    32: 42 / 62 / 29     64: 71 / 98 / 38
+//   333 x 26, batch 100    1: 93 / 39 / 39    16: 121 / 74 / 60   32: 126 / 105 / 64   64: 237 / 171 / 118
+//   5000 x 4, batch 4      1: 34 / 31 / 31    16: 35 / 53 / 34    32: 38 / 75 / 36     64: 65 / 118 / 46
+// The line of 4096 products: a round of 16 x 2, batch 1, 32 workers with its
+// merge and pull took 62 us with 512 threads, 40 with 128.
+struct ClVariant {
+  int NT, K;
+};
+ClVariant cluster_variant(int D, int C, int B, int W) {
+  const ClVariant all[3] = {{512, 1}, {256, 2}, {128, 4}}, few[2] = {{128, 2}, {128, 4}};
+  const bool small = cluster_threads_alone(D, C, B) == 128;
+  const ClVariant* v = small ? few : all;
+  if (W == 1) return v[0];
+  ClVariant best = v[0];
+  int least = 1 << 30;
+  for (int i = 0; i < (small ? 2 : 3) && least > 1; ++i) {
+    int k = static_cast<int>(kSmSmem / (cluster_smem_bytes(D, C, B, v[i].NT) + kCtaSmem));
+    k = k > v[i].K ? v[i].K : k < 1 ? 1 : k;
+    const int room = cluster_room(k), waves = (W + room - 1) / room;
+    if (waves < least) {
+      least = waves;
+      best = v[i];
+    }
+  }
+  return best;
+}
+
+template <int CC, int NT, int K>
+cudaError_t launch_cluster_nt(const SoftregArgs& a, int W, cudaStream_t s) {
+  const size_t smem = cluster_smem_bytes(a.D, a.C, a.B, NT);
+  cudaError_t e = cudaFuncSetAttribute(softreg_cluster_round_kernel<CC, NT, K>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t cfg = cluster_config<CC, NT, K>(&attr, W, smem, s);
+  return cudaLaunchKernelEx(&cfg, softreg_cluster_round_kernel<CC, NT, K>, a);
 }
 
 template <int CC>
 cudaError_t launch_cluster(const SoftregArgs& a, int W, cudaStream_t s) {
-  return cluster_threads(a.D, a.C, a.B) == kClSmall ? launch_cluster_nt<CC, kClSmall>(a, W, s)
-                                                    : launch_cluster_nt<CC, kClThreads>(a, W, s);
+  const ClVariant v = cluster_variant(a.D, a.C, a.B, W);
+  return v.NT == 512  ? launch_cluster_nt<CC, 512, 1>(a, W, s)
+         : v.NT == 256 ? launch_cluster_nt<CC, 256, 2>(a, W, s)
+         : v.K == 2    ? launch_cluster_nt<CC, 128, 2>(a, W, s)
+                       : launch_cluster_nt<CC, 128, 4>(a, W, s);
 }
 }  // namespace
 
 bool softreg_cluster_supported(int D, int C, int B) {
-  return B <= kSoftregMaxBatch && cluster_smem_bytes(D, C, B) <= 220 * 1024;
+  return B <= kSoftregMaxBatch && cluster_smem_bytes(D, C, B, cluster_threads_alone(D, C, B)) <= 220 * 1024;
 }
 
 cudaError_t launch_softreg_cluster_round(const SoftregArgs& a, int W, cudaStream_t s) {

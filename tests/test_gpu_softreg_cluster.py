@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 import torch
 
-import synth
+import paper_2102_08550_gb300 as P
 from tests.test_zz_no_alloc import call, check, oracle_steps
 
 pytestmark = pytest.mark.gpu
@@ -48,3 +48,64 @@ def test_cluster_steps_match_oracle(cuda_device, D, C, B, n, tau):
     again = torch.empty_like(out)
     call(p, again, xd, yd, n, cursor, tau, D, C, B, 0.05, loss)
     torch.testing.assert_close(again, out, rtol=0, atol=0)   # fixed summation order
+
+
+def _shared_shard(D, C, B, n=300):
+    rng = np.random.default_rng(D * 1000 + C * 10 + B)
+    X = rng.standard_normal((n, D)).astype(np.float32)
+    y = rng.integers(0, C, n).astype(np.int32)
+    flat = np.concatenate([rng.uniform(-1, 1, C * D) / np.sqrt(D), rng.uniform(-0.1, 0.1, C)]).astype(np.float32)
+    return X, y, flat
+
+
+def _context(D, C, B, W, X, y, flat, dev, tau):
+    xd, yd = torch.from_numpy(X).to(dev), torch.from_numpy(y).to(dev)
+    ctx = P.OscarsContext(num_workers=W, dims=[D, C], batch=B, lr=0.05, bf16=False, shards=[(xd, yd)] * W, M=8,
+                          init_params=torch.from_numpy(flat).to(dev), t_ticks=[1] * W,
+                          stream=torch.cuda.current_stream().cuda_stream)
+    ctx.set_local_steps(tau)
+    return ctx
+
+
+# 512, 256 and 128 threads a CTA, and more workers than any of them runs at once
+@pytest.mark.parametrize("D,C,B", [(784, 10, 8), (333, 26, 100), (60, 25, 65), (16, 2, 1), (40, 32, 33)])
+@pytest.mark.parametrize("W", [3, 17, 40, 150])
+def test_cluster_round_workers_share_sms(cuda_device, D, C, B, W):
+    X, y, flat = _shared_shard(D, C, B)
+    tau = [1 + k % 3 for k in range(W)]
+    ctx = _context(D, C, B, W, X, y, flat, cuda_device, tau)
+    _, losses = ctx.local_steps()
+    got = torch.empty(W, flat.size, device=cuda_device)
+    for k in range(W):
+        ctx.read_replica(k, got[k])
+    torch.cuda.synchronize()
+    ctx.close()
+    for t in range(1, 4):
+        ref, ref_loss = oracle_steps(flat, X, y, 0, t, D, C, B, 0.05)
+        check(got[t - 1].cpu().numpy(), losses[t - 1], ref, ref_loss, C, D)
+        for k in range(t - 1, W, 3):
+            assert torch.equal(got[k], got[t - 1]) and losses[k] == losses[t - 1]
+
+
+@pytest.mark.parametrize("D,C,B", [(784, 10, 8), (64, 10, 64), (1500, 3, 16)])
+def test_thirty_workers_take_one_wave(cuda_device, D, C, B):
+    """30 workers run side by side: far less than the two waves (2.0 to 2.4
+    times one worker's round) of one CTA an SM; 1.1 to 1.5 when they share SMs."""
+    X, y, flat = _shared_shard(D, C, B)
+
+    def us(W):
+        ctx = _context(D, C, B, W, X, y, flat, cuda_device, [8] * W)
+        best = float("inf")
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(10):
+                ctx.local_steps(want_loss=False)
+                ctx.push_merge()
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 100)
+        ctx.close()
+        return best
+
+    assert us(30) < 1.8 * us(1)
