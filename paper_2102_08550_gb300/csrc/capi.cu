@@ -13,6 +13,7 @@
 // Inside a slot every W_l and b_l starts on a 64-element boundary; the
 // padding stays zero.
 #include <algorithm>
+#include <atomic>
 #include <limits>
 #include <cstdio>
 #include <cstring>
@@ -42,16 +43,36 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
+  static std::atomic<EncodeTiledFn> fn{nullptr};
+  if (!fn.load(std::memory_order_relaxed)) {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
             cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
+      fn.store(reinterpret_cast<EncodeTiledFn>(p), std::memory_order_relaxed);
   }
-  return fn;
+  return fn.load(std::memory_order_relaxed);
+}
+
+// One tensor map.  A host thread that has made no CUDA call yet has no context
+// bound, which the driver's encoder wants (the runtime's calls bind it
+// themselves): bind the device's primary one then.
+bool encode_map(CUtensorMap* m, CUtensorMapDataType type, uint32_t rank, const void* base, const cuuint64_t* dims,
+                const cuuint64_t* strides, const cuuint32_t* box, CUtensorMapSwizzle swz) {
+  EncodeTiledFn f = encode_fn();
+  if (!f) return false;
+  const cuuint32_t es[4] = {1, 1, 1, 1};
+  auto encode = [&] {
+    return f(m, type, rank, const_cast<void*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  CUresult r = encode();
+  if (r == CUDA_ERROR_INVALID_CONTEXT || r == CUDA_ERROR_NOT_INITIALIZED) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess) r = encode();
+  }
+  return r == CUDA_SUCCESS;
 }
 
 // 3-D bf16 tensor map: element (x, y, z) at base + z*stride_z + y*stride_y +
@@ -59,58 +80,38 @@ EncodeTiledFn encode_fn() {
 // outside the extents.
 bool make_map(CUtensorMap* m, const void* base, uint64_t dx, uint64_t dy, uint64_t dz, uint64_t stride_y,
               uint64_t stride_z, uint32_t box_y) {
-  EncodeTiledFn f = encode_fn();
-  if (!f) return false;
   cuuint64_t dims[3] = {dx, dy, dz};
   cuuint64_t strides[2] = {stride_y, stride_z};
   cuuint32_t box[3] = {64, box_y, 1};
-  cuuint32_t es[3] = {1, 1, 1};
-  return f(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return encode_map(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 // 4-D bf16 tensor map, boxes of 64 x box_y x 1 x 1, 128-byte swizzle
 bool make_map4(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t d3, uint64_t s1,
                uint64_t s2, uint64_t s3, uint32_t box_y) {
-  EncodeTiledFn f = encode_fn();
-  if (!f) return false;
   cuuint64_t dims[4] = {d0, d1, d2, d3};
   cuuint64_t strides[3] = {s1, s2, s3};
   cuuint32_t box[4] = {64, box_y, 1, 1};
-  cuuint32_t es[4] = {1, 1, 1, 1};
-  return f(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return encode_map(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 // 4-D bf16 tensor map with an explicit box, 128-byte swizzle, zero fill
 bool make_map_box4(CUtensorMap* m, const void* base, const uint64_t (&d)[4], const uint64_t (&st)[3],
                    const uint32_t (&box)[4]) {
-  EncodeTiledFn f = encode_fn();
-  if (!f) return false;
   cuuint64_t dims[4] = {d[0], d[1], d[2], d[3]};
   cuuint64_t strides[3] = {st[0], st[1], st[2]};
   cuuint32_t bx[4] = {box[0], box[1], box[2], box[3]};
-  cuuint32_t es[4] = {1, 1, 1, 1};
-  return f(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, bx, es,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return encode_map(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, bx, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 // 3-D fp32 tensor map, boxes of 32 x box_y x 1 (128-byte rows), 128-byte swizzle
 bool make_map_f32(CUtensorMap* m, const void* base, uint64_t dx, uint64_t dy, uint64_t dz, uint64_t stride_y,
                   uint64_t stride_z, uint32_t box_y, uint32_t box_x = 32,
                   CUtensorMapSwizzle swz = CU_TENSOR_MAP_SWIZZLE_128B) {
-  EncodeTiledFn f = encode_fn();
-  if (!f) return false;
   cuuint64_t dims[3] = {dx, dy, dz};
   cuuint64_t strides[2] = {stride_y, stride_z};
   cuuint32_t box[3] = {box_x, box_y, 1};
-  cuuint32_t es[3] = {1, 1, 1};
-  return f(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, es,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return encode_map(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, swz);
 }
 
 struct Layer {
