@@ -897,11 +897,11 @@ cudaError_t launch_conv_igemm(int mode, const CUtensorMap& mIn, const CUtensorMa
                               const ConvArgs& a, int n_active, int cpw, cudaStream_t s) {
   const dim3 grid(cpw, n_active);
   if (mode == 0) {
-    cudaError_t e = cudaFuncSetAttribute(conv_igemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGSmem);
+    cudaError_t e = allow_smem(conv_igemm_kernel<0>, kGSmem);
     if (e != cudaSuccess) return e;
     conv_igemm_kernel<0><<<grid, kGT, kGSmem, s>>>(mIn, mW, mm, a);
   } else {
-    cudaError_t e = cudaFuncSetAttribute(conv_igemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGSmem);
+    cudaError_t e = allow_smem(conv_igemm_kernel<1>, kGSmem);
     if (e != cudaSuccess) return e;
     conv_igemm_kernel<1><<<grid, kGT, kGSmem, s>>>(mIn, mW, mm, a);
   }
@@ -916,7 +916,7 @@ int conv_wgrad_chunks(int B, int n_active, int sms) {
 
 cudaError_t launch_conv_wgrad(const CUtensorMap& mIn, const CUtensorMap& mDz, const WgradArgs& a, int n_active,
                               cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(conv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem2);
+  cudaError_t e = allow_smem(conv_wgrad_kernel, kWSmem2);
   if (e != cudaSuccess) return e;
   conv_wgrad_kernel<<<dim3(a.n_chunks, n_active), kWT, kWSmem2, s>>>(mIn, mDz, a);
   return cudaGetLastError();
@@ -944,7 +944,7 @@ static size_t cnn_head_smem(int B, int K) {
 
 cudaError_t launch_cnn_head(const CnnHeadArgs& a, int n_active, cudaStream_t s) {
   const size_t smem = cnn_head_smem(a.B, a.K);
-  cudaError_t e = cudaFuncSetAttribute(cnn_head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(cnn_head_kernel, smem);
   if (e != cudaSuccess) return e;
   cnn_head_kernel<<<n_active, kHeadT, smem, s>>>(a);
   return cudaGetLastError();
@@ -953,8 +953,7 @@ cudaError_t launch_cnn_head(const CnnHeadArgs& a, int n_active, cudaStream_t s) 
 cudaError_t launch_cnn_head_loss(const float* pool_part, const int32_t* labels, int lanes, int B, int64_t n_img, int K,
                                  const float* master, int64_t offWf, int64_t offBf, float* out, cudaStream_t s) {
   const size_t smem = sizeof(float) * (static_cast<size_t>(B) * kGld + K * kCC);
-  cudaError_t e = cudaFuncSetAttribute(cnn_head_loss_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(cnn_head_loss_kernel, smem);
   if (e != cudaSuccess) return e;
   cnn_head_loss_kernel<<<lanes, 256, smem, s>>>(pool_part, labels, B, n_img, K, master, offWf, offBf, out);
   return cudaGetLastError();

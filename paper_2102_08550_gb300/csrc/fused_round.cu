@@ -1116,8 +1116,7 @@ template <int B, int S>
 cudaError_t launch_bs(const CUtensorMap& mX, const CUtensorMap& mXT, const CUtensorMap& mW0f, const CUtensorMap& mRep32,
                       const CUtensorMap& mRep16, const FusedArgs& a, int priority, cudaStream_t s) {
   using Cfg = FCfg<B, S>;
-  cudaError_t e = cudaFuncSetAttribute(fused_mlp2_round_kernel<B, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       Cfg::kSmem);
+  cudaError_t e = allow_smem(fused_mlp2_round_kernel<B, S>, Cfg::kSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.n_clusters, S * (a.H / kFU), 1);
@@ -1171,9 +1170,7 @@ namespace {
 template <int B, int S>
 int max_clusters_bs(int H) {
   using Cfg = FCfg<B, S>;
-  if (cudaFuncSetAttribute(fused_mlp2_round_kernel<B, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem) !=
-      cudaSuccess)
-    return 0;
+  if (allow_smem(fused_mlp2_round_kernel<B, S>, Cfg::kSmem) != cudaSuccess) return 0;
   cudaLaunchConfig_t cfg = {};
   const int ncl = S * (H / kFU);
   cfg.gridDim = dim3(1, ncl, 1);

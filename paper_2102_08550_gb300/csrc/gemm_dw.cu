@@ -290,7 +290,7 @@ cudaError_t launch_gemm_dw(const DwMaps& maps, DwArgs a, int sms, cudaStream_t s
     if (ly.M % kDwTile != 0 || ly.N % 8 != 0) return cudaErrorInvalidValue;
     a.first_tile[l + 1] = a.first_tile[l] + a.n_active * (ly.M / kDwTile) * ((ly.N + kDwTile - 1) / kDwTile);
   }
-  cudaError_t e = cudaFuncSetAttribute(gemm_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDwSmem);
+  cudaError_t e = allow_smem(gemm_dw_kernel, kDwSmem);
   if (e != cudaSuccess) return e;
   const int tiles = a.first_tile[a.n_layers];
   cudaLaunchConfig_t cfg = {};

@@ -50,7 +50,8 @@ constexpr int kRMaxStages = 8;
 constexpr int kRStg = 4096;                       // one staging box: 32 rows x 128 bytes
 constexpr int kRStgBytes = 4 * 2 * kRStg;         // two per epilogue warp
 constexpr int kRBarBytes = 256;
-constexpr int kRRing = 227 * 1024 - 1024 - kRBarBytes - kRStgBytes;
+constexpr int kRSmem = 227 * 1024;                // at most
+constexpr int kRRing = kRSmem - 1024 - kRBarBytes - kRStgBytes;
 
 struct RowsBars {
   uint64_t full[kRMaxStages], empty[kRMaxStages], accf[2], acce[2];
@@ -385,8 +386,7 @@ void device_room(int& sms, int& pairs) {
   cudaLaunchAttribute attr[1];
   const size_t smem = rows_smem(rows_stages(kRMaxBN, 64, 2), kRMaxBN, 2);
   pairs = 0;
-  if (cudaFuncSetAttribute(gemm_rows_kernel<kRowsStore, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(smem)) == cudaSuccess) {
+  if (allow_smem(gemm_rows_kernel<kRowsStore, 2>, kRSmem) == cudaSuccess) {
     cudaLaunchConfig_t cfg = rows_config<kRowsStore, 2>(attr, 2, smem, nullptr);
     if (cudaOccupancyMaxActiveClusters(&pairs, gemm_rows_kernel<kRowsStore, 2>, &cfg) != cudaSuccess) pairs = 0;
   }
@@ -410,8 +410,7 @@ template <int EPI, int CL>
 cudaError_t launch_rows_t(const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mD, const RowsArgs& a,
                           int grid, cudaStream_t s) {
   const size_t smem = rows_smem(a.stages, a.BN, CL);
-  cudaError_t e = cudaFuncSetAttribute(gemm_rows_kernel<EPI, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(gemm_rows_kernel<EPI, CL>, kRSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = rows_config<EPI, CL>(attr, grid, smem, s);

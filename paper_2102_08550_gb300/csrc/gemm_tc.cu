@@ -512,8 +512,7 @@ cudaError_t launch_tile(const GemmMaps& m, const GemmArgs& a, int n_active, cuda
   size_t smem = 1024 + static_cast<size_t>(stages) * Cfg::kStageBytes + kBarrierBytes + red_bytes;
   const size_t floor_b = smem_floor_for_tmem(Cfg::kTmemCols);
   if (smem < floor_b) smem = floor_b;
-  cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, SPLIT, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(gemm_tc_kernel<BN, EPI, SPLIT, TT>, smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;

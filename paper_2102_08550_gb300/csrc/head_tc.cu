@@ -567,7 +567,7 @@ template <int NH, int NC, int CT>
 cudaError_t launch_head_tc_nh(const CUtensorMap& mH, const CUtensorMap& mW2, const CUtensorMap& mGT,
                               const HeadArgs& a, int n_active, cudaStream_t s) {
   using Cfg = HTCfg<NH, NC>;
-  cudaError_t e = cudaFuncSetAttribute(head_tc_kernel<NH, NC, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem);
+  cudaError_t e = allow_smem(head_tc_kernel<NH, NC, CT>, Cfg::kSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_active, a.H / Cfg::F, 1);

@@ -8,6 +8,18 @@
 
 namespace oscars {
 
+// Lets `kernel` take `bytes` of dynamic shared memory.  The limit belongs to the
+// kernel in the process, not to a launch: set to each launch's own size, a host
+// thread could lower it between another one's setting and its launch, which then
+// fails.  So every launch sets the same limit, all of an SM's shared memory but
+// room for static variables (only kernels that always pass one constant take more).
+constexpr size_t kSmemLimit = 225 * 1024;
+template <typename F>
+cudaError_t allow_smem(F* kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(bytes > kSmemLimit ? bytes : kSmemLimit));
+}
+
 constexpr int kMaxMergeWorkers = 256;   // pointer table of the merge kernel
 constexpr int kMaxWorkersMLP = 64;
 constexpr int kMaxClasses = 32;

@@ -747,8 +747,7 @@ cudaError_t launch_stage_round(const StageArgs& a, const int32_t* tau, int W, in
 cudaError_t launch_head_fwd(const HeadArgs& a, int n_active, cudaStream_t s) {
   if (a.H % 8 != 0 || a.H > 32 * 8 * kHeadMaxH8) return cudaErrorInvalidValue;
   const size_t smem = sizeof(float) * static_cast<size_t>(a.C) * a.H;
-  cudaError_t e = cudaFuncSetAttribute(head_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(head_fwd_kernel, smem);
   if (e != cudaSuccess) return e;
   dim3 grid(n_active, a.B / kRowsPerLossChunk);
   head_fwd_kernel<<<grid, kHeadFwdThreads, smem, s>>>(a);
@@ -758,8 +757,7 @@ cudaError_t launch_head_fwd(const HeadArgs& a, int n_active, cudaStream_t s) {
 cudaError_t launch_head_bwd(const HeadArgs& a, int n_active, cudaStream_t s) {
   if (a.B % (8 * kHBGroups) != 0 || a.H % 8 != 0) return cudaErrorInvalidValue;
   const size_t smem = head_bwd_smem(a.B, a.C);
-  cudaError_t e = cudaFuncSetAttribute(head_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(head_bwd_kernel, smem);
   if (e != cudaSuccess) return e;
   dim3 grid(n_active, (a.H + kHB - 1) / kHB);
   head_bwd_kernel<<<grid, kHeadBwdThreads, smem, s>>>(a);
@@ -774,8 +772,7 @@ bool head_fused_supported(int H, int B, int C) {
 cudaError_t launch_head_fused(const HeadArgs& a, int n_active, cudaStream_t s) {
   if (!head_fused_supported(a.H, a.B, a.C)) return cudaErrorInvalidValue;
   const size_t smem = head_fused_smem(a.B, a.C);
-  cudaError_t e = cudaFuncSetAttribute(head_fused_kernel<kHFClasses>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(head_fused_kernel<kHFClasses>, smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_active, a.H / kHF, 1);

@@ -788,8 +788,7 @@ size_t softreg_smem_bytes(int D, int C, int B) {
 
 cudaError_t launch_softreg_round(const SoftregArgs& a, int W, cudaStream_t s) {
   const size_t smem = softreg_smem_bytes(a.D, a.C, a.B);
-  cudaError_t e = cudaFuncSetAttribute(softreg_round_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(softreg_round_kernel, smem);
   if (e != cudaSuccess) return e;
   softreg_round_kernel<<<W, kThreads, smem, s>>>(a);
   return cudaGetLastError();
@@ -890,8 +889,7 @@ ClVariant cluster_variant(int D, int C, int B, int W) {
 template <int CC, int NT, int K>
 cudaError_t launch_cluster_nt(const SoftregArgs& a, int W, cudaStream_t s) {
   const size_t smem = cluster_smem_bytes(a.D, a.C, a.B, NT);
-  cudaError_t e = cudaFuncSetAttribute(softreg_cluster_round_kernel<CC, NT, K>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(softreg_cluster_round_kernel<CC, NT, K>, smem);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr;
   const cudaLaunchConfig_t cfg = cluster_config<CC, NT, K>(&attr, W, smem, s);
@@ -931,8 +929,7 @@ namespace {
 template <int CC, int G>
 cudaError_t launch_eval(const SoftregEvalArgs& a, int blocks, cudaStream_t s) {
   const size_t smem = sizeof(float) * a.C * static_cast<size_t>(a.D);
-  cudaError_t e = cudaFuncSetAttribute(softreg_eval_kernel<CC, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(softreg_eval_kernel<CC, G>, smem);
   if (e != cudaSuccess) return e;
   softreg_eval_kernel<CC, G><<<blocks, kEvalThreads, smem, s>>>(a);
   return cudaGetLastError();

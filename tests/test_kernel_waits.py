@@ -6,7 +6,9 @@ missing one shows only as a fault or a hang, and only now and then, on a GPU).
   the first remote load, store or arrival.
 * A warp that runs a loop together and elects a lane to issue (elect.sync with a
   full mask) must stay together: such a loop is not left on a wait, which may run
-  out in some lanes and not in the others."""
+  out in some lanes and not in the others.
+
+Beside them, what a launch must not set by its own size."""
 import os
 import re
 
@@ -135,3 +137,11 @@ def test_a_lane_wise_wait_is_caught():
     assert lanes_that_leave_alone(kernel % ("", "if (!(ok = mbar_wait(b, i))) break")) == ["k"]
     assert lanes_that_leave_alone(kernel % ("ok && ", "ok = mbar_wait(b, i)")) == ["k"]
     assert lanes_that_leave_alone(kernel % ("", "mbar_wait_keep(ok, b, i)")) == []
+
+
+def test_shared_memory_limits_do_not_depend_on_a_launch():
+    """The limit on dynamic shared memory is the kernel's, in the whole process: a launch that set it to its
+    own size could lower it under another thread's.  It is set in one place, to one value."""
+    sets = {f: len(re.findall(r"cudaFuncAttributeMaxDynamicSharedMemorySize", _clean(_read(f))))
+            for f in sorted(os.listdir(CSRC)) if f.endswith((".cu", ".h", ".cuh"))}
+    assert {f for f, n in sets.items() if n} == {"internal.h"} and sets["internal.h"] == 1
