@@ -208,6 +208,7 @@ struct FCfg {
   static constexpr int oBar = (oLab + B * 4 + 15) / 16 * 16;
   static constexpr int kBarBytes = 256;
   static constexpr int kSmem = oBar + kBarBytes + 1024;      // + alignment slack
+  static_assert(no_cluster_beside(kSmem), "all of the tensor memory: no other cluster's CTA beside one");
   static_assert(S == 1 || kUPC * kZs * 4 <= kHsBytes, "the incoming partials must fit the h tile they alias");
   static_assert(S == 1 || kZBytes <= kFRing, "own partials must fit the F ring");
 };

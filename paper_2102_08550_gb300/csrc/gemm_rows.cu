@@ -345,10 +345,13 @@ struct DevInfo {
 };
 DevInfo g_dev[kMaxDevices];
 
-// at least 120 KB: one CTA per SM, so that a tcgen05.alloc of all 512 columns never waits
+// at least 164 KB: one CTA per SM and none of another kernel's clusters beside it,
+// so that a tcgen05.alloc of all 512 columns never waits for one
+constexpr size_t kRLeastSmem = 164 * 1024;
+static_assert(no_cluster_beside(kRLeastSmem), "the pair's CTAs meet no other cluster's");
 size_t rows_smem(int stages, int BN, int cl) {
   const size_t b = 1024 + kRStgBytes + static_cast<size_t>(stages) * (kRABytes + BN / cl * 128) + kRBarBytes;
-  return b < 120 * 1024 ? 120 * 1024 : b;
+  return b < kRLeastSmem ? kRLeastSmem : b;
 }
 int rows_stages(int BN, int nk, int cl) {
   int st = kRRing / (kRABytes + BN / cl * 128);

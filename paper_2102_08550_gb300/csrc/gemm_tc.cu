@@ -508,6 +508,8 @@ cudaError_t launch_tile(const GemmMaps& m, const GemmArgs& a, int n_active, cuda
   const int budget = SPLIT > 1 ? 150 * 1024 : ctas > sms ? 100 * 1024 : 200 * 1024;
   const int max_stages = budget / Cfg::kStageBytes;
   int stages = nk < max_stages ? nk : (max_stages < 8 ? max_stages : 8);
+  static_assert(SPLIT == 1 || (4 * Cfg::kStageBytes >= kLeastClusterSmem && 4 * Cfg::kStageBytes <= 150 * 1024),
+                "at least 4 K-blocks a CTA (split_for), so 4 stages: see kLeastClusterSmem");
   if (stages < 2) stages = nk < 2 ? nk : 2;
   size_t smem = 1024 + static_cast<size_t>(stages) * Cfg::kStageBytes + kBarrierBytes + red_bytes;
   const size_t floor_b = smem_floor_for_tmem(Cfg::kTmemCols);

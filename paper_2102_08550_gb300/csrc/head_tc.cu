@@ -80,6 +80,7 @@ struct HTCfg {
   static constexpr int oBar = oB2 + NC * 4;            // tma, mma barriers, TMEM slot
   static constexpr int kSmem = oBar + 64 + 1024;
   static constexpr uint32_t kTmemCols = 128 * NH;
+  static_assert(kSmem >= kLeastClusterSmem, "a kernel on clusters with tensor memory");
 };
 
 // element (row b, feature f) of the h tile (K-major, 128-byte swizzle, one box per 64 features)

@@ -20,6 +20,17 @@ cudaError_t allow_smem(F* kernel, size_t bytes) {
                               static_cast<int>(bytes > kSmemLimit ? bytes : kSmemLimit));
 }
 
+// Two kernels on clusters that together want more than an SM's tensor memory must
+// not meet on an SM: a tcgen05.alloc waits without a limit, and two clusters of
+// different streams, each with one CTA that has its columns and one that waits
+// for the other's, would wait for ever.  Every kernel on clusters that allocates
+// tensor memory takes at least kLeastClusterSmem of dynamic shared memory, and one
+// that allocates all of it leaves less on its SM.  (The others wait for nobody, so
+// a wait for their columns ends.)
+constexpr size_t kLeastClusterSmem = 64 * 1024;
+constexpr size_t kSmSmem = 228 * 1024, kCtaSmem = 1024;   // shared memory of an SM; taken by each CTA beside its own
+constexpr bool no_cluster_beside(size_t smem) { return smem + kCtaSmem + kLeastClusterSmem + kCtaSmem > kSmSmem; }
+
 constexpr int kMaxMergeWorkers = 256;   // pointer table of the merge kernel
 constexpr int kMaxWorkersMLP = 64;
 constexpr int kMaxClasses = 32;

@@ -824,7 +824,6 @@ cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, int W, size_t smem,
 // Clusters that run at once with k CTAs an SM, k <= 4 (not k SMs / 8: the SMs of
 // a cluster share a processor cluster).  Queried once per device.
 constexpr int kMaxDevices = 64;
-constexpr size_t kSmSmem = 228 * 1024, kCtaSmem = 1024;   // shared memory of an SM; taken by each CTA beside its own
 std::atomic<int> g_room[kMaxDevices][4];
 template <int NT, int K>
 int query_room(size_t smem) {
