@@ -177,18 +177,19 @@ __global__ void __launch_bounds__(kGT, 1) conv_igemm_kernel(const __grid_constan
     }
   } else if (warp == 1) {   // converged, one elected lane issues: see elect_one
     constexpr uint32_t idesc = idesc_bf16_f32(128, kCC), idesc3 = idesc_bf16_f32(128, 3 * kCC);
-    bool ok = mbar_wait(wfull, 0, a.err, kDevTimeoutFull);
+    uint32_t limit = kSpinLimit;
+    mbar_wait_keep(limit, wfull, 0, a.err, kDevTimeoutFull);
     tc_fence_after();
     const uint64_t wb = smem_desc_k128(smem_u32(wts));
     for (int k = 0; k < my_tiles; ++k) {
       const int buf = k & 1, use = k >> 1, sl = k % kGSlots;
-      if (use >= 1) mbar_wait_keep(ok, &acce[buf], (use - 1) & 1, a.err, kDevTimeoutAccum);
-      mbar_wait_keep(ok, &full[sl], (k / kGSlots) & 1, a.err, kDevTimeoutFull);
+      if (use >= 1) mbar_wait_keep(limit, &acce[buf], (use - 1) & 1, a.err, kDevTimeoutAccum);
+      mbar_wait_keep(limit, &full[sl], (k / kGSlots) & 1, a.err, kDevTimeoutFull);
       tc_fence_after();
       // descriptors count 16 bytes: 2 for the 32 bytes of a K slice
       const uint64_t sa = smem_desc_k128(smem_u32(slots + sl * kGBox));
       const uint32_t acc = tmem + buf * kGAcc;
-      if (elect_one() && ok) {
+      if (elect_one() && limit > 1) {
         if (one_tap) {
 #pragma unroll
           for (int j = 0; j < kCC / 16; ++j) umma_bf16(acc, sa + 2 * j, wb + 2 * j, idesc, j != 0 ? 1u : 0u);
@@ -444,14 +445,14 @@ __global__ void __launch_bounds__(kWT, 1) conv_wgrad_kernel(const __grid_constan
     }
   } else if (warp == 1) {   // converged, one elected lane issues: see elect_one
     constexpr uint32_t idesc1 = idesc_bf16_f32_mn(128, kCC), idesc3 = idesc_bf16_f32_mn(128, 3 * kCC);
-    bool ok = true;
+    uint32_t limit = kSpinLimit;
     for (int kb = 0; kb < nk; ++kb) {
       const int st = kb % kWStages2;
-      mbar_wait_keep(ok, &full[st], (kb / kWStages2) & 1, a.err, kDevTimeoutFull);
+      mbar_wait_keep(limit, &full[st], (kb / kWStages2) & 1, a.err, kDevTimeoutFull);
       tc_fence_after();
       const uint32_t sa = smem_u32(sm + st * kWStage2);
       const uint64_t ad = smem_desc_mn128(sa, kWRow), bd = smem_desc_mn128(sa + kWBox, kWTile);
-      if (elect_one() && ok) {
+      if (elect_one() && limit > 1) {
         // K = 16 pixels per MMA: two 8-row groups, 2048 bytes (descriptors count 16)
         if (a.im2col) {   // A's upper atom (the next row) is not read back
 #pragma unroll

@@ -75,12 +75,22 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
 // A converged warp that issues through an elected lane (elect_one), or reads
 // tensor memory, must stay together even when a wait runs out, and it may run
 // out in some lanes only.  A loop that elects a lane is therefore never left on
-// a wait: a lane whose wait ran out goes through the rest of it without waiting
-// (mbar_wait_keep), and the elected lane issues nothing any more once its own
-// has.  A branch around a warp-wide instruction takes one answer for all lanes
-// (mbar_wait_warp; in the loops its vote cost 1 to 2% of a round).
-__device__ __forceinline__ void mbar_wait_keep(bool& ok, uint64_t* bar, uint32_t parity, int* err, int code) {
-  if (ok) ok = mbar_wait(bar, parity, err, code);
+// a wait: a lane whose wait ran out sets its limit to 1 and goes through the rest
+// of the loop with one poll a wait, and the elected lane issues nothing any more
+// once its own has (limit > 1).  This costs nothing (128 x 8192 x 3072: 14.7 us, as
+// with a loop left lane by lane; 15.5 with a flag tested before each wait, 15.8
+// with a vote after it).  A branch around a warp-wide instruction takes one
+// answer for all lanes (mbar_wait_warp).
+__device__ __forceinline__ void mbar_wait_keep(uint32_t& limit, uint64_t* bar, uint32_t parity, int* err, int code) {
+  uint32_t i = 0;
+  while (!mbar_try_wait(bar, parity)) {
+    if (++i >= limit) {
+      limit = 1;
+      if (err) atomicCAS(err, 0, code);
+      break;
+    }
+    if (i > 64) __nanosleep(64);
+  }
 }
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err, int code) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, code));

@@ -484,10 +484,10 @@ __global__ void __launch_bounds__(kFT, 1) fused_mlp2_round_kernel(const __grid_c
         if (producer_ok) producer_ok = issue_d(s, 0, pre_d);     // the first X^T tiles of step D
       } else if (warp == 1) {   // converged, one elected lane issues: see elect_one
         constexpr uint32_t idesc = idesc_bf16_f32(128, B);
-        bool ok = true;
+        uint32_t limit = kSpinLimit;
         for (int kb = 0; kb < nkf; ++kb) {
           const int c = sg * nkf + kb, st = c % Cfg::kStagesF;
-          mbar_wait_keep(ok, &fullF[st], (c / Cfg::kStagesF) & 1, a.err, kDevTimeoutFull);
+          mbar_wait_keep(limit, &fullF[st], (c / Cfg::kStagesF) & 1, a.err, kDevTimeoutFull);
           tc_fence_after();
           const uint32_t wa = smem_u32(w0s + kb * kW0Blk);
           const uint32_t xb = smem_u32(fring + st * Cfg::kBBytes);
@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(kFT, 1) fused_mlp2_round_kernel(const __grid_c
           // operands) are not issued
           const int kleft = D - (kb_begin + kb) * kFBK;
           const uint64_t ad = smem_desc_k128(wa), bd = smem_desc_k128(xb);
-          if (elect_one() && ok) {
+          if (elect_one() && limit > 1) {
 #pragma unroll
             for (int j = 0; j < kFBK / 16; ++j)   // 32 bytes along K: 2 in the descriptor's address field
               if (j * 16 < kleft) umma_bf16(tmem + kTAcc, ad + 2 * j, bd + 2 * j, idesc, (kb | j) != 0 ? 1u : 0u);

@@ -167,26 +167,26 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
     // ---- MMA issuer: the warp converged, one elected lane issues (see elect_one)
     constexpr uint32_t idesc = idesc_bf16_f32(kDwTile, kDwTile);
     int kc = 0, it = 0;
-    bool ok = true;
+    uint32_t limit = kSpinLimit;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {
       const int b = it & 1;
-      if (it >= 2) mbar_wait_keep(ok, &bars->aempty[b], ((it >> 1) + 1) & 1, a.err, kDevTimeoutAccum);
+      if (it >= 2) mbar_wait_keep(limit, &bars->aempty[b], ((it >> 1) + 1) & 1, a.err, kDevTimeoutAccum);
       tc_fence_after();
       const uint32_t acc = tmem + static_cast<uint32_t>(b * kDwTile);
       for (int kb = 0; kb < nk; ++kb, ++kc) {
         const int s = kc & 1;
-        mbar_wait_keep(ok, &bars->full[s], (kc >> 1) & 1, a.err, kDevTimeoutFull);
+        mbar_wait_keep(limit, &bars->full[s], (kc >> 1) & 1, a.err, kDevTimeoutFull);
         tc_fence_after();
         const uint64_t ad = smem_desc_k128(smem_u32(sOps + s * kDwOpBytes));
         const uint64_t bd = smem_desc_k128(smem_u32(sOps + s * kDwOpBytes + kDwOpBytes / 2));
-        if (elect_one() && ok) {
+        if (elect_one() && limit > 1) {
 #pragma unroll
           for (int j = 0; j < kDwBK / 16; ++j) umma_bf16(acc, ad + 2 * j, bd + 2 * j, idesc, (kb | j) != 0 ? 1u : 0u);
           umma_commit(&bars->empty[s]);
         }
         __syncwarp();
       }
-      if (elect_one() && ok) umma_commit(&bars->afull[b]);
+      if (elect_one() && limit > 1) umma_commit(&bars->afull[b]);
       __syncwarp();
     }
     if (elect_one()) umma_commit(&bars->mma_done);   // every product issued above has landed before TMEM is released

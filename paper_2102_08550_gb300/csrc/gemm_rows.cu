@@ -190,18 +190,18 @@ __global__ void __launch_bounds__(kRThreads, 1) gemm_rows_kernel(const __grid_co
     const uint32_t idesc = idesc_bf16_f32(kRM * CL, a.BN);
     const uint32_t ring0 = smem_u32(ring);
     int s = 0, ph = 0, t = 0;
-    bool ok = true;
+    uint32_t limit = kSpinLimit;
     for (int u = u0; u < units; u += ustep, ++t) {
       const int b = t & 1;
-      if (t >= 2) mbar_wait_keep(ok, &bars->acce[b], ((t >> 1) + 1) & 1, a.err, kDevTimeoutAccum);
+      if (t >= 2) mbar_wait_keep(limit, &bars->acce[b], ((t >> 1) + 1) & 1, a.err, kDevTimeoutAccum);
       tc_fence_after();
       const uint32_t acc = tmem + static_cast<uint32_t>(b * kRMaxBN);
       for (int kb = 0; kb < nk; ++kb) {
-        mbar_wait_keep(ok, &bars->full[s], ph, a.err, kDevTimeoutFull);
+        mbar_wait_keep(limit, &bars->full[s], ph, a.err, kDevTimeoutFull);
         tc_fence_after();
         const uint64_t ad = smem_desc_k128(ring0 + s * stage_bytes);
         const uint64_t bd = smem_desc_k128(ring0 + s * stage_bytes + kRABytes);
-        if (elect_one() && ok) {
+        if (elect_one() && limit > 1) {
 #pragma unroll
           for (int j = 0; j < kRK / 16; ++j) {   // 32 bytes along K: 2 in the descriptor's address field
             if (CL > 1) umma_bf16_pair(acc, ad + 2 * j, bd + 2 * j, idesc, (kb | j) != 0 ? 1u : 0u);
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kRThreads, 1) gemm_rows_kernel(const __grid_co
           ph ^= 1;
         }
       }
-      if (elect_one() && ok) {
+      if (elect_one() && limit > 1) {
         if (CL > 1) umma_commit_pair(&bars->accf[b]);
         else umma_commit(&bars->accf[b]);
       }

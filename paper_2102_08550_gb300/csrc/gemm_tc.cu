@@ -248,10 +248,10 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
     // B MN-major (bit 16) when it is read from its transpose
     const bool bmn = a.b_mn;
     const uint32_t idesc = idesc_bf16_f32(BM, BN) | (EPI == kEpiDh ? (1u << 15) : 0u) | (bmn ? (1u << 16) : 0u);
-    bool ok = true;
+    uint32_t limit = kSpinLimit;
     for (int kb = 0; kb < nk; ++kb) {
       const int s = kb % stages;
-      mbar_wait_keep(ok, &full[s], (kb / stages) & 1, a.err, kDevTimeoutFull);
+      mbar_wait_keep(limit, &full[s], (kb / stages) & 1, a.err, kDevTimeoutFull);
       tc_fence_after();
       const uint32_t a_base = smem_u32(sA + s * kABytes);
       const uint32_t b_base = smem_u32(sB + s * Cfg::kBBytes);
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
       const uint64_t ad = EPI == kEpiDh ? smem_desc_mn128(a_base, kABytes / 2) : smem_desc_k128(a_base);
       const uint64_t bd = bmn ? smem_desc_mn128(b_base, 8192) : smem_desc_k128(b_base);
       const uint32_t astep = EPI == kEpiDh ? 128 : 2, bstep = bmn ? 128 : 2;
-      if (elect_one() && ok) {
+      if (elect_one() && limit > 1) {
 #pragma unroll
         for (int j = 0; j < BK / 16; ++j)
           umma_bf16(tmem, ad + j * astep, bd + j * bstep, idesc, (kb | j) != 0 ? 1u : 0u);

@@ -133,10 +133,10 @@ def test_issuing_warps_leave_their_loops_together(f):
 
 
 def test_a_lane_wise_wait_is_caught():
-    kernel = "__global__ void __launch_bounds__(32) k(int* p) {\n for (int i = 0; %si < 4; ++i) {\n %s;\n if (elect_one() && ok) { go(); }\n }\n}\n"
+    kernel = "__global__ void __launch_bounds__(32) k(int* p) {\n for (int i = 0; %si < 4; ++i) {\n %s;\n if (elect_one() && limit > 1) { go(); }\n }\n}\n"
     assert lanes_that_leave_alone(kernel % ("", "if (!(ok = mbar_wait(b, i))) break")) == ["k"]
     assert lanes_that_leave_alone(kernel % ("ok && ", "ok = mbar_wait(b, i)")) == ["k"]
-    assert lanes_that_leave_alone(kernel % ("", "mbar_wait_keep(ok, b, i)")) == []
+    assert lanes_that_leave_alone(kernel % ("", "mbar_wait_keep(limit, b, i)")) == []
 
 
 def test_shared_memory_limits_do_not_depend_on_a_launch():
