@@ -2222,8 +2222,9 @@ oscars_status oscars_gemm_bf16_nt(const void* A, const void* B, float* C, int32_
                                   void* stream) {
   if (!A || !B || !C || M < 128 || M % 128 != 0 || N < 1 || K < 8 || K % 8 != 0) return OSCARS_EINVAL;
   if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) return OSCARS_EINVAL;
-  const RowsPlan p = gemm_rows_plan(kRowsStore, M, N, K);
   const int tma = N % 4 == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
+  const RowsEpi epi = !tma && N <= 32 ? kRowsNarrow : kRowsStore;
+  const RowsPlan p = gemm_rows_plan(epi, M, N, K);
   CUtensorMap mA, mB, mC;
   if (!make_map(&mA, A, K, M, 1, K * 2ull, static_cast<uint64_t>(M) * K * 2ull, 128) ||
       !make_map(&mB, B, K, N, 1, K * 2ull, static_cast<uint64_t>(N) * K * 2ull, p.BN / p.cl))
@@ -2236,8 +2237,8 @@ oscars_status oscars_gemm_bf16_nt(const void* A, const void* B, float* C, int32_
   g.K = K;
   g.C = C;
   g.tma_store = tma;
-  return launch_gemm_rows(kRowsStore, p, mA, mB, mC, g, static_cast<cudaStream_t>(stream)) == cudaSuccess ? OSCARS_OK
-                                                                                                         : OSCARS_ECUDA;
+  return launch_gemm_rows(epi, p, mA, mB, mC, g, static_cast<cudaStream_t>(stream)) == cudaSuccess ? OSCARS_OK
+                                                                                                  : OSCARS_ECUDA;
 }
 
 int32_t oscars_phase_times(oscars_ctx* c, int32_t cap, double* us) {

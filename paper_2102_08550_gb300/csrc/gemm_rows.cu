@@ -4,6 +4,7 @@
 // held-out set), where m is a sample and all samples go in one launch.
 //
 //  kRowsStore  C[m][n] fp32 row-major
+//  kRowsNarrow the same for at most 32 columns whose rows are not 16-byte aligned
 //  kRowsRelu   out[m][n] = bf16(relu(D + bias[n])) row-major
 //  kRowsLoss   n = class: softmax cross-entropy of row m against its label,
 //              summed over the 32 rows of a warp into loss_part
@@ -128,7 +129,7 @@ __global__ void __launch_bounds__(kRThreads, 1) gemm_rows_kernel(const __grid_co
   if (threadIdx.x == 0) {
     prefetch_tmap(&mapA);
     prefetch_tmap(&mapB);
-    if (EPI != kRowsLoss) prefetch_tmap(&mapD);
+    if (EPI == kRowsStore || EPI == kRowsRelu) prefetch_tmap(&mapD);
     for (int i = 0; i < a.stages; ++i) {
       mbar_init(&bars->full[i], 1);
       mbar_init(&bars->empty[i], 1);
@@ -266,6 +267,13 @@ __global__ void __launch_bounds__(kRThreads, 1) gemm_rows_kernel(const __grid_co
           }
           ++nst;
         }
+      } else if constexpr (EPI == kRowsNarrow) {   // a thread's row as it is (staged as above it took a warp 32 turns)
+        float v[32];
+        tmem_ld_32x32b_x32(row, v);
+        float* out = a.C + static_cast<int64_t>(m0 + lane) * a.N;
+#pragma unroll
+        for (int c = 0; c < 32; ++c)
+          if (c < a.N && m0 + lane < a.M) out[c] = v[c];
       } else if constexpr (EPI == kRowsRelu) {
         for (int c0 = 0; c0 < a.BN && n0 + c0 < a.N; c0 += 64) {   // BN and N are multiples of 64
           float v0[32], v1[32];
@@ -401,12 +409,17 @@ void device_room(int& sms, int& pairs) {
 
 // relative time of a launch with tiles of BN columns: waves x the longer of a
 // k-block's products (BN cycles) and loads (bytes at 60 a cycle), plus a
-// tile's fixed part
+// tile's fixed part, plus what a launch on clusters takes longer (start and end
+// barriers, both SMs' tensor memory): 1500 cycles, so that products of few
+// K-blocks run on CTAs alone.  Device time of a launch, one 128 x BN tile a CTA
+// without clusters before this kernel / pairs wherever the row tiles are even /
+// this rule, us: 1024 x 1 x 64: 3.0 / 4.5 / 2.8; 4096 x 64 x 64: 3.8 / 4.2 / 3.2;
+// 1024 x 1 x 784: 7.4 / 8.4 / 7.1; 1024 x 1000 x 784: 9.9 / 8.5 / 7.4.
 double rows_cost(int mt, int N, int nk, int BN, int CL, int room) {
   const int units = mt / CL * ((N + BN - 1) / BN);
   const int waves = (units + room - 1) / room;
   const double load = (kRABytes + BN * 128.0 / CL) / 60.0, mma = BN;
-  return waves * (nk * (load > mma ? load : mma) + 4.0 * BN + 600.0);
+  return waves * (nk * (load > mma ? load : mma) + 4.0 * BN + 600.0) + (CL > 1 ? 1500.0 : 0.0);
 }
 
 template <int EPI, int CL>
@@ -464,6 +477,8 @@ cudaError_t launch_gemm_rows(int epi, const RowsPlan& p, const CUtensorMap& mA, 
   const int grid = static_cast<int>(units < room ? units : room) * p.cl;
   if (epi == kRowsStore)
     return p.cl == 2 ? launch_rows_t<kRowsStore, 2>(mA, mB, mD, a, grid, s) : launch_rows_t<kRowsStore, 1>(mA, mB, mD, a, grid, s);
+  if (epi == kRowsNarrow)
+    return p.cl == 2 ? launch_rows_t<kRowsNarrow, 2>(mA, mB, mD, a, grid, s) : launch_rows_t<kRowsNarrow, 1>(mA, mB, mD, a, grid, s);
   if (epi == kRowsRelu)
     return p.cl == 2 ? launch_rows_t<kRowsRelu, 2>(mA, mB, mD, a, grid, s) : launch_rows_t<kRowsRelu, 1>(mA, mB, mD, a, grid, s);
   return launch_rows_t<kRowsLoss, 1>(mA, mB, mD, a, grid, s);

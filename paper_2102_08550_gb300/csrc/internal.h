@@ -190,14 +190,14 @@ struct GemmMaps {
 cudaError_t launch_gemm(int epi, const GemmMaps& m, const GemmArgs& a, int n_active, cudaStream_t s);
 
 // One large product D[m][n] = sum_k A[m][k] B[n][k] (csrc/gemm_rows.cu).
-enum RowsEpi { kRowsStore = 0, kRowsRelu = 1, kRowsLoss = 2 };
+enum RowsEpi { kRowsStore = 0, kRowsRelu = 1, kRowsLoss = 2, kRowsNarrow = 3 };
 struct RowsPlan {
   int BN, cl;              // columns per tile, CTAs per tile (row tiles of 128 each)
 };
 struct RowsArgs {
   int M, N, K;
   int BN, stages, mt, nt;  // set by the launcher
-  float* C;                // kRowsStore: [M][N] (when tma_store is 0)
+  float* C;                // kRowsStore (when tma_store is 0), kRowsNarrow: [M][N]
   int tma_store;           // kRowsStore: 1 = through mD (N % 4 == 0 and C 16-byte aligned)
   const float* bias;       // kRowsRelu, kRowsLoss: [N]
   const int32_t* labels;   // kRowsLoss: [M]
@@ -205,7 +205,7 @@ struct RowsArgs {
   int* err;
   int pdl;                 // launch as a programmatic dependent of the previous kernel on the stream
 };
-// kRowsRelu: N a multiple of 64, bias 16-byte aligned; kRowsLoss: N <= 32
+// kRowsRelu: N a multiple of 64, bias 16-byte aligned; kRowsLoss, kRowsNarrow: N <= 32
 RowsPlan gemm_rows_plan(int epi, int M, int N, int K);
 // mA: [M][K] bf16, box {64, 128}; mB: [N][K] bf16, box {64, BN / cl}; mD: the
 // result, boxes of 32 rows x 128 bytes (kRowsStore fp32, kRowsRelu bf16); all
