@@ -50,6 +50,8 @@
 // the loops, the early code and the h^T tile); 3072-1024-1024-10, 32 workers:
 // 1579 -> 1573.  (Both models' rounds have become shorter by other kernels
 // since.)
+#include <atomic>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -222,8 +224,9 @@ __device__ __forceinline__ void head_softmax(const HeadArgs& a, uint8_t* sm, int
   }
 }
 
-template <int NH, int NC, int CT>
-__global__ void __launch_bounds__(kHTThreads) head_tc_kernel(const __grid_constant__ CUtensorMap mH,
+// K CTAs share an SM (registers): see head_per_sm
+template <int NH, int NC, int CT, int K>
+__global__ void __launch_bounds__(kHTThreads, K) head_tc_kernel(const __grid_constant__ CUtensorMap mH,
                                                               const __grid_constant__ CUtensorMap mW2,
                                                               const __grid_constant__ CUtensorMap mGT,
                                                               const __grid_constant__ HeadArgs a) {
@@ -564,35 +567,72 @@ bool head_tc_supported(int H, int B, int C) {
 int head_tc_class_rows(int C) { return C <= 16 ? 16 : 32; }
 
 namespace {
-template <int NH, int NC, int CT>
-cudaError_t launch_head_tc_nh(const CUtensorMap& mH, const CUtensorMap& mW2, const CUtensorMap& mGT,
-                              const HeadArgs& a, int n_active, cudaStream_t s) {
-  using Cfg = HTCfg<NH, NC>;
-  cudaError_t e = allow_smem(head_tc_kernel<NH, NC, CT>, Cfg::kSmem);
-  if (e != cudaSuccess) return e;
+template <int NH, int NC, int CT, int K>
+cudaLaunchConfig_t head_config(cudaLaunchAttribute* attr, int clusters, int size, int pdl, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n_active, a.H / Cfg::F, 1);
+  cfg.gridDim = dim3(clusters, size, 1);
   cfg.blockDim = dim3(kHTThreads, 1, 1);
-  cfg.dynamicSmemBytes = Cfg::kSmem;
+  cfg.dynamicSmemBytes = HTCfg<NH, NC>::kSmem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 1;
-  attr[0].val.clusterDim.y = a.H / Cfg::F;
+  attr[0].val.clusterDim.y = size;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = a.pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, head_tc_kernel<NH, NC, CT>, mH, mW2, mGT, a);
+  cfg.numAttrs = pdl ? 2 : 1;
+  return cfg;
+}
+
+// CTAs an SM: one with all the registers it likes (175 to 246 a thread), or two
+// with 128 where the workers' clusters are more than run at once with one
+// (queried once per device).  2048 features, 10 classes, batch 32, 16 workers on
+// clusters of 8: 25 us with one CTA an SM, two waves; 17.5 with two.  1024
+// features, where one wave does: 15.7 and 16.4.  With more than 16 classes 128
+// registers spill (2048 x 32, batch 32, a round of one worker 38 -> 44 us, of 64
+// 308 -> 360): always one.
+constexpr int kMaxDevices = 64;
+std::atomic<int> g_head_room[kMaxDevices][kHTMaxCluster + 1];
+template <int NH>
+int head_per_sm(int size, int clusters) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) dev = 0;
+  std::atomic<int>& r = g_head_room[dev][size];
+  int room = r.load(std::memory_order_relaxed);
+  if (room == 0) {
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = head_config<NH, 16, 10, 1>(attr, 1, size, 0, nullptr);
+    if (allow_smem(head_tc_kernel<NH, 16, 10, 1>, HTCfg<NH, 16>::kSmem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&room, head_tc_kernel<NH, 16, 10, 1>, &cfg) != cudaSuccess || room < 1) {
+      cudaGetLastError();
+      room = 1;
+    }
+    r.store(room, std::memory_order_relaxed);
+  }
+  return clusters > room ? 2 : 1;
+}
+
+template <int NH, int NC, int CT, int K>
+cudaError_t launch_head_tc_k(const CUtensorMap& mH, const CUtensorMap& mW2, const CUtensorMap& mGT,
+                             const HeadArgs& a, int n_active, cudaStream_t s) {
+  using Cfg = HTCfg<NH, NC>;
+  cudaError_t e = allow_smem(head_tc_kernel<NH, NC, CT, K>, Cfg::kSmem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr[2];
+  const cudaLaunchConfig_t cfg = head_config<NH, NC, CT, K>(attr, n_active, a.H / Cfg::F, a.pdl, s);
+  return cudaLaunchKernelEx(&cfg, head_tc_kernel<NH, NC, CT, K>, mH, mW2, mGT, a);
 }
 
 template <int NH>
 cudaError_t launch_head_tc_c(const CUtensorMap& mH, const CUtensorMap& mW2, const CUtensorMap& mGT,
                              const HeadArgs& a, int n_active, cudaStream_t s) {
-  return a.C == 10   ? launch_head_tc_nh<NH, 16, 10>(mH, mW2, mGT, a, n_active, s)
-         : a.C <= 16 ? launch_head_tc_nh<NH, 16, 0>(mH, mW2, mGT, a, n_active, s)
-                     : launch_head_tc_nh<NH, 32, 0>(mH, mW2, mGT, a, n_active, s);
+  if (a.C > 16) return launch_head_tc_k<NH, 32, 0, 1>(mH, mW2, mGT, a, n_active, s);
+  const int k = head_per_sm<NH>(a.H / (kHT * NH), n_active);
+  if (a.C == 10) return k == 2 ? launch_head_tc_k<NH, 16, 10, 2>(mH, mW2, mGT, a, n_active, s)
+                               : launch_head_tc_k<NH, 16, 10, 1>(mH, mW2, mGT, a, n_active, s);
+  return k == 2 ? launch_head_tc_k<NH, 16, 0, 2>(mH, mW2, mGT, a, n_active, s)
+                : launch_head_tc_k<NH, 16, 0, 1>(mH, mW2, mGT, a, n_active, s);
 }
 }  // namespace
 

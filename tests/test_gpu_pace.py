@@ -33,3 +33,10 @@ def test_input_gradient_keeps_its_mask_loads_in_flight(cuda_device):
     """1024 x 1024, 256 samples: 1.6 times the forward with the mask loads woven into the stores, 1.2 ahead of them."""
     t = _profile([1024, 1024, 1024, 10], 256, 32, cuda_device)
     assert t["gemm_dh"] < 1.4 * t["gemm_fwd"], t
+
+
+def test_sixteen_heads_on_clusters_of_eight_take_one_wave(cuda_device):
+    """2048 features: 8 workers' clusters run at once with one CTA an SM, 16 only with two (1.5 times as long
+    in two waves, 1.1 in one)."""
+    t8, t16 = (_profile([784, 2048, 10], 32, W, cuda_device)["head_fused"] for W in (8, 16))
+    assert t16 < 1.3 * t8, (t8, t16)
