@@ -112,13 +112,15 @@ __device__ __forceinline__ void epi_dh_mask(const GemmArgs& a, int wid, int m, i
   for (int c = 0; c < 32; ++c) mk[c] = __ldg(hm + static_cast<int64_t>(c) * a.M);
 }
 
+template <bool kTest>
 __device__ __forceinline__ float epi_dh(const GemmArgs& a, int wid, int m, int n0, const float (&v)[32],
                                         const unsigned short (&mk)[32]) {
-  // the row-major copy: always written here, but a test around its stores keeps
-  // the compiler from weaving them into the next chunk's mask loads (64
-  // registers and few loads in flight instead of 144: 1024 x 1024, 256 samples,
-  // 32 workers: 43 us so, 31 with the test)
-  __nv_bfloat16* out = a.out ? a.out + static_cast<int64_t>(wid) * a.N * a.M : nullptr;
+  // the row-major copy: always written here, but with eight chunks a thread
+  // (kTest) a test around its stores keeps the compiler from weaving them into
+  // the next chunk's mask loads (64 registers and few loads in flight instead of
+  // 144: 1024 x 1024, 256 samples, 32 workers: 43 us so, 31 with the test); with
+  // one it costs (17-class round, batch 32: 315.8 us without, 319.3 with)
+  __nv_bfloat16* out = a.out + static_cast<int64_t>(wid) * a.N * a.M;
   uint32_t pk[16];
   float gsum = 0.f;
 #pragma unroll
@@ -130,7 +132,7 @@ __device__ __forceinline__ float epi_dh(const GemmArgs& a, int wid, int m, int n
     gsum += g0;
     gsum += g1;
     const __nv_bfloat162 p = __floats2bfloat162_rn(g0, g1);
-    if (out) {
+    if (!kTest || a.out) {
       out[e0] = p.x;
       out[e1] = p.y;
     }
@@ -365,7 +367,7 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
       } else {
         unsigned short mk[32];
         epi_dh_mask(a, wid, m, n0 + c0, mk);
-        gpart[rl * (BN / 32) + c0 / 32] = epi_dh(a, wid, m, n0 + c0, v, mk);
+        gpart[rl * (BN / 32) + c0 / 32] = epi_dh<false>(a, wid, m, n0 + c0, v, mk);
       }
     }
     if constexpr (EPI == kEpiDh) {
@@ -457,7 +459,7 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
 #pragma unroll
         for (int c = 0; c < 32; ++c) cur[c] = mk[c];
         if (c0 + 32 < BN) epi_dh_mask(a, wid, m, n0 + c0 + 32, mk);
-        gsum += epi_dh(a, wid, m, n0 + c0, v, cur);
+        gsum += epi_dh<BN == 256>(a, wid, m, n0 + c0, v, cur);
       }
       a.gb_out[static_cast<int64_t>(wid) * a.M + m] = gsum;
     } else {
