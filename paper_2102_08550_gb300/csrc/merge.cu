@@ -30,7 +30,10 @@
 // 16 bytes.  When they share one offset that is not 0, the first (up to 3)
 // elements of a segment are peeled off; those and the tail are single
 // elements that threads of the same launch take after their chunks.  Only
-// buffers with different offsets take single elements throughout.
+// buffers with different offsets take single elements throughout, four a thread
+// at a time: one at a time, 5 M elements of 1 and 3 workers took 23 and 45 us (19
+// and 43 on a kernel of their own before), 12.5 and 20.8 now; of 16 workers 57
+// (206), 52 now.
 #include <atomic>
 
 #include "common.cuh"
@@ -76,29 +79,64 @@ __device__ __forceinline__ void merge_group(const MergeArgs& a, int k, int64_t p
   }
 }
 
-// The same for single element p.
-template <int G, bool kReplica>
-__device__ __forceinline__ void merge_group1(const MergeArgs& a, int k, int64_t p, float x, float& acc) {
-  float v[G];
+// The same for E single elements p.
+template <int G, int E, bool kReplica>
+__device__ __forceinline__ void merge_singles(const MergeArgs& a, int k, int64_t at, const int64_t (&p)[E],
+                                              const float (&x)[E], float (&acc)[E]) {
+  float v[G][E];
 #pragma unroll
-  for (int j = 0; j < G; ++j) v[j] = __ldcs(a.src[k + j] + p);
+  for (int g = 0; g < G; ++g)
 #pragma unroll
-  for (int j = 0; j < G; ++j) acc = fmaf(a.w[k + j], kReplica ? v[j] - x : v[j], acc);
+    for (int j = 0; j < E; ++j) v[g][j] = __ldcs(a.src[k + g] + at + p[j]);
+#pragma unroll
+  for (int g = 0; g < G; ++g)
+#pragma unroll
+    for (int j = 0; j < E; ++j) acc[j] = fmaf(a.w[k + g], kReplica ? v[g][j] - x[j] : v[g][j], acc[j]);
 }
 
+// E single elements q, q + stride, ... of a segment, G E loads in flight
+template <int G, int E, bool kReplica>
+__device__ __forceinline__ void merge_at(const MergeArgs& a, const MergeSeg& sg, float* __restrict__ x_g, float eta,
+                                         __nv_bfloat16* __restrict__ shadow, int64_t q, int64_t stride) {
+  int64_t p[E];
+  float x[E], acc[E];
+#pragma unroll
+  for (int j = 0; j < E; ++j) {
+    const int64_t at = q + j * stride;
+    p[j] = at < sg.head ? at : at + 4 * sg.n4;
+    x[j] = x_g[sg.dst + p[j]];
+    acc[j] = 0.f;
+  }
+  int k = 0;
+  for (; k + G <= a.W; k += G) merge_singles<G, E, kReplica>(a, k, sg.src, p, x, acc);
+  for (; k < a.W; ++k) merge_singles<1, E, kReplica>(a, k, sg.src, p, x, acc);
+#pragma unroll
+  for (int j = 0; j < E; ++j) {
+    const float out = fmaf(eta, acc[j], x[j]);
+    x_g[sg.dst + p[j]] = out;
+    if (shadow) shadow[sg.dst + p[j]] = __float2bfloat16_rn(out);
+  }
+}
+
+// Up to N segments: 1, 8 or kMaxMergeSegs.  The pointer and weight tables are 3 KB;
+// with a table of 32 segments beside them, and the code for single elements in a
+// kernel that has none, a launch took 0.3 us longer (device time of 1000
+// elements, 16 workers, us: 1.8, 2.1 with both, 1.9 now; 400 000: 2.9, 3.2, 2.9).
+template <int N>
 struct MergeSegs {
-  MergeSeg s[kMaxMergeSegs];
-  int first_block[kMaxMergeSegs + 1];   // segment i runs on blocks [first_block[i], first_block[i + 1])
+  MergeSeg s[N];
+  int first_block[N + 1];   // segment i runs on blocks [first_block[i], first_block[i + 1])
   int n;
 };
 
-template <bool kReplica>
+// kSingle: some segment has single elements (any may, with N > 1)
+template <bool kReplica, int N, bool kSingle>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) merge_vec4_kernel(const __grid_constant__ MergeArgs a,
-                                                                     const __grid_constant__ MergeSegs segs,
+                                                                     const __grid_constant__ MergeSegs<N> segs,
                                                                      float* __restrict__ x_g, float eta,
                                                                      __nv_bfloat16* __restrict__ shadow) {
   int si = 0;
-  while (si + 1 < segs.n && static_cast<int>(blockIdx.x) >= segs.first_block[si + 1]) ++si;
+  while (N > 1 && si + 1 < segs.n && static_cast<int>(blockIdx.x) >= segs.first_block[si + 1]) ++si;
   const MergeSeg& sg = segs.s[si];
   const int64_t stride = static_cast<int64_t>(segs.first_block[si + 1] - segs.first_block[si]) * kThreads;
   const int64_t t0 = static_cast<int64_t>(blockIdx.x - segs.first_block[si]) * kThreads + threadIdx.x;
@@ -133,20 +171,14 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) merge_vec4_kernel(const 
     if (shadow)   // the bf16 operand copy of the new global model, same pass
       reinterpret_cast<uint2*>(shadow + go)[i] = make_uint2(pack_bf16x2(out.x, out.y), pack_bf16x2(out.z, out.w));
   }
+  if (!kSingle) return;
   // single elements: [0, head) and [head + 4 n4, n), from the segment's last
-  // threads (the ones with the fewest chunks)
-  const int64_t tail = sg.head + 4 * sg.n4, count = sg.head + (sg.n - tail);
-  for (int64_t q = stride - 1 - t0; q < count; q += stride) {
-    const int64_t p = q < sg.head ? q : tail + (q - sg.head);
-    const float x = x_g[sg.dst + p];
-    float acc = 0.f;
-    int k = 0;
-    for (; k + 8 <= a.W; k += 8) merge_group1<8, kReplica>(a, k, sg.src + p, x, acc);
-    for (; k < a.W; ++k) merge_group1<1, kReplica>(a, k, sg.src + p, x, acc);
-    const float out = fmaf(eta, acc, x);
-    x_g[sg.dst + p] = out;
-    if (shadow) shadow[sg.dst + p] = __float2bfloat16_rn(out);
-  }
+  // threads (the ones with the fewest chunks); four a thread at a time where
+  // there are that many (buffers with different offsets)
+  const int64_t count = sg.n - 4 * sg.n4;
+  int64_t q = stride - 1 - t0;
+  for (; q + 3 * stride < count; q += 4 * stride) merge_at<4, 4, kReplica>(a, sg, x_g, eta, shadow, q, stride);
+  for (; q < count; q += stride) merge_at<8, 1, kReplica>(a, sg, x_g, eta, shadow, q, stride);
 }
 
 constexpr int kMaxDevices = 64;
@@ -170,10 +202,11 @@ int sm_count() {
 
 }  // namespace
 
-cudaError_t launch_merge_segs(const MergeArgs& a, const MergeSeg* seg, int nseg, float* x_g, float eta, bool replica,
-                              cudaStream_t s, __nv_bfloat16* shadow) {
-  if (nseg < 0 || nseg > kMaxMergeSegs) return cudaErrorInvalidValue;
-  MergeSegs m;
+namespace {
+template <int N>
+cudaError_t launch_merge_n(const MergeArgs& a, const MergeSeg* seg, int nseg, float* x_g, float eta, bool replica,
+                           cudaStream_t s, __nv_bfloat16* shadow) {
+  MergeSegs<N> m;
   m.n = 0;
   m.first_block[0] = 0;
   // every pushed buffer at the same offset modulo 16 bytes?
@@ -208,9 +241,28 @@ cudaError_t launch_merge_segs(const MergeArgs& a, const MergeSeg* seg, int nseg,
   }
   if (m.n == 0) return cudaSuccess;
   const unsigned nb = static_cast<unsigned>(m.first_block[m.n]);
-  if (replica) merge_vec4_kernel<true><<<nb, kThreads, 0, s>>>(a, m, x_g, eta, shadow);
-  else merge_vec4_kernel<false><<<nb, kThreads, 0, s>>>(a, m, x_g, eta, shadow);
+  if constexpr (N == 1) {
+    // no single elements, and less than a full grid: without their code (see
+    // above; a full grid is bound by memory, and 25.6 M elements of 64 workers
+    // took 955 us without that code, 943 with it)
+    if (m.s[0].head == 0 && m.s[0].n == 4 * m.s[0].n4 && nb < static_cast<unsigned>(most)) {
+      if (replica) merge_vec4_kernel<true, 1, false><<<nb, kThreads, 0, s>>>(a, m, x_g, eta, shadow);
+      else merge_vec4_kernel<false, 1, false><<<nb, kThreads, 0, s>>>(a, m, x_g, eta, shadow);
+      return cudaGetLastError();
+    }
+  }
+  if (replica) merge_vec4_kernel<true, N, true><<<nb, kThreads, 0, s>>>(a, m, x_g, eta, shadow);
+  else merge_vec4_kernel<false, N, true><<<nb, kThreads, 0, s>>>(a, m, x_g, eta, shadow);
   return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_merge_segs(const MergeArgs& a, const MergeSeg* seg, int nseg, float* x_g, float eta, bool replica,
+                              cudaStream_t s, __nv_bfloat16* shadow) {
+  if (nseg < 0 || nseg > kMaxMergeSegs) return cudaErrorInvalidValue;
+  return nseg <= 1   ? launch_merge_n<1>(a, seg, nseg, x_g, eta, replica, s, shadow)
+         : nseg <= 8 ? launch_merge_n<8>(a, seg, nseg, x_g, eta, replica, s, shadow)
+                     : launch_merge_n<kMaxMergeSegs>(a, seg, nseg, x_g, eta, replica, s, shadow);
 }
 
 cudaError_t launch_merge(const MergeArgs& a, float* x_g, int64_t P, float eta, bool replica, cudaStream_t s,

@@ -111,3 +111,23 @@ def test_merge_full_size_p25m_w64(cuda_device):
 @pytest.mark.parametrize("rule", ["uniform", "localsteps"])
 def test_merge_full_size_p340m_w8(cuda_device, rule):
     assert _full_size_merge(cuda_device, synth.CFG5, rule) <= PARAM_RTOL
+
+
+# one to four single elements a thread, and their edges (152 SMs x 3 blocks x 224 threads = 102144 at a time)
+@pytest.mark.parametrize("Pn", [1, 5, 102143, 102145, 306432, 306433, 408576, 409001, 1000003])
+@pytest.mark.parametrize("W", [1, 3, 8, 13])
+def test_merge_buffers_with_different_offsets(cuda_device, W, Pn):
+    """Element by element, bit for bit what the same buffers give from 16-byte chunks: both add in worker order."""
+    g = torch.Generator(device=cuda_device).manual_seed(W * 7 + Pn)
+    x = torch.randn(Pn, device=cuda_device, generator=g)
+    d = [torch.randn(Pn, device=cuda_device, generator=g) for _ in range(W)]
+    w, s = [1.0 / (k + 2) for k in range(W)], torch.cuda.current_stream().cuda_stream
+    bufs = [torch.zeros(Pn + 8, device=cuda_device) for _ in range(W)]
+    moved = [b[(k + 1) % 4:][:Pn].copy_(v) for k, (b, v) in enumerate(zip(bufs, d))]
+    guard = torch.full((Pn + 8,), 5.0, device=cuda_device)
+    y = guard[4:4 + Pn].copy_(x)
+    P.oscars_merge(x.data_ptr(), [v.data_ptr() for v in d], w, Pn, 0.75, s)
+    P.oscars_merge(y.data_ptr(), [v.data_ptr() for v in moved], w, Pn, 0.75, s)
+    torch.cuda.synchronize()
+    assert torch.equal(x, y)
+    assert (guard[:4] == 5.0).all() and (guard[4 + Pn:] == 5.0).all()
