@@ -2045,13 +2045,16 @@ oscars_status eval_cnn(oscars_ctx* c, const float* x, const int32_t* y, int64_t 
   if (st != OSCARS_OK) return st;
   for (int64_t lane0 = 0; lane0 < *parts; lane0 += W) {
     const int na = static_cast<int>(std::min<int64_t>(W, *parts - lane0));
+    // a lane alone holds only the images that are left (one image, batches of
+    // 256: 59 us a call; 112 with the lane filled up)
+    const int Bc = na == 1 ? static_cast<int>(std::min<int64_t>(B, n - lane0 * B)) : B;
     CnnStageArgs a{};
     a.x1 = x;
     a.y1 = y;
     a.n1 = n;
     a.eval_base = lane0 * B;
     a.wid = c->lane_ids;
-    a.B = B;
+    a.B = Bc;
     a.Cin = c->dims[2];
     a.im2col = c->cnn_im2col ? 1 : 0;
     a.out = c->cnn_buf[0];
@@ -2062,7 +2065,7 @@ oscars_status eval_cnn(oscars_ctx* c, const float* x, const int32_t* y, int64_t 
       std::memset(&ca, 0, sizeof(ca));
       ca.wid = c->lane_ids;
       ca.src = c->global_src;
-      ca.B = B;
+      ca.B = Bc;
       ca.bias = c->slab;
       ca.slot_stride = c->P_pad;
       ca.off_bias = c->cnn_offB[layer];
@@ -2072,7 +2075,7 @@ oscars_status eval_cnn(oscars_ctx* c, const float* x, const int32_t* y, int64_t 
       ca.im2col = layer == 0 && c->cnn_im2col ? 1 : 0;
       return launch_conv_igemm(0, ca.im2col ? c->cnn_m4[in] : c->cnn_m6[in], c->cnn_mw[layer],
                                ConvMaps{c->cnn_m4[add >= 0 ? add : out], c->cnn_m4[out], c->cnn_m1[out]}, ca, na,
-                               conv_ctas_per_worker(B, na, c->sms), c->stream);
+                               conv_ctas_per_worker(Bc, na, c->sms), c->stream);
     };
     if (e == cudaSuccess) e = conv(0, 0, -1, 1, nullptr);
     for (int k = 0; e == cudaSuccess && k < c->cnn_blocks; ++k) {
@@ -2081,7 +2084,7 @@ oscars_status eval_cnn(oscars_ctx* c, const float* x, const int32_t* y, int64_t 
       if (e == cudaSuccess) e = conv(2 + 2 * k, 2 + 2 * k, h, 3 + 2 * k, k == c->cnn_blocks - 1 ? c->cnn_pool : nullptr);
     }
     if (e == cudaSuccess)
-      e = launch_cnn_head_loss(c->cnn_pool, c->labels, na, B, n - lane0 * B, c->C, c->slab + g, c->cnn_offWf, c->cnn_offBf,
+      e = launch_cnn_head_loss(c->cnn_pool, c->labels, na, Bc, n - lane0 * B, c->C, c->slab + g, c->cnn_offWf, c->cnn_offBf,
                                c->eval_part + lane0, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "eval");
   }

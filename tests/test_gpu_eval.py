@@ -71,7 +71,7 @@ def test_eval_softreg(cuda_device, D, C, n):
     ctx.close()
 
 
-@pytest.mark.parametrize("n,W", [(1, 2), (17, 2), (100, 3)])
+@pytest.mark.parametrize("n,W", [(1, 2), (17, 2), (100, 3), (7, 1), (33, 2), (48, 1)])   # a lane alone, whole or not, and others
 def test_eval_cnn(cuda_device, n, W):
     B, dev = 16, cuda_device
     w = synth.ConvWorkload("cnn-eval", W, [32 * 32 * 3, 10], B, 0.05, B, 4, 1, clip=3.0, blocks=1, in_ch=3)
