@@ -668,8 +668,11 @@ __global__ void __launch_bounds__(NT + NT / 4, K) softreg_cluster_round_kernel(c
   }
   // a wait that ran out, in any lane, shows as a NaN loss (the allocation-free entry has no error word)
   alive = __all_sync(0xffffffffu, alive);
-  if (!fetcher && lane == 0)
-    lsum[warp] = alive ? static_cast<double>(loss_hi) + static_cast<double>(loss_lo) : static_cast<double>(NAN);
+  if (!fetcher && lane == 0) {
+    double sum = static_cast<double>(loss_hi);
+    if (isfinite(loss_hi)) sum += static_cast<double>(loss_lo);   // an infinite row has made it inf - inf
+    lsum[warp] = alive ? sum : static_cast<double>(NAN);
+  }
   __syncthreads();
   // push: this CTA's columns into the replica
   for (int c = warp; c < C; c += (NT + NF) / 32)

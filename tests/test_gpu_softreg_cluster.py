@@ -109,3 +109,24 @@ def test_thirty_workers_take_one_wave(cuda_device, D, C, B):
         return best
 
     assert us(30) < 1.8 * us(1)
+
+
+@pytest.mark.parametrize("D,C,B,steps", [(4, 3, 5, 1), (784, 10, 32, 3), (60, 32, 512, 1)])   # the cluster kernel, and one CTA
+def test_infinite_loss_stays_infinite(cuda_device, D, C, B, steps):
+    """A label whose logit is minus infinity has an infinite loss (and a finite gradient); so has the step and the
+    round.  NaN is for undefined values and for a wait that ran out."""
+    dev = cuda_device
+    p = torch.zeros(C * D + C, device=dev)
+    p[0] = -1e38
+    x, y = torch.zeros(2 * B, D, device=dev), torch.ones(2 * B, dtype=torch.int32, device=dev)
+    x[1, 0], y[1] = 100.0, 0          # logits (-inf, 0, ...), label 0
+    out, loss = torch.empty_like(p), torch.empty(1, device=dev)
+    call(p, out, x, y, 2 * B, 0, steps, D, C, B, 0.05, loss)
+    assert loss.item() == float("inf")
+    assert torch.isfinite(out).all()
+    ctx = P.OscarsContext(num_workers=2, dims=[D, C], batch=B, lr=0.05, bf16=False, shards=[(x, y)] * 2, M=8,
+                          init_params=p, t_ticks=[1, 1], stream=torch.cuda.current_stream().cuda_stream)
+    ctx.set_local_steps([steps] * 2)
+    _, losses = ctx.local_steps()
+    ctx.close()
+    assert losses == [float("inf")] * 2
