@@ -243,7 +243,12 @@ oscars_status oscars_set_iteration_ticks(oscars_ctx* ctx, const int64_t* t_iter)
 /*
  * oscars_eval_loss - mean softmax cross-entropy of the global model on n
  * samples x [n][dims[0]] fp32 and labels y [n] (both device pointers), with
- * the same operand precision as training.  MLP mode; n >= 1; *loss is host.
+ * the same operand precision as training.  MLP and CNN mode; n >= 1 (for an MLP
+ * with hidden layers a multiple of the batch); *loss is host.  Synchronises.
+ * For an MLP with hidden layers the context keeps, until it is destroyed, the
+ * samples and the outputs of one or two layers in bf16 for up to 16384 samples
+ * at a time (fewer where the device has no room for them).  Errors: EINVAL,
+ * ENOTSUP, ESTATE (no such model), ENOMEM, ECUDA, ETIMEOUT.
  */
 oscars_status oscars_eval_loss(oscars_ctx* ctx, const float* x, const int32_t* y, int64_t n,
                                float* loss);

@@ -114,6 +114,9 @@ bool make_map_f32(CUtensorMap* m, const void* base, uint64_t dx, uint64_t dy, ui
   return encode_map(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, swz);
 }
 
+constexpr int64_t kEvalRows = 16384;   // samples of one pass over the layers, where memory allows
+constexpr int64_t kEvalLeast = 128;    // and at least
+
 struct Layer {
   int in, out;
   int64_t offW, offB;
@@ -174,6 +177,7 @@ struct oscars_ctx {
   __nv_bfloat16* eval_x = nullptr;
   __nv_bfloat16* eval_h[2] = {};
   int64_t eval_rows = 0;
+  int64_t eval_most = kEvalRows;        // rows they may have
   // tensor maps per layer
   std::vector<CUtensorMap> mShadow, mShadowMN, mA, mG, mGT, mAT;
   // G^T [lane][out][B] and H^T [lane][in][B] in boxes of 64 x 64: the MN-major B
@@ -1964,8 +1968,6 @@ oscars_status oscars_set_iteration_ticks(oscars_ctx* c, const int64_t* t_iter) {
 
 namespace {
 
-constexpr int64_t kEvalRows = 16384;   // samples of one pass over the layers
-
 oscars_status eval_parts(oscars_ctx* c, int64_t count) {
   if (c->eval_part_cap >= count) return OSCARS_OK;
   c->eval_part_cap = 0;
@@ -1982,26 +1984,36 @@ oscars_status eval_parts(oscars_ctx* c, int64_t count) {
 // of the 784-512-10 model, 277 us; four launches and one synchronisation, 37.
 oscars_status eval_mlp(oscars_ctx* c, const float* x, const int32_t* y, int64_t n, int64_t* parts) {
   const int L = c->L, D = c->dims[0];
-  const int64_t rows = std::min(n, kEvalRows);
-  if (c->eval_rows < rows) {
+  const int64_t want = std::min(n, c->eval_most);
+  if (c->eval_rows < want) {
     int widest = 0;
     for (int l = 1; l < L; ++l) widest = std::max(widest, c->dims[l]);
     c->eval_rows = 0;
-    dev_release(c, &c->eval_x);
-    for (auto& h : c->eval_h) dev_release(c, &h);
-    if (!dev_alloc(c, &c->eval_x, static_cast<size_t>(rows) * D) ||
-        !dev_alloc(c, &c->eval_h[0], static_cast<size_t>(rows) * widest) ||
-        (L > 2 && !dev_alloc(c, &c->eval_h[1], static_cast<size_t>(rows) * widest)))
-      return fail(c, OSCARS_ENOMEM, "eval scratch");
-    c->eval_rows = rows;
+    for (int64_t r = want;; r = std::max(r / 2, kEvalLeast)) {   // fewer samples a pass where the device is full
+      dev_release(c, &c->eval_x);
+      for (auto& h : c->eval_h) dev_release(c, &h);
+      if (dev_alloc(c, &c->eval_x, static_cast<size_t>(r) * D) &&
+          dev_alloc(c, &c->eval_h[0], static_cast<size_t>(r) * widest) &&
+          (L == 2 || dev_alloc(c, &c->eval_h[1], static_cast<size_t>(r) * widest))) {
+        c->eval_rows = r;
+        if (r < want) c->eval_most = r;   // later evaluations do not try again
+        break;
+      }
+      if (r <= kEvalLeast) {
+        dev_release(c, &c->eval_x);
+        for (auto& h : c->eval_h) dev_release(c, &h);
+        return fail(c, OSCARS_ENOMEM, "eval scratch");
+      }
+    }
   }
+  const int64_t rows = std::min(n, c->eval_rows);
   const int64_t per = (rows + 127) / 128 * 4;   // loss partials of a pass
-  const oscars_status st = eval_parts(c, (n + kEvalRows - 1) / kEvalRows * per);
+  const oscars_status st = eval_parts(c, (n + rows - 1) / rows * per);
   if (st != OSCARS_OK) return st;
   const int64_t g = static_cast<int64_t>(c->W) * c->P_pad;
   *parts = 0;
-  for (int64_t base = 0; base < n; base += kEvalRows) {
-    const int m = static_cast<int>(std::min(kEvalRows, n - base));
+  for (int64_t base = 0; base < n; base += rows) {
+    const int m = static_cast<int>(std::min(rows, n - base));
     cudaError_t e = launch_cast_rows(x + base * D, c->eval_x, static_cast<int64_t>(m) * D, c->sms, c->stream);
     for (int l = 0; e == cudaSuccess && l < L; ++l) {
       const Layer& ly = c->layers[l];

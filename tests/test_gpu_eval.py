@@ -113,3 +113,33 @@ def test_eval_between_rounds_changes_nothing(cuda_device, dims, flags):
         ctx.close()
     assert out[0][0] == out[1][0]
     torch.testing.assert_close(out[0][1], out[1][1], rtol=0, atol=0)
+
+
+def test_eval_on_a_nearly_full_device(cuda_device):
+    """A layer of 16384 outputs: two buffers of 16384 samples want 1.1 GB.  With 400 MB left the evaluation takes
+    fewer samples a pass, and gives the same loss (sums of the same 32-sample partials)."""
+    dims, B, n, dev = [64, 16384, 128, 10], 32, 16384 + 96, cuda_device
+    rng = np.random.default_rng(3)
+    flat = torch.from_numpy(synth.flatten_layers(
+        [(rng.uniform(-1, 1, (o, i)).astype(np.float32) / np.float32(np.sqrt(i)), np.zeros(o, np.float32))
+         for i, o in zip(dims[:-1], dims[1:])])).to(dev)
+    X, y = _set(dims[0], dims[-1], n, 5)
+    x, yd = torch.from_numpy(X).to(dev), torch.from_numpy(y).to(dev)
+    ctx = _ctx(dims, B, 1, dev, flat=flat)
+    want = ctx.eval_loss(x, yd)
+    ctx.close()
+    ctx = _ctx(dims, B, 1, dev, flat=flat)
+    ctx.eval_loss(x[:B], yd[:B])
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    hold = torch.empty(max(free - 400 * 2 ** 20, 1), dtype=torch.uint8, device=dev)
+    try:
+        first = ctx.eval_loss(x, yd)
+        again = ctx.eval_loss(x, yd)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    later = ctx.eval_loss(x[:n - 96], yd[:n - 96])
+    ctx.close()
+    assert first == again and abs(first - want) <= 1e-6 * abs(want), (first, again, want)
+    assert abs(later - want) <= 0.05 * abs(want)
