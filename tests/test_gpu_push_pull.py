@@ -18,6 +18,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("dims,bf16,W,shifts", [
     ([333, 26], False, 5, [0]), ([333, 26], False, 3, [1]), ([18, 3], False, 2, [0, 2]),
     ([64, 128, 10], True, 4, [0]), ([72, 128, 128, 17], True, 3, [3]), ([64, 128, 10], True, 2, [0, 1]),
+    ([72, 128, 128, 128, 128, 17], True, 3, [0]), ([72] + [128] * 14 + [17], True, 2, [1, 0]),   # 10 and 30 tensors
 ], ids=lambda v: "-".join(map(str, v)) if isinstance(v, list) else str(v))
 @pytest.mark.parametrize("dst_shift", [0, 1])
 def test_push_deltas_and_pull(cuda_device, dims, bf16, W, shifts, dst_shift):
