@@ -473,11 +473,14 @@ oscars_status oscars_gemm_bf16_nt(const void* A, const void* B, float* C, int32_
  * partial per step); larger tau, classes outside [2, 32] or bad pointers give
  * EINVAL; batch > 512, or shapes whose weights plus one batch exceed shared
  * memory, ENOTSUP.
- * The first call on a device looks up the scratch address (once per device);
- * make that first call before any stream capture.  Every call shares the one
- * scratch array and leaves its contents behind; each call writes all it reads
- * first, so nothing needs clearing, but calls that overlap on the GPU (other
- * streams, other threads) race on it.
+ * Make the first call on a device before any stream capture (it loads the
+ * kernel, and for the single-CTA kernel looks up the scratch address).  Calls on
+ * the cluster kernel keep nothing in the library, so calls with buffers of their
+ * own may overlap on the GPU (other streams, other threads).  Calls on the
+ * single-CTA kernel (batches from about 390 with 17 classes and more, 470 with
+ * 15) share the one scratch array and leave its contents behind; each writes all
+ * it reads first, so nothing needs clearing, but such calls must not overlap:
+ * they race on it.
  */
 oscars_status oscars_softreg_steps_noalloc(const float* params_in, float* params_out, const float* x,
                                            const int32_t* y, int64_t n, int64_t cursor, int32_t tau,

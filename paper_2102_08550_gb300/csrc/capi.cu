@@ -699,8 +699,8 @@ const CUtensorMap& step_inputs_t(oscars_ctx* c, int step) {
 }
 const int32_t* step_labels(oscars_ctx* c) { return c->ahead_mlp ? c->labb[c->cur_buf] : c->labels_all; }
 
-// forward layers 0..L-2 for `na` lanes (training step or evaluation)
-cudaError_t enqueue_forward(oscars_ctx* c, const int* wid, const int* src, int na, cudaStream_t st, int step = 0) {
+// forward layers 0..L-2 of local step `step` for `na` lanes
+cudaError_t enqueue_forward(oscars_ctx* c, const int* wid, const int* src, int na, cudaStream_t st, int step) {
   for (int l = 0; l + 1 < c->L; ++l) {
     const Layer& ly = c->layers[l];
     GemmArgs g = gemm_base(c, wid, src);
@@ -829,8 +829,6 @@ StageArgs stage_args(oscars_ctx* c, int buf, const int32_t* ahead) {
   sa.y = c->dy_tab;
   sa.n = c->dn_tab;
   sa.start = c->cursor;
-  sa.row_add = 0;
-  sa.wid = nullptr;
   sa.D = c->dims[0];
   sa.B = c->B;
   sa.A0 = c->A0b[buf];
@@ -888,8 +886,6 @@ cudaError_t enqueue_round_mlp(oscars_ctx* c, cudaStream_t st) {
     sa.y = c->dy_tab;
     sa.n = c->dn_tab;
     sa.start = c->cursor;
-    sa.row_add = 0;
-    sa.wid = nullptr;
     sa.D = c->dims[0];
     sa.B = c->B;
     sa.A0 = c->A0all;
@@ -1213,7 +1209,7 @@ oscars_status layout_cnn(oscars_ctx* c, const oscars_config* cfg) {
          static_cast<int64_t>(K) * C + K;
   c->cnn_wt_slot = static_cast<int64_t>(2 * c->cnn_blocks) * 9 * 64 * 64;
   c->cnn_im2col = 9 * Cin <= 64;   // layer 0 then uses the first 64 x 64 of its 64 x 9 x 64 block
-  c->cnn_chunks = c->B;   // capacity: at most one image per chunk
+  c->cnn_chunks = c->B;   // capacity: conv_wgrad_chunks gives at most B (ranges of 2-row blocks, which may cross images)
   return OSCARS_OK;
 }
 
@@ -2048,7 +2044,7 @@ oscars_status eval_mlp(oscars_ctx* c, const float* x, const int32_t* y, int64_t 
 
 // CNN: W lanes of B images at a time with the global model's weights (1024
 // images, 16 workers, batch 32: 2035 us one lane at a time with a
-// synchronisation each, 434 now)
+// synchronisation each, 316 now)
 oscars_status eval_cnn(oscars_ctx* c, const float* x, const int32_t* y, int64_t n, int64_t* parts) {
   const int W = c->W, B = c->B;
   const int64_t g = static_cast<int64_t>(W) * c->P_pad;

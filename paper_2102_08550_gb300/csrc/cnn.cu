@@ -81,7 +81,9 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 // stores of a pixel's row by its thread touched 32 lines an instruction: they
 // took the load/store unit about 2000 clocks a tile, four times the MMAs, and
 // the kernels ran at 41 us (forward) and 60 us (input gradient) a launch of
-// up to 16 workers; 36 and 48 us with this epilogue.
+// up to 16 workers; 36 and 48 us with this epilogue.  In the input gradient a
+// thread also keeps 64 channel sums over its tiles: 168 registers at 320 threads,
+// and 52 bytes spilled.
 constexpr int kGT = 320;                    // warp 0 TMA, warp 1 MMA, warps 2-5 and 6-9 epilogue
 constexpr int kGSlots = 4;                  // input boxes in flight (one a tile)
 constexpr int kGAcc = 256;                  // TMEM columns of an accumulator (192 used)

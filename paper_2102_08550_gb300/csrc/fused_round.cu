@@ -78,8 +78,8 @@
 // workers, which it runs one after the other (the host deals them by
 // decreasing tau to the cluster with the least work so far).
 //
-// Warp roles (384 threads): warp 0 lane 0 issues TMA, warp 1 lane 0 issues
-// tcgen05.mma (in step D warps 1 and 3 issue one chain each), warp 2 owns the
+// Warp roles (384 threads): warp 0 lane 0 issues TMA, an elected lane of warp 1
+// issues tcgen05.mma (in step D warps 1 and 3 issue one chain each), warp 2 owns the
 // TMEM allocation (all 512 columns: one CTA per SM), warps 4..11 are the two
 // epilogue warpgroups (each covering the 128 TMEM lanes), all warps share the
 // CUDA-core work of step H.

@@ -17,7 +17,7 @@
 //  * warp 0 lane 0 (TMA producer) loads each tile's fp32 master block into
 //    one of two buffers (four 32-column boxes, 128-byte swizzle) as soon as
 //    that buffer is free, and the operand k-blocks through a 2-slot ring;
-//  * warp 1 lane 0 issues tcgen05.mma into one of two TMEM accumulators of
+//  * warp 1 (an elected lane) issues tcgen05.mma into one of two TMEM accumulators of
 //    128 columns, so tile i + 1's products run under tile i's epilogue;
 //  * warp 2 owns the TMEM allocation;
 //  * warps 4-11 (two per TMEM lane quarter, 32 rows x 64 columns each)
@@ -116,7 +116,8 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
   // this kernel, a merge) has completed, because every kernel of the chain
   // waits for its predecessor before it lets its successor start.  A round of
   // 1000-384-256-17, 5 workers: 309.6 -> 306.2 us; 3072-1024-1024-10, 32
-  // workers: 1521 -> 1510 (both buffers: 1510).
+  // workers: 1521 -> 1510 (both buffers: 1510); timed in a loop over two prepared
+  // contexts, which reads 1 to 2% lower than passes on changing inputs.
   auto load_master = [&](int ly, int src, int m0, int n0, int b) {
     mbar_arrive_expect_tx(&bars->mfull[b], kDwMasterBytes);
 #pragma unroll

@@ -8,7 +8,7 @@
 // One CTA computes one 128 x BN tile of one active worker (grid z = worker).
 // Warp 0 lane 0 streams K-blocks of 64 with TMA (128-byte swizzle, 3-D
 // tensor maps whose z coordinate selects the worker's buffer or the
-// parameter slot), warp 1 lane 0 issues tcgen05.mma (M=128, N=BN, K=16) into
+// parameter slot), warp 1 (an elected lane) issues tcgen05.mma (M=128, N=BN, K=16) into
 // a TMEM accumulator and frees each stage with tcgen05.commit, warp 2 owns
 // the TMEM allocation; then all four warps read their 32 TMEM lanes
 // (one output row per thread) and run the epilogue:
@@ -80,7 +80,6 @@ __device__ __forceinline__ void sts128(uint32_t addr, const uint32_t* r) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
 }
 
-template <int EPI>
 __device__ __forceinline__ void epi_fwd(const GemmArgs& a, int wid, int src, int m, int n0,
                                         const float (&v)[32]) {
   const float bias = a.master[static_cast<int64_t>(src) * a.slot_stride + a.offB + m];
@@ -363,7 +362,7 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
 #pragma unroll
         for (int q = 0; q < 4; ++q) outT[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
       } else if constexpr (EPI == kEpiFwd) {
-        epi_fwd<EPI>(a, wid, src, m, n0 + c0, v);
+        epi_fwd(a, wid, src, m, n0 + c0, v);
       } else {
         unsigned short mk[32];
         epi_dh_mask(a, wid, m, n0 + c0, mk);
@@ -467,7 +466,7 @@ __global__ void __launch_bounds__(kWarps * 32) gemm_tc_kernel(const __grid_const
       for (int c0 = 0; c0 < BN; c0 += 32) {
         float v[32];
         tmem_ld_32x32b_x32(trow + c0, v);
-        epi_fwd<EPI>(a, wid, src, m, n0 + c0, v);
+        epi_fwd(a, wid, src, m, n0 + c0, v);
       }
     }
   }
@@ -589,13 +588,9 @@ cudaError_t launch_epi(int bn, const GemmMaps& m, const GemmArgs& a, int n_activ
 
 }  // namespace
 
-int gemm_bn_for(int epi, int N) {
-  return N;  // forward / input gradient: the whole batch in one tile
-}
-
 cudaError_t launch_gemm(int epi, const GemmMaps& m, const GemmArgs& a, int n_active, cudaStream_t s) {
   if (a.M % BM != 0) return cudaErrorInvalidValue;
-  const int bn = gemm_bn_for(epi, a.N);
+  const int bn = a.N;   // the whole batch in one tile
   return epi == kEpiFwd ? launch_epi<kEpiFwd>(bn, m, a, n_active, s) : launch_epi<kEpiDh>(bn, m, a, n_active, s);
 }
 

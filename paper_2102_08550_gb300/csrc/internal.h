@@ -131,16 +131,16 @@ int softreg_eval_blocks(int64_t n, int sms);   // loss_sum entries
 cudaError_t launch_softreg_eval(const SoftregEvalArgs& a, int blocks, cudaStream_t s);
 
 // ---------------------------------------------------------------- MLP (bf16 GEMMs)
-// Rows of one step's work: active lane i uses activation buffers of lane
+// In the step kernels below active lane i uses activation buffers of lane
 // `wid[i]` and reads parameters from slot `src[i]` (the global slot on the
 // first local step: the fused pull), writing them to slot `wid[i]`.
+
+// Staging of a round's mini-batches: fp32 rows to bf16, both layouts
 struct StageArgs {
   const float* const* x;   // [lanes] sample matrix per lane (device pointers)
   const int32_t* const* y;
   const int64_t* n;        // [lanes] rows available
   const int64_t* start;    // [lanes] first row (cursor)
-  int64_t row_add;         // added to start (step * B)
-  const int* wid;          // [n_active]
   int D, B;
   __nv_bfloat16* A0;       // [lanes][B][D]
   __nv_bfloat16* A0T;      // [lanes][D][B]
@@ -154,10 +154,10 @@ cudaError_t launch_cast_rows(const float* x, __nv_bfloat16* out, int64_t count, 
 // all mini-batches of a round: step s of worker w (s < tau[w]) at slot s * W + w
 // (grid z over a.slots when given, else over all max_tau * W slots)
 cudaError_t launch_stage_round(const StageArgs& a, const int32_t* tau, int W, int max_tau, cudaStream_t s);
-// the same with a launch priority (cudaLaunchAttributePriority)
 // the same staging from `blocks` blocks striding over the tiles (bounded footprint beside other kernels)
 cudaError_t launch_stage_round_strided(const StageArgs& a, const int32_t* tau, int W, int max_tau, int blocks,
                                        int priority, cudaStream_t s);
+// the first form with a launch priority (cudaLaunchAttributePriority)
 cudaError_t launch_stage_round_priority(const StageArgs& a, const int32_t* tau, int W, int max_tau, int priority,
                                         cudaStream_t s);
 
@@ -248,7 +248,6 @@ struct DwMaps {
 };
 // `sms`: the device's multiprocessors (one CTA each at most)
 cudaError_t launch_gemm_dw(const DwMaps& maps, DwArgs a, int sms, cudaStream_t s);
-int gemm_bn_for(int epi, int N);
 
 struct HeadArgs {
   const int* wid;

@@ -1,8 +1,9 @@
 // One worker's fp32 softmax-regression local steps without any device
-// allocation: the same round kernel as oscars_local_steps runs with its
-// global scratch (the one-worker argument tables and the per-step loss
-// partials) placed in a fixed array that the library reserves when it is
-// loaded.
+// allocation: the kernel that oscars_local_steps runs, the cluster kernel with
+// the worker's values in its arguments, or, where that kernel's exchange buffers
+// do not fit shared memory, the single-CTA kernel with its global scratch (the
+// one-worker argument tables and the per-step loss partials) in a fixed array
+// that the library reserves when it is loaded.
 //
 // Who needs this: a caller that must not allocate device memory at the point
 // of the call.  Examples: code running while a CUDA graph is being captured

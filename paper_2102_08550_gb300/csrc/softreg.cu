@@ -10,8 +10,8 @@
 // exchange data inside a round.  Two kernels: softreg_cluster_round_kernel
 // puts each worker on a cluster of 8 CTAs that split the input columns;
 // softreg_round_kernel puts each worker on one CTA (only where the cluster's
-// exchange buffers do not fit: about 400 rows and more with 17 or more
-// classes).
+// exchange buffers do not fit: from about 390 rows with 17 classes and more, 470
+// with 15; 241 us a step of 100 x 20 with 400 rows).
 //
 // Per step: logits z[b][c] = sum_k x[b][k] W[c][k] + bias[c] (warp-level dot
 // products), p = softmax(z), loss_b = logsumexp(z_b) - z_b[y_b],
@@ -263,8 +263,8 @@ __global__ void __launch_bounds__(kThreads) softreg_round_kernel(const __grid_co
 // sends dz(s + 1) only after it has received every CTA's partials(s + 1),
 // which a CTA sends after its last read of dz(s).
 //
-// What bounds it: the latency of the chain (issue slots 39% busy, 0.3% of
-// DRAM).  Eight steps of one 784 x 10 worker, batch 32: 203 us on one CTA,
+// What bounds it: the latency of the chain (784 x 10, 4 workers: issue slots 30%
+// busy, 0.3% of DRAM).  Eight steps of one 784 x 10 worker, batch 32: 203 us on one CTA,
 // 35 us here (about 3.3 us a step).  A round of 333 x 26, batch 100, 12
 // workers, with its merge and pull: 373 us with the earlier cluster kernel
 // (cluster barrier, remote reads, one-thread row loops), 128 us now.
